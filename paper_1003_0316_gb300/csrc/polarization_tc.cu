@@ -542,12 +542,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // all items), so the barrier waits of one issuing thread overlap the tensor-core work of
       // the other. Each round is one drain period: SUB chunks x 2 K steps x 3 MMAs into a
       // fresh accumulator.
-      const uint32_t mpar = uint32_t(warp - MMA_WARP);
-      if (lane == 0) {
+      // The whole warp runs the loop and one elected lane issues (tc::elect_one): against a loop
+      // under `lane == 0`, TF32x3 on one q of K = 102,400 11.68 -> 11.21 ms, BF16x3 on two q of
+      // K = 409,600 52.3 -> 51.7 ms, the quadratic form of 8 q x 16 frequencies 7.1 -> 5.9 ms. One
+      // issuer for every round, in order, was slower (13.1 and 55.3 ms): with two accumulators
+      // its waits for a drained one are no longer hidden behind the other issuer's MMAs.
+      const uint32_t mpar = tc::uniform(uint32_t(warp - MMA_WARP));
+      const uint32_t tm = tc::uniform(tmem);
+      {
         uint64_t g = 0;
         uint32_t kb = 0;              // periods issued on this warp's accumulator
-        const uint64_t desc0 = tc::smem_desc(tc::smem_u32(ring), 512, 4);
-        const uint32_t d = tmem + ACC_COL + mpar * TN;
+        const uint64_t desc0 = tc::smem_desc(tc::uniform(tc::smem_u32(ring)), 512, 4);
+        const uint32_t d = tm + ACC_COL + mpar * TN;
         bool ok = true;
         const uint64_t hp0 = hp_now();
         uint64_t hp_wb = 0, hp_wa = 0, hp_wc = 0, hp_n = 0;
@@ -570,17 +576,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint64_t gg = g + uint64_t(r);
             const int st = int(gg % NSB), slot = int(gg % NSA);
             const uint64_t t0 = hp_now();
-            if (!tc::mbar_wait(&fullB[st], uint32_t(gg / NSB) & 1, &s_abort, WAIT_LIMIT)) {
+            if (!tc::mbar_wait_warp(&fullB[st], uint32_t(gg / NSB) & 1, &s_abort, WAIT_LIMIT)) {
               ok = false;
               break;
             }
             const uint64_t t1 = hp_now();
-            if (!tc::mbar_wait(&fullA[slot], uint32_t(gg / NSA) & 1, &s_abort, WAIT_LIMIT)) {
+            if (!tc::mbar_wait_warp(&fullA[slot], uint32_t(gg / NSA) & 1, &s_abort, WAIT_LIMIT)) {
               ok = false;
               break;
             }
             const uint64_t t2 = hp_now();
-            if (pstart && !tc::mbar_wait(&acce_bar[mpar], (kb & 1) ^ 1, &s_abort, WAIT_LIMIT)) {
+            if (pstart && !tc::mbar_wait_warp(&acce_bar[mpar], (kb & 1) ^ 1, &s_abort, WAIT_LIMIT)) {
               ok = false;
               break;
             }
@@ -589,49 +595,52 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             hp_wc += hp_now() - t2;
             ++hp_n;
             tc::tc_fence_after();
-            const uint32_t a0 = tmem + A_COL + slot * (SUB * 32);
+            const uint32_t a0 = tm + A_COL + slot * (SUB * 32);
             // descriptor address field is (addr >> 4): advancing the address adds to the low bits
             const uint64_t dst = desc0 + uint64_t((st * STAGE_BYTES) >> 4);
+            if (tc::elect_one()) {
 #pragma unroll
-            for (int u = 0; u < SUB; ++u) {
+              for (int u = 0; u < SUB; ++u) {
 #pragma unroll
-              for (int ks = 0; ks < 2; ++ks) {
-                const uint64_t dBh = dst + uint64_t((u * CHUNK_BYTES + ks * 32) >> 4);
-                const uint64_t dBl = dst + uint64_t((u * CHUNK_BYTES + B_TILE + ks * 32) >> 4);
-                const uint32_t ah = a0 + u * 32 + ks * 8, al = a0 + u * 32 + 16 + ks * 8;
-                const uint32_t acc0 = (pstart && u == 0 && ks == 0) ? 0u : 1u;
-                if (BF16) {
-                  tc::mma_f16_ta(d, al, dBh, IDESC, acc0);
-                  tc::mma_f16_ta(d, ah, dBl, IDESC, 1u);
-                  tc::mma_f16_ta(d, ah, dBh, IDESC, 1u);
-                } else {
-                  tc::mma_tf32_ta(d, al, dBh, IDESC, acc0);
-                  tc::mma_tf32_ta(d, ah, dBl, IDESC, 1u);
-                  tc::mma_tf32_ta(d, ah, dBh, IDESC, 1u);
+                for (int ks = 0; ks < 2; ++ks) {
+                  const uint64_t dBh = dst + uint64_t((u * CHUNK_BYTES + ks * 32) >> 4);
+                  const uint64_t dBl = dst + uint64_t((u * CHUNK_BYTES + B_TILE + ks * 32) >> 4);
+                  const uint32_t ah = a0 + u * 32 + ks * 8, al = a0 + u * 32 + 16 + ks * 8;
+                  const uint32_t acc0 = (pstart && u == 0 && ks == 0) ? 0u : 1u;
+                  if (BF16) {
+                    tc::mma_f16_ta(d, al, dBh, IDESC, acc0);
+                    tc::mma_f16_ta(d, ah, dBl, IDESC, 1u);
+                    tc::mma_f16_ta(d, ah, dBh, IDESC, 1u);
+                  } else {
+                    tc::mma_tf32_ta(d, al, dBh, IDESC, acc0);
+                    tc::mma_tf32_ta(d, ah, dBl, IDESC, 1u);
+                    tc::mma_tf32_ta(d, ah, dBh, IDESC, 1u);
+                  }
                 }
               }
+              tc::mma_commit(&emptyB[st]);
+              tc::mma_commit(&emptyA[slot]);
+              if (pend) tc::mma_commit(&accf_bar[mpar]);
             }
-            tc::mma_commit(&emptyB[st]);
-            tc::mma_commit(&emptyA[slot]);
-            if (pend) {
-              tc::mma_commit(&accf_bar[mpar]);
-              ++kb;
-            }
+            __syncwarp();
+            if (pend) ++kb;
           }
           g += uint64_t(nr);
         }
-        if (!ok && !s_abort) {
+        if (lane == 0 && !ok && !s_abort) {
           s_abort = 1;
           raise_status(status, ST_ETIMEOUT);
         }
-        if (kWaitProfile) {
+        if (kWaitProfile && lane == 0) {
           hp_flush(HP_MMA_TOTAL, hp_now() - hp0);
           hp_flush(HP_MMA_WAIT_B, hp_wb);
           hp_flush(HP_MMA_WAIT_A, hp_wa);
           hp_flush(HP_MMA_WAIT_ACC, hp_wc);
           hp_flush(HP_MMA_ROUNDS, hp_n);
         }
-        tc::mma_commit(&done_bar[mpar]);
+        // the same lane as above issued every MMA, so its commit covers them all
+        if (tc::elect_one()) tc::mma_commit(&done_bar[mpar]);
+        __syncwarp();
         int never = 0;
         tc::mbar_wait(&done_bar[mpar], 0, reinterpret_cast<volatile int*>(&never), WAIT_LIMIT);
       }

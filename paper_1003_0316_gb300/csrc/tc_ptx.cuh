@@ -72,6 +72,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The same by a whole converged warp: every lane waits, the result is warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                               uint64_t limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, limit_ns)) != 0;
+}
+
 // ------------------------------------------------------------------ packed FP32 pairs
 // Two FP32 values in one 64-bit register (low word first) and the paired sm_100-family
 // instructions on them; each lane of a pair is rounded to nearest exactly as the scalar
@@ -94,6 +100,18 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+
+// One lane of a converged warp (elect.sync). The MMA issuers run their loops with the whole warp
+// and guard only the tcgen05 instructions by it: control flow, addresses and descriptors are then
+// warp-uniform for the compiler, which keeps them in uniform registers; under a divergent
+// `lane == 0` branch every descriptor of every MMA is moved there first.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// a value the whole warp holds, made warp-uniform for the compiler
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // ------------------------------------------------------------------ proxies
 __device__ __forceinline__ void fence_async_smem() {
@@ -207,6 +225,18 @@ __device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uin
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
       "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+// 32 lanes x 8 columns as packed pairs of 32-bit values (tcgen05.ld and its wait).
+__device__ __forceinline__ void tmem_ld8p(uint32_t taddr, uint64_t (&v)[4]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = f2_pack(r[2 * i], r[2 * i + 1]);
 }
 
 // 32 lanes x 16 columns load / 32 lanes x 8 columns store of 32-bit values.
