@@ -1,0 +1,1082 @@
+// FP64 products on the tensor cores: the polarization (a2) and the pair coefficients (a5) of the
+// FP64 precision, as error-free sliced products (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms
+// 59, 2012).
+//
+// GB300 executes FP64 multiply-adds at 1/64 of its FP32 rate (1.17 TFLOP/s measured), so the
+// plain FP64 kernels are bound by that pipe whatever their data movement. Here every FP64
+// operand x of a column (of A or B) and K range (superblock) with |x| < 2^E becomes a 56-bit
+// fixed-point integer cut into seven signed 8-bit digits, x = 2^(E-7) sum_i d_i 256^(1-i), each
+// digit exact in BF16. A product x y is the sum of the 28 digit products with i + j <= 8 (what is
+// left out is near 2^-56 of the largest product of the range); products of equal i + j = g form
+// one group:
+//   g = 2 .. 5 (g - 1 digit pairs): integer multiples of 256^(2-g), summed exactly by the FP32
+//     accumulators of the tensor core while pairs x K x 2^14 <= 2^24: 32, 16, 8 and 8 stages of
+//     K = 32 between drains (g = 5 is drained every 2, see below);
+//   g = 6, 7, 8 (18 pairs, "low") together in one accumulator, 2^-32 below the leading group: their
+//     truncating FP32 chain stays near 2^-50 of the result, where FP64 sums round as well.
+// The epilogue keeps three FP32 sums per element, s (groups 2-4), c (exact rounding errors of s,
+// and group 5) and d (exact rounding errors of c, and the low groups), by two-sums, so nothing
+// above 2^-24 of the low groups is lost; a superblock's result (s + c) + d goes to FP64 with the
+// power of two of its row and column exponents.
+//
+// Measured: one q of K = 102,400, N_b = 600, 2 frequencies 314 ms (FP64 kernel, 0.94 TFLOP/s) ->
+// 7.2 ms (41 TFLOP/s FP64-equivalent): k_oz_gemm 5.8 ms, slices 1.05, scales 0.25; relative error of
+// P against 64-bit sums 1.1e-15 -> 5e-16. K = 896, N_b = 64, 8 frequencies 3.7 -> 0.14 ms. The MMAs
+// take about 85 cycles instead of 64 (both operands from shared memory) and set the pace.
+//
+// What an input may contain: the scale kernels see every operand first. A non-finite value, one
+// outside [2^-100, 2^100], or a column whose largest entry exceeds 1024 times its mean magnitude
+// (where fixed-point slices would lose what FP64 keeps) sets a device flag: the sliced kernels
+// then return at once and the FP64 kernel, launched behind them and otherwise empty, does the work.
+//
+// Layout and roles of k_oz_gemm (384 threads, one persistent CTA per SM): 128 x 128 tiles; per stage
+// (K = 32) 7 slices of A and of B, pre-split in global memory as 8 KB K-major, 64-byte-swizzled
+// tiles, copied by bulk async copies into two shared-memory stages of 112 KB, each in two parts
+// (slices 1-4 and 5-7). One warp issues the MMAs (both operands from shared memory). TMEM holds four
+// accumulators (512 columns): C4, C3, C2 for the groups 4, 3, 2 and D, which alternates between
+// the low groups and group 5 so that each is drained while C's MMAs run:
+//   even stage: g4; low, drain; g3, g2; g5
+//   odd stage:  g5 (continuing), drain; g4, g3, g2 (drains due every 8 stages); low, drain
+// (low starts afresh in every stage, its smallest products first: continuing it over a second
+// stage adds 26 truncating MMAs to a large accumulator and cost 3x the error of P)
+// Eight epilogue warps drain (two per lane quadrant, 64 columns each).
+#include <algorithm>
+#include <vector>
+
+#include "gw_internal.cuh"
+#include "fp64_tc.cuh"
+#include "tc_ptx.cuh"
+
+namespace gw {
+namespace {
+
+constexpr int OT = 128;                     // tile edge
+constexpr int OKS = 32;                     // K per stage
+constexpr int OSL = 7;                      // digit slices
+constexpr int SLB = OT * 64;                // one slice of one operand and stage: 8 KB
+constexpr int NHI = 4;                      // slices 1-4: the stage's first part
+constexpr int HIB = NHI * SLB, LOB = (OSL - NHI) * SLB;   // bytes of the parts, per operand
+constexpr int OBLK = HIB + LOB;             // one operand's stage
+constexpr int OSTAGE = 2 * OBLK;            // A 1-4, B 1-4, A 5-7, B 5-7
+constexpr int ONST = 2;                     // stages in shared memory
+constexpr int SBMAX = 256;                  // stages per superblock at most (K = 8192)
+constexpr int OTHREADS = 384;
+constexpr int EPI_WARPS = 8;
+constexpr int REG_E = 232, REG_P = 40;      // 256 x 232 + 128 x 40 = 384 x 168
+static_assert(256 * REG_E + 128 * REG_P == OTHREADS * 168, "register split");
+constexpr uint64_t OWAIT = 2000000000ull;   // ns per bounded wait
+constexpr int CHROWS = 64;                  // rows per scale chunk (superblocks are multiples)
+constexpr float RATIO_MAX = 1024.0f;        // largest entry against the mean magnitude of a column
+
+__device__ __forceinline__ uint32_t swz64(int n, int kc) {
+  return uint32_t((n >> 3) * 512 + (n & 7) * 64 + ((kc ^ ((n & 7) >> 1)) << 4));
+}
+
+// One problem: a q point's polarization over a range of rows and frequencies, or (QF) the pair
+// coefficients of a range of pairs and frequencies.
+struct OzProb {
+  // inputs
+  const double2* M;         // polarization: the pass's first row
+  const double* delta;      // ... of the whole q (Kall entries), with dbar and f or NULL
+  const double* dbar;
+  const double* f;
+  double* w;                // s_tj [nw][Kall]; wp: of the pass's first row and frequency
+  const double* wp;
+  const double* x;          // QF: rows of the real operand [nrow][ncol]
+  int* flag;                // set: the FP64 kernel does this problem
+  // workspace
+  float2* part;             // scale partials
+  int* EA;                  // exponents [operand block][superblock][128]
+  int* EB;
+  char* A;                  // slices: [f (polarization)][block][stage][56 KB]
+  char* B;                  // [f (QF)][block][stage][56 KB]
+  double* G;                // polarization: [split][f][C, S][nbp][nbp], transposed tiles
+  double* cpart;            // QF: [f][2 nbj][nrow]
+  double2* P;               // polarization: the pass's first frequency
+  int64_t Kall, K;          // rows of the q, rows of the pass
+  int64_t nrow, ncol;       // QF
+  int nb, nf;
+  int nst, nsb, sbst;       // stages, superblocks, stages per superblock
+  int sps, splits;          // superblocks per split, splits
+  int nbi, nbj;             // QF: row and column blocks; polarization: nbj = ceil(N_b / 128)
+  int ntile;
+};
+constexpr int OZQ = 16;     // problems per launch
+struct OzBatch {
+  OzProb q[OZQ];
+  int64_t item0[OZQ + 1];
+  float* s;                 // per CTA: the sums s of its tile, [column][row]
+  int nq;
+  int add;                  // G += instead of G =
+};
+
+// polarization: tiles of C = Mr^T D Mi (all) and S = (Mr+Mi)^T D (Mr+Mi) (upper), the layout of the
+// split-precision polarization; quadratic form: every (row block, column block)
+template <bool QF>
+__device__ __forceinline__ const OzProb& oz_item(const OzBatch& batch, int64_t item, int& f, int& sp,
+                                                 int& bi, int& bj, int& kind) {
+  int q = 0;
+  while (q + 1 < batch.nq && item >= batch.item0[q + 1]) ++q;
+  const OzProb& L = batch.q[q];
+  item -= batch.item0[q];
+  int u = int(item % L.ntile);
+  item /= L.ntile;
+  f = int(item % L.nf);
+  sp = int(item / L.nf);
+  if (QF) {
+    bi = u % L.nbi;
+    bj = u / L.nbi;
+    kind = 2;
+    return L;
+  }
+  const int nbb = L.nbj;
+  if (u < nbb * nbb) {
+    bi = u % nbb;
+    bj = u / nbb;
+    kind = 0;
+    return L;
+  }
+  u -= nbb * nbb;
+  bj = 0;
+  while (u > bj) {
+    u -= bj + 1;
+    ++bj;
+  }
+  bi = u + nbb;
+  bj += nbb;
+  kind = 1;
+  return L;
+}
+
+__device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                        unsigned* status) {
+  int ok = 0;
+  if ((threadIdx.x & 31) == 0) {
+    ok = (!*abort && tc::mbar_wait(bar, parity, abort, OWAIT)) ? 1 : 0;
+    if (!ok && !*abort) {
+      *abort = 1;
+      raise_status(status, ST_ETIMEOUT);
+    }
+  }
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// FP64 of a register sum, and a global load, in volatile asm: they stay in program order, since
+// 64 elements' conversions and loads moved up front would not fit beside the sums
+__device__ __forceinline__ double to_f64(float v) {
+  double r;
+  asm volatile("cvt.f64.f32 %0, %1;" : "=d"(r) : "f"(v));
+  return r;
+}
+// (s + c) + d of element i (c, d packed)
+__device__ __forceinline__ double sum_f64(float s, const uint64_t (&c)[32], const uint64_t (&d)[32],
+                                          int i) {
+  auto part = [i](uint64_t x) {
+    float l, h;
+    tc::f2_unpack(x, l, h);
+    return to_f64(i & 1 ? h : l);
+  };
+  return (to_f64(s) + part(c[i / 2])) + part(d[i / 2]);
+}
+__device__ __forceinline__ float ld_f32(const float* p) {
+  float r;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p) : "memory");
+  return r;
+}
+__device__ __forceinline__ double ld_f64(const double* p) {
+  double r;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(r) : "l"(p) : "memory");
+  return r;
+}
+__device__ __forceinline__ int4 ld_exp4(const int* p) {
+  int4 r;
+  asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p));
+  return r;
+}
+
+template <bool QF>
+__global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm(const __grid_constant__ OzBatch batch, unsigned* status) {
+  constexpr uint32_t IDESC = tc::instr_desc(1u, OT, OT);
+  extern __shared__ __align__(1024) char dsmem[];
+  char* ring = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
+  // full/empty per stage part (0: slices 1-4, 1: slices 5-7); D and C: the accumulators
+  __shared__ __align__(8) uint64_t full[ONST][2], empty[ONST][2], fullD, emptyD, fullC, emptyC, done;
+  __shared__ uint32_t s_tmem;
+  __shared__ volatile int s_abort;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < ONST; ++i)
+      for (int h = 0; h < 2; ++h) {
+        tc::mbar_init(&full[i][h], 1);
+        tc::mbar_init(&empty[i][h], 1);
+      }
+    tc::mbar_init(&fullD, 1);
+    tc::mbar_init(&emptyD, EPI_WARPS);
+    tc::mbar_init(&fullC, 1);
+    tc::mbar_init(&emptyC, EPI_WARPS);
+    tc::mbar_init(&done, 1);
+    s_abort = 0;
+    tc::mbar_fence_init();
+  }
+  if (warp == 0) {
+    tc::tmem_alloc(&s_tmem, 512);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tmem = s_tmem;               // columns: D, C4, C3, C2 (128 each)
+  const int64_t nitems = batch.item0[batch.nq];
+
+  // the stage range of an item (the quadratic form's column block bj needs K < 128 (bj + 1))
+  auto range = [&](const OzProb& L, int sp, int bj, int& st0, int& st1) {
+    st0 = sp * L.sps * L.sbst;
+    st1 = min(L.nst, st0 + L.sps * L.sbst);
+    if (QF) st1 = min(st1, (bj + 1) * (OT / OKS));
+  };
+
+  if (warp < EPI_WARPS) {
+    tc::setmaxnreg_inc<REG_E>();
+    const int qd = warp & 3, c0 = (warp >> 2) * 64;
+    const int r = qd * 32 + lane;
+    const uint32_t base = tmem + (uint32_t(qd * 32) << 16) + c0;
+    uint64_t c[32], d[32];                    // packed FP32 pairs: columns 2 i, 2 i + 1
+    // s is touched every 8 stages only: in L2 (64 KB per CTA, this thread's own entries), since
+    // three sums of 64 columns leave too few registers for the two-sums (they spilled in
+    // every drain)
+    float* sp_s = batch.s + (size_t(blockIdx.x) * OT + c0) * OT + r;
+    uint32_t gD = 0, gC = 0;                  // phases of fullD, fullC
+    bool stop = false;
+    // Paired FP32 adds in volatile asm, element by element: the compiler would otherwise move the
+    // next chunks' work up and spill. add: x += v; two_sum: x + v = x' + e exactly (Knuth).
+    auto add = [](uint64_t& x, uint64_t v) {
+      asm volatile("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(v));
+    };
+    auto two_sum = [](uint64_t& x, uint64_t v) {
+      uint64_t e;
+      asm volatile(
+          "{\n.reg .b64 t, b, p, q;\nadd.rn.f32x2 t, %0, %2;\nsub.rn.f32x2 b, t, %0;\n"
+          "sub.rn.f32x2 p, t, b;\nsub.rn.f32x2 p, %0, p;\nsub.rn.f32x2 q, %2, b;\n"
+          "add.rn.f32x2 %1, p, q;\nmov.b64 %0, t;\n}\n"
+          : "+l"(x), "=l"(e)
+          : "l"(v));
+      return e;
+    };
+    auto drain_c = [&](uint32_t col, bool fresh) {   // groups 2-4: s, then its error into c, then d
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        float sv[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sv[i] = fresh ? 0.0f : ld_f32(sp_s + (h * 16 + i) * OT);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          uint64_t v[4];
+          tc::tmem_ld8p(base + col + h * 16 + g * 8, v);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int e2 = g * 8 + 2 * i, k2 = h * 8 + g * 4 + i;
+            uint64_t x = tc::f2_pack(__float_as_uint(sv[e2]), __float_as_uint(sv[e2 + 1]));
+            const uint64_t e = two_sum(x, v[i]);
+            tc::f2_unpack(x, sv[e2], sv[e2 + 1]);
+            add(d[k2], two_sum(c[k2], e));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sp_s[(h * 16 + i) * OT] = sv[i];
+      }
+    };
+    // D: group 5 into c, the low groups into d; false after an expired wait
+    auto drain_d = [&](bool g5) {
+      if (!oz_wait(&fullD, gD & 1, &s_abort, status)) return false;
+      ++gD;
+      tc::tc_fence_after();
+      if (g5) {
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          uint64_t v[4];
+          tc::tmem_ld8p(base + h * 8, v);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) add(d[h * 4 + i], two_sum(c[h * 4 + i], v[i]));
+        }
+      } else {
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          uint64_t v[4];
+          tc::tmem_ld8p(base + h * 8, v);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) add(d[h * 4 + i], v[i]);
+        }
+      }
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&emptyD);
+      return true;
+    };
+    for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x) {
+      int f, sp, bi, bj, kind;
+      const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
+      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
+      int st0, st1;
+      range(L, sp, bj, st0, st1);
+      double qsum = 0.0;
+      bool first = true;
+      for (int sb0 = st0; sb0 < st1 && !stop; sb0 += L.sbst) {
+        const int n = min(L.sbst, st1 - sb0);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) c[i] = d[i] = 0;
+        bool fresh = true;                    // s is zero
+        for (int k = 0; k < n; ++k) {
+          const bool last = k == n - 1;
+          if (!drain_d(k & 1)) {               // even: low, odd: group 5
+            stop = true;
+            break;
+          }
+          if ((k & 7) == 7 || last) {
+            if (!oz_wait(&fullC, gC & 1, &s_abort, status)) {
+              stop = true;
+              break;
+            }
+            ++gC;
+            tc::tc_fence_after();
+            const int ng = last || (k & 31) == 31 ? 3 : (k & 15) == 15 ? 2 : 1;
+#pragma unroll 1
+            for (int gi = 1; gi <= ng; ++gi) {
+              drain_c(gi * OT, fresh);
+              fresh = false;
+            }
+            tc::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&emptyC);
+          }
+          // odd: low; even: group 5, which the next odd stage continues
+          if (((k & 1) || last) && !drain_d(!(k & 1))) {
+            stop = true;
+            break;
+          }
+        }
+        if (stop) break;
+        // the superblock in FP64: ((s + c) + d) 2^(EA + EB - 14)
+        const int sb = sb0 / L.sbst;
+        const int* eb = L.EB + (size_t(QF ? f * L.nbj + bj : bj) * L.nsb + sb) * OT + c0;
+        const int ea =
+            L.EA[(size_t(QF ? bi : f * 2 * L.nbj + bi) * L.nsb + sb) * OT + r] - 14 + 1023;
+        if (QF) {
+          const int64_t p = int64_t(bi) * OT + r;
+          const int64_t col = int64_t(bj) * OT + c0;
+          if (p < L.nrow) {
+            const double* xr = L.x + p * L.ncol + col;
+#pragma unroll
+            for (int g4 = 0; g4 < 16; ++g4) {
+              const int4 e4 = ld_exp4(eb + 4 * g4);
+              const int e[4] = {e4.x, e4.y, e4.z, e4.w};
+              double x[4];
+              float sv[4];
+#pragma unroll
+              for (int t = 0; t < 4; ++t) sv[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
+#pragma unroll
+              for (int t = 0; t < 4; ++t) x[t] = col + 4 * g4 + t < L.ncol ? ld_f64(xr + 4 * g4 + t) : 0.0;
+#pragma unroll
+              for (int t = 0; t < 4; ++t) {
+                const double v = sum_f64(sv[t], c, d, 4 * g4 + t);
+                qsum = fma(v * __hiloint2double((ea + e[t]) << 20, 0), x[t], qsum);
+              }
+            }
+          }
+        } else {
+          const size_t nbp = size_t(L.nbj) * OT;
+          const int a = (kind ? bi - L.nbj : bi) * OT + r;
+          const int b0 = (kind ? bj - L.nbj : bj) * OT + c0;
+          double* g = L.G + ((size_t(sp) * L.nf + f) * 2 + kind) * nbp * nbp + size_t(b0) * nbp + a;
+          const bool add = batch.add || !first;
+#pragma unroll
+          for (int g4 = 0; g4 < 16; ++g4) {
+            const int4 e4 = ld_exp4(eb + 4 * g4);
+            const int e[4] = {e4.x, e4.y, e4.z, e4.w};
+            double o[4] = {0.0, 0.0, 0.0, 0.0};
+            float sv[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) sv[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
+            if (add) {
+#pragma unroll
+              for (int t = 0; t < 4; ++t) o[t] = ld_f64(g + size_t(4 * g4 + t) * nbp);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const double v = sum_f64(sv[t], c, d, 4 * g4 + t);
+              g[size_t(4 * g4 + t) * nbp] = fma(v, __hiloint2double((ea + e[t]) << 20, 0), o[t]);
+            }
+          }
+        }
+        first = false;
+      }
+      if (QF && !stop) {
+        const int64_t p = int64_t(bi) * OT + r;
+        if (p < L.nrow)
+          L.cpart[(size_t(f) * 2 * L.nbj + 2 * bj + (c0 ? 1 : 0)) * L.nrow + p] = qsum;
+      }
+    }
+  } else {
+    tc::setmaxnreg_dec<REG_P>();
+    if (warp == EPI_WARPS && lane == 0) {
+      // ---------------------------------------------- bulk copies of the slices
+      uint32_t g = 0;
+      bool ok = true;
+      for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+        int f, sp, bi, bj, kind;
+        const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
+      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
+        int st0, st1;
+        range(L, sp, bj, st0, st1);
+        const char* a = L.A + size_t(QF ? bi : f * 2 * L.nbj + bi) * L.nst * OBLK;
+        const char* b = L.B + size_t(QF ? f * L.nbj + bj : bj) * L.nst * OBLK;
+        for (int st = st0; st < st1 && ok; ++st, ++g) {
+          const int slot = g % ONST;
+          const uint32_t par = ((g / ONST) & 1) ^ 1;
+          char* dst = ring + slot * OSTAGE;
+#pragma unroll
+          for (int h = 1; h >= 0; --h) {              // slices 5-7 are free first
+            if (!tc::mbar_wait(&empty[slot][h], par, &s_abort, OWAIT)) {
+              ok = false;
+              break;
+            }
+            const int nb = h ? LOB : HIB;
+            char* to = dst + (h ? 2 * HIB : 0);
+            const size_t off = size_t(st) * OBLK + (h ? HIB : 0);
+            tc::mbar_arrive_expect_tx(&full[slot][h], 2 * nb);
+            tc::bulk_g2s(to, a + off, nb, &full[slot][h]);
+            tc::bulk_g2s(to + nb, b + off, nb, &full[slot][h]);
+          }
+        }
+      }
+      if (!ok && !s_abort) {
+        s_abort = 1;
+        raise_status(status, ST_ETIMEOUT);
+      }
+    } else if (warp == EPI_WARPS + 1) {
+      // ---------------------------------------------- MMA issue (tc::elect_one)
+      const uint32_t tm = tc::uniform(tmem);
+      uint32_t g = 0, nD = 0, nC = 0;          // stages; drains of D and C so far
+      bool ok = true;
+      const uint64_t desc0 = tc::smem_desc(tc::uniform(tc::smem_u32(ring)), 512, 4);
+      for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+        int f, sp, bi, bj, kind;
+        const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
+      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
+        int st0, st1;
+        range(L, sp, bj, st0, st1);
+        for (int sb0 = st0; sb0 < st1 && ok; sb0 += L.sbst) {
+          const int n = min(L.sbst, st1 - sb0);
+          for (int k = 0; k < n; ++k, ++g) {
+            const int slot = g % ONST;
+            const uint32_t par = (g / ONST) & 1;
+            const bool last = k == n - 1, odd = k & 1, due = (k & 7) == 7 || last;
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+              return ok = tc::mbar_wait_warp(bar, parity, &s_abort, OWAIT);
+            };
+            if (!wait(&full[slot][1], par) || !wait(&full[slot][0], par)) break;
+            tc::tc_fence_after();
+            const uint64_t sd = desc0 + uint64_t((slot * OSTAGE) >> 4);
+            // slice i (1-based) of A and of B in the stage
+            auto da = [&](int i) {
+              return sd + uint64_t((i <= NHI ? (i - 1) * SLB : 2 * HIB + (i - 1 - NHI) * SLB) >> 4);
+            };
+            auto db = [&](int i) { return da(i) + uint64_t((i <= NHI ? HIB : LOB) >> 4); };
+            auto group = [&](int gg, uint32_t dst, uint32_t acc) {
+#pragma unroll
+              for (int i = 1; i <= OSL; ++i) {
+                const int j = gg - i;
+                if (j < 1 || j > OSL) continue;
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                  tc::mma_f16(dst, da(i) + uint64_t((ks * 32) >> 4), db(j) + uint64_t((ks * 32) >> 4),
+                              IDESC, acc);
+                  acc = 1u;
+                }
+              }
+            };
+            auto low = [&]() {                          // a fresh D, the smallest products first
+              group(8, tm, 0u);
+              group(7, tm, 1u);
+              group(6, tm, 1u);
+              tc::mma_commit(&empty[slot][1]);
+              tc::mma_commit(&fullD);
+            };
+            auto g4 = [&]() { group(4, tm + OT, (k & 7) ? 1u : 0u); };
+            auto g32 = [&]() {
+              group(3, tm + 2 * OT, (k & 15) ? 1u : 0u);
+              group(2, tm + 3 * OT, (k & 31) ? 1u : 0u);
+              if (due) tc::mma_commit(&fullC);
+            };
+            if (odd) {
+              if (tc::elect_one()) {
+                group(5, tm, 1u);
+                tc::mma_commit(&fullD);
+              }
+              __syncwarp();
+              ++nD;
+              if (!wait(&emptyC, (nC & 1) ^ 1)) break;
+              tc::tc_fence_after();
+              if (tc::elect_one()) {
+                g4();
+                g32();
+              }
+              __syncwarp();
+              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
+              tc::tc_fence_after();
+              if (tc::elect_one()) {
+                low();
+                tc::mma_commit(&empty[slot][0]);
+              }
+              __syncwarp();
+              ++nD;
+            } else {
+              if (!wait(&emptyC, (nC & 1) ^ 1)) break;
+              tc::tc_fence_after();
+              if (tc::elect_one()) g4();
+              __syncwarp();
+              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
+              tc::tc_fence_after();
+              if (tc::elect_one()) {
+                low();
+                g32();
+              }
+              __syncwarp();
+              ++nD;
+              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
+              tc::tc_fence_after();
+              if (tc::elect_one()) {
+                group(5, tm, 0u);
+                tc::mma_commit(&empty[slot][0]);
+                if (last) tc::mma_commit(&fullD);
+              }
+              __syncwarp();
+              if (last) ++nD;
+            }
+            if (due) ++nC;
+          }
+        }
+      }
+      if (lane == 0 && !ok && !s_abort) {
+        s_abort = 1;
+        raise_status(status, ST_ETIMEOUT);
+      }
+      if (tc::elect_one()) tc::mma_commit(&done);
+      __syncwarp();
+      int never = 0;
+      tc::mbar_wait(&done, 0, reinterpret_cast<volatile int*>(&never), OWAIT);
+    }
+    __syncwarp();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
+// ------------------------------------------------------------------ digits
+// Digits of 8 consecutive K values with exponent E (|v| < 0.996 2^E): for every slice 8 BF16
+// values d_i 256^(1-i), packed in K order. The fixed-point value X = round(v 2^(55-E)) plus the
+// bias 128 sum 256^k has the digits (plus 128) as its bytes; a byte put into the low mantissa bits
+// of a float of the slice's exponent, minus that float with the byte at 128, is the digit's value.
+// Integer arithmetic throughout: the FP64 pipe would take as long as the products.
+__device__ __forceinline__ void digits8(const double (&v)[8], int E, uint32_t (&w)[OSL][4]) {
+  constexpr unsigned long long BIAS = 128ull * (((1ull << 56) - 1) / 255);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    float f[2][OSL];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned long long b = __double_as_longlong(v[2 * p + h]);
+      const int ex = int(b >> 52) & 0x7ff;
+      const int sh = min(E + 1022 - ex, 60);
+      unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 2;
+      // sh >= 0 by the choice of E; below the last digit (and for zero): zero
+      m = ex == 0 ? 0ull : (m + ((1ull << sh) >> 1)) >> sh;
+      const unsigned long long y = (b >> 63) ? BIAS - m : BIAS + m;
+      const uint32_t lo = uint32_t(y), hi = uint32_t(y >> 32);
+#pragma unroll
+      for (int i = 0; i < OSL; ++i) {
+        const uint32_t mg = 0x4B000000u - (uint32_t(8 * i) << 23);
+        // byte 6 - i of y in place of mg's lowest byte
+        const uint32_t bits = i < 3 ? __byte_perm(hi, mg, 0x7650u | uint32_t(2 - i))
+                                    : __byte_perm(lo, mg, 0x7650u | uint32_t(6 - i));
+        f[h][i] = __fsub_rn(__uint_as_float(bits), __uint_as_float(mg | 128u));
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < OSL; ++i) w[i][p] = tc::cvt_bf16x2(f[0][i], f[1][i]);
+  }
+}
+
+// 16 bytes of every slice of row n at K chunk kc of a stage's block
+__device__ __forceinline__ void store_digits(char* blk, int n, int kc, const uint32_t (&w)[OSL][4]) {
+  const uint32_t off = swz64(n, kc);
+#pragma unroll
+  for (int i = 0; i < OSL; ++i)
+    *reinterpret_cast<uint4*>(blk + i * SLB + off) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+}
+
+// the exponent of a range: E with (largest magnitude) < 0.996 2^E, or a raised flag
+__device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool ratio, int* flag) {
+  if (!(sum <= 3.0e38f) || !(mx < 1.2676506e30f)) {        // not finite, or from 2^100 on
+    *flag = 1;
+    return 0;
+  }
+  if (mx == 0.0f) return 0;
+  if (mx < 7.8886091e-31f || (ratio && mx * n > RATIO_MAX * sum)) {
+    *flag = 1;
+    return 0;
+  }
+  return ilogbf(mx * 1.005f) + 1;       // 1.005 mx < 2^E
+}
+
+// s_tj = prefactor f_t 2 Delta / (Delta^2 + w^2) (minus the same at Delta_bar with the extrapolar
+// correction), FP64, [nw][K]
+__global__ void k_oz_weights(const __grid_constant__ OzBatch batch, double pref, int nw, OmegaArr om,
+                             unsigned* status) {
+  const OzProb& L = batch.q[blockIdx.y];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *L.flag = 0;
+  for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < L.Kall;
+       t += int64_t(gridDim.x) * blockDim.x) {
+    const double d = L.delta[t];
+    if (!(d > 0.0)) raise_status(status, ST_EINVAL);
+    const double p2 = 2.0 * pref * (L.f ? L.f[t] : 1.0);
+    const double db = L.dbar ? L.dbar[t] : 0.0;
+    if (L.dbar && !(db > 0.0)) raise_status(status, ST_EINVAL);
+    for (int j = 0; j < nw; ++j) {
+      const double w2 = om.v[j] * om.v[j];
+      double s = p2 * d / (d * d + w2);
+      if (L.dbar) s -= p2 * db / (db * db + w2);
+      L.w[size_t(j) * L.Kall + t] = s;
+    }
+  }
+}
+
+// |v| rounded up to FP32 by integer arithmetic (the FP64 pipe's conversions cost three times the
+// reads of the scale kernel): the exponent re-biased, the top 23 mantissa bits plus one. Zero and
+// magnitudes below 2^-126 become 2^-126, those above the FP32 range (and non-finite ones) infinite.
+__device__ __forceinline__ float abs_up(double v) {
+  const unsigned long long b = __double_as_longlong(v) & 0x7fffffffffffffffull;
+  const long long f = (long long)(b >> 29) - (896ll << 23) + 1;      // FP32 bits of the next value up
+  const int bits = f < 0x00800000ll ? 0x00800000 : f > 0x7f800000ll ? 0x7f800000 : int(f);
+  return __int_as_float(b ? bits : 0);
+}
+
+// Bounds (within 2^-21) of the largest magnitude and of the magnitude sum of every column over
+// chunks of 64 rows, in FP32: operand types 0 Mi, 1 Mr + Mi (B), 2 + 2 f and 3 + 2 f: s_f Mr,
+// s_f (Mr + Mi) (A). Thread = column; grid (column blocks, chunks). Bound by the read of M.
+__global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch batch) {
+  __shared__ float sw[4][CHROWS];
+  const OzProb& L = batch.q[blockIdx.z];
+  const double2* __restrict__ M = L.M;
+  const double* __restrict__ w = L.wp;
+  const int64_t K = L.K, wld = L.Kall;
+  const int nb = L.nb, nf = L.nf, ncolp = L.nbj * OT;
+  if (int(blockIdx.x) >= L.nbj || int64_t(blockIdx.y) * CHROWS >= K) return;   // whole CTA
+  const int col = blockIdx.x * OT + threadIdx.x;
+  const int64_t t0 = int64_t(blockIdx.y) * CHROWS;
+  const int n = int(K - t0 < CHROWS ? K - t0 : CHROWS);
+  const int ntype = 2 + 2 * nf;
+  float2* out = L.part + size_t(blockIdx.y) * ntype * ncolp + col;
+  for (int f0 = 0; f0 < nf; f0 += 4) {
+    const int nj = min(4, nf - f0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 4 * CHROWS; e += OT) {
+      const int j = e / CHROWS, t = e % CHROWS;
+      sw[j][t] = j < nj && t < n ? abs_up(w[size_t(f0 + j) * wld + t0 + t]) : 0.0f;
+    }
+    __syncthreads();
+    float mi = 0.f, ms = 0.f, si = 0.f, ss = 0.f, ma[4][2] = {}, sa[4][2] = {};
+    if (col < nb) {
+#pragma unroll 8
+      for (int t = 0; t < n; ++t) {
+        const double2 x = __ldg(M + (t0 + t) * nb + col);
+        const float r = abs_up(x.x), i = abs_up(x.y);
+        // |Mr + Mi| of the rounded parts, plus their rounding
+        const bool same = (__double2hiint(x.x) ^ __double2hiint(x.y)) >= 0;
+        const float s = (same ? r + i : fabsf(r - i)) + 4.7683716e-7f * (r + i);
+        mi = fmaxf(mi, i);
+        si += i;
+        ms = fmaxf(ms, s);
+        ss += s;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float pr = r * sw[j][t], ps = s * sw[j][t];
+          ma[j][0] = fmaxf(ma[j][0], pr);
+          sa[j][0] += pr;
+          ma[j][1] = fmaxf(ma[j][1], ps);
+          sa[j][1] += ps;
+        }
+      }
+    }
+    if (f0 == 0) {
+      out[0] = make_float2(mi, si);
+      out[ncolp] = make_float2(ms, ss);
+    }
+    for (int j = 0; j < nj; ++j) {
+      out[size_t(2 + 2 * (f0 + j)) * ncolp] = make_float2(ma[j][0], sa[j][0]);
+      out[size_t(3 + 2 * (f0 + j)) * ncolp] = make_float2(ma[j][1], sa[j][1]);
+    }
+  }
+}
+
+// exponents of every (type, column, superblock) from the chunk partials
+__global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  const float2* __restrict__ part = L.part;
+  const int64_t K = L.K;
+  const int nbb = L.nbj, nf = L.nf, nsb = L.nsb, sbst = L.sbst;
+  int *EA = L.EA, *EB = L.EB;
+  const int ncolp = nbb * OT, ntype = 2 + 2 * nf;
+  const int64_t total = int64_t(ntype) * ncolp * nsb;
+  const int cps = sbst * OKS / CHROWS;              // chunks per superblock
+  const int nch = int((K + CHROWS - 1) / CHROWS);
+  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
+       e += int64_t(gridDim.x) * blockDim.x) {
+    const int col = int(e % ncolp), type = int(e / ncolp % ntype), sb = int(e / ncolp / ntype);
+    float mx = 0.f, sum = 0.f;
+    const int ch1 = min(nch, (sb + 1) * cps);
+    for (int ch = sb * cps; ch < ch1; ++ch) {
+      const float2 p = part[(size_t(ch) * ntype + type) * ncolp + col];
+      mx = fmaxf(mx, p.x);
+      sum += p.y;
+    }
+    const int64_t r0 = int64_t(sb) * sbst * OKS;
+    const float rows = float(min(int64_t(sbst) * OKS, K - r0));
+    const int E = range_exponent(mx, sum, rows, true, L.flag);
+    const int cb = col / OT, n = col % OT;
+    if (type < 2)
+      EB[(size_t(type * nbb + cb) * nsb + sb) * OT + n] = E;
+    else
+      EA[(size_t((type - 2) / 2 * 2 * nbb + (type & 1) * nbb + cb) * nsb + sb) * OT + n] = E;
+  }
+}
+
+// The digit slices of one stage (32 rows) and 32 basis functions: B (Mi, Mr + Mi) and, per
+// frequency, A (s Mr, s (Mr + Mi)). Four lanes per basis function, 8 rows each: a warp reads 128
+// contiguous bytes per row and writes 512 per slice. (One lane per basis function wrote half
+// sectors: 3.46 ms for one q of K = 102,400, N_b = 600, 2 frequencies.)
+__global__ void __launch_bounds__(OT) k_oz_slice(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.z];
+  const int nst = L.nst, nsb = L.nsb, sbst = L.sbst, nbb = L.nbj, nb = L.nb, nf = L.nf;
+  if (int(blockIdx.x) >= nst || int(blockIdx.y) >= 4 * nbb || __ldg(L.flag)) return;
+  const double2* __restrict__ M = L.M;
+  const double* __restrict__ w = L.wp;
+  const int64_t K = L.K, wld = L.Kall;
+  const int* __restrict__ EA = L.EA;
+  const int* __restrict__ EB = L.EB;
+  char* __restrict__ A = L.A;
+  char* __restrict__ B = L.B;
+  const int cb = blockIdx.y >> 2, st = blockIdx.x, kc = threadIdx.x & 3;
+  const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
+  const int col = cb * OT + n, sb = st / sbst;
+  const size_t e0 = size_t(sb) * OT + n, eld = size_t(nsb) * OT;
+  const int64_t t0 = int64_t(st) * OKS + kc * 8;
+  double xr[8], xi[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const double2 x = t0 + k < K && col < nb ? __ldg(M + (t0 + k) * nb + col) : make_double2(0., 0.);
+    xr[k] = x.x;
+    xi[k] = x.y;
+  }
+  uint32_t dg[OSL][4];
+  digits8(xi, EB[cb * eld + e0], dg);
+  store_digits(B + (size_t(cb) * nst + st) * OBLK, n, kc, dg);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) xi[k] = xr[k] + xi[k];
+  digits8(xi, EB[(nbb + cb) * eld + e0], dg);
+  store_digits(B + (size_t(nbb + cb) * nst + st) * OBLK, n, kc, dg);
+  for (int f = 0; f < nf; ++f) {
+    double y[8], wk[8];
+    const size_t blk = size_t(f) * 2 * nbb + cb;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      wk[k] = t0 + k < K ? __ldg(w + size_t(f) * wld + t0 + k) : 0.0;
+      y[k] = xr[k] * wk[k];
+    }
+    digits8(y, EA[blk * eld + e0], dg);
+    store_digits(A + (blk * nst + st) * OBLK, n, kc, dg);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) y[k] = xi[k] * wk[k];
+    digits8(y, EA[(blk + nbb) * eld + e0], dg);
+    store_digits(A + ((blk + nbb) * nst + st) * OBLK, n, kc, dg);
+  }
+}
+
+// P (or P +=) from the tiles of C and S summed over the splits in order:
+// P_ab = -S_ab + C_ab + C_ba + i (C_ab - C_ba), Hermitian exactly (S from its upper element)
+__global__ void k_oz_combine(const __grid_constant__ OzBatch batch, int accumulate) {
+  const OzProb& L = batch.q[blockIdx.y];
+  if (__ldg(L.flag)) return;
+  double2* __restrict__ P = L.P;
+  const double* __restrict__ G = L.G;
+  const int nb = L.nb, nbp = L.nbj * OT, nf = L.nf, splits = L.splits;
+  const int64_t n2 = int64_t(nb) * nb, total = n2 * nf;
+  const size_t p2 = size_t(nbp) * nbp;
+  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
+       e += int64_t(gridDim.x) * blockDim.x) {
+    const int f = int(e / n2);
+    const int64_t rem = e % n2;
+    const int a = int(rem / nb), b = int(rem % nb);
+    const size_t ab = size_t(b) * nbp + a, ba = size_t(a) * nbp + b;
+    double cab = 0.0, cba = 0.0, sab = 0.0;
+    for (int sp = 0; sp < splits; ++sp) {
+      const double* C = G + (size_t(sp) * nf + f) * 2 * p2;
+      cab += C[ab];
+      cba += C[ba];
+      sab += C[p2 + (a <= b ? ab : ba)];
+    }
+    double re = (cab + cba) - sab, im = cab - cba;
+    if (accumulate) {
+      const double2 o = P[e];
+      re += o.x;
+      im += o.y;
+    }
+    P[e] = make_double2(re, im);
+  }
+}
+
+size_t oz_smem() { return size_t(ONST) * OSTAGE + 1024; }
+
+template <bool QF>
+int launch_oz(const OzBatch& batch, cudaStream_t s, const DeviceCtx& ctx) {
+  const int64_t items = batch.item0[batch.nq];
+  if (items == 0) return GW_OK;
+  int rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_oz_gemm<QF>), oz_smem(), ctx.device);
+  if (rc) return rc;
+  const unsigned grid = unsigned(std::min<int64_t>(items, ctx.sm_count));
+  k_oz_gemm<QF><<<grid, OTHREADS, oz_smem(), s>>>(batch, ctx.status);
+  GW_LAUNCH_CHECK("k_oz_gemm");
+  return GW_OK;
+}
+
+// ------------------------------------------------------------------ polarization plan
+// A q is done in passes over frequency chunks (nf) and K ranges (rows): the digit slices of a pass
+// stay within DIGIT_BUDGET where a pass of one superblock and one frequency allows. q points
+// of one pass share their launches, up to OZQ of them within the budget.
+constexpr size_t DIGIT_BUDGET = size_t(6) << 30;
+
+struct OzPlan {
+  int nbb, ntile, nf, nst, sbst, nsb, sps, splits;
+  int64_t rows;                     // per pass
+  int npass, nchunk;                // K ranges and frequency chunks
+  size_t digits;
+  size_t b_w, b_part, b_ea, b_eb, b_A, b_B, b_G;
+  size_t total() const {
+    return b_w + b_part + size_t(npass) * nchunk * (b_ea + b_eb) + b_A + b_B + b_G;
+  }
+};
+
+OzPlan oz_plan(int64_t K, int nb, int nw) {
+  OzPlan p;
+  p.nbb = (nb + OT - 1) / OT;
+  p.ntile = p.nbb * p.nbb + p.nbb * (p.nbb + 1) / 2;
+  const size_t blk_row = size_t(2) * p.nbb * OT * 2 * OSL;       // digit bytes per row and operand
+  const int64_t unit = int64_t(SBMAX) * OKS;
+  const int64_t one = std::min<int64_t>(K, unit);
+  p.nf = int(std::max<int64_t>(1, std::min<int64_t>(nw, int64_t(DIGIT_BUDGET / (blk_row * one)) - 1)));
+  const int64_t fit = int64_t(DIGIT_BUDGET / (blk_row * (p.nf + 1)));
+  p.rows = std::min(K, std::max<int64_t>(1, fit / unit) * unit);
+  p.nst = int((p.rows + OKS - 1) / OKS);
+  p.npass = int((K + p.rows - 1) / p.rows);
+  p.nchunk = (nw + p.nf - 1) / p.nf;
+  p.digits = blk_row * size_t(p.nst) * OKS * (p.nf + 1);
+  return p;
+}
+
+// Splits of the pass's K and the buffer sizes, for a share of `sm` SMs: every CTA takes about the
+// same time per item, so whole waves of CTAs; at least 8 stages each, among the counts that give 3
+// to 12 waves the best filled last one.
+void oz_splits(OzPlan& p, int64_t K, int nw, int sm) {
+  const int64_t items = int64_t(p.ntile) * p.nf;
+  const int most = int(std::max<int64_t>(1, std::min<int64_t>((12 * int64_t(sm)) / items, (p.nst + 7) / 8)));
+  const int least = int(std::min<int64_t>(most, (3 * int64_t(sm) + items - 1) / items));
+  int pick = std::max(1, least);
+  double best = 0.0;
+  for (int sp = pick; sp <= most; ++sp) {
+    const int sb = std::min(SBMAX, ((p.nst + sp - 1) / sp + 7) / 8 * 8);
+    const int nsb = (p.nst + sb - 1) / sb, sps = (nsb + sp - 1) / sp;
+    const int64_t it = items * ((nsb + sps - 1) / sps);
+    const double fill = double(it) / double((it + sm - 1) / sm * sm);
+    if (fill > best + 0.02) {
+      best = fill;
+      pick = sp;
+    }
+  }
+  p.sbst = std::min(SBMAX, ((p.nst + pick - 1) / pick + 7) / 8 * 8);
+  p.nsb = (p.nst + p.sbst - 1) / p.sbst;
+  p.sps = (p.nsb + pick - 1) / pick;
+  p.splits = (p.nsb + p.sps - 1) / p.sps;
+  const int64_t nch = (p.rows + CHROWS - 1) / CHROWS;
+  p.b_w = ws_round(size_t(nw) * size_t(K) * 8);
+  p.b_part = ws_round(size_t(nch) * (2 + 2 * p.nf) * p.nbb * OT * sizeof(float2));
+  p.b_ea = ws_round(size_t(p.nf) * 2 * p.nbb * p.nsb * OT * 4);
+  p.b_eb = ws_round(size_t(2) * p.nbb * p.nsb * OT * 4);
+  p.b_A = ws_round(size_t(p.nf) * 2 * p.nbb * p.nst * OBLK);
+  p.b_B = ws_round(size_t(2) * p.nbb * p.nst * OBLK);
+  p.b_G = ws_round(size_t(p.splits) * p.nf * 2 * p.nbb * OT * p.nbb * OT * 8);
+}
+
+// plans of one group of q points
+std::vector<OzPlan> oz_plans(const std::vector<int>& qs, const int64_t* K, const int* nb, int nw, int sm) {
+  std::vector<OzPlan> p;
+  int64_t items = 0;
+  for (int q : qs) {
+    p.push_back(oz_plan(K[q], nb[q], nw));
+    items += int64_t(p.back().ntile) * p.back().nf;
+  }
+  for (size_t i = 0; i < qs.size(); ++i) {
+    const int64_t mine = int64_t(p[i].ntile) * p[i].nf;
+    oz_splits(p[i], K[qs[i]], nw, int(std::max<int64_t>(1, (sm * mine + items / 2) / items)));
+  }
+  return p;
+}
+
+size_t oz_sum_bytes(int sm) { return ws_round(size_t(sm) * OT * OT * sizeof(float)); }
+
+}  // namespace
+
+// From one stage of 32 rows on: K = 32, N_b = 8, 4 frequencies 0.08 ms against 0.14 with the FP64
+// kernel, K = 128, N_b = 24 0.11 against 0.54 (16 such q in one call 0.18 against 0.55); fewer rows
+// would be mostly padding.
+bool oz_pol_eligible(int64_t K) { return K >= OKS; }
+
+std::vector<std::vector<int>> oz_pol_groups(const std::vector<int>& qs, const int64_t* K, const int* nb,
+                                            int nw) {
+  std::vector<std::vector<int>> g;
+  size_t bytes = 0;
+  bool open = false;
+  for (int q : qs) {
+    const OzPlan p = oz_plan(K[q], nb[q], nw);
+    const bool single = p.npass * p.nchunk == 1;
+    if (!open || !single || int(g.back().size()) == OZQ || bytes + p.digits > DIGIT_BUDGET) {
+      g.push_back({});
+      bytes = 0;
+    }
+    g.back().push_back(q);
+    bytes += p.digits;
+    open = single;
+  }
+  return g;
+}
+
+size_t oz_pol_workspace(const std::vector<int>& group, const int64_t* K, const int* nb, int nw, int sm) {
+  size_t b = 256 + oz_sum_bytes(sm);
+  for (const OzPlan& p : oz_plans(group, K, nb, nw, sm)) b += p.total();
+  return b;
+}
+
+int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, const OmegaArr& om,
+           bool accumulate, void* ws, size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx,
+           PolOpts& o) {
+  const int n = int(group.size());
+  std::vector<int64_t> K;
+  std::vector<int> nb, idx;
+  for (int i = 0; i < n; ++i) {
+    K.push_back(qs[group[i]].K);
+    nb.push_back(qs[group[i]].nb);
+    idx.push_back(i);
+  }
+  const std::vector<OzPlan> plans = oz_plans(idx, K.data(), nb.data(), nw, ctx.sm_count);
+  WsCursor cur{static_cast<char*>(ws), ws_bytes, 0};
+  int* flags = static_cast<int*>(cur.take(256));
+  OzBatch b{};
+  b.nq = n;
+  b.s = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));
+  std::vector<char*> exps(n);
+  int64_t kmax = 0;
+  for (int i = 0; i < n; ++i) {
+    const OzPlan& p = plans[i];
+    const PolQ& Q = qs[group[i]];
+    OzProb& L = b.q[i];
+    L.flag = flags + i;
+    L.w = static_cast<double*>(cur.take(p.b_w));
+    L.part = static_cast<float2*>(cur.take(p.b_part));
+    exps[i] = static_cast<char*>(cur.take(size_t(p.npass) * p.nchunk * (p.b_ea + p.b_eb)));
+    L.A = static_cast<char*>(cur.take(p.b_A));
+    L.B = static_cast<char*>(cur.take(p.b_B));
+    L.G = static_cast<double*>(cur.take(p.b_G));
+    if (!flags || !b.s || !L.w || !L.part || !exps[i] || !L.A || !L.B || !L.G)
+      return set_error(GW_EWORKSPACE, "internal: FP64 slice workspace too small");
+    L.delta = Q.delta;
+    L.dbar = Q.dbar;
+    L.f = Q.f;
+    L.Kall = Q.K;
+    L.nb = Q.nb;
+    L.nbi = L.nbj = p.nbb;
+    L.ntile = p.ntile;
+    L.sbst = p.sbst;
+    L.sps = p.sps;
+    kmax = std::max(kmax, Q.K);
+  }
+  // the problems of a frequency chunk and K range (several only for a group of one q)
+  const int npass = plans[0].npass, nchunk = plans[0].nchunk;
+  auto set_pass = [&](int ch, int ps) {
+    for (int i = 0; i < n; ++i) {
+      const OzPlan& p = plans[i];
+      const PolQ& Q = qs[group[i]];
+      OzProb& L = b.q[i];
+      const int f0 = ch * p.nf;
+      const int64_t t0 = ps * p.rows;
+      L.nf = std::min(p.nf, nw - f0);
+      L.K = std::min(p.rows, Q.K - t0);
+      L.nst = int((L.K + OKS - 1) / OKS);
+      L.nsb = (L.nst + p.sbst - 1) / p.sbst;
+      L.splits = (L.nsb + p.sps - 1) / p.sps;
+      L.M = static_cast<const double2*>(Q.M) + t0 * Q.nb;
+      L.wp = L.w + size_t(f0) * Q.K + t0;
+      L.EA = reinterpret_cast<int*>(exps[i] + (size_t(ch) * npass + ps) * (p.b_ea + p.b_eb));
+      L.EB = reinterpret_cast<int*>(reinterpret_cast<char*>(L.EA) + p.b_ea);
+      L.P = reinterpret_cast<double2*>(Q.P) + size_t(f0) * Q.nb * Q.nb;
+      b.item0[i + 1] = b.item0[i] + int64_t(p.ntile) * L.nf * L.splits;
+    }
+    b.add = ps > 0;                     // the first pass has the most splits: it writes every tile
+  };
+  auto over = [&](auto get) {           // the largest of a per-problem count
+    int64_t m = 0;
+    for (int i = 0; i < n; ++i) m = std::max<int64_t>(m, get(b.q[i]));
+    return m;
+  };
+  const unsigned nq = unsigned(n);
+  const int64_t cap = int64_t(ctx.sm_count) * 8;
+  k_oz_weights<<<dim3(unsigned(std::min<int64_t>((kmax + 255) / 256, cap)), nq), 256, 0, s>>>(
+      b, pref, nw, om, ctx.status);
+  GW_LAUNCH_CHECK("k_oz_weights");
+  // the exponents of the whole call first, so that the flags are final before P is touched
+  for (int ch = 0; ch < nchunk; ++ch)
+    for (int ps = 0; ps < npass; ++ps) {
+      set_pass(ch, ps);
+      const unsigned bl = unsigned(over([](const OzProb& L) { return int64_t(L.nbj); }));
+      k_oz_scale<<<dim3(bl, unsigned(over([](const OzProb& L) { return (L.K + CHROWS - 1) / CHROWS; })), nq),
+                   OT, 0, s>>>(b);
+      GW_LAUNCH_CHECK("k_oz_scale");
+      const int64_t ne = over([](const OzProb& L) { return int64_t(2 + 2 * L.nf) * L.nbj * OT * L.nsb; });
+      k_oz_exps<<<dim3(unsigned((ne + 255) / 256), nq), 256, 0, s>>>(b);
+      GW_LAUNCH_CHECK("k_oz_exps");
+    }
+  for (int ch = 0; ch < nchunk; ++ch) {
+    for (int ps = 0; ps < npass; ++ps) {
+      set_pass(ch, ps);
+      k_oz_slice<<<dim3(unsigned(over([](const OzProb& L) { return int64_t(L.nst); })),
+                        unsigned(over([](const OzProb& L) { return int64_t(4 * L.nbj); })), nq),
+                   OT, 0, s>>>(b);
+      GW_LAUNCH_CHECK("k_oz_slice");
+      int rc = record_herk_event(o, o.launches, false, s);
+      if (rc) return rc;
+      if ((rc = launch_oz<false>(b, s, ctx))) return rc;
+      if ((rc = record_herk_event(o, o.launches, true, s))) return rc;
+      ++o.launches;
+    }
+    set_pass(ch, 0);                    // the splits of the first pass
+    const int64_t tot = over([](const OzProb& L) { return int64_t(L.nf) * L.nb * L.nb; });
+    k_oz_combine<<<dim3(unsigned(std::min<int64_t>((tot + 255) / 256, cap)), nq), 256, 0, s>>>(
+        b, accumulate ? 1 : 0);
+    GW_LAUNCH_CHECK("k_oz_combine");
+  }
+  return GW_OK;
+}
+
+}  // namespace gw

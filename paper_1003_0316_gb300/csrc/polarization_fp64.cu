@@ -1,7 +1,8 @@
 // a1 transition weights and the FP64 path of a2, the polarization
 // P_IJ(q, i w_j) = sum_t w_tj M_tI conj(M_tJ)  (Eq. polar_MB at w = i omega).
 //
-// FP64 path: one CTA per (q, upper 64x64 tile, frequency, K-split). Each CTA
+// FP64 kernel (q points of fewer than 32 rows, and those whose values fall outside the range of the
+// digit slices of fp64_tc.cu): one CTA per (q, upper 64x64 tile, frequency, K-split). Each CTA
 // streams its slice of transitions through shared memory in chunks of 8 rows,
 // scales the I-side rows by w_tj (computed on the fly from Delta_t), and
 // accumulates 4x4 complex outputs per thread with DFMA. Partial tiles go to the
@@ -11,6 +12,7 @@
 #include <algorithm>
 
 #include "gw_internal.cuh"
+#include "fp64_tc.cuh"
 
 namespace gw {
 
@@ -104,10 +106,12 @@ __device__ __forceinline__ void tile_of(int u, int T, int* ti, int* tj) {
 }
 
 __global__ void __launch_bounds__(256) k_herk_fp64(PolLaunch L, double pref, OmegaArr om,
-                                                  double2* __restrict__ part, unsigned* status) {
+                                                  double2* __restrict__ part, unsigned* status,
+                                                  const int* __restrict__ only_if) {
   int64_t item = blockIdx.x;
   int q = 0;
   while (q + 1 < L.nq && item >= L.item0[q + 1]) ++q;
+  if (only_if && !only_if[q]) return;         // whole CTA: the sliced path has this q's result
   int64_t local = item - L.item0[q];
   const int S = L.splits[q];
   const int T = L.tside[q];
@@ -203,7 +207,8 @@ __global__ void __launch_bounds__(256) k_herk_fp64(PolLaunch L, double pref, Ome
 
 // Sum the K-splits of one (q, j, tile) and write the tile and its mirror.
 __global__ void __launch_bounds__(256) k_herk_reduce(PolLaunch L, const double2* __restrict__ part,
-                                                     bool accumulate) {
+                                                     bool accumulate,
+                                                     const int* __restrict__ only_if) {
   int64_t blk = blockIdx.x;  // one block per (q, tile, j)
   int q = 0;
   // item0 counts (tile, j, split); blocks count (tile, j)
@@ -213,6 +218,7 @@ __global__ void __launch_bounds__(256) k_herk_reduce(PolLaunch L, const double2*
     if (blk < acc_blocks + nblk) break;
     acc_blocks += nblk;
   }
+  if (only_if && !only_if[q]) return;
   int64_t rest = blk - acc_blocks;
   const int S = L.splits[q];
   const int nw = L.nw;
@@ -285,22 +291,53 @@ static void plan_fp64(int nq, const int64_t* K, const int* nb, int nw, int sm_co
     splits[q] = int(std::max<int64_t>(1, std::min<int64_t>(pick, std::max<int64_t>(1, K[q] / 512))));
 }
 
-size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o) {
+static size_t plain_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, int sm,
+                                   int waves) {
   std::vector<int> splits;
   std::vector<int64_t> tiles;
-  int sm = 152;
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-  cudaGetLastError();
-  plan_fp64(nq, K, nb, nw, sm, o.fp64_waves, splits, tiles);
+  plan_fp64(nq, K, nb, nw, sm, waves, splits, tiles);
   size_t ntile = 0;
   for (int q = 0; q < nq; ++q) ntile += size_t(tiles[q]) * nw * splits[q];
   return ws_round(ntile * HT * HT * sizeof(double2));
 }
 
-int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, void* ws,
-             size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx, PolOpts& o) {
+// The q points of a call in two sets: those of the sliced tensor-core path (fp64_tc.cu), group by
+// group, and the rest in one launch of the FP64 kernel. The workspace is the largest of the
+// steps; a sliced group also has room for the FP64 kernel that takes over the q points whose flag
+// is set (behind the flags' 256 bytes).
+static void split_q(int nq, const int64_t* K, std::vector<int>& oz, std::vector<int>& plain) {
+  for (int q = 0; q < nq; ++q) (oz_pol_eligible(K[q]) ? oz : plain).push_back(q);
+}
+
+size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o) {
+  int sm = 152;
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+  cudaGetLastError();
+  std::vector<int> oz, plain;
+  split_q(nq, K, oz, plain);
+  auto plain_need = [&](const std::vector<int>& qs) {
+    std::vector<int64_t> Kp;
+    std::vector<int> nbp;
+    for (int q : qs) {
+      Kp.push_back(K[q]);
+      nbp.push_back(nb[q]);
+    }
+    return plain_fp64_workspace(int(qs.size()), Kp.data(), nbp.data(), nw, sm, o.fp64_waves);
+  };
+  size_t need = plain.empty() ? 0 : plain_need(plain);
+  for (const std::vector<int>& g : oz_pol_groups(oz, K, nb, nw))
+    need = std::max({need, oz_pol_workspace(g, K, nb, nw, sm), 256 + plain_need(g)});
+  return need;
+}
+
+// the FP64 kernel over the given q points; only_if: one device word per q point (MAXQ at most), whose
+// work is empty when it is zero (these launches are not counted as HERK launches)
+static int pol_fp64_plain(const std::vector<PolQ>& qs, double pref, int nw, const OmegaArr& om,
+                          void* ws, size_t ws_bytes, const int* only_if, cudaStream_t s,
+                          const DeviceCtx& ctx, PolOpts& o) {
+  const int nq = int(qs.size());
   std::vector<int64_t> K(nq);
   std::vector<int> nb(nq);
   for (int q = 0; q < nq; ++q) {
@@ -310,10 +347,6 @@ int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, vo
   std::vector<int> splits;
   std::vector<int64_t> tiles;
   plan_fp64(nq, K.data(), nb.data(), nw, ctx.sm_count, o.fp64_waves, splits, tiles);
-  if (o.input_events)                  // every q's inputs before the first launch
-    for (int q = 0; q < nq; ++q)
-      if (o.input_events[q])
-        GW_CUDA_TRY(cudaStreamWaitEvent(s, static_cast<cudaEvent_t>(o.input_events[q]), 0));
   for (int q0 = 0; q0 < nq; q0 += MAXQ) {
     int n = std::min(MAXQ, nq - q0);
     PolLaunch L{};
@@ -343,18 +376,49 @@ int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, vo
     if (part * HT * HT * sizeof(double2) > ws_bytes)
       return set_error(GW_EWORKSPACE, "internal: FP64 partial buffer exceeds workspace");
     double2* pbuf = static_cast<double2*>(ws);
-    int rc = record_herk_event(o, o.launches, false, s);
-    if (rc) return rc;
-    k_herk_fp64<<<unsigned(item), 256, 0, s>>>(L, pref, om, pbuf, ctx.status);
+    int rc = GW_OK;
+    if (!only_if && (rc = record_herk_event(o, o.launches, false, s))) return rc;
+    k_herk_fp64<<<unsigned(item), 256, 0, s>>>(L, pref, om, pbuf, ctx.status, only_if);
     GW_LAUNCH_CHECK("k_herk_fp64");
-    if ((rc = record_herk_event(o, o.launches, true, s))) return rc;
-    ++o.launches;
+    if (!only_if) {
+      if ((rc = record_herk_event(o, o.launches, true, s))) return rc;
+      ++o.launches;
+    }
     int64_t nblk = 0;
     for (int q = 0; q < n; ++q) nblk += tiles[q0 + q] * nw;
-    k_herk_reduce<<<unsigned(nblk), 256, 0, s>>>(L, pbuf, o.accumulate);
+    k_herk_reduce<<<unsigned(nblk), 256, 0, s>>>(L, pbuf, o.accumulate, only_if);
     GW_LAUNCH_CHECK("k_herk_reduce");
   }
   return GW_OK;
+}
+
+int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, void* ws,
+             size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx, PolOpts& o) {
+  if (o.input_events)                  // every q's inputs before the first launch
+    for (int q = 0; q < nq; ++q)
+      if (o.input_events[q])
+        GW_CUDA_TRY(cudaStreamWaitEvent(s, static_cast<cudaEvent_t>(o.input_events[q]), 0));
+  std::vector<int64_t> K(nq);
+  std::vector<int> nb(nq);
+  for (int q = 0; q < nq; ++q) {
+    K[q] = qs[q].K;
+    nb[q] = qs[q].nb;
+  }
+  std::vector<int> oz, plain;
+  split_q(nq, K.data(), oz, plain);
+  for (const std::vector<int>& g : oz_pol_groups(oz, K.data(), nb.data(), nw)) {
+    int rc = oz_pol(g, qs, pref, nw, om, o.accumulate, ws, ws_bytes, s, ctx, o);
+    if (rc) return rc;
+    std::vector<PolQ> again;
+    for (int q : g) again.push_back(qs[q]);
+    rc = pol_fp64_plain(again, pref, nw, om, static_cast<char*>(ws) + 256, ws_bytes - 256,
+                        static_cast<const int*>(ws), s, ctx, o);
+    if (rc) return rc;
+  }
+  if (plain.empty()) return GW_OK;
+  std::vector<PolQ> rest;
+  for (int q : plain) rest.push_back(qs[q]);
+  return pol_fp64_plain(rest, pref, nw, om, ws, ws_bytes, nullptr, s, ctx, o);
 }
 
 }  // namespace gw
