@@ -22,7 +22,8 @@
 // Measured: one q of K = 102,400, N_b = 600, 2 frequencies 314 ms (FP64 kernel, 0.94 TFLOP/s) ->
 // 7.2 ms (41 TFLOP/s FP64-equivalent): k_oz_gemm 5.8 ms, slices 1.05, scales 0.25; relative error of
 // P against 64-bit sums 1.1e-15 -> 5e-16. K = 896, N_b = 64, 8 frequencies 3.7 -> 0.14 ms. The MMAs
-// take about 85 cycles instead of 64 (both operands from shared memory) and set the pace.
+// take about 85 cycles instead of 64 (both operands from shared memory) and set the pace. Pair
+// coefficients of 6,656 pairs, N_b = 600, 16 frequencies: 262 -> 5.9 ms (k_oz_gemm 5.5 ms).
 //
 // What an input may contain: the scale kernels see every operand first. A non-finite value, one
 // outside [2^-100, 2^100], or a column whose largest entry exceeds 1024 times its mean magnitude
@@ -125,7 +126,7 @@ __device__ __forceinline__ const OzProb& oz_item(const OzBatch& batch, int64_t i
   sp = int(item / L.nf);
   if (QF) {
     bi = u % L.nbi;
-    bj = u / L.nbi;
+    bj = L.nbj - 1 - u / L.nbi;         // the longest items (K < 128 (bj + 1)) first
     kind = 2;
     return L;
   }
@@ -364,10 +365,13 @@ __global__ void __launch_bounds__(OTHREADS, 1)
         const int ea =
             L.EA[(size_t(QF ? bi : f * 2 * L.nbj + bi) * L.nsb + sb) * OT + r] - 14 + 1023;
         if (QF) {
+          // this row's part of x . (x U) over the tile's columns: x 2^(EA + EB - 14) by integer
+          // exponent arithmetic, s and c against it in FP64, d (2^-40 of s) in FP32
           const int64_t p = int64_t(bi) * OT + r;
           const int64_t col = int64_t(bj) * OT + c0;
           if (p < L.nrow) {
             const double* xr = L.x + p * L.ncol + col;
+            float qd = 0.0f;
 #pragma unroll
             for (int g4 = 0; g4 < 16; ++g4) {
               const int4 e4 = ld_exp4(eb + 4 * g4);
@@ -380,10 +384,28 @@ __global__ void __launch_bounds__(OTHREADS, 1)
               for (int t = 0; t < 4; ++t) x[t] = col + 4 * g4 + t < L.ncol ? ld_f64(xr + 4 * g4 + t) : 0.0;
 #pragma unroll
               for (int t = 0; t < 4; ++t) {
-                const double v = sum_f64(sv[t], c, d, 4 * g4 + t);
-                qsum = fma(v * __hiloint2double((ea + e[t]) << 20, 0), x[t], qsum);
+                const int i = 4 * g4 + t;
+                const int hi = __double2hiint(x[t]), xe = (hi >> 20) & 0x7ff;
+                const int ex = xe + ea - 1023 + e[t];
+                const bool z = xe == 0 || ex < 1;                  // zero or underflow
+                const double xs = z ? 0.0 : __hiloint2double(hi + ((ea - 1023 + e[t]) << 20),
+                                                             __double2loint(x[t]));
+                float cl, ch, dl, dh;
+                tc::f2_unpack(c[i / 2], cl, ch);
+                tc::f2_unpack(d[i / 2], dl, dh);
+                qsum = fma(to_f64(sv[t]), xs, qsum);
+                qsum = fma(to_f64(i & 1 ? ch : cl), xs, qsum);
+                if (xe != 0 && ex >= 897 && ex <= 1120) {
+                  const float xf = __int_as_float((hi & 0x80000000) | ((ex - 896) << 23) |
+                                                  ((hi & 0xfffff) << 3) |
+                                                  int(uint32_t(__double2loint(x[t])) >> 29));
+                  qd = fmaf(i & 1 ? dh : dl, xf, qd);
+                } else {
+                  qsum = fma(to_f64(i & 1 ? dh : dl), xs, qsum);   // outside the FP32 range
+                }
               }
             }
+            qsum += to_f64(qd);
           }
         } else {
           const size_t nbp = size_t(L.nbj) * OT;
@@ -839,6 +861,134 @@ __global__ void k_oz_combine(const __grid_constant__ OzBatch batch, int accumula
   }
 }
 
+// ------------------------------------------------------------------ quadratic form
+// c_p = x_p R x_p^T of the pair projections' real rows x and the real form R of W^c (R[2I+a][2J+b] =
+// Re W_IJ for a = b, -Im W_IJ for (0,1), Im W_IJ for (1,0)), as x U x^T with U the upper triangle
+// U_kk = R_kk, U_kc = R_kc + R_ck (k < c), so that column block bj needs K < 128 (bj + 1) only.
+__device__ __forceinline__ double u_entry(const double2* __restrict__ W, int nb, int k, int c) {
+  if (k > c || c >= 2 * nb) return 0.0;
+  const int I = k >> 1, a = k & 1, J = c >> 1, b = c & 1;
+  const double2 w = __ldg(W + size_t(I) * nb + J);
+  const double u = a == b ? w.x : a == 0 ? -w.y : w.y;
+  if (k == c) return u;
+  const double2 t = __ldg(W + size_t(J) * nb + I);
+  return u + (a == b ? t.x : b == 0 ? -t.y : t.y);
+}
+
+// exponents of the rows of x, one warp per row and superblock (rows beyond nrow: zeros)
+__global__ void __launch_bounds__(256) k_oz_rowexps(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  const int64_t rows = int64_t(L.nbi) * OT;
+  for (int64_t e = blockIdx.x * 8 + (threadIdx.x >> 5); e < rows * L.nsb; e += int64_t(gridDim.x) * 8) {
+    const int64_t row = e / L.nsb;
+    const int sb = int(e % L.nsb);
+    float mx = 0.f, sum = 0.f;
+    if (row < L.nrow) {
+      const int64_t c0 = int64_t(sb) * L.sbst * OKS, c1 = min(L.ncol, c0 + int64_t(L.sbst) * OKS);
+      for (int64_t c = c0 + lane; c < c1; c += 32) {
+        const float v = abs_up(__ldg(L.x + row * L.ncol + c));
+        mx = fmaxf(mx, v);
+        sum += v;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    if (lane == 0)
+      L.EA[(size_t(row / OT) * L.nsb + sb) * OT + row % OT] = range_exponent(mx, sum, 1.0f, false, L.flag);
+  }
+}
+
+// digit slices of x: grid (stages, row blocks x 4, problems), four lanes per row
+__global__ void __launch_bounds__(OT) k_oz_slice_rows(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.z];
+  if (int(blockIdx.x) >= L.nst || int(blockIdx.y) >= 4 * L.nbi || __ldg(L.flag)) return;
+  const int bi = blockIdx.y >> 2, st = blockIdx.x, kc = threadIdx.x & 3;
+  const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
+  const int64_t row = int64_t(bi) * OT + n, c0 = int64_t(st) * OKS + kc * 8;
+  double v[8];
+#pragma unroll
+  for (int k = 0; k < 8; k += 2) {            // ncol is even: whole pairs
+    const double2 x = row < L.nrow && c0 + k < L.ncol
+                          ? __ldg(reinterpret_cast<const double2*>(L.x + row * L.ncol + c0 + k))
+                          : make_double2(0., 0.);
+    v[k] = x.x;
+    v[k + 1] = x.y;
+  }
+  uint32_t dg[OSL][4];
+  digits8(v, L.EA[(size_t(bi) * L.nsb + st / L.sbst) * OT + n], dg);
+  store_digits(L.A + (size_t(bi) * L.nst + st) * OBLK, n, kc, dg);
+}
+
+// largest magnitude of the columns of U over 128 of its rows: grid (column blocks, row chunks,
+// problems x frequencies); thread = column. W: the problem's first frequency.
+__global__ void __launch_bounds__(OT) k_oz_uscale(const __grid_constant__ OzBatch batch, int nfmax) {
+  const OzProb& L = batch.q[blockIdx.z / nfmax];
+  const int f = blockIdx.z % nfmax, cb = blockIdx.x, ch = blockIdx.y;
+  if (f >= L.nf || cb >= L.nbj || ch > cb) return;
+  const double2* W = L.M + size_t(f) * L.nb * L.nb;
+  const int c = cb * OT + threadIdx.x;
+  float mx = 0.f, sum = 0.f;
+  for (int k = ch * OT; k < (ch + 1) * OT && k <= c; ++k) {
+    const float v = abs_up(u_entry(W, L.nb, k, c));
+    mx = fmaxf(mx, v);
+    sum += v;
+  }
+  L.part[(size_t(f) * L.nbj + ch) * (size_t(L.nbj) * OT) + c] = make_float2(mx, sum);
+}
+
+__global__ void k_oz_uexps(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  const int ncolp = L.nbj * OT, cps = L.sbst * OKS / OT;
+  const int64_t total = int64_t(L.nf) * ncolp * L.nsb;
+  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
+       e += int64_t(gridDim.x) * blockDim.x) {
+    const int c = int(e % ncolp), sb = int(e / ncolp % L.nsb), f = int(e / ncolp / L.nsb);
+    const int cb = c / OT;
+    float mx = 0.f, sum = 0.f;
+    for (int ch = sb * cps; ch < (sb + 1) * cps && ch <= cb; ++ch) {
+      const float2 p = L.part[(size_t(f) * L.nbj + ch) * ncolp + c];
+      mx = fmaxf(mx, p.x);
+      sum += p.y;
+    }
+    L.EB[(size_t(f * L.nbj + cb) * L.nsb + sb) * OT + c % OT] = range_exponent(mx, sum, 1.0f, false, L.flag);
+  }
+}
+
+// digit slices of U: grid (stages, column blocks x 4, problems x frequencies)
+__global__ void __launch_bounds__(OT) k_oz_slice_u(const __grid_constant__ OzBatch batch, int nfmax) {
+  const OzProb& L = batch.q[blockIdx.z / nfmax];
+  const int f = blockIdx.z % nfmax, cb = blockIdx.y >> 2, st = blockIdx.x;
+  if (f >= L.nf || cb >= L.nbj || st >= L.nst || st * OKS > cb * OT + OT - 1 || __ldg(L.flag)) return;
+  const double2* W = L.M + size_t(f) * L.nb * L.nb;
+  const int kc = threadIdx.x & 3, n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
+  const int c = cb * OT + n, k0 = st * OKS + kc * 8;
+  double v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = u_entry(W, L.nb, k0 + k, c);
+  uint32_t dg[OSL][4];
+  const size_t blk = size_t(f) * L.nbj + cb;
+  digits8(v, L.EB[(blk * L.nsb + st / L.sbst) * OT + n], dg);
+  store_digits(L.B + (blk * L.nst + st) * OBLK, n, kc, dg);
+}
+
+// c[f][p] from the column blocks' parts in order; ldc: pairs of the whole q
+__global__ void k_oz_pair_reduce(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  if (__ldg(L.flag)) return;
+  const int64_t total = L.nrow * L.nf;
+  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
+       e += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t f = e / L.nrow, p = e % L.nrow;
+    double v = 0.0;
+    for (int b = 0; b < 2 * L.nbj; ++b) v += L.cpart[(f * 2 * L.nbj + b) * L.nrow + p];
+    L.G[f * L.Kall + p] = v;
+  }
+}
+
 size_t oz_smem() { return size_t(ONST) * OSTAGE + 1024; }
 
 template <bool QF>
@@ -1075,6 +1225,142 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
     k_oz_combine<<<dim3(unsigned(std::min<int64_t>((tot + 255) / 256, cap)), nq), 256, 0, s>>>(
         b, accumulate ? 1 : 0);
     GW_LAUNCH_CHECK("k_oz_combine");
+  }
+  return GW_OK;
+}
+
+// ------------------------------------------------------------------ pair coefficients
+namespace {
+
+// One problem per q, range of pairs and range of frequencies: the slices of x within half of the
+// budget, those of U within the other half where one frequency allows; problems share launches.
+struct PairPlan {
+  int q, f0, nf;
+  int64_t p0, np;
+  int nst, nsb, nbi, nbj;
+  size_t digits, b_part, b_ea, b_eb, b_A, b_B, b_c;
+  size_t total() const { return b_part + b_ea + b_eb + b_A + b_B + b_c; }
+};
+
+std::vector<std::vector<PairPlan>> pair_batches(int nq, const int64_t* npair, const int* nb, int nw) {
+  std::vector<std::vector<PairPlan>> out;
+  size_t bytes = 0;
+  for (int q = 0; q < nq; ++q) {
+    if (npair[q] == 0) continue;
+    const int nst = (2 * nb[q] + OKS - 1) / OKS, nbj = (2 * nb[q] + OT - 1) / OT;
+    const size_t a1 = size_t(nst) * OBLK, u1 = size_t(nbj) * nst * OBLK;
+    // (four grid rows per row block)
+    const int64_t rmax = std::min<int64_t>(16000, std::max<int64_t>(1, int64_t(DIGIT_BUDGET / 2 / a1))) * OT;
+    const int fmax = int(std::max<int64_t>(1, int64_t(DIGIT_BUDGET / 2 / u1)));
+    for (int64_t p0 = 0; p0 < npair[q]; p0 += rmax)
+      for (int f0 = 0; f0 < nw; f0 += fmax) {
+        PairPlan p;
+        p.q = q;
+        p.f0 = f0;
+        p.nf = std::min(fmax, nw - f0);
+        p.p0 = p0;
+        p.np = std::min(rmax, npair[q] - p0);
+        p.nst = nst;
+        p.nsb = (nst + SBMAX - 1) / SBMAX;
+        p.nbi = int((p.np + OT - 1) / OT);
+        p.nbj = nbj;
+        p.b_A = ws_round(p.nbi * a1);
+        p.b_B = ws_round(p.nf * u1);
+        p.digits = p.b_A + p.b_B;
+        p.b_part = ws_round(size_t(p.nf) * nbj * nbj * OT * sizeof(float2));
+        p.b_ea = ws_round(size_t(p.nbi) * p.nsb * OT * 4);
+        p.b_eb = ws_round(size_t(p.nf) * nbj * p.nsb * OT * 4);
+        p.b_c = ws_round(size_t(p.nf) * 2 * nbj * size_t(p.np) * 8);
+        if (out.empty() || int(out.back().size()) == OZQ || bytes + p.digits > DIGIT_BUDGET) {
+          out.push_back({});
+          bytes = 0;
+        }
+        out.back().push_back(p);
+        bytes += p.digits;
+      }
+  }
+  return out;
+}
+
+}  // namespace
+
+size_t oz_pair_workspace(int nq, const int64_t* npair, const int* nb, int nw, int sm) {
+  size_t need = 0;
+  for (const std::vector<PairPlan>& v : pair_batches(nq, npair, nb, nw)) {
+    size_t b = 0;
+    for (const PairPlan& p : v) b += p.total();
+    need = std::max(need, b);
+  }
+  return need + ws_round(size_t(nq) * sizeof(int)) + oz_sum_bytes(sm);
+}
+
+int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig, int nw,
+            const double* const* Wc, double* const* c, void* ws, size_t ws_bytes, cudaStream_t s,
+            const DeviceCtx& ctx) {
+  WsCursor cur{static_cast<char*>(ws), ws_bytes, 0};
+  int* flags = static_cast<int*>(cur.take(ws_round(size_t(nq) * sizeof(int))));
+  float* ssum = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));
+  if (!flags || !ssum) return set_error(GW_EWORKSPACE, "internal: FP64 pair workspace too small");
+  GW_CUDA_TRY(cudaMemsetAsync(flags, 0, size_t(nq) * sizeof(int), s));
+  const size_t base = cur.used;
+  for (const std::vector<PairPlan>& v : pair_batches(nq, npair, nb, nw)) {
+    cur.used = base;
+    OzBatch b{};
+    b.nq = int(v.size());
+    b.s = ssum;
+    int64_t nst = 0, nbi = 0, nbj = 0, nf = 0, nsb = 0, nred = 0;
+    for (int i = 0; i < b.nq; ++i) {
+      const PairPlan& p = v[i];
+      OzProb& L = b.q[i];
+      L.flag = flags + p.q;
+      L.part = static_cast<float2*>(cur.take(p.b_part));
+      L.EA = static_cast<int*>(cur.take(p.b_ea));
+      L.EB = static_cast<int*>(cur.take(p.b_eb));
+      L.A = static_cast<char*>(cur.take(p.b_A));
+      L.B = static_cast<char*>(cur.take(p.b_B));
+      L.cpart = static_cast<double*>(cur.take(p.b_c));
+      if (!L.part || !L.EA || !L.EB || !L.A || !L.B || !L.cpart)
+        return set_error(GW_EWORKSPACE, "internal: FP64 pair workspace too small");
+      L.nb = nb[p.q];
+      L.ncol = 2 * int64_t(nb[p.q]);
+      L.nrow = p.np;
+      L.x = static_cast<const double*>(Msig[p.q]) + p.p0 * L.ncol;
+      L.M = reinterpret_cast<const double2*>(Wc[p.q]) + size_t(p.f0) * L.nb * L.nb;
+      L.G = c[p.q] + size_t(p.f0) * npair[p.q] + p.p0;
+      L.Kall = npair[p.q];
+      L.nf = p.nf;
+      L.nst = p.nst;
+      L.nsb = p.nsb;
+      L.sbst = SBMAX;
+      L.sps = p.nsb;
+      L.splits = 1;
+      L.nbi = p.nbi;
+      L.nbj = p.nbj;
+      L.ntile = p.nbi * p.nbj;
+      b.item0[i + 1] = b.item0[i] + int64_t(L.ntile) * L.nf;
+      nst = std::max<int64_t>(nst, p.nst);
+      nbi = std::max<int64_t>(nbi, p.nbi);
+      nbj = std::max<int64_t>(nbj, p.nbj);
+      nf = std::max<int64_t>(nf, p.nf);
+      nsb = std::max<int64_t>(nsb, p.nsb);
+      nred = std::max<int64_t>(nred, p.np * p.nf);
+    }
+    const unsigned nq_ = unsigned(b.nq), nz = unsigned(b.nq * nf);
+    const int64_t cap = int64_t(ctx.sm_count) * 16;
+    k_oz_rowexps<<<dim3(unsigned(std::min<int64_t>((nbi * OT * nsb + 7) / 8, cap)), nq_), 256, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_rowexps");
+    k_oz_uscale<<<dim3(unsigned(nbj), unsigned(nbj), nz), OT, 0, s>>>(b, int(nf));
+    GW_LAUNCH_CHECK("k_oz_uscale");
+    k_oz_uexps<<<dim3(unsigned(std::min<int64_t>((nf * nbj * OT * nsb + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_uexps");
+    k_oz_slice_rows<<<dim3(unsigned(nst), unsigned(4 * nbi), nq_), OT, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_slice_rows");
+    k_oz_slice_u<<<dim3(unsigned(nst), unsigned(4 * nbj), nz), OT, 0, s>>>(b, int(nf));
+    GW_LAUNCH_CHECK("k_oz_slice_u");
+    int rc = launch_oz<true>(b, s, ctx);
+    if (rc) return rc;
+    k_oz_pair_reduce<<<dim3(unsigned(std::min<int64_t>((nred + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_pair_reduce");
   }
   return GW_OK;
 }

@@ -1,7 +1,7 @@
 // a5 pair coefficients and a6 frequency convolution of the correlation self-energy
 // (Eq. SEc_AC and the paragraph after it).
 //
-// a5 (FP64 path): for each (q, frequency) the CTA tile computes
+// a5 (FP64 kernel, for what fp64_tc.cu hands back): for each (q, frequency) the CTA tile computes
 //   Y[p][I] = sum_J m[p][J] W^c[I][J]      (64 pairs x 64 basis functions)
 // and folds it at once into c_p += Re sum_I conj(m[p][I]) Y[p][I]; partial sums per
 // I-tile are reduced in a fixed order.
@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "gw_internal.cuh"
+#include "fp64_tc.cuh"
 
 namespace gw {
 
@@ -35,14 +36,19 @@ struct PairLaunch {
   int itiles[SMAXQ];
   int64_t blk0[SMAXQ + 1];   // first block of q: blocks ordered (j, ptile, itile)
   size_t part0[SMAXQ];       // first partial double of q
+  double* c[SMAXQ];
   int nq;
   int nw;
 };
 
-__global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __restrict__ part) {
+// only_if: one device word per q of the launch; a q's work is empty when its word is zero (the sliced
+// tensor-core path has its result)
+__global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __restrict__ part,
+                                                       const int* __restrict__ only_if) {
   int64_t blk = blockIdx.x;
   int q = 0;
   while (q + 1 < L.nq && blk >= L.blk0[q + 1]) ++q;
+  if (!only_if[q]) return;
   int64_t loc = blk - L.blk0[q];
   const int it = int(loc % L.itiles[q]);
   loc /= L.itiles[q];
@@ -118,25 +124,35 @@ __global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __r
 }
 
 __global__ void k_paircoef_reduce(PairLaunch L, const double* __restrict__ part,
-                                  double* const* __restrict__ cout_unused, double* c0, int q,
-                                  int64_t np, int itiles, size_t part0, int nw) {
-  int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-  if (e >= np * nw) return;
-  int j = int(e / np);
-  int64_t p = e % np;
-  double s = 0.0;
-  for (int it = 0; it < itiles; ++it) s += part[part0 + (size_t(j) * itiles + it) * np + p];
-  c0[size_t(j) * np + p] = s;
+                                  const int* __restrict__ only_if) {
+  const int q = blockIdx.y;
+  if (!only_if[q]) return;
+  const int64_t np = L.npair[q];
+  for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < np * L.nw;
+       e += int64_t(gridDim.x) * blockDim.x) {
+    const int j = int(e / np);
+    const int64_t p = e % np;
+    double s = 0.0;
+    for (int it = 0; it < L.itiles[q]; ++it)
+      s += part[L.part0[q] + (size_t(j) * L.itiles[q] + it) * np + p];
+    L.c[q][size_t(j) * np + p] = s;
+  }
 }
 
+// FP64: the sliced tensor-core path (fp64_tc.cu), and the FP64 kernel for the q points whose flag it
+// raised, with its partial sums behind the flags.
 size_t paircoef_workspace(int nq, const int64_t* npair, const int* nb, int nw, int precision) {
   if (precision != GW_FP64) return quad_tc_workspace(nq, npair, nb, nw, precision);
+  int sm = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+  cudaGetLastError();
   size_t b = 0;
   for (int q = 0; q < nq; ++q) {
     int it = (nb[q] + ST - 1) / ST;
     b += size_t(nw) * it * size_t(npair[q]);
   }
-  return ws_round(b * sizeof(double));
+  return std::max(ws_round(size_t(nq) * sizeof(int)) + ws_round(b * sizeof(double)),
+                  oz_pair_workspace(nq, npair, nb, nw, sm));
 }
 
 int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msig, int dtype,
@@ -145,7 +161,10 @@ int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msi
   if (precision != GW_FP64)
     return quad_tc(nq, npair, nb, Msig, nw, Wc, c, precision, dtype == GW_R32, ws, ws_bytes, s,
                    ctx);
-  double* part = static_cast<double*>(ws);
+  int rc = oz_pair(nq, npair, nb, Msig, nw, Wc, c, ws, ws_bytes, s, ctx);
+  if (rc) return rc;
+  const int* flags = static_cast<const int*>(ws);
+  double* part = reinterpret_cast<double*>(static_cast<char*>(ws) + ws_round(size_t(nq) * sizeof(int)));
   for (int q0 = 0; q0 < nq; q0 += SMAXQ) {
     int n = std::min(SMAXQ, nq - q0);
     PairLaunch L{};
@@ -157,6 +176,7 @@ int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msi
       int Q = q0 + q;
       L.M[q] = static_cast<const double2*>(Msig[Q]);
       L.W[q] = reinterpret_cast<const double2*>(Wc[Q]);
+      L.c[q] = c[Q];
       L.npair[q] = npair[Q];
       L.nb[q] = nb[Q];
       L.ptiles[q] = int((npair[Q] + ST - 1) / ST);
@@ -167,18 +187,11 @@ int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msi
       p0 += size_t(nw) * L.itiles[q] * size_t(npair[Q]);
     }
     L.blk0[n] = blk;
-    if (blk > 0) {
-      k_paircoef_fp64<<<unsigned(blk), 256, 0, s>>>(L, part);
-      GW_LAUNCH_CHECK("k_paircoef_fp64");
-    }
-    for (int q = 0; q < n; ++q) {
-      int64_t np = L.npair[q];
-      if (np == 0) continue;
-      int64_t tot = np * nw;
-      k_paircoef_reduce<<<unsigned((tot + 255) / 256), 256, 0, s>>>(
-          L, part, nullptr, c[q0 + q], q, np, L.itiles[q], L.part0[q], nw);
-      GW_LAUNCH_CHECK("k_paircoef_reduce");
-    }
+    if (blk == 0) continue;
+    k_paircoef_fp64<<<unsigned(blk), 256, 0, s>>>(L, part, flags + q0);
+    GW_LAUNCH_CHECK("k_paircoef_fp64");
+    k_paircoef_reduce<<<dim3(unsigned(ctx.sm_count), unsigned(n)), 256, 0, s>>>(L, part, flags + q0);
+    GW_LAUNCH_CHECK("k_paircoef_reduce");
   }
   return GW_OK;
 }

@@ -117,3 +117,62 @@ def test_inputs_outside_the_digits_range_take_the_fp64_kernel(gw, what):
         # entry by entry against the sum of magnitudes, which fixed-point digits would miss
         mag = reference(bad.abs().to(torch.complex128), d2, om, 0.25).abs()
         assert float(((Pb - R).abs() / mag).max()) <= 1e-14
+
+
+# ---------------------------------------------------------------- pair coefficients
+def pair_inputs(npair, nb, nw, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    M, _ = inputs(npair, nb, seed)
+    W = torch.view_as_complex(torch.randn((nw, nb, nb, 2), generator=g, dtype=torch.float64, device="cuda"))
+    dec = 1.0 / (1.0 + torch.arange(nb, device="cuda", dtype=torch.float64))
+    return M, W * (dec[:, None] * dec[None, :]).sqrt()
+
+
+def pair_reference(M, W):
+    """c and the sum of the magnitudes of its terms (no assumption on W's symmetry)."""
+    c = torch.stack([((M @ w.T) * M.conj()).sum(1).real for w in W])
+    a = torch.stack([((M.abs() @ w.abs().T) * M.abs()).sum(1) for w in W])
+    return c, a
+
+
+@pytest.mark.parametrize("npair,nb,nw", [(1, 1, 4), (127, 15, 4), (128, 64, 5), (129, 65, 4), (300, 200, 3),
+                                         (1000, 97, 17)])
+def test_pair_coefficients_edges(gw, npair, nb, nw):
+    """|dc| <= 1e-14 of the sum of the magnitudes of the terms (the digits' bound of the module
+    docstring; the largest entry of a column of W is below 2^6 times its mean square here)."""
+    M, W = pair_inputs(npair, nb, nw, npair + nb)
+    c = gw.sigma_pair_coeffs([M], [W])[0]
+    gw.check()
+    r, a = pair_reference(M, W)
+    assert float(((c - r).abs() / a).max()) <= 1e-14
+
+
+def test_pair_coefficients_batch_and_scales(gw):
+    """q points of unequal size (one empty) and of very different scales in one call."""
+    ins = [pair_inputs(n, nb, 4, 50 + i) for i, (n, nb) in enumerate([(40, 30), (0, 8), (700, 70), (5, 129)])]
+    ins[2] = (ins[2][0] * 1e-25, ins[2][1] * 1e-25)
+    ins[3] = (ins[3][0] * 1e25, ins[3][1])
+    cs = gw.sigma_pair_coeffs([m for m, _ in ins], [w for _, w in ins])
+    gw.check()
+    for (M, W), c in zip(ins, cs):
+        if M.shape[0]:
+            r, a = pair_reference(M, W)
+            assert float(((c - r).abs() / a).max()) <= 1e-14
+
+
+@pytest.mark.parametrize("what", ["nan", "huge"])
+def test_pair_coefficients_fall_back(gw, what):
+    M, W = pair_inputs(200, 40, 4, 3)
+    M2, W2 = M.clone(), W.clone()
+    if what == "nan":
+        W2[1, 3, 5] = float("nan")
+    else:
+        M2 *= 1e40
+    c, c2 = gw.sigma_pair_coeffs([M, M2], [W, W2])
+    gw.check()
+    r, a = pair_reference(M, W)
+    assert float(((c - r).abs() / a).max()) <= 1e-14
+    r2, a2 = pair_reference(M2, W2)
+    assert torch.equal(torch.isfinite(c2), torch.isfinite(r2))
+    ok = torch.isfinite(r2)
+    assert float(((c2 - r2).abs() / a2)[ok].max()) <= 1e-14
