@@ -12,6 +12,8 @@
 // relative cost decrease is <= 1e-14, when C <= 1e-28 * (1/2 sum |y|^2), or after
 // 200 iterations. Default start: w_p = s (0.5, 2, 5, 10, 20)_p - 0.1 i s (s the sign
 // of the state energy) with residues from the linear least-squares problem.
+#include <algorithm>
+
 #include "gw_internal.cuh"
 #include "fit_common.cuh"
 
@@ -268,12 +270,376 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
   status_out[cidx] = st;
 }
 
+// ---- many curves: four or eight lanes per curve, eight or four curves per warp --------------------
+// GB300's FP64 pipe takes as long for an instruction with one active lane as for a full one (16
+// cycles per warp instruction and SM), and the warp-per-curve kernel issues most of its FP64
+// instructions with few (the pivots with one, the sweeps with at most P = 4 N_p, the points with nw
+// of 32). Here several curves share a warp's instructions, with the same operations in the same
+// order (sums over points as the warp's butterfly forms them, everything else through shared
+// memory as there), so the results are bit-identical. A block draws its curves from a contiguous
+// range through a counter, the lanes of a curve taking the next one when their fit ends; each trip
+// of the loop is damped solve, cost, accept or reject, and the Jacobian for the curves that
+// accepted. Still bound by the FP64 pipe. One lane per curve was not faster (270 ms for 1e5 curves:
+// its registers hold one curve's matrix, few warps run) and rounds differently.
+// Two-pole fits on 24 points, this kernel against one warp per curve: 1e5 curves 440 -> 248 ms,
+// 32,000 144 -> 91.5, 8,192 40.3 -> 33.6, 6,500 32.7 -> 30.3 ms. Below about 6,000 curves there are too
+// few warps (5,000: 26.5 -> 30.9 ms), and from 8,192 on four lanes per curve are the faster split
+// (16,000: 57.4 -> 55.5 ms, 1e5: 276 -> 248 ms). More than 32 points take too much shared
+// memory per curve (9,000 curves on 64 points: 82 -> 167 ms), as do four poles and more.
+constexpr int LM_GROUPS_MIN = 6144;   // curves from which this kernel is taken
+constexpr int LM_GROUPS4_MIN = 8192;  // ... with four lanes per curve
+constexpr int LM_GROUPS_MAXNW = 32;
+
+// doubles of shared memory per curve (odd, so that the curves of a warp start in other banks)
+__host__ __device__ constexpr int lm_group_doubles(int nw, int P) {
+  return (2 * nw * P + 2 * nw + P * (P + 1) + 3 * P) | 1;
+}
+
+// the sum the butterfly of warp_sum forms of the lanes' values c(l), l = sub + G k held in c[k]
+template <int G>
+__device__ __forceinline__ double group_butterfly(double (&c)[32 / G]) {
+#pragma unroll
+  for (int n = 16 / G; n > 0; n /= 2)
+#pragma unroll
+    for (int k = 0; k < n; ++k) c[k] += c[k + n];
+  double v = c[0];
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+template <int G>
+__device__ __forceinline__ double group_max(double v) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+template <int NPOLE, int LMG>
+__global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __grid_constant__ OmegaArr om,
+                                                   const double2* __restrict__ sigma,
+                                                   const double* __restrict__ sign,
+                                                   const double* theta_init, double* params,
+                                                   double* __restrict__ cost_out,
+                                                   int* __restrict__ iters_out,
+                                                   int* __restrict__ status_out, int keep_better) {
+  constexpr int npole = NPOLE;
+  constexpr int P = 4 * npole;
+  constexpr int NP = P * (P + 1) / 2;
+  constexpr int EPL = (NP + LMG - 1) / LMG;     // packed entries per lane
+  constexpr int NL = 32 / LMG;                  // lanes of the warp kernel per lane
+  extern __shared__ double lsm[];
+  __shared__ int next;
+  const int lane = threadIdx.x & 31, sub = lane & (LMG - 1);
+  double* rowR = lsm + size_t(threadIdx.x / LMG) * lm_group_doubles(nw, P);
+  double* rowI = rowR + nw * P;
+  double* res = rowI + nw * P;
+  double* sA = res + 2 * nw;
+  double* Ld = sA + NP;
+  double* sg = Ld + NP;
+  double* sb = sg + P;
+  double* dinv = sb + P;
+  const int per = (ncurve + int(gridDim.x) - 1) / int(gridDim.x);
+  const int c_end = min(ncurve, (int(blockIdx.x) + 1) * per);
+  if (threadIdx.x == 0) next = int(blockIdx.x) * per;
+  __syncthreads();
+  // the packed entries e = sub + 8 h of A this lane sums: row ea[h], column eb[h]
+  int ea[EPL], eb[EPL];
+#pragma unroll
+  for (int h = 0; h < EPL; ++h) {
+    const int e = sub + LMG * h;
+    int a = 0;
+    while ((a + 1) * (a + 2) / 2 <= e) ++a;
+    ea[h] = e < NP ? a : 0;
+    eb[h] = e < NP ? e - a * (a + 1) / 2 : 0;
+  }
+  // per curve, the same in its eight lanes
+  int cidx = 0, it = 0, st = 1;
+  bool active = false, done = false, init = false;
+  double th[P], thn[P], C = 0.0, cscale = 0.0, mu = -1.0;
+  for (int k = 0; k < P; ++k) th[k] = thn[k] = 0.0;
+  const double2* y = sigma;
+  while (true) {
+    const bool want = !active && !done;
+    if (__any_sync(0xffffffffu, want)) {
+      int c = 0;
+      if (want && sub == 0) c = atomicAdd(&next, 1);
+      c = __shfl_sync(0xffffffffu, c, 0, LMG);
+      if (want) {
+        if (c >= c_end) {
+          done = true;
+        } else {
+          cidx = c;
+          active = init = true;
+          it = 0;
+          st = 1;
+          mu = -1.0;
+          y = sigma + size_t(cidx) * nw;
+          if (theta_init) {
+            for (int k = 0; k < P; ++k) thn[k] = theta_init[size_t(cidx) * P + k];
+          } else if (sub == 0) {
+            const double s = sign ? (sign[cidx] >= 0.0 ? 1.0 : -1.0) : 1.0;
+            lm_default_start(om.v, y, nw, npole, s, sb);
+          }
+        }
+      }
+      __syncwarp();
+      if (init && !theta_init)
+        for (int k = 0; k < P; ++k) thn[k] = sb[k];
+      double c4[NL];
+#pragma unroll
+      for (int k = 0; k < NL; ++k) {
+        const int l = sub + LMG * k;
+        const double2 a = init && l < nw ? y[l] : make_double2(0.0, 0.0);
+        const double2 b = init && l + 32 < nw ? y[l + 32] : make_double2(0.0, 0.0);
+        c4[k] = a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y;
+      }
+      const double cs = 0.5 * group_butterfly<LMG>(c4);
+      if (init) cscale = cs;
+      if (!__any_sync(0xffffffffu, active)) break;
+    }
+    const bool solve = active && !init;
+    bool ok = true;
+    if (__any_sync(0xffffffffu, solve)) {
+      if (solve) {
+        for (int e = sub; e < NP; e += LMG) Ld[e] = sA[e];
+      }
+      __syncwarp();
+      if (solve) {
+        for (int i = sub; i < P; i += LMG) {
+          Ld[i * (i + 1) / 2 + i] += mu * sA[i * (i + 1) / 2 + i];
+          sb[i] = -sg[i];
+        }
+      }
+      __syncwarp();
+      // Cholesky, column by column: the pivot by the curve's first lane, the rows below it by its lanes
+      for (int jc = 0; jc < P; ++jc) {
+        if (solve && sub == 0) {
+          double d = Ld[jc * (jc + 1) / 2 + jc];
+          for (int k = 0; k < jc; ++k) d -= Ld[jc * (jc + 1) / 2 + k] * Ld[jc * (jc + 1) / 2 + k];
+          if (!(d > 0.0)) ok = false;
+          const double r = d > 0.0 ? sqrt(d) : 1.0;
+          Ld[jc * (jc + 1) / 2 + jc] = r;
+          dinv[jc] = 1.0 / r;
+        }
+        __syncwarp();
+        if (solve) {
+          for (int i = jc + 1 + sub; i < P; i += LMG) {
+            double v = Ld[i * (i + 1) / 2 + jc];
+            for (int k = 0; k < jc; ++k) v -= Ld[i * (i + 1) / 2 + k] * Ld[jc * (jc + 1) / 2 + k];
+            Ld[i * (i + 1) / 2 + jc] = v * dinv[jc];
+          }
+        }
+        __syncwarp();
+      }
+      ok = __shfl_sync(0xffffffffu, int(ok), 0, LMG) != 0;
+      // L z = b by column sweeps, then L^T x = z
+      for (int k = 0; k < P; ++k) {
+        const double zk = sb[k] * dinv[k];
+        __syncwarp();
+        if (solve) {
+          for (int i = k + 1 + sub; i < P; i += LMG) sb[i] -= Ld[i * (i + 1) / 2 + k] * zk;
+          if (sub == 0) sb[k] = zk;
+        }
+        __syncwarp();
+      }
+      for (int k = P - 1; k >= 0; --k) {
+        const double xk = sb[k] * dinv[k];
+        __syncwarp();
+        if (solve) {
+          for (int i = sub; i < k; i += LMG) sb[i] -= Ld[k * (k + 1) / 2 + i] * xk;
+          if (sub == 0) sb[k] = xk;
+        }
+        __syncwarp();
+      }
+      if (solve)
+        for (int k = 0; k < P; ++k) thn[k] = th[k] + sb[k];
+    }
+    // the cost at thn
+    double c4[NL];
+#pragma unroll
+    for (int k4 = 0; k4 < NL; ++k4) {
+      double c = 0.0;
+      for (int h = 0; h < 2; ++h) {
+        const int j = sub + LMG * k4 + 32 * h;
+        if (j >= nw || !active) break;
+        double fx = 0.0, fy = 0.0;
+        for (int p = 0; p < npole; ++p) {
+          const double dx = -thn[4 * p + 2], dy = om.v[j] - thn[4 * p + 3];
+          const double inv = 1.0 / (dx * dx + dy * dy);
+          const double px = dx * inv, py = -dy * inv;          // phi = 1 / (i w_j - w_p)
+          fx += thn[4 * p] * px - thn[4 * p + 1] * py;
+          fy += thn[4 * p] * py + thn[4 * p + 1] * px;
+        }
+        const double2 yj = y[j];
+        const double rx = fx - yj.x, ry = fy - yj.y;
+        c += rx * rx + ry * ry;
+      }
+      c4[k4] = c;
+    }
+    const double Cn = 0.5 * group_butterfly<LMG>(c4);
+    bool jac = false, end = false;
+    if (active) {
+      bool accepted = init;
+      double dec = 0.0, Cold = 0.0;
+      if (!init) {
+        accepted = ok && Cn < C;
+        if (accepted) {
+          mu = fmax(mu / 10.0, LM_MU_MIN);
+          dec = C - Cn;
+          Cold = C;
+        } else {
+          mu *= 10.0;
+          if (mu > LM_MU_MAX) {
+            st = 2;
+            end = true;
+          }
+        }
+      }
+      if (accepted) {
+        for (int k = 0; k < P; ++k) th[k] = thn[k];
+        C = Cn;
+        if (!init) {
+          ++it;
+          if (dec <= LM_FTOL * Cold) {
+            st = 0;
+            end = true;
+          } else if (it >= LM_MAXIT) {
+            end = true;
+          }
+        }
+        init = false;
+        if (!end) {
+          if (C <= LM_CTOL * cscale) {
+            st = 0;
+            end = true;
+          } else {
+            jac = true;
+          }
+        }
+      }
+    }
+    if (__any_sync(0xffffffffu, jac)) {
+      // Jacobian rows and residuals of this lane's points
+      if (jac) {
+        for (int j = sub; j < nw; j += LMG) {
+          double fx = 0.0, fy = 0.0;
+          for (int p = 0; p < npole; ++p) {
+            const double ax = th[4 * p], ay = th[4 * p + 1];
+            const double dx = -th[4 * p + 2], dy = om.v[j] - th[4 * p + 3];
+            const double inv = 1.0 / (dx * dx + dy * dy);
+            const double px = dx * inv, py = -dy * inv;        // phi
+            const double tx = ax * px - ay * py, ty = ax * py + ay * px;   // a phi
+            fx += tx;
+            fy += ty;
+            const double qx = tx * px - ty * py, qy = tx * py + ty * px;   // a phi^2
+            double* R = rowR + j * P + 4 * p;
+            double* I = rowI + j * P + 4 * p;
+            R[0] = px;
+            I[0] = py;
+            R[1] = -py;
+            I[1] = px;
+            R[2] = qx;
+            I[2] = qy;
+            R[3] = -qy;
+            I[3] = qx;
+          }
+          const double2 yj = y[j];
+          res[2 * j] = fx - yj.x;
+          res[2 * j + 1] = fy - yj.y;
+        }
+      }
+      __syncwarp();
+      // A (packed lower) and g, summed over points
+      double gm = 0.0, dm = 0.0;
+      if (jac) {
+        double v[EPL];
+#pragma unroll
+        for (int h = 0; h < EPL; ++h) v[h] = 0.0;
+#pragma unroll 2
+        for (int j = 0; j < nw; ++j) {
+          const double* R = rowR + j * P;
+          const double* I = rowI + j * P;
+#pragma unroll
+          for (int h = 0; h < EPL; ++h) v[h] += R[ea[h]] * R[eb[h]] + I[ea[h]] * I[eb[h]];
+        }
+#pragma unroll
+        for (int h = 0; h < EPL; ++h) {
+          const int e = sub + LMG * h;
+          if (e < NP) {
+            sA[e] = v[h];
+            if (ea[h] == eb[h]) dm = fmax(dm, v[h]);
+          }
+        }
+        for (int a = sub; a < P; a += LMG) {
+          double w = 0.0;
+          for (int j = 0; j < nw; ++j) w += rowR[j * P + a] * res[2 * j] + rowI[j * P + a] * res[2 * j + 1];
+          sg[a] = w;
+          gm = fmax(gm, fabs(w));
+        }
+      }
+      __syncwarp();
+      gm = group_max<LMG>(gm);
+      dm = group_max<LMG>(dm);
+      if (jac) {
+        if (gm <= LM_GTOL) {
+          st = 0;
+          end = true;
+        }
+        if (mu < 0.0) mu = 1e-3 * dm;
+      }
+    }
+    if (end) {
+      active = false;
+      // the other start's result stays when it is not worse
+      if (sub == 0 && (!keep_better || C < cost_out[cidx])) {
+        for (int k = 0; k < P; ++k) params[size_t(cidx) * P + k] = th[k];
+        cost_out[cidx] = C;
+        iters_out[cidx] = it;
+        status_out[cidx] = st;
+      }
+    }
+  }
+}
+
+template <int NPOLE, int G>
+static int launch_lm_groups(int ncurve, int nw, const OmegaArr& om, const double2* y, const double* sign,
+                            const double* theta_init, double* params, double* cost, int* iters,
+                            int* status, int keep_better, cudaStream_t s, const DeviceCtx& ctx) {
+  const auto kern = k_lm_groups<NPOLE, G>;
+  const size_t per_warp = size_t(32 / G) * lm_group_doubles(nw, 4 * NPOLE) * sizeof(double);
+  const int warps = int(std::max<size_t>(1, std::min<size_t>(4, (100u << 10) / per_warp)));
+  const size_t smem = warps * per_warp;
+  int rc = set_max_dyn_smem(reinterpret_cast<const void*>(kern), smem, ctx.device);
+  if (rc) return rc;
+  int fit = 0;                        // resident blocks per SM
+  GW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem));
+  const int curves = warps * 32 / G;
+  const int blocks = int(std::min<int64_t>((int64_t(ncurve) + curves - 1) / curves,
+                                           int64_t(ctx.sm_count) * std::max(1, fit)));
+  kern<<<blocks, 32 * warps, smem, s>>>(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status,
+                                       keep_better);
+  GW_LAUNCH_CHECK("k_lm_groups");
+  return GW_OK;
+}
+
 int launch_lm(int ncurve, int nw, const OmegaArr& om, const double* sigma, const double* sign,
               int npole, const double* theta_init, double* params, double* cost, int* iters,
               int* status, int keep_better, cudaStream_t s) {
   if (ncurve == 0) return GW_OK;
   if (nw > LM_WMAXNW) return set_error(GW_EINVAL, "the fit takes at most %d frequencies", LM_WMAXNW);
   const double2* y = reinterpret_cast<const double2*>(sigma);
+  if (npole <= 3 && nw <= LM_GROUPS_MAXNW && ncurve >= LM_GROUPS_MIN) {
+    DeviceCtx ctx;
+    int rc = device_ctx(&ctx);
+    if (rc) return rc;
+    auto run = [&](auto f) {
+      return f(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status, keep_better, s, ctx);
+    };
+    const bool four = ncurve >= LM_GROUPS4_MIN;
+    if (npole == 1) return run(four ? launch_lm_groups<1, 4> : launch_lm_groups<1, 8>);
+    if (npole == 2) return run(four ? launch_lm_groups<2, 4> : launch_lm_groups<2, 8>);
+    return run(four ? launch_lm_groups<3, 4> : launch_lm_groups<3, 8>);
+  }
   auto go = [&](auto kern) {
     kern<<<ncurve, 32, 0, s>>>(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status,
                                keep_better);
