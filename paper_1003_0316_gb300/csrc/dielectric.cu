@@ -6,16 +6,15 @@
 //   W^c = v^1/2 (Z^H Z - 1) v^1/2
 //
 // The caller-workspace entry points factorise a workspace copy of eps right-looking over many
-// CTAs (per 32-wide panel: the diagonal block, the panel below it, the trailing update of the
-// lower 32x32 tiles), invert the factor by block columns (the diagonal blocks first, then one
-// CTA per (system, block column) for the forward substitution of that column) and form W^c
-// with one CTA per (system, 32-row block), so every phase uses every SM; each thread owns one
-// row and four columns of a 32x32 tile staged in shared memory. About 4 N^3 real flops per
-// system (N^3/6 complex multiply-adds per phase). Storage and the small steps (diagonal
-// blocks, their inverses) are FP64; the tile products and the panel solve run in float-float
-// arithmetic on the FP32 pipe, which GB300 executes 64 times faster than FP64 (see FF below):
-// about 2^-48 relative per operation. The no-allocation entry point keeps the factorisation
-// and the inverse inside one CTA per system, in FP64.
+// CTAs (per 32-wide panel: the diagonal block and its inverse, the panel below it, the trailing
+// update of the lower 32x32 tiles), invert the factor by block columns (one CTA per (system, block
+// column) for the forward substitution of that column) and form W^c with one CTA per (system,
+// 32-row block), so every phase uses every SM; each thread owns one row and four columns of a
+// 32x32 tile staged in shared memory. About 4 N^3 real flops per system (N^3/6 complex
+// multiply-adds per phase). Storage and arithmetic are float-float on the FP32 pipe, which GB300
+// executes 64 times faster than FP64 (see FF below): about 2^-48 relative per operation; P, v and
+// W^c are FP64. The no-allocation entry point keeps the factorisation and the inverse inside one
+// CTA per system, in FP64.
 #include <vector>
 #include <algorithm>
 #include <mutex>
@@ -186,9 +185,32 @@ __device__ __forceinline__ void ff_csubmul_conj(FAccC& a, FFC x, FFC l) {
   ff_mac(a.im, ff_neg(x.im), l.re);
   ff_mac(a.im, x.re, l.im);
 }
-__device__ __forceinline__ double ff_to_d(FF x) { return double(x.h) + double(x.l); }
-__device__ __forceinline__ double ff_to_t(FF x) { return ff_to_d(x); }
-__device__ __forceinline__ double2 ff_to_t(FFC x) { return make_double2(ff_to_d(x.re), ff_to_d(x.im)); }
+// acc -= x y
+__device__ __forceinline__ void ff_csubmul(FAcc& a, FF x, FF y) { ff_mac(a, ff_neg(x), y); }
+__device__ __forceinline__ void ff_csubmul(FAccC& a, FFC x, FFC y) {
+  ff_mac(a.re, ff_neg(x.re), y.re);
+  ff_mac(a.re, x.im, y.im);
+  ff_mac(a.im, ff_neg(x.re), y.im);
+  ff_mac(a.im, ff_neg(x.im), y.re);
+}
+__device__ __forceinline__ FF ff_re(FF x) { return x; }
+__device__ __forceinline__ FF ff_re(FFC x) { return x.re; }
+template <typename FT> __device__ __forceinline__ FT ff_real(FF x);
+template <> __device__ __forceinline__ FF ff_real<FF>(FF x) { return x; }
+template <> __device__ __forceinline__ FFC ff_real<FFC>(FF x) { return FFC{x, FF{0.0f, 0.0f}}; }
+// 1 / sqrt(d) for a positive d: the FP32 approximation y and one Newton step
+// y + y (1 - d y^2) / 2 with the residual in float-float (relative error near 2^-46)
+__device__ __forceinline__ FF ff_rsqrt(FF d) {
+  const float y = rsqrtf(d.h);
+  FAcc r = {1.0f, 0.0f};
+  const float p = __fmul_rn(y, y);
+  ff_mac(r, ff_neg(d), FF{p, __fmaf_rn(y, y, -p)});          // 1 - d y^2
+  const FF e = ff_renorm(r);
+  const float c = __fmul_rn(0.5f * y, e.h);
+  // the second-order term 3/8 y e^2 keeps the result at the float-float level
+  const float c2 = __fmaf_rn(__fmul_rn(0.375f * y, e.h), e.h, __fmul_rn(0.5f * y, e.l));
+  return ff_renorm(FAcc{y, __fadd_rn(c, __fadd_rn(c2, __fmaf_rn(0.5f * y, e.h, -c)))});
+}
 
 // e - a rounded to float-float (e a float-float value, a an accumulator)
 __device__ __forceinline__ FF ff_sub_acc(FF e, FAcc a) {
@@ -206,8 +228,7 @@ __device__ __forceinline__ FFC ff_negate(FFC x) { return FFC{ff_neg(x.re), ff_ne
 
 // The caller-workspace path keeps eps, its factor, the inverse factor and the inverted
 // diagonal blocks in float-float form (the bytes of the FP64 element: complex FFC, real FF),
-// so the tile products load them without FP64 conversions; the diagonal blocks are factorised
-// and inverted in FP64 and the output W^c is FP64.
+// so the tile products load them without FP64 conversions; the output W^c is FP64.
 template <typename T>
 using StorOf = typename FFOf<T>::tile;
 template <typename T>
@@ -229,19 +250,6 @@ __device__ __forceinline__ void load_tile_s(FT* S, const FT* A, int ld, int n_ro
     S[r * DLD + c] = v;
   }
 }
-// the same into FP64 shared memory
-template <typename T>
-__device__ __forceinline__ void load_tile_s2d(T* S, const StorOf<T>* A, int ld, int n_rows,
-                                              int n_cols, int r0, int c0, int mode) {
-  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS) {
-    int r = e / DB, c = e % DB;
-    int R = r0 + r, C = c0 + c;
-    T v = T{};
-    if (R < n_rows && C < n_cols && (mode == 0 || C <= R)) v = ff_to_t(A[size_t(R) * ld + C]);
-    S[r * DLD + c] = v;
-  }
-}
-
 // load_tile into float-float shared memory
 template <typename T>
 __device__ __forceinline__ void load_tile_ff(typename FFOf<T>::tile* S, const T* A, int ld,
@@ -273,8 +281,7 @@ struct DieBatchT {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(DTHREADS) k_dielectric(const DieBatchT<T> batch, unsigned* status,
-                                                         bool invert) {
+__global__ void __launch_bounds__(DTHREADS) k_dielectric(const DieBatchT<T> batch, unsigned* status) {
   extern __shared__ __align__(16) unsigned char dsm_raw[];
   T* smem = reinterpret_cast<T*>(dsm_raw);
   T* SA = smem;
@@ -387,7 +394,6 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric(const DieBatchT<T> batc
     if (tid == 0) raise_status(status, (s_fail & 1) ? ST_ENOTHPD : ST_ENONFINITE);
     return;
   }
-  if (!invert) return;   // the inverse follows by block columns (k_dielectric_dinv, _zcol)
 
   // ---- phase 2: Z = L^{-1}, lower, in place --------------------------------
   for (int kt = nt - 1; kt >= 0; --kt) {
@@ -521,43 +527,8 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_w(const DieBatchT<T> ba
 }
 
 // ---- the inverse Z = L^{-1} by block columns (the columns of Z are independent forward
-// substitutions L Z_c = I_c): first every diagonal block inverted, one CTA per (system, block)
-template <typename T>
-__global__ void __launch_bounds__(DTHREADS) k_dielectric_dinv(const DieBatchT<T> batch) {
-  extern __shared__ __align__(16) unsigned char dsm_raw[];
-  T* SD = reinterpret_cast<T*>(dsm_raw);
-  const DieSysT<T> sys = batch.s[blockIdx.x];
-  const int n = sys.n;
-  const int nt = (n + DB - 1) / DB;
-  const int r = blockIdx.y;
-  if (r >= nt) return;
-  const int k0 = r * DB;
-  const int kb = min(DB, n - k0);
-  load_tile_s2d(SD, stor(sys.E), n, n, n, k0, k0, 1);
-  __syncthreads();
-  if (threadIdx.x < DB) {
-    const int c = threadIdx.x;
-    T z[DB];
-#pragma unroll
-    for (int i = 0; i < DB; ++i) z[i] = T{};
-    if (c < kb) {
-      z[c] = real_of<T>(1.0 / re_(SD[c * DLD + c]));
-#pragma unroll
-      for (int i = 0; i < DB; ++i) {
-        if (i > c && i < kb) {
-          T acc = T{};
-          for (int k = c; k < i; ++k) cfma(acc, SD[i * DLD + k], z[k]);
-          z[i] = scal(acc, -1.0 / re_(SD[i * DLD + i]));
-        }
-      }
-    }
-    StorOf<T>* Dr = stor(sys.D) + size_t(r) * DB * DB;
-#pragma unroll
-    for (int i = 0; i < DB; ++i) Dr[i * DB + c] = to_ff_t(z[i]);
-  }
-}
-
-// then one CTA per (system, block column c): for r = c, c + 1, ...
+// substitutions L Z_c = I_c); the diagonal blocks D_r were inverted by k_chol_diag.
+// One CTA per (system, block column c): for r = c, c + 1, ...
 //   Z[r][c] = D_r (delta_rc - sum_{k = c}^{r-1} L[r][k] Z[k][c])
 // with the earlier blocks Z[k][c] of the same column read back from global memory.
 template <typename T>
@@ -652,91 +623,96 @@ __global__ void __launch_bounds__(DTHREADS) k_eps_fill(const DieBatchT<T> batch,
   if (bad) raise_status(status, ST_ENONFINITE);
 }
 
-// in-place Cholesky of the kb x kb lower block held in shared memory (SD, ld DLD); returns
-// false (through *fail) on a non-positive or non-finite pivot, which is replaced by 1
-template <typename T>
-__device__ void chol_block_smem(T* SD, int kb, int* fail) {
-  const int tid = threadIdx.x;
-  for (int c = 0; c < kb; ++c) {
-    if (tid == 0) {
-      double d = re_(SD[c * DLD + c]);
-      if (!(d > 0.0) || !isfinite(d)) {
-        *fail = 1;
-        d = 1.0;
-      }
-      SD[c * DLD + c] = real_of<T>(sqrt(d));
-    }
-    __syncthreads();
-    const double dinv = 1.0 / re_(SD[c * DLD + c]);
-    for (int r = c + 1 + tid; r < kb; r += DTHREADS) SD[r * DLD + c] = scal(SD[r * DLD + c], dinv);
-    __syncthreads();
-    for (int e = tid; e < DB * DB; e += DTHREADS) {
-      const int r = e / DB, s = e % DB;
-      if (r < kb && s > c && s <= r) {
-        T x = SD[r * DLD + s];
-        csubmul(x, SD[r * DLD + c], cconj(SD[s * DLD + c]));
-        SD[r * DLD + s] = x;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// step 1 of panel kt: the diagonal block, one CTA per system
+// step 1 of panel kt: the diagonal block's factor and its inverse D_kt, one CTA per system, in
+// float-float. Right-looking over the columns c: with y = 1 / sqrt(pivot), column c of L and row c of
+// the inverse Z (which starts as the identity) are scaled by y, then every entry (r, s) below row c
+// takes one product: x_rs -= L_rc conj(L_sc) for s > c, Z_rs -= L_rc Z_cs for s <= c. (In FP64, with
+// one thread on each pivot and one on each column of the inverse, the two took 57 and about 50 us
+// per panel of 128 systems; this takes 34, bound by its serial columns.)
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS) k_chol_diag(const DieBatchT<T> batch, int kt,
                                                         unsigned* status) {
-  __shared__ T SD[DB * DLD];
-  __shared__ int s_fail;
+  using FT = typename FFOf<T>::tile;
+  using FA = typename FFOf<T>::acc;
+  __shared__ __align__(16) unsigned char raw[2 * DB * DLD * sizeof(FT)];
+  FT* SD = reinterpret_cast<FT*>(raw);
+  FT* SZ = SD + DB * DLD;
   const DieSysT<T>& sys = batch.s[blockIdx.x];
   const int n = sys.n, nt = (n + DB - 1) / DB;
   if (kt >= nt) return;                      // whole CTA, before any barrier
-  const int k0 = kt * DB, kb = min(DB, n - k0);
-  if (threadIdx.x == 0) s_fail = 0;
-  load_tile_s2d(SD, stor(sys.E), n, n, n, k0, k0, 1);
-  __syncthreads();
-  chol_block_smem(SD, kb, &s_fail);
-  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS) {
-    const int r = e / DB, c = e % DB;
-    if (r < kb && c <= r) stor(sys.E)[size_t(k0 + r) * n + k0 + c] = to_ff_t(SD[r * DLD + c]);
+  const int k0 = kt * DB, kb = min(DB, n - k0), tid = threadIdx.x;
+  load_tile_s(SD, stor(sys.E), n, n, n, k0, k0, 1);
+  for (int e = tid; e < DB * DB; e += DTHREADS) SZ[(e / DB) * DLD + e % DB] = FT{};
+  bool fail = false;
+  for (int c = 0; c < kb; ++c) {
+    __syncthreads();
+    FF d = ff_re(SD[c * DLD + c]);
+    if (!(d.h > 0.0f) || !isfinite(d.h)) {   // not positive definite: a pivot of 1
+      fail = true;
+      d = FF{1.0f, 0.0f};
+    }
+    const FF y = ff_rsqrt(d);
+    __syncthreads();                          // the pivot is read
+    if (tid < DB) {
+      const int r = tid;
+      if (r > c && r < kb) SD[r * DLD + c] = ff_scale(SD[r * DLD + c], y);
+      if (r == c) SD[c * DLD + c] = ff_real<FT>(ff_mul(d, y));
+    } else if (tid < 2 * DB) {
+      const int q = tid - DB;
+      if (q < c) SZ[c * DLD + q] = ff_scale(SZ[c * DLD + q], y);
+      if (q == c) SZ[c * DLD + c] = ff_real<FT>(y);
+    }
+    __syncthreads();
+    for (int e = tid; e < DB * DB; e += DTHREADS) {
+      const int r = e / DB, q = e % DB;
+      if (r <= c || r >= kb || q > r) continue;
+      FT* x = (q > c ? SD : SZ) + r * DLD + q;
+      FA acc = ff_acc(*x);
+      const FT l = SD[r * DLD + c];
+      if (q > c) ff_csubmul_conj(acc, l, SD[q * DLD + c]);
+      else ff_csubmul(acc, l, SZ[c * DLD + q]);
+      *x = ff_renorm_t(acc);
+    }
   }
-  if (threadIdx.x == 0 && s_fail) raise_status(status, ST_ENOTHPD);
+  __syncthreads();
+  FT* E = stor(sys.E);
+  FT* Dr = stor(sys.D) + size_t(kt) * DB * DB;
+  for (int e = tid; e < DB * DB; e += DTHREADS) {
+    const int r = e / DB, c = e % DB;
+    if (r < kb && c <= r) E[size_t(k0 + r) * n + k0 + c] = SD[r * DLD + c];
+    Dr[e] = SZ[r * DLD + c];
+  }
+  if (tid == 0 && fail) raise_status(status, ST_ENOTHPD);
 }
 
-// step 2: the panel X L_kk^H = A_ik below the diagonal block, one row per thread, in
-// float-float (the reciprocals of the diagonal in FP64); grid (256-row blocks of the trailing
-// rows, system)
+// step 2: the panel X = A_ik L_kk^{-H} = A_ik D_kt^H below the diagonal block, in float-float; one
+// CTA per (32-row block, system): 1.3 ms for the 18 panels of 128 systems of N_b = 600. (A row per
+// thread solving against L_kk took 4.1 ms, one dependent chain of 26,000 FP32 operations per row.)
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS) k_chol_panel(const DieBatchT<T> batch, int kt) {
   using FT = typename FFOf<T>::tile;
   using FA = typename FFOf<T>::acc;
-  __shared__ FT SD[DB * DLD];
-  __shared__ FF rinv[DB];
+  extern __shared__ __align__(16) unsigned char dsm_raw[];
+  FT* SA = reinterpret_cast<FT*>(dsm_raw);
+  FT* SB = SA + DB * DLD;
   const DieSysT<T>& sys = batch.s[blockIdx.y];
   const int n = sys.n, nt = (n + DB - 1) / DB;
-  if (kt >= nt - 1) return;                  // no rows below the last block
+  const int it = kt + 1 + blockIdx.x;
+  if (it >= nt) return;                      // whole CTA, before any barrier
   const int k0 = kt * DB;                    // a full block: kt < nt - 1
-  const int r0 = k0 + DB + blockIdx.x * DTHREADS;
-  if (r0 >= n) return;                       // whole CTA, before any barrier
-  load_tile_s(SD, stor(sys.E), n, n, n, k0, k0, 1);
-  if (threadIdx.x < DB)
-    rinv[threadIdx.x] = to_ff(1.0 / re_(ff_to_t(stor(sys.E)[size_t(k0 + threadIdx.x) * n + k0 + threadIdx.x])));
+  FT* E = stor(sys.E);
+  load_tile_s(SA, E, n, n, n, it * DB, k0, 0);
+  const FT* Dr = stor(sys.D) + size_t(kt) * DB * DB;
+  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS)       // SB[k][c] = conj(D[c][k])
+    SB[(e % DB) * DLD + e / DB] = ff_conj(Dr[e]);
   __syncthreads();
-  const int r = r0 + threadIdx.x;
-  if (r < n) {
-    FT x[DB];
-    FT* row = stor(sys.E) + size_t(r) * n + k0;
+  const int tr = threadIdx.x >> 3, tc = threadIdx.x & 7;
+  FA acc[4] = {};
+  tile_mac_ff<false>(acc, SA, SB, tr, tc);
+  const int R = it * DB + tr;
+  if (R < n) {
 #pragma unroll
-    for (int c = 0; c < DB; ++c) x[c] = row[c];
-#pragma unroll
-    for (int c = 0; c < DB; ++c) {
-      FA acc = ff_acc(x[c]);
-#pragma unroll
-      for (int k = 0; k < c; ++k) ff_csubmul_conj(acc, x[k], SD[c * DLD + k]);
-      x[c] = ff_scale(ff_renorm_t(acc), rinv[c]);
-    }
-#pragma unroll
-    for (int c = 0; c < DB; ++c) row[c] = x[c];
+    for (int b = 0; b < 4; ++b) E[size_t(R) * n + k0 + tc + 8 * b] = ff_renorm_t(acc[b]);
   }
 }
 
@@ -787,6 +763,7 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
                                 const DeviceCtx& ctx) {
   const size_t smem_u = 2 * DB * DLD * sizeof(T);
   int rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_chol_update<T>), smem_u, ctx.device);
+  if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_chol_panel<T>), smem_u, ctx.device);
   if (rc) return rc;
   int nmax = 0;
   for (int i = 0; i < nsys; ++i) nmax = std::max(nmax, batch.s[i].n);
@@ -796,12 +773,10 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
   for (int kt = 0; kt < ntmax; ++kt) {
     k_chol_diag<T><<<unsigned(nsys), DTHREADS, 0, s>>>(batch, kt, ctx.status);
     GW_LAUNCH_CHECK("k_chol_diag");
-    const int rows = nmax - (kt + 1) * DB;
-    if (rows <= 0) continue;
-    const unsigned pb = unsigned((rows + DTHREADS - 1) / DTHREADS);
-    k_chol_panel<T><<<dim3(pb, unsigned(nsys)), DTHREADS, 0, s>>>(batch, kt);
-    GW_LAUNCH_CHECK("k_chol_panel");
     const int64_t m = ntmax - kt - 1;
+    if (m <= 0) continue;
+    k_chol_panel<T><<<dim3(unsigned(m), unsigned(nsys)), DTHREADS, smem_u, s>>>(batch, kt);
+    GW_LAUNCH_CHECK("k_chol_panel");
     k_chol_update<T><<<dim3(unsigned(m * (m + 1) / 2), unsigned(nsys)), DTHREADS, smem_u, s>>>(batch, kt);
     GW_LAUNCH_CHECK("k_chol_update");
   }
@@ -834,13 +809,11 @@ static int launch_dielectric(std::vector<DieSysT<T>>& sys, cudaStream_t s, const
       if (rc) return rc;
     } else {
       // no-allocation entry: factorisation and inverse inside one CTA per system
-      k_dielectric<T><<<unsigned(nb_), DTHREADS, smem, s>>>(batch, ctx.status, true);
+      k_dielectric<T><<<unsigned(nb_), DTHREADS, smem, s>>>(batch, ctx.status);
       GW_LAUNCH_CHECK("k_dielectric");
     }
     if (by_columns) {
       const dim3 g2(static_cast<unsigned>(nb_), static_cast<unsigned>(ntmax));
-      k_dielectric_dinv<T><<<g2, DTHREADS, DB * DLD * sizeof(T), s>>>(batch);
-      GW_LAUNCH_CHECK("k_dielectric_dinv");
       k_dielectric_zcol<T><<<g2, DTHREADS, smem_w, s>>>(batch);
       GW_LAUNCH_CHECK("k_dielectric_zcol");
     }
