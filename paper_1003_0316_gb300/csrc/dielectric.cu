@@ -5,20 +5,21 @@
 //   Z   = L^{-1}                  blocked triangular inversion
 //   W^c = v^1/2 (Z^H Z - 1) v^1/2
 //
-// The caller-workspace entry points factorise a workspace copy of eps right-looking over many
-// CTAs (per 32-wide panel: the diagonal block and its inverse, the panel below it, the trailing
-// update of the lower 32x32 tiles), invert the factor by block columns (one CTA per (system, block
-// column) for the forward substitution of that column) and form W^c with one CTA per (system,
-// 32-row block), so every phase uses every SM; each thread owns one row and four columns of a
-// 32x32 tile staged in shared memory. About 4 N^3 real flops per system (N^3/6 complex
-// multiply-adds per phase). Storage and arithmetic are float-float on the FP32 pipe, which GB300
-// executes 64 times faster than FP64 (see FF below): about 2^-48 relative per operation; P, v and
-// W^c are FP64. The no-allocation entry point keeps the factorisation and the inverse inside one
-// CTA per system, in FP64.
+// The caller-workspace entry points factorise a workspace copy of eps over many CTAs (per 32-wide
+// panel: the diagonal block and its inverse, the panel below it, the trailing update of the lower
+// 32x32 tiles), invert the factor by block columns and form W^c with one CTA per (system, 32-row
+// block); each thread owns one row and four columns of a 32x32 tile staged in shared memory. About
+// 4 N^3 real flops per system (N^3/6 complex multiply-adds per phase). Storage and arithmetic are
+// float-float on the FP32 pipe, which GB300 executes 64 times faster than FP64 (see FF below): about
+// 2^-48 relative per operation; P, v and W^c are FP64. For larger systems all products outside the
+// diagonal 128-blocks and the current 128-column panel run on the tensor cores (DzChunk below). The
+// no-allocation entry point keeps the factorisation and the inverse inside one CTA per system, in
+// FP64.
 #include <vector>
 #include <algorithm>
 #include <mutex>
 
+#include "fp64_slices.cuh"
 #include "gw_internal.cuh"
 
 namespace gw {
@@ -46,6 +47,8 @@ struct DieSysT {
 // scalar operations for the complex and the real systems
 __device__ __forceinline__ double re_(double2 a) { return a.x; }
 __device__ __forceinline__ double re_(double a) { return a; }
+__device__ __forceinline__ double im_(double2 a) { return a.y; }
+__device__ __forceinline__ double im_(double) { return 0.0; }
 __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double cconj(double a) { return a; }
 __device__ __forceinline__ void cfma(double2& acc, double2 a, double2 b) {
@@ -130,6 +133,23 @@ __device__ __forceinline__ FF to_ff(double x) {
   const float h = __double2float_rn(x);
   return FF{h, __double2float_rn(x - double(h))};
 }
+// to_ff by integer arithmetic (each FP64 conversion occupies the FP64 pipe like a multiply-add): h
+// from the magnitude rounded to 24 bits (to nearest, ties to even), l from the remaining bits, whose
+// integer difference is exact. l of a value below 2^-73 is zero.
+__device__ __forceinline__ FF split_ff(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x)) & 0x7fffffffffffffffull;
+  const unsigned long long hb = (b + 0x0fffffffull + ((b >> 29) & 1ull)) & ~0x1fffffffull;
+  const int ex = int(b >> 52);                                   // biased by 1023
+  const uint32_t sign = static_cast<uint32_t>(__double2hiint(x)) & 0x80000000u;
+  const long long hf = static_cast<long long>(hb >> 29) - (896ll << 23);
+  const uint32_t hbits = hf < 0x00800000ll ? 0u : hf > 0x7f800000ll ? 0x7f800000u : uint32_t(hf);
+  const float d = float(int(static_cast<long long>(b) - static_cast<long long>(hb)));
+  const int se = ex - 1023 - 52 + 127;                           // 2^(e - 52)
+  const float l = hbits == 0u || se < 1 ? 0.0f : d * __int_as_float(se << 23);
+  return FF{__uint_as_float(hbits | sign), __uint_as_float(__float_as_uint(l) ^ sign)};
+}
+__device__ __forceinline__ FF split_ff_t(double x) { return split_ff(x); }
+__device__ __forceinline__ FFC split_ff_t(double2 x) { return FFC{split_ff(x.x), split_ff(x.y)}; }
 __device__ __forceinline__ FF to_ff_t(double x) { return to_ff(x); }
 __device__ __forceinline__ FFC to_ff_t(double2 x) { return FFC{to_ff(x.x), to_ff(x.y)}; }
 __device__ __forceinline__ FF ff_neg(FF x) { return FF{-x.h, -x.l}; }
@@ -530,9 +550,10 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_w(const DieBatchT<T> ba
 // substitutions L Z_c = I_c); the diagonal blocks D_r were inverted by k_chol_diag.
 // One CTA per (system, block column c): for r = c, c + 1, ...
 //   Z[r][c] = D_r (delta_rc - sum_{k = c}^{r-1} L[r][k] Z[k][c])
+// (with a group, only the rows of the column's group of blocks: the inverses of the diagonal groups)
 // with the earlier blocks Z[k][c] of the same column read back from global memory.
 template <typename T>
-__global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T> batch) {
+__global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T> batch, int group) {
   using FT = typename FFOf<T>::tile;
   using FA = typename FFOf<T>::acc;
   extern __shared__ __align__(16) unsigned char dsm_raw[];
@@ -547,7 +568,8 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T>
   const int tr = tid >> 3, tc = tid & 7;
   StorOf<T>* Z = stor(sys.Z);
   const StorOf<T>* L = stor(sys.E);
-  for (int r = c; r < nt; ++r) {
+  const int r_end = group ? min(nt, (c / group + 1) * group) : nt;
+  for (int r = c; r < r_end; ++r) {
     FT out[4] = {FT{}, FT{}, FT{}, FT{}};
     if (r == c) {
       const FT* Dr = stor(sys.D) + size_t(r) * DB * DB;
@@ -593,9 +615,11 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T>
 // SM takes part however few systems there are (20 systems of N_b = 4096 would leave 132 of
 // 152 SMs idle with one CTA per system).
 
-// eps = 1 - v^1/2 P v^1/2 over the full matrix: grid (32-row blocks, system); the square roots
-// of v are taken once per row and column block (FP64 square roots are costly on GB300's FP64
-// pipe) and kept in shared memory
+// the lower triangle of eps = 1 - v^1/2 P v^1/2 (what the factorisation reads), with the whole of P
+// checked for non-finite values: grid (32-row blocks, system). Three FP64 multiplications per
+// complex entry; the square roots of v are taken once per row and column block and the split into
+// float-float is integer work, since the FP64 pipe set the pace (128 systems of N_b = 600, the full
+// matrix with FP64 conversions: 1.28 ms).
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS) k_eps_fill(const DieBatchT<T> batch, unsigned* status) {
   __shared__ double svr[DB], svc[DTHREADS];
@@ -605,19 +629,29 @@ __global__ void __launch_bounds__(DTHREADS) k_eps_fill(const DieBatchT<T> batch,
   if (r0 >= n) return;                       // whole CTA, before any barrier
   const int tid = threadIdx.x;
   if (tid < DB) svr[tid] = r0 + tid < n ? sqrt(sys.v[r0 + tid]) : 0.0;
-  bool bad = false;
+  // exponent bits all ones: infinite or NaN
+  auto bad_of = [](double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; };
+  bool bad = tid < DB && r0 + tid < n && bad_of(sys.v[r0 + tid]);
   for (int c0 = 0; c0 < n; c0 += DTHREADS) {
     __syncthreads();                          // the previous chunk's svc is read
     svc[tid] = c0 + tid < n ? sqrt(sys.v[c0 + tid]) : 0.0;
     __syncthreads();
     const int c = c0 + tid;
     if (c >= n) continue;
-    for (int rr = 0; rr < DB && r0 + rr < n; ++rr) {
+    const double sc = svc[tid];
+#pragma unroll 4
+    for (int rr = 0; rr < DB; ++rr) {
+      if (r0 + rr >= n) break;
       const size_t e = size_t(r0 + rr) * n + c;
-      T x = scal(from_c<T>(sys.P[e]), -(svr[rr] * svc[tid]));
+      const T p = from_c<T>(sys.P[e]);
+      if (c > r0 + rr) {
+        bad = bad || bad_of(re_(p)) || bad_of(im_(p));
+        continue;
+      }
+      T x = scal(p, -(svr[rr] * sc));
       if (r0 + rr == c) x = add_re(x, 1.0);
-      if (!fin(x)) bad = true;
-      stor(sys.E)[e] = to_ff_t(x);
+      bad = bad || bad_of(re_(x)) || bad_of(im_(x));
+      stor(sys.E)[e] = split_ff_t(x);
     }
   }
   if (bad) raise_status(status, ST_ENONFINITE);
@@ -719,7 +753,7 @@ __global__ void __launch_bounds__(DTHREADS) k_chol_panel(const DieBatchT<T> batc
 // step 3: the trailing update A_ij -= L_ik L_jk^H for kt < j <= i (lower tiles; the diagonal
 // tiles keep their lower triangle); grid (tiles of the largest system, system)
 template <typename T>
-__global__ void __launch_bounds__(DTHREADS) k_chol_update(const DieBatchT<T> batch, int kt) {
+__global__ void __launch_bounds__(DTHREADS) k_chol_update(const DieBatchT<T> batch, int kt, int jend) {
   using FT = typename FFOf<T>::tile;
   using FA = typename FFOf<T>::acc;
   extern __shared__ __align__(16) unsigned char dsm_raw[];
@@ -729,13 +763,21 @@ __global__ void __launch_bounds__(DTHREADS) k_chol_update(const DieBatchT<T> bat
   const int n = sys.n, nt = (n + DB - 1) / DB;
   const int m = nt - kt - 1;                 // trailing block rows
   const int64_t t = blockIdx.x;
-  if (m <= 0 || t >= int64_t(m) * (m + 1) / 2) return;   // whole CTA, before any barrier
-  // t -> (ii, jj), 0 <= jj <= ii < m, row by row
-  int ii = int((sqrt(8.0 * double(t) + 1.0) - 1.0) * 0.5);
-  while (int64_t(ii + 1) * (ii + 2) / 2 <= t) ++ii;
-  while (int64_t(ii) * (ii + 1) / 2 > t) --ii;
-  const int jj = int(t - int64_t(ii) * (ii + 1) / 2);
-  const int it = kt + 1 + ii, jt = kt + 1 + jj;
+  int it, jt;
+  if (jend < nt) {                           // tile columns kt + 1 .. jend - 1 only
+    int u = int(t);
+    for (jt = kt + 1; jt < jend && u >= nt - jt; ++jt) u -= nt - jt;
+    if (jt >= jend) return;                  // whole CTA, before any barrier
+    it = jt + u;
+  } else {
+    if (m <= 0 || t >= int64_t(m) * (m + 1) / 2) return;   // whole CTA, before any barrier
+    // t -> (ii, jj), 0 <= jj <= ii < m, row by row
+    int ii = int((sqrt(8.0 * double(t) + 1.0) - 1.0) * 0.5);
+    while (int64_t(ii + 1) * (ii + 2) / 2 <= t) ++ii;
+    while (int64_t(ii) * (ii + 1) / 2 > t) --ii;
+    it = kt + 1 + ii;
+    jt = kt + 1 + int(t - int64_t(ii) * (ii + 1) / 2);
+  }
   const int k0 = kt * DB;
   const int tid = threadIdx.x, tr = tid >> 3, tc = tid & 7;
   FT* E = stor(sys.E);
@@ -777,14 +819,523 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
     if (m <= 0) continue;
     k_chol_panel<T><<<dim3(unsigned(m), unsigned(nsys)), DTHREADS, smem_u, s>>>(batch, kt);
     GW_LAUNCH_CHECK("k_chol_panel");
-    k_chol_update<T><<<dim3(unsigned(m * (m + 1) / 2), unsigned(nsys)), DTHREADS, smem_u, s>>>(batch, kt);
+    k_chol_update<T><<<dim3(unsigned(m * (m + 1) / 2), unsigned(nsys)), DTHREADS, smem_u, s>>>(batch, kt, ntmax);
     GW_LAUNCH_CHECK("k_chol_update");
   }
   return GW_OK;
 }
 
+// ---- large systems: the products on the tensor cores ------------------------------------------
+// The float-float tile products take 52 FP32 operations per complex multiply-add and keep the FP32
+// pipe 80 % busy. For larger systems the products run as digit-slice products of 128 x 128 tiles on
+// the tensor cores instead (fp64_slices.cuh, k_oz_gemm_cplx: 56-bit digits, more than the 48 of
+// the float-float storage): the float-float operands are cut into slices, a launch forms the products
+// C1, C2, S of all systems' tiles, and k_dz_combine turns them into W^c or float-float blocks.
+
+// What to slice: blocks of 128 lines (columns of M, or rows with DZ_ROWS) and stages of 32 values
+// along each line, of a float-float matrix M (row-major n x n); DZ_LOWER: entries above the
+// diagonal count as zero, DZ_CONJ: the conjugate.
+enum : int { DZ_ROWS = 1, DZ_LOWER = 2, DZ_CONJ = 4 };
+struct DzSlice {
+  const void* M;            // FFC or FF entries
+  char* out;                // (set, block, stage) = (0, 0, 0)
+  float* mx;                // largest magnitude per line (block 0), zeroed before k_dz_max
+  int64_t set, blk;         // strides in bytes
+  int n, mode;
+  int blk0, nblk, st0, nst;
+};
+constexpr int DZ_MAX = 256;
+struct DzSliceBatch {
+  DzSlice j[DZ_MAX];
+};
+
+__device__ __forceinline__ FFC ff_cplx(FFC x) { return x; }
+__device__ __forceinline__ FFC ff_cplx(FF x) { return FFC{x, FF{0.0f, 0.0f}}; }
+
+// entry k of line `line`, or zero outside the matrix (and the triangle)
+template <typename FT>
+__device__ __forceinline__ FFC dz_entry(const DzSlice& J, int line, int k) {
+  const FT* M = static_cast<const FT*>(J.M);
+  const bool in = line < J.n && k < J.n &&
+                  (!(J.mode & DZ_LOWER) || ((J.mode & DZ_ROWS) ? k <= line : k >= line));
+  if (!in) return FFC{};
+  return ff_cplx((J.mode & DZ_ROWS) ? M[size_t(line) * J.n + k] : M[size_t(k) * J.n + line]);
+}
+
+// whether values k0 .. k0 + 31 of a block's lines are all above the diagonal (never read)
+__device__ __forceinline__ bool dz_empty(const DzSlice& J, int blk, int k0) {
+  return (J.mode & DZ_LOWER) && ((J.mode & DZ_ROWS) ? k0 >= (blk + 1) * OT : k0 + OKS <= blk * OT);
+}
+
+// largest magnitude of the parts per line, over 128 values: grid (blocks, value chunks, jobs)
+template <typename FT>
+__global__ void __launch_bounds__(OT) k_dz_max(const __grid_constant__ DzSliceBatch batch) {
+  const DzSlice& J = batch.j[blockIdx.z];
+  constexpr int SPB = OT / OKS;
+  if (int(blockIdx.x) >= J.nblk || int(blockIdx.y) * SPB >= J.nst) return;
+  const int line0 = (J.blk0 + blockIdx.x) * OT;
+  const int k0 = (J.st0 + int(blockIdx.y) * SPB) * OKS;
+  const int k1 = min(k0 + OT, (J.st0 + J.nst) * OKS);
+  if (dz_empty(J, J.blk0 + blockIdx.x, (J.mode & DZ_ROWS) ? k0 : k1 - OKS)) return;
+  auto mag = [](FFC x) { return fmaxf(fabsf(x.re.h), fabsf(x.im.h)); };
+  if (J.mode & DZ_ROWS) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = warp; i < OT; i += OT / 32) {
+      float m = 0.0f;
+      for (int k = k0 + lane; k < k1; k += 32) m = fmaxf(m, mag(dz_entry<FT>(J, line0 + i, k)));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) atomicMax(reinterpret_cast<int*>(J.mx) + line0 + i, __float_as_int(m));
+    }
+  } else {
+    const int line = line0 + threadIdx.x;
+    float m = 0.0f;
+    for (int k = k0; k < k1; ++k) m = fmaxf(m, mag(dz_entry<FT>(J, line, k)));
+    atomicMax(reinterpret_cast<int*>(J.mx) + line, __float_as_int(m));
+  }
+}
+
+// the slices: grid (stages, blocks x 4, jobs), four lanes per line
+template <typename FT>
+__global__ void __launch_bounds__(OT) k_dz_slice(const __grid_constant__ DzSliceBatch batch) {
+  const DzSlice& J = batch.j[blockIdx.z];
+  const int b = blockIdx.y >> 2;
+  if (int(blockIdx.x) >= J.nst || b >= J.nblk) return;
+  const int st = J.st0 + blockIdx.x, kc = threadIdx.x & 3;
+  if (dz_empty(J, J.blk0 + b, st * OKS)) return;
+  const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
+  const int line = (J.blk0 + b) * OT + n, k0 = st * OKS + kc * 8;
+  const int E = exponent_of(J.mx[line]);
+  char* out = J.out + (J.blk0 + b) * J.blk + int64_t(st) * OBLK;
+  long long xr[8], xi[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const FFC x = dz_entry<FT>(J, line, k0 + k);
+    xr[k] = fixed_f32(x.re.h, E) + fixed_f32(x.re.l, E);
+    if constexpr (sizeof(FT) == sizeof(FFC)) {
+      const long long v = fixed_f32(x.im.h, E) + fixed_f32(x.im.l, E);
+      xi[k] = (J.mode & DZ_CONJ) ? -v : v;
+    }
+  }
+  uint32_t w[OSL][4];
+  fixed_digits8(xr, w);
+  store_digits(out, n, kc, w);
+  if constexpr (sizeof(FT) == sizeof(FFC)) {
+    fixed_digits8(xi, w);
+    store_digits(out + J.set, n, kc, w);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) xi[k] += xr[k];
+    fixed_digits8(xi, w);
+    store_digits(out + 2 * J.set, n, kc, w);
+  }
+}
+
+// What becomes of the product tiles out_ab of one problem (rows I of a, columns J of b):
+//   DZ_W:    W^c_IJ = sqrt(v_I v_J) (out_IJ - delta_IJ) for I <= J, and its Hermitian mirror
+//   DZ_SUB:  M_IJ -= conj(out_IJ) for I >= J
+//   DZ_PUT:  M_IJ = conj(out_IJ);  DZ_NEG: M_IJ = -out_IJ
+struct DzCombine {
+  const float2* G;
+  void* M;                  // float-float matrix, row-major n x n
+  double2* Wc;
+  const double* v;
+  int n, nprod, ntile;
+  int a0, a1, b0, b1, flags;
+};
+constexpr int DZC_MAX = 256;
+struct DzCombineBatch {
+  DzCombine j[DZC_MAX];
+};
+enum : int { DZ_W, DZ_SUB, DZ_PUT, DZ_NEG };
+template <typename FT> __device__ __forceinline__ FT ff_from(FFC x);
+template <> __device__ __forceinline__ FFC ff_from<FFC>(FFC x) { return x; }
+template <> __device__ __forceinline__ FF ff_from<FF>(FFC x) { return x.re; }
+
+__device__ __forceinline__ FF ff_load(float2 x) { return FF{x.x, x.y}; }
+
+template <typename FT, int WHAT>
+__global__ void __launch_bounds__(256) k_dz_combine(const __grid_constant__ DzCombineBatch batch) {
+  constexpr bool CPLX = sizeof(FT) == sizeof(FFC);
+  const DzCombine& J = batch.j[blockIdx.y];
+  const int t = blockIdx.x;
+  if (t >= J.ntile) return;                  // whole CTA, before any barrier
+  OzC L;
+  L.a0 = J.a0;
+  L.a1 = J.a1;
+  L.b0 = J.b0;
+  L.b1 = J.b1;
+  L.flags = J.flags;
+  int a, b;
+  oz_tile(L, t, a, b);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = J.n;
+  __shared__ double2 sW[32][33];             // a 32 x 32 block, transposed (FP64 W^c or float-float)
+  __shared__ double sv[2][OT];               // square roots of v of the tile's rows and columns
+  FFC (*sF)[33] = reinterpret_cast<FFC(*)[33]>(&sW[0][0]);
+  if constexpr (WHAT == DZ_W) {
+    const int g = (threadIdx.x < OT ? a : b) * OT + (threadIdx.x & (OT - 1));
+    sv[threadIdx.x / OT][threadIdx.x & (OT - 1)] = g < n ? sqrt(J.v[g]) : 0.0;
+    __syncthreads();
+  }
+  const size_t pstride = size_t(J.ntile) * OT * OT;
+  const float2* G = J.G + size_t(t) * OT * OT;
+  for (int s = 0; s < 16; ++s) {
+    const int rl = (s & 3) * 32, cl = (s >> 2) * 32, r0 = a * OT + rl, c0 = b * OT + cl;
+    if (r0 >= n || c0 >= n) continue;                        // whole CTA
+    if (WHAT == DZ_W && r0 > c0 + 31) continue;
+    if (WHAT == DZ_SUB && r0 + 31 < c0) continue;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int cc = warp + 8 * i, I = r0 + lane, Jc = c0 + cc;
+      const size_t e = size_t(cl + cc) * OT + rl + lane;
+      FFC out;
+      if constexpr (CPLX) {
+        const FF c1 = ff_load(G[e]), c2 = ff_load(G[pstride + e]), ss = ff_load(G[2 * pstride + e]);
+        out.re = ff_sub_acc(ff_sub_acc(ss, ff_acc(c1)), ff_acc(c2));
+        out.im = ff_sub_acc(c1, ff_acc(c2));
+      } else {
+        out.re = ff_load(G[e]);
+        out.im = FF{0.0f, 0.0f};
+      }
+      if constexpr (WHAT == DZ_W) {
+        double2 x = make_double2(double(out.re.h) + double(out.re.l), 0.0);
+        if (CPLX && I != Jc) x.y = double(out.im.h) + double(out.im.l);
+        if (I == Jc) x.x -= 1.0;
+        const double sc = sv[0][rl + lane] * sv[1][cl + cc];
+        x = make_double2(x.x * sc, x.y * sc);
+        if (I < n && Jc < n && I <= Jc)
+          J.Wc[size_t(Jc) * n + I] = make_double2(x.x, -x.y);   // the mirror, lanes along I
+        sW[cc][lane] = x;
+      } else {
+        sF[cc][lane] = out;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {                            // lanes along J
+      const int rr = warp + 8 * i, Ir = r0 + rr, Jc = c0 + lane;
+      if (Ir >= n || Jc >= n) continue;
+      if constexpr (WHAT == DZ_W) {
+        if (Ir <= Jc) J.Wc[size_t(Ir) * n + Jc] = sW[lane][rr];
+      } else {
+        const FFC o = sF[lane][rr];
+        FT* m = static_cast<FT*>(J.M) + size_t(Ir) * n + Jc;
+        if (WHAT == DZ_SUB) {
+          if (Ir >= Jc) *m = ff_sub_acc_t(*m, ff_acc(ff_from<FT>(ff_conj(o))));
+        } else if (WHAT == DZ_PUT) {
+          *m = ff_from<FT>(ff_conj(o));
+        } else {
+          *m = ff_from<FT>(ff_negate(o));
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Systems that take this path, and the slice workspace of one of them. Chunks of systems share a
+// launch while their slices stay within DZ_BUDGET. Float-float tiles against slices, whole solve:
+// complex N = 200 (20 systems) 0.93 / 1.00 ms, 300 (30) 2.07 / 1.97, 450 (32) 5.54 / 3.33, 600 (128)
+// 30.3 / 12.3, 2048 (2) 39.8 / 9.9; real N = 333 (32) 1.16 / 1.38, 600 (128) 9.72 / 5.63, 1100 (3)
+// 5.6 / 3.5 (a real product is a third of a complex one, but its slicing costs half).
+constexpr int DZ_MIN_N = 257, DZ_MIN_N_REAL = 449;
+constexpr size_t DZ_BUDGET = size_t(6) << 30;
+struct DzPlan {
+  int nbb, nst, nset, levels, ntile;
+  size_t b_x, b_mx, b_g;
+  DzPlan(int n, bool cplx) {
+    nbb = (n + OT - 1) / OT;
+    nst = (n + OKS - 1) / OKS;
+    nset = cplx ? 3 : 1;
+    levels = 0;
+    while ((1 << levels) < nbb) ++levels;
+    ntile = oz_tiles(0, nbb, 0, nbb, OZC_UPPER);
+    b_x = ws_round(size_t(nset) * nbb * nst * OBLK);            // one operand's slices
+    b_mx = size_t(2 + 3 * levels) * nbb * OT * sizeof(float);   // magnitudes: L, Z, per level Z11, T, Z22
+    b_g = ws_round(size_t(nset) * ntile * OT * OT * sizeof(float2));
+  }
+  size_t total() const { return 2 * b_x + b_mx + 256 + b_g; }
+  int64_t set() const { return int64_t(nbb) * nst * OBLK; }
+  int64_t blk() const { return int64_t(nst) * OBLK; }
+};
+static bool dz_takes(int n, bool cplx) { return n >= (cplx ? DZ_MIN_N : DZ_MIN_N_REAL); }
+
+// slice workspace of a list of systems: every chunk stays within the budget or is one system
+static size_t dz_workspace(const std::vector<int>& ns, bool cplx, int sm) {
+  size_t all = 0, one = 0;
+  for (int n : ns) {
+    const size_t b = DzPlan(n, cplx).total();
+    all += b;
+    one = std::max(one, b);
+  }
+  return std::min(all, std::max(one, DZ_BUDGET)) + oz_sum_bytes(sm);
+}
+
+template <typename FT>
+static int dz_launch_slices(const std::vector<DzSlice>& jobs, cudaStream_t s, bool find_max) {
+  for (size_t j0 = 0; j0 < jobs.size(); j0 += DZ_MAX) {
+    const int n = int(std::min<size_t>(DZ_MAX, jobs.size() - j0));
+    DzSliceBatch b;
+    int nblk = 0, nst = 0;
+    for (int i = 0; i < n; ++i) {
+      b.j[i] = jobs[j0 + i];
+      nblk = std::max(nblk, b.j[i].nblk);
+      nst = std::max(nst, b.j[i].nst);
+    }
+    if (nblk == 0 || nst == 0) continue;
+    constexpr int SPB = OT / OKS;
+    if (find_max) {
+      k_dz_max<FT><<<dim3(unsigned(nblk), unsigned((nst + SPB - 1) / SPB), unsigned(n)), OT, 0, s>>>(b);
+      GW_LAUNCH_CHECK("k_dz_max");
+    }
+    k_dz_slice<FT><<<dim3(unsigned(nst), unsigned(4 * nblk), unsigned(n)), OT, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_dz_slice");
+  }
+  return GW_OK;
+}
+
+template <typename FT, int WHAT>
+static int dz_launch_combine(const std::vector<DzCombine>& jobs, cudaStream_t s) {
+  for (size_t j0 = 0; j0 < jobs.size(); j0 += DZC_MAX) {
+    const int n = int(std::min<size_t>(DZC_MAX, jobs.size() - j0));
+    DzCombineBatch b;
+    int nt = 0;
+    for (int i = 0; i < n; ++i) {
+      b.j[i] = jobs[j0 + i];
+      nt = std::max(nt, b.j[i].ntile);
+    }
+    k_dz_combine<FT, WHAT><<<dim3(unsigned(nt), unsigned(n)), 256, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_dz_combine");
+  }
+  return GW_OK;
+}
+
+// magnitudes of the rows of L: |L_ik| <= sqrt(eps_ii), from the diagonal of eps
+template <typename FT>
+__global__ void k_dz_diag(const __grid_constant__ DzSliceBatch batch) {
+  const DzSlice& J = batch.j[blockIdx.y];
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < J.n) J.mx[i] = sqrtf(fmaxf(ff_re(static_cast<const FT*>(J.M)[size_t(i) * J.n + i]).h, 0.0f));
+}
+
+// One chunk of large systems from eps to W^c:
+//   Cholesky, left-looking over panels of 128 columns: the panel's rows take the products with all
+//     columns before them (slices of L, cut once per panel; rows scaled by sqrt(eps_ii)), then the
+//     panel is factorised with the 32-wide float-float steps;
+//   Z = L^{-1}: the diagonal 128-blocks in float-float, then doubling: for neighbouring diagonal
+//     groups with inverses Z11, Z22 the block below is Z21 = -Z22 (L21 Z11);
+//   W^c from Z^H Z.
 template <typename T>
-static int launch_dielectric(std::vector<DieSysT<T>>& sys, cudaStream_t s, const DeviceCtx& ctx) {
+struct DzChunk {
+  using FT = StorOf<T>;
+  static constexpr bool CPLX = sizeof(FT) == sizeof(FFC);
+  struct Sys {
+    DieSysT<T> S;
+    DzPlan p;
+    char *X1, *X2;          // slices of row operands (L, then Z22) and column operands (Z11, T, Z)
+    float2* G;
+    float* mx;              // [2 + 3 levels][128 nbb]
+    float* mag(int i) const { return mx + size_t(i) * p.nbb * OT; }
+  };
+  std::vector<Sys> sys;
+  float* ssum;
+  cudaStream_t s;
+  const DeviceCtx& ctx;
+
+  DzChunk(float* ss, cudaStream_t st, const DeviceCtx& c) : ssum(ss), s(st), ctx(c) {}
+
+  int place(const std::vector<DieSysT<T>>& list, WsCursor cur) {
+    size_t mxb = 0;
+    for (const DieSysT<T>& S : list) mxb += DzPlan(S.n, CPLX).b_mx;
+    float* mx = static_cast<float*>(cur.take(mxb));
+    if (!mx) return set_error(GW_EWORKSPACE, "internal: dielectric slice workspace too small");
+    GW_CUDA_TRY(cudaMemsetAsync(mx, 0, mxb, s));
+    for (const DieSysT<T>& S : list) {
+      Sys y{S, DzPlan(S.n, CPLX), nullptr, nullptr, nullptr, mx};
+      mx += y.p.b_mx / sizeof(float);
+      y.X1 = static_cast<char*>(cur.take(y.p.b_x));
+      y.X2 = static_cast<char*>(cur.take(y.p.b_x));
+      y.G = static_cast<float2*>(cur.take(y.p.b_g));
+      if (!y.X1 || !y.X2 || !y.G)
+        return set_error(GW_EWORKSPACE, "internal: dielectric slice workspace too small");
+      sys.push_back(y);
+    }
+    return GW_OK;
+  }
+  static DzSlice slice(const Sys& y, const T* M, char* out, float* mx, int mode, int blk0, int nblk,
+                       int st0, int nst) {
+    DzSlice j{};
+    j.M = M;
+    j.out = out;
+    j.mx = mx;
+    j.set = y.p.set();
+    j.blk = y.p.blk();
+    j.n = y.S.n;
+    j.mode = mode;
+    j.blk0 = blk0;
+    j.nblk = nblk;
+    j.st0 = st0;
+    j.nst = nst;
+    return j;
+  }
+  static OzC product(const Sys& y, const char* X, const float* mx, const char* Y, const float* my, int a0,
+                     int a1, int b0, int b1, int k0, int k1, int flags) {
+    OzC q{};
+    q.X = X;
+    q.Y = Y;
+    q.mx = mx;
+    q.my = my;
+    q.G = y.G;
+    q.xset = q.yset = y.p.set();
+    q.xblk = q.yblk = y.p.blk();
+    q.a0 = a0;
+    q.a1 = a1;
+    q.b0 = b0;
+    q.b1 = b1;
+    q.k0 = k0;
+    q.k1 = k1;
+    q.flags = flags;
+    q.nprod = y.p.nset;
+    q.ntile = oz_tiles(a0, a1, b0, b1, flags);
+    return q;
+  }
+  static DzCombine combine(const Sys& y, const OzC& q, T* M) {
+    DzCombine c{};
+    c.G = q.G;
+    c.M = M;
+    c.Wc = y.S.Wc;
+    c.v = y.S.v;
+    c.n = y.S.n;
+    c.nprod = q.nprod;
+    c.ntile = q.ntile;
+    c.a0 = q.a0;
+    c.a1 = q.a1;
+    c.b0 = q.b0;
+    c.b1 = q.b1;
+    c.flags = q.flags;
+    return c;
+  }
+  template <int WHAT>
+  int run(const std::vector<OzC>& pr, const std::vector<DzCombine>& cb) {
+    if (pr.empty()) return GW_OK;
+    int rc = oz_cplx(pr.data(), int(pr.size()), ssum, s, ctx);
+    return rc ? rc : dz_launch_combine<FT, WHAT>(cb, s);
+  }
+
+  static constexpr int SPB = OT / OKS;       // stages per 128-block
+  static constexpr int TPB = OT / DB;        // 32-blocks per 128-block
+
+  int cholesky(const DieBatchT<T>& batch, int ntmax) {
+    const unsigned nsys = unsigned(sys.size());
+    const size_t smem_u = 2 * DB * DLD * sizeof(T);
+    int nmax = 0, nbbmax = 0;
+    std::vector<DzSlice> dg;
+    for (const Sys& y : sys) {
+      nmax = std::max(nmax, y.S.n);
+      nbbmax = std::max(nbbmax, y.p.nbb);
+      dg.push_back(slice(y, y.S.E, nullptr, y.mag(0), 0, 0, 0, 0, 0));
+    }
+    k_eps_fill<T><<<dim3(unsigned((nmax + DB - 1) / DB), nsys), DTHREADS, 0, s>>>(batch, ctx.status);
+    GW_LAUNCH_CHECK("k_eps_fill");
+    for (size_t j0 = 0; j0 < dg.size(); j0 += DZ_MAX) {
+      const unsigned n = unsigned(std::min<size_t>(DZ_MAX, dg.size() - j0));
+      DzSliceBatch b;
+      std::copy(dg.begin() + j0, dg.begin() + j0 + n, b.j);
+      k_dz_diag<FT><<<dim3(unsigned((nmax + 127) / 128), n), 128, 0, s>>>(b);
+      GW_LAUNCH_CHECK("k_dz_diag");
+    }
+    for (int kb = 0; kb < nbbmax; ++kb) {
+      std::vector<OzC> pr;
+      std::vector<DzCombine> cb;
+      std::vector<DzSlice> sl;
+      for (const Sys& y : sys) {
+        if (kb > 0 && kb < y.p.nbb) {
+          pr.push_back(product(y, y.X1, y.mag(0), y.X1, y.mag(0), kb, y.p.nbb, kb, kb + 1, 0, SPB * kb, 0));
+          cb.push_back(combine(y, pr.back(), y.S.E));
+        }
+        if (kb + 1 < y.p.nbb)
+          sl.push_back(slice(y, y.S.E, y.X1, y.mag(0), DZ_ROWS, kb + 1, y.p.nbb - kb - 1, SPB * kb, SPB));
+      }
+      int rc = run<DZ_SUB>(pr, cb);
+      if (rc) return rc;
+      for (int kt = TPB * kb; kt < std::min(ntmax, TPB * (kb + 1)); ++kt) {
+        k_chol_diag<T><<<nsys, DTHREADS, 0, s>>>(batch, kt, ctx.status);
+        GW_LAUNCH_CHECK("k_chol_diag");
+        const int m = ntmax - kt - 1;
+        if (m <= 0) continue;
+        k_chol_panel<T><<<dim3(unsigned(m), nsys), DTHREADS, smem_u, s>>>(batch, kt);
+        GW_LAUNCH_CHECK("k_chol_panel");
+        const int jend = TPB * (kb + 1);
+        int64_t tiles = 0;
+        for (int jt = kt + 1; jt < std::min(jend, ntmax); ++jt) tiles += ntmax - jt;
+        if (tiles == 0) continue;
+        k_chol_update<T><<<dim3(unsigned(tiles), nsys), DTHREADS, smem_u, s>>>(batch, kt, jend);
+        GW_LAUNCH_CHECK("k_chol_update");
+      }
+      if ((rc = dz_launch_slices<FT>(sl, s, false))) return rc;
+    }
+    return GW_OK;
+  }
+
+  // Z from the inverses of its diagonal 128-blocks
+  int inverse() {
+    int lmax = 0;
+    for (const Sys& y : sys) lmax = std::max(lmax, y.p.levels);
+    for (int l = 0; l < lmax; ++l) {
+      const int g = 1 << l;
+      std::vector<DzSlice> s1, s2;
+      std::vector<OzC> p1, p2;
+      std::vector<DzCombine> c1, c2;
+      for (const Sys& y : sys) {
+        if (l >= y.p.levels) continue;
+        float *m11 = y.mag(2 + 3 * l), *mt = y.mag(3 + 3 * l), *m22 = y.mag(4 + 3 * l);
+        int tile0 = 0;
+        for (int j = 0; j + g < y.p.nbb; j += 2 * g) {
+          const int e = std::min(j + 2 * g, y.p.nbb), h = j + g;   // groups [j, h) and [h, e)
+          const int ks1 = SPB * h, ks2 = std::min(SPB * e, y.p.nst);
+          // conj(L21 Z11) from L and conj(Z11); T = L21 Z11 goes where Z21 will be
+          s1.push_back(slice(y, y.S.Z, y.X2, m11, DZ_LOWER | DZ_CONJ, j, g, SPB * j, ks1 - SPB * j));
+          OzC q = product(y, y.X1, y.mag(0), y.X2, m11, h, e, j, h, SPB * j, ks1, OZC_KB);
+          q.G += size_t(tile0) * q.nprod * OT * OT;
+          p1.push_back(q);
+          c1.push_back(combine(y, q, y.S.Z));
+          // -Z22 T from conj(Z22) and T
+          s2.push_back(slice(y, y.S.Z, y.X2, mt, 0, j, g, ks1, ks2 - ks1));
+          s2.push_back(slice(y, y.S.Z, y.X1, m22, DZ_ROWS | DZ_LOWER | DZ_CONJ, h, e - h, ks1, ks2 - ks1));
+          q = product(y, y.X1, m22, y.X2, mt, h, e, j, h, ks1, ks2, OZC_KTOP);
+          q.G += size_t(tile0) * q.nprod * OT * OT;
+          p2.push_back(q);
+          c2.push_back(combine(y, q, y.S.Z));
+          tile0 += q.ntile;
+        }
+      }
+      int rc = dz_launch_slices<FT>(s1, s, true);
+      if (!rc) rc = run<DZ_PUT>(p1, c1);
+      if (!rc) rc = dz_launch_slices<FT>(s2, s, true);
+      if (!rc) rc = run<DZ_NEG>(p2, c2);
+      if (rc) return rc;
+    }
+    return GW_OK;
+  }
+
+  int screened() {
+    std::vector<DzSlice> sl;
+    std::vector<OzC> pr;
+    std::vector<DzCombine> cb;
+    for (const Sys& y : sys) {
+      sl.push_back(slice(y, y.S.Z, y.X2, y.mag(1), DZ_LOWER, 0, y.p.nbb, 0, y.p.nst));
+      pr.push_back(product(y, y.X2, y.mag(1), y.X2, y.mag(1), 0, y.p.nbb, 0, y.p.nbb, 0, y.p.nst,
+                           OZC_UPPER | OZC_KA | OZC_KB));
+      cb.push_back(combine(y, pr.back(), nullptr));
+    }
+    int rc = dz_launch_slices<FT>(sl, s, true);
+    return rc ? rc : run<DZ_W>(pr, cb);
+  }
+};
+
+// dz: the slice workspace (caller-workspace entry points); ssum: the slice products' scratch
+template <typename T>
+static int launch_dielectric(std::vector<DieSysT<T>>& sys, WsCursor dz, float* ssum, cudaStream_t s,
+                             const DeviceCtx& ctx) {
   const size_t smem = 3 * DB * DLD * sizeof(T);
   const size_t smem_w = 2 * DB * DLD * sizeof(T);
   {
@@ -792,49 +1343,75 @@ static int launch_dielectric(std::vector<DieSysT<T>>& sys, cudaStream_t s, const
     if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_dielectric_w<T, true>), smem_w, ctx.device);
     if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_dielectric_w<T, false>), smem_w, ctx.device);
     if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_dielectric_zcol<T>), smem_w, ctx.device);
+    if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_chol_update<T>), smem_w, ctx.device);
+    if (!rc) rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_chol_panel<T>), smem_w, ctx.device);
     if (rc) return rc;
   }
+  constexpr bool CPLX = sizeof(T) == sizeof(double2);
   const bool by_columns = !sys.empty() && sys[0].D != nullptr;
-  for (size_t b0 = 0; b0 < sys.size(); b0 += DMAXSYS) {
-    size_t nb_ = std::min<size_t>(DMAXSYS, sys.size() - b0);
+  for (size_t b0 = 0; b0 < sys.size();) {
+    // up to DMAXSYS systems; those of the sliced path apart from the others, within the slice budget
+    const bool sliced = by_columns && dz_takes(sys[b0].n, CPLX);
+    size_t nb_ = 0, bytes = 0;
     DieBatchT<T> batch;
     int ntmax = 1;
-    for (size_t i = 0; i < nb_; ++i) {
-      batch.s[i] = sys[b0 + i];
-      ntmax = std::max(ntmax, (batch.s[i].n + DB - 1) / DB);
+    while (b0 + nb_ < sys.size() && nb_ < DMAXSYS) {
+      const DieSysT<T>& S = sys[b0 + nb_];
+      if (by_columns && dz_takes(S.n, CPLX) != sliced) break;
+      if (sliced) {
+        const size_t need = DzPlan(S.n, CPLX).total();
+        if (nb_ > 0 && bytes + need > DZ_BUDGET) break;
+        bytes += need;
+      }
+      batch.s[nb_++] = S;
+      ntmax = std::max(ntmax, (S.n + DB - 1) / DB);
     }
-    if (by_columns) {
+    const dim3 g2(static_cast<unsigned>(nb_), static_cast<unsigned>(ntmax));
+    if (sliced) {
+      DzChunk<T> c(ssum, s, ctx);
+      int rc = c.place(std::vector<DieSysT<T>>(sys.begin() + b0, sys.begin() + b0 + nb_), dz);
+      if (!rc) rc = c.cholesky(batch, ntmax);
+      if (rc) return rc;
+      k_dielectric_zcol<T><<<g2, DTHREADS, smem_w, s>>>(batch, DzChunk<T>::TPB);
+      GW_LAUNCH_CHECK("k_dielectric_zcol");
+      rc = c.inverse();
+      if (!rc) rc = c.screened();
+      if (rc) return rc;
+    } else if (by_columns) {
       // caller workspace: the factorisation over many CTAs, then the inverse by block columns
       int rc = launch_cholesky_grid<T>(batch, int(nb_), ntmax, s, ctx);
       if (rc) return rc;
+      k_dielectric_zcol<T><<<g2, DTHREADS, smem_w, s>>>(batch, 0);
+      GW_LAUNCH_CHECK("k_dielectric_zcol");
+      k_dielectric_w<T, true><<<g2, DTHREADS, smem_w, s>>>(batch);
     } else {
       // no-allocation entry: factorisation and inverse inside one CTA per system
       k_dielectric<T><<<unsigned(nb_), DTHREADS, smem, s>>>(batch, ctx.status);
       GW_LAUNCH_CHECK("k_dielectric");
+      k_dielectric_w<T, false><<<g2, DTHREADS, smem_w, s>>>(batch);
     }
-    if (by_columns) {
-      const dim3 g2(static_cast<unsigned>(nb_), static_cast<unsigned>(ntmax));
-      k_dielectric_zcol<T><<<g2, DTHREADS, smem_w, s>>>(batch);
-      GW_LAUNCH_CHECK("k_dielectric_zcol");
-    }
-    if (by_columns)
-      k_dielectric_w<T, true><<<dim3(unsigned(nb_), unsigned(ntmax)), DTHREADS, smem_w, s>>>(batch);
-    else
-      k_dielectric_w<T, false><<<dim3(unsigned(nb_), unsigned(ntmax)), DTHREADS, smem_w, s>>>(batch);
     GW_LAUNCH_CHECK("k_dielectric_w");
+    b0 += nb_;
   }
   return GW_OK;
 }
 
+// E, Z, D of every system
 template <typename T>
 static size_t dielectric_ws_t(int nq, const int* nb, int nw) {
   size_t b = 0;
+  std::vector<int> large;
   for (int q = 0; q < nq; ++q) {
     size_t n = size_t(nb[q]);
     const size_t nt = (n + DB - 1) / DB;
-    b += size_t(nw) * ws_round((2 * n * n + nt * DB * DB) * sizeof(T));   // E, Z, D
+    b += size_t(nw) * ws_round((2 * n * n + nt * DB * DB) * sizeof(T));
+    if (dz_takes(nb[q], sizeof(T) == sizeof(double2))) large.insert(large.end(), nw, nb[q]);
   }
-  return b;
+  if (large.empty()) return b;
+  int sm = 152, dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
+  cudaGetLastError();
+  return b + dz_workspace(large, sizeof(T) == sizeof(double2), sm);
 }
 
 template <typename T>
@@ -861,7 +1438,14 @@ static int dielectric_t(int nq, const int* nb, int nw, const double* const* v,
       sys.push_back(d);
     }
   }
-  return launch_dielectric<T>(sys, s, ctx);
+  float* ssum = nullptr;
+  bool large = false;
+  for (int q = 0; q < nq; ++q) large = large || dz_takes(nb[q], sizeof(T) == sizeof(double2));
+  if (large) {
+    ssum = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));
+    if (!ssum) return set_error(GW_EWORKSPACE, "internal: dielectric workspace too small");
+  }
+  return launch_dielectric<T>(sys, cur, ssum, s, ctx);
 }
 
 size_t dielectric_workspace(int nq, const int* nb, int nw) {
@@ -929,7 +1513,7 @@ int dielectric_wc_noalloc(int nb, int nw, const double* v, const double* P, doub
       d.D = nullptr;
       d.n = nb;
     }
-    rc = launch_dielectric<double2>(sys, s, ctx);
+    rc = launch_dielectric<double2>(sys, WsCursor{nullptr, 0, 0}, nullptr, s, ctx);
     if (rc) return rc;
   }
   return GW_OK;

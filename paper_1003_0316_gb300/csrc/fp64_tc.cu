@@ -30,7 +30,7 @@
 // (where fixed-point slices would lose what FP64 keeps) sets a device flag: the sliced kernels
 // then return at once and the FP64 kernel, launched behind them and otherwise empty, does the work.
 //
-// Layout and roles of k_oz_gemm (384 threads, one persistent CTA per SM): 128 x 128 tiles; per stage
+// Layout and roles of k_oz_gemm_* (384 threads, one persistent CTA per SM): 128 x 128 tiles; per stage
 // (K = 32) 7 slices of A and of B, pre-split in global memory as 8 KB K-major, 64-byte-swizzled
 // tiles, copied by bulk async copies into two shared-memory stages of 112 KB, each in two parts
 // (slices 1-4 and 5-7). One warp issues the MMAs (both operands from shared memory). TMEM holds four
@@ -45,20 +45,13 @@
 #include <vector>
 
 #include "gw_internal.cuh"
+#include "fp64_slices.cuh"
 #include "fp64_tc.cuh"
 #include "tc_ptx.cuh"
 
 namespace gw {
 namespace {
 
-constexpr int OT = 128;                     // tile edge
-constexpr int OKS = 32;                     // K per stage
-constexpr int OSL = 7;                      // digit slices
-constexpr int SLB = OT * 64;                // one slice of one operand and stage: 8 KB
-constexpr int NHI = 4;                      // slices 1-4: the stage's first part
-constexpr int HIB = NHI * SLB, LOB = (OSL - NHI) * SLB;   // bytes of the parts, per operand
-constexpr int OBLK = HIB + LOB;             // one operand's stage
-constexpr int OSTAGE = 2 * OBLK;            // A 1-4, B 1-4, A 5-7, B 5-7
 constexpr int ONST = 2;                     // stages in shared memory
 constexpr int SBMAX = 256;                  // stages per superblock at most (K = 8192)
 constexpr int OTHREADS = 384;
@@ -68,10 +61,6 @@ static_assert(256 * REG_E + 128 * REG_P == OTHREADS * 168, "register split");
 constexpr uint64_t OWAIT = 2000000000ull;   // ns per bounded wait
 constexpr int CHROWS = 64;                  // rows per scale chunk (superblocks are multiples)
 constexpr float RATIO_MAX = 1024.0f;        // largest entry against the mean magnitude of a column
-
-__device__ __forceinline__ uint32_t swz64(int n, int kc) {
-  return uint32_t((n >> 3) * 512 + (n & 7) * 64 + ((kc ^ ((n & 7) >> 1)) << 4));
-}
 
 // One problem: a q point's polarization over a range of rows and frequencies, or (QF) the pair
 // coefficients of a range of pairs and frequencies.
@@ -110,43 +99,99 @@ struct OzBatch {
   int nq;
   int add;                  // G += instead of G =
 };
+struct OzCBatch {
+  OzC q[OZC_MAX];
+  int item0[OZC_MAX + 1];
+  float* s;
+  int nq;
+};
+static_assert(sizeof(OzCBatch) < 32000, "kernel parameter space");
+
+// k_oz_gemm's modes: polarization, quadratic form, complex products
+enum : int { OZ_POL, OZ_QUAD, OZ_CPLX };
+template <int MODE> struct OzBatchOf { using B = OzBatch; using P = OzProb; };
+template <> struct OzBatchOf<OZ_CPLX> { using B = OzCBatch; using P = OzC; };
+
+// One work item: its problem, operand slices (stage 0), stage range, stages per superblock, and the
+// indexes that its output needs.
+template <int MODE>
+struct OzItem {
+  const typename OzBatchOf<MODE>::P* L;
+  const char *a, *b;
+  int st0, st1, sbst;
+  int f, sp, bi, bj, kind;
+};
 
 // polarization: tiles of C = Mr^T D Mi (all) and S = (Mr+Mi)^T D (Mr+Mi) (upper), the layout of the
-// split-precision polarization; quadratic form: every (row block, column block)
-template <bool QF>
-__device__ __forceinline__ const OzProb& oz_item(const OzBatch& batch, int64_t item, int& f, int& sp,
-                                                 int& bi, int& bj, int& kind) {
+// split-precision polarization; quadratic form: every (row block, column block), whose column block
+// bj needs K < 128 (bj + 1). False: the FP64 kernel does this problem.
+template <int MODE>
+__device__ __forceinline__ bool oz_item(const OzBatch& batch, int64_t item, OzItem<MODE>& it) {
   int q = 0;
   while (q + 1 < batch.nq && item >= batch.item0[q + 1]) ++q;
   const OzProb& L = batch.q[q];
+  it.L = &L;
   item -= batch.item0[q];
   int u = int(item % L.ntile);
   item /= L.ntile;
-  f = int(item % L.nf);
-  sp = int(item / L.nf);
-  if (QF) {
-    bi = u % L.nbi;
-    bj = L.nbj - 1 - u / L.nbi;         // the longest items (K < 128 (bj + 1)) first
-    kind = 2;
-    return L;
+  it.f = int(item % L.nf);
+  it.sp = int(item / L.nf);
+  it.st0 = it.sp * L.sps * L.sbst;
+  it.st1 = min(L.nst, it.st0 + L.sps * L.sbst);
+  it.sbst = L.sbst;
+  if (MODE == OZ_QUAD) {
+    it.bi = u % L.nbi;
+    it.bj = L.nbj - 1 - u / L.nbi;      // the longest items first
+    it.kind = 2;
+    it.st1 = min(it.st1, (it.bj + 1) * (OT / OKS));
+    it.a = L.A + size_t(it.bi) * L.nst * OBLK;
+    it.b = L.B + size_t(it.f * L.nbj + it.bj) * L.nst * OBLK;
+  } else {
+    const int nbb = L.nbj;
+    if (u < nbb * nbb) {
+      it.bi = u % nbb;
+      it.bj = u / nbb;
+      it.kind = 0;
+    } else {
+      u -= nbb * nbb;
+      int bj = 0;
+      while (u > bj) {
+        u -= bj + 1;
+        ++bj;
+      }
+      it.bi = u + nbb;
+      it.bj = bj + nbb;
+      it.kind = 1;
+    }
+    it.a = L.A + size_t(it.f * 2 * nbb + it.bi) * L.nst * OBLK;
+    it.b = L.B + size_t(it.bj) * L.nst * OBLK;
   }
-  const int nbb = L.nbj;
-  if (u < nbb * nbb) {
-    bi = u % nbb;
-    bj = u / nbb;
-    kind = 0;
-    return L;
+  return !__ldg(L.flag);
+}
+// complex products: kind: the product, f: the tile's index, (bi, bj): the tile
+template <int MODE>
+__device__ __forceinline__ bool oz_item(const OzCBatch& batch, int64_t item, OzItem<MODE>& it) {
+  int lo = 0, hi = batch.nq - 1;        // the last problem that starts at or before the item
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (item >= batch.item0[mid]) lo = mid;
+    else hi = mid - 1;
   }
-  u -= nbb * nbb;
-  bj = 0;
-  while (u > bj) {
-    u -= bj + 1;
-    ++bj;
-  }
-  bi = u + nbb;
-  bj += nbb;
-  kind = 1;
-  return L;
+  const OzC& L = batch.q[lo];
+  it.L = &L;
+  const int u = int(item - batch.item0[lo]);
+  it.f = u / L.nprod;
+  it.kind = u - it.f * L.nprod;
+  it.sp = 0;
+  oz_tile(L, it.f, it.bi, it.bj);
+  const int sx = L.nprod == 1 ? 0 : it.kind, sy = L.nprod == 1 ? 0 : it.kind == 2 ? 2 : 1 - it.kind;
+  it.a = L.X + sx * L.xset + it.bi * L.xblk;
+  it.b = L.Y + sy * L.yset + it.bj * L.yblk;
+  constexpr int SPB = OT / OKS;         // stages per block
+  it.st0 = max(L.k0, max((L.flags & OZC_KA) ? SPB * it.bi : 0, (L.flags & OZC_KB) ? SPB * it.bj : 0));
+  it.st1 = (L.flags & OZC_KTOP) ? min(L.k1, SPB * (it.bi + 1)) : L.k1;
+  it.sbst = SBMAX;
+  return it.st1 > it.st0;
 }
 
 __device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
@@ -197,9 +242,8 @@ __device__ __forceinline__ int4 ld_exp4(const int* p) {
   return r;
 }
 
-template <bool QF>
-__global__ void __launch_bounds__(OTHREADS, 1)
-    k_oz_gemm(const __grid_constant__ OzBatch batch, unsigned* status) {
+template <int MODE>
+__device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch, unsigned* status) {
   constexpr uint32_t IDESC = tc::instr_desc(1u, OT, OT);
   extern __shared__ __align__(1024) char dsmem[];
   char* ring = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
@@ -231,13 +275,6 @@ __global__ void __launch_bounds__(OTHREADS, 1)
   tc::tc_fence_after();
   const uint32_t tmem = s_tmem;               // columns: D, C4, C3, C2 (128 each)
   const int64_t nitems = batch.item0[batch.nq];
-
-  // the stage range of an item (the quadratic form's column block bj needs K < 128 (bj + 1))
-  auto range = [&](const OzProb& L, int sp, int bj, int& st0, int& st1) {
-    st0 = sp * L.sps * L.sbst;
-    st1 = min(L.nst, st0 + L.sps * L.sbst);
-    if (QF) st1 = min(st1, (bj + 1) * (OT / OKS));
-  };
 
   if (warp < EPI_WARPS) {
     tc::setmaxnreg_inc<REG_E>();
@@ -317,15 +354,14 @@ __global__ void __launch_bounds__(OTHREADS, 1)
       return true;
     };
     for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x) {
-      int f, sp, bi, bj, kind;
-      const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
-      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
-      int st0, st1;
-      range(L, sp, bj, st0, st1);
+      OzItem<MODE> w;
+      if (!oz_item<MODE>(batch, item, w)) continue;
+      const auto& L = *w.L;
+      const int f = w.f, sp = w.sp, bi = w.bi, bj = w.bj, kind = w.kind;
       double qsum = 0.0;
       bool first = true;
-      for (int sb0 = st0; sb0 < st1 && !stop; sb0 += L.sbst) {
-        const int n = min(L.sbst, st1 - sb0);
+      for (int sb0 = w.st0; sb0 < w.st1 && !stop; sb0 += w.sbst) {
+        const int n = min(w.sbst, w.st1 - sb0);
 #pragma unroll
         for (int i = 0; i < 32; ++i) c[i] = d[i] = 0;
         bool fresh = true;                    // s is zero
@@ -359,46 +395,78 @@ __global__ void __launch_bounds__(OTHREADS, 1)
           }
         }
         if (stop) break;
+        if constexpr (MODE == OZ_CPLX) {
+          // the product tile in float-float: s + c + d renormalised, times 2^(EX + EY - 14)
+          const int ex = exponent_of(__ldg(L.mx + bi * OT + r)) - 14;
+          const float* my = L.my + bj * OT + c0;
+          float2* g = L.G + ((size_t(kind) * L.ntile + f) * OT + c0) * OT + r;
+          float s16[16];
+#pragma unroll
+          for (int i = 0; i < 64; ++i) {
+            if (i % 16 == 0) {                // 16 loads in flight (the volatile loads keep their order)
+#pragma unroll
+              for (int t = 0; t < 16; ++t) s16[t] = ld_f32(sp_s + (i + t) * OT);
+            }
+            const float sv = s16[i % 16];
+            const int e = ex + exponent_of(__ldg(my + i)), e1 = max(-126, min(127, e >> 1)),
+                      e2 = max(-126, min(127, e - e1));
+            const float f1 = __int_as_float((e1 + 127) << 23), f2 = __int_as_float((e2 + 127) << 23);
+            float cl, ch, dl, dh;
+            tc::f2_unpack(c[i / 2], cl, ch);
+            tc::f2_unpack(d[i / 2], dl, dh);
+            const float cv = i & 1 ? ch : cl, dv = i & 1 ? dh : dl;
+            const float h = __fadd_rn(sv, cv), b = __fsub_rn(h, sv);
+            const float lo = __fadd_rn(__fadd_rn(__fsub_rn(sv, __fsub_rn(h, b)), __fsub_rn(cv, b)), dv);
+            const float hh = __fadd_rn(h, lo);
+            g[size_t(i) * OT] = make_float2(__fmul_rn(__fmul_rn(hh, f1), f2),
+                                            __fmul_rn(__fmul_rn(__fsub_rn(lo, __fsub_rn(hh, h)), f1), f2));
+          }
+          continue;
+        } else {
         // the superblock in FP64: ((s + c) + d) 2^(EA + EB - 14)
-        const int sb = sb0 / L.sbst;
-        const int* eb = L.EB + (size_t(QF ? f * L.nbj + bj : bj) * L.nsb + sb) * OT + c0;
+        const int sb = sb0 / w.sbst;
+        const int* eb = L.EB + (size_t(MODE == OZ_QUAD ? f * L.nbj + bj : bj) * L.nsb + sb) * OT + c0;
         const int ea =
-            L.EA[(size_t(QF ? bi : f * 2 * L.nbj + bi) * L.nsb + sb) * OT + r] - 14 + 1023;
-        if (QF) {
+            L.EA[(size_t(MODE == OZ_QUAD ? bi : f * 2 * L.nbj + bi) * L.nsb + sb) * OT + r] - 14 + 1023;
+        if constexpr (MODE == OZ_QUAD) {
           // this row's part of x . (x U) over the tile's columns: x 2^(EA + EB - 14) by integer
           // exponent arithmetic, s and c against it in FP64, d (2^-40 of s) in FP32
           const int64_t p = int64_t(bi) * OT + r;
           const int64_t col = int64_t(bj) * OT + c0;
           if (p < L.nrow) {
             const double* xr = L.x + p * L.ncol + col;
-            float qd = 0.0f;
+            float qd = 0.0f, s16[16];
+            double x8[8];
 #pragma unroll
             for (int g4 = 0; g4 < 16; ++g4) {
               const int4 e4 = ld_exp4(eb + 4 * g4);
               const int e[4] = {e4.x, e4.y, e4.z, e4.w};
-              double x[4];
-              float sv[4];
+              if (g4 % 4 == 0) {
 #pragma unroll
-              for (int t = 0; t < 4; ++t) sv[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
+                for (int t = 0; t < 16; ++t) s16[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
+              }
+              if (g4 % 2 == 0) {
 #pragma unroll
-              for (int t = 0; t < 4; ++t) x[t] = col + 4 * g4 + t < L.ncol ? ld_f64(xr + 4 * g4 + t) : 0.0;
+                for (int t = 0; t < 8; ++t) x8[t] = col + 4 * g4 + t < L.ncol ? ld_f64(xr + 4 * g4 + t) : 0.0;
+              }
 #pragma unroll
               for (int t = 0; t < 4; ++t) {
                 const int i = 4 * g4 + t;
-                const int hi = __double2hiint(x[t]), xe = (hi >> 20) & 0x7ff;
+                const double xv = x8[4 * (g4 % 2) + t];
+                const int hi = __double2hiint(xv), xe = (hi >> 20) & 0x7ff;
                 const int ex = xe + ea - 1023 + e[t];
                 const bool z = xe == 0 || ex < 1;                  // zero or underflow
                 const double xs = z ? 0.0 : __hiloint2double(hi + ((ea - 1023 + e[t]) << 20),
-                                                             __double2loint(x[t]));
+                                                             __double2loint(xv));
                 float cl, ch, dl, dh;
                 tc::f2_unpack(c[i / 2], cl, ch);
                 tc::f2_unpack(d[i / 2], dl, dh);
-                qsum = fma(to_f64(sv[t]), xs, qsum);
+                qsum = fma(to_f64(s16[4 * (g4 % 4) + t]), xs, qsum);
                 qsum = fma(to_f64(i & 1 ? ch : cl), xs, qsum);
                 if (xe != 0 && ex >= 897 && ex <= 1120) {
                   const float xf = __int_as_float((hi & 0x80000000) | ((ex - 896) << 23) |
                                                   ((hi & 0xfffff) << 3) |
-                                                  int(uint32_t(__double2loint(x[t])) >> 29));
+                                                  int(uint32_t(__double2loint(xv)) >> 29));
                   qd = fmaf(i & 1 ? dh : dl, xf, qd);
                 } else {
                   qsum = fma(to_f64(i & 1 ? dh : dl), xs, qsum);   // outside the FP32 range
@@ -413,30 +481,33 @@ __global__ void __launch_bounds__(OTHREADS, 1)
           const int b0 = (kind ? bj - L.nbj : bj) * OT + c0;
           double* g = L.G + ((size_t(sp) * L.nf + f) * 2 + kind) * nbp * nbp + size_t(b0) * nbp + a;
           const bool add = batch.add || !first;
+          float s16[16];
 #pragma unroll
           for (int g4 = 0; g4 < 16; ++g4) {
+            if (g4 % 4 == 0) {
+#pragma unroll
+              for (int t = 0; t < 16; ++t) s16[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
+            }
             const int4 e4 = ld_exp4(eb + 4 * g4);
             const int e[4] = {e4.x, e4.y, e4.z, e4.w};
             double o[4] = {0.0, 0.0, 0.0, 0.0};
-            float sv[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) sv[t] = ld_f32(sp_s + (4 * g4 + t) * OT);
             if (add) {
 #pragma unroll
               for (int t = 0; t < 4; ++t) o[t] = ld_f64(g + size_t(4 * g4 + t) * nbp);
             }
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-              const double v = sum_f64(sv[t], c, d, 4 * g4 + t);
+              const double v = sum_f64(s16[4 * (g4 % 4) + t], c, d, 4 * g4 + t);
               g[size_t(4 * g4 + t) * nbp] = fma(v, __hiloint2double((ea + e[t]) << 20, 0), o[t]);
             }
           }
         }
+        }
         first = false;
       }
-      if (QF && !stop) {
+      if constexpr (MODE == OZ_QUAD) {
         const int64_t p = int64_t(bi) * OT + r;
-        if (p < L.nrow)
+        if (!stop && p < L.nrow)
           L.cpart[(size_t(f) * 2 * L.nbj + 2 * bj + (c0 ? 1 : 0)) * L.nrow + p] = qsum;
       }
     }
@@ -447,14 +518,10 @@ __global__ void __launch_bounds__(OTHREADS, 1)
       uint32_t g = 0;
       bool ok = true;
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        int f, sp, bi, bj, kind;
-        const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
-      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
-        int st0, st1;
-        range(L, sp, bj, st0, st1);
-        const char* a = L.A + size_t(QF ? bi : f * 2 * L.nbj + bi) * L.nst * OBLK;
-        const char* b = L.B + size_t(QF ? f * L.nbj + bj : bj) * L.nst * OBLK;
-        for (int st = st0; st < st1 && ok; ++st, ++g) {
+        OzItem<MODE> w;
+        if (!oz_item<MODE>(batch, item, w)) continue;
+        const char *a = w.a, *b = w.b;
+        for (int st = w.st0; st < w.st1 && ok; ++st, ++g) {
           const int slot = g % ONST;
           const uint32_t par = ((g / ONST) & 1) ^ 1;
           char* dst = ring + slot * OSTAGE;
@@ -484,13 +551,10 @@ __global__ void __launch_bounds__(OTHREADS, 1)
       bool ok = true;
       const uint64_t desc0 = tc::smem_desc(tc::uniform(tc::smem_u32(ring)), 512, 4);
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-        int f, sp, bi, bj, kind;
-        const OzProb& L = oz_item<QF>(batch, item, f, sp, bi, bj, kind);
-      if (__ldg(L.flag)) continue;          // the FP64 kernel does this problem
-        int st0, st1;
-        range(L, sp, bj, st0, st1);
-        for (int sb0 = st0; sb0 < st1 && ok; sb0 += L.sbst) {
-          const int n = min(L.sbst, st1 - sb0);
+        OzItem<MODE> w;
+        if (!oz_item<MODE>(batch, item, w)) continue;
+        for (int sb0 = w.st0; sb0 < w.st1 && ok; sb0 += w.sbst) {
+          const int n = min(w.sbst, w.st1 - sb0);
           for (int k = 0; k < n; ++k, ++g) {
             const int slot = g % ONST;
             const uint32_t par = (g / ONST) & 1;
@@ -598,49 +662,20 @@ __global__ void __launch_bounds__(OTHREADS, 1)
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// ------------------------------------------------------------------ digits
-// Digits of 8 consecutive K values with exponent E (|v| < 0.996 2^E): for every slice 8 BF16
-// values d_i 256^(1-i), packed in K order. The fixed-point value X = round(v 2^(55-E)) plus the
-// bias 128 sum 256^k has the digits (plus 128) as its bytes; a byte put into the low mantissa bits
-// of a float of the slice's exponent, minus that float with the byte at 128, is the digit's value.
-// Integer arithmetic throughout: the FP64 pipe would take as long as the products.
-__device__ __forceinline__ void digits8(const double (&v)[8], int E, uint32_t (&w)[OSL][4]) {
-  constexpr unsigned long long BIAS = 128ull * (((1ull << 56) - 1) / 255);
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    float f[2][OSL];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const unsigned long long b = __double_as_longlong(v[2 * p + h]);
-      const int ex = int(b >> 52) & 0x7ff;
-      const int sh = min(E + 1022 - ex, 60);
-      unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 2;
-      // sh >= 0 by the choice of E; below the last digit (and for zero): zero
-      m = ex == 0 ? 0ull : (m + ((1ull << sh) >> 1)) >> sh;
-      const unsigned long long y = (b >> 63) ? BIAS - m : BIAS + m;
-      const uint32_t lo = uint32_t(y), hi = uint32_t(y >> 32);
-#pragma unroll
-      for (int i = 0; i < OSL; ++i) {
-        const uint32_t mg = 0x4B000000u - (uint32_t(8 * i) << 23);
-        // byte 6 - i of y in place of mg's lowest byte
-        const uint32_t bits = i < 3 ? __byte_perm(hi, mg, 0x7650u | uint32_t(2 - i))
-                                    : __byte_perm(lo, mg, 0x7650u | uint32_t(6 - i));
-        f[h][i] = __fsub_rn(__uint_as_float(bits), __uint_as_float(mg | 128u));
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < OSL; ++i) w[i][p] = tc::cvt_bf16x2(f[0][i], f[1][i]);
-  }
+__global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm_pol(const __grid_constant__ OzBatch batch, unsigned* status) {
+  oz_gemm<OZ_POL>(batch, status);
+}
+__global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm_quad(const __grid_constant__ OzBatch batch, unsigned* status) {
+  oz_gemm<OZ_QUAD>(batch, status);
+}
+__global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm_cplx(const __grid_constant__ OzCBatch batch, unsigned* status) {
+  oz_gemm<OZ_CPLX>(batch, status);
 }
 
-// 16 bytes of every slice of row n at K chunk kc of a stage's block
-__device__ __forceinline__ void store_digits(char* blk, int n, int kc, const uint32_t (&w)[OSL][4]) {
-  const uint32_t off = swz64(n, kc);
-#pragma unroll
-  for (int i = 0; i < OSL; ++i)
-    *reinterpret_cast<uint4*>(blk + i * SLB + off) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
-}
-
+// ------------------------------------------------------------------ digits (fp64_slices.cuh)
 // the exponent of a range: E with (largest magnitude) < 0.996 2^E, or a raised flag
 __device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool ratio, int* flag) {
   if (!(sum <= 3.0e38f) || !(mx < 1.2676506e30f)) {        // not finite, or from 2^100 on
@@ -991,14 +1026,14 @@ __global__ void k_oz_pair_reduce(const __grid_constant__ OzBatch batch) {
 
 size_t oz_smem() { return size_t(ONST) * OSTAGE + 1024; }
 
-template <bool QF>
-int launch_oz(const OzBatch& batch, cudaStream_t s, const DeviceCtx& ctx) {
+template <typename B>
+int launch_oz(void (*kern)(B, unsigned*), const B& batch, cudaStream_t s, const DeviceCtx& ctx) {
   const int64_t items = batch.item0[batch.nq];
   if (items == 0) return GW_OK;
-  int rc = set_max_dyn_smem(reinterpret_cast<const void*>(k_oz_gemm<QF>), oz_smem(), ctx.device);
+  int rc = set_max_dyn_smem(reinterpret_cast<const void*>(kern), oz_smem(), ctx.device);
   if (rc) return rc;
   const unsigned grid = unsigned(std::min<int64_t>(items, ctx.sm_count));
-  k_oz_gemm<QF><<<grid, OTHREADS, oz_smem(), s>>>(batch, ctx.status);
+  kern<<<grid, OTHREADS, oz_smem(), s>>>(batch, ctx.status);
   GW_LAUNCH_CHECK("k_oz_gemm");
   return GW_OK;
 }
@@ -1085,9 +1120,25 @@ std::vector<OzPlan> oz_plans(const std::vector<int>& qs, const int64_t* K, const
   return p;
 }
 
+}  // namespace
+
 size_t oz_sum_bytes(int sm) { return ws_round(size_t(sm) * OT * OT * sizeof(float)); }
 
-}  // namespace
+int oz_cplx(const OzC* probs, int n, float* s, cudaStream_t st, const DeviceCtx& ctx) {
+  for (int p0 = 0; p0 < n; p0 += OZC_MAX) {
+    OzCBatch b;
+    b.nq = std::min(OZC_MAX, n - p0);
+    b.s = s;
+    b.item0[0] = 0;
+    for (int i = 0; i < b.nq; ++i) {
+      b.q[i] = probs[p0 + i];
+      b.item0[i + 1] = b.item0[i] + b.q[i].ntile * b.q[i].nprod;
+    }
+    int rc = launch_oz<OzCBatch>(k_oz_gemm_cplx, b, st, ctx);
+    if (rc) return rc;
+  }
+  return GW_OK;
+}
 
 // From one stage of 32 rows on: K = 32, N_b = 8, 4 frequencies 0.08 ms against 0.14 with the FP64
 // kernel, K = 128, N_b = 24 0.11 against 0.54 (16 such q in one call 0.18 against 0.55); fewer rows
@@ -1216,7 +1267,7 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
       GW_LAUNCH_CHECK("k_oz_slice");
       int rc = record_herk_event(o, o.launches, false, s);
       if (rc) return rc;
-      if ((rc = launch_oz<false>(b, s, ctx))) return rc;
+      if ((rc = launch_oz<OzBatch>(k_oz_gemm_pol, b, s, ctx))) return rc;
       if ((rc = record_herk_event(o, o.launches, true, s))) return rc;
       ++o.launches;
     }
@@ -1357,7 +1408,7 @@ int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig
     GW_LAUNCH_CHECK("k_oz_slice_rows");
     k_oz_slice_u<<<dim3(unsigned(nst), unsigned(4 * nbj), nz), OT, 0, s>>>(b, int(nf));
     GW_LAUNCH_CHECK("k_oz_slice_u");
-    int rc = launch_oz<true>(b, s, ctx);
+    int rc = launch_oz<OzBatch>(k_oz_gemm_quad, b, s, ctx);
     if (rc) return rc;
     k_oz_pair_reduce<<<dim3(unsigned(std::min<int64_t>((nred + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_pair_reduce");
