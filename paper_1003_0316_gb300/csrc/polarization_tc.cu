@@ -1050,6 +1050,7 @@ __global__ void __launch_bounds__(128) k_prep_quad(const double2* __restrict__ W
   char* __restrict__ bsp = bsp0 + size_t(blockIdx.z) * size_t(jstride);
   const int cb = blockIdx.y;
   const int64_t ch = blockIdx.x;
+  if (ch * CH >= int64_t(cb + 1) * TN) return;   // K blocks that no item of this column block reads
   const int n = threadIdx.x;
   const int c = cb * TN + n;
   const int ncol = REAL ? nb : 2 * nb;

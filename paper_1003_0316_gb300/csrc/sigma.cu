@@ -207,8 +207,14 @@ __device__ __forceinline__ cplx operator*(cplx a, cplx b) {
   return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ cplx operator*(double s, cplx a) { return mk(s * a.x, s * a.y); }
+__device__ __forceinline__ double cnorm(cplx a) { return fma(a.x, a.x, a.y * a.y); }
+// a / b: one division by |b|^2, and Smith's scaled form where that would leave the FP64 range
 __device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
-  // Smith's algorithm
+  const double n = cnorm(b);
+  if (n > 1e-280 && n < 1e280) {
+    const double i = 1.0 / n;
+    return mk(fma(a.x, b.x, a.y * b.y) * i, fma(a.y, b.x, -a.x * b.y) * i);
+  }
   if (fabs(b.x) >= fabs(b.y)) {
     double r = b.y / b.x, d = b.x + b.y * r;
     return mk((a.x + a.y * r) / d, (a.y - a.x * r) / d);
@@ -217,8 +223,11 @@ __device__ __forceinline__ cplx cdiv(cplx a, cplx b) {
     return mk((a.x * r + a.y) / d, (a.y * r - a.x) / d);
   }
 }
-__device__ __forceinline__ double cabs_(cplx a) { return hypot(a.x, a.y); }
-__device__ __forceinline__ cplx clog_(cplx a) { return mk(log(hypot(a.x, a.y)), atan2(a.y, a.x)); }
+__device__ __forceinline__ cplx clog_(cplx a) {
+  const double n = cnorm(a);
+  const double l = n > 1e-280 && n < 1e280 ? 0.5 * log(n) : log(hypot(a.x, a.y));
+  return mk(l, atan2(a.y, a.x));
+}
 
 // 1/k for k = 1..60 (the series below multiply by these instead of dividing)
 __constant__ double kInvInt[60] = {1.0, 0.5, 0.3333333333333333, 0.25, 0.2, 0.16666666666666666, 0.14285714285714285, 0.125, 0.1111111111111111, 0.1, 0.09090909090909091, 0.08333333333333333, 0.07692307692307693, 0.07142857142857142, 0.06666666666666667, 0.0625, 0.058823529411764705, 0.05555555555555555, 0.05263157894736842, 0.05, 0.047619047619047616, 0.045454545454545456, 0.043478260869565216, 0.041666666666666664, 0.04, 0.038461538461538464, 0.037037037037037035, 0.03571428571428571, 0.034482758620689655, 0.03333333333333333, 0.03225806451612903, 0.03125, 0.030303030303030304, 0.029411764705882353, 0.02857142857142857, 0.027777777777777776, 0.02702702702702703, 0.02631578947368421, 0.02564102564102564, 0.025, 0.024390243902439025, 0.023809523809523808, 0.023255813953488372, 0.022727272727272728, 0.022222222222222223, 0.021739130434782608, 0.02127659574468085, 0.020833333333333332, 0.02040816326530612, 0.02, 0.0196078431372549, 0.019230769230769232, 0.018867924528301886, 0.018518518518518517, 0.01818181818181818, 0.017857142857142856, 0.017543859649122806, 0.017241379310344827, 0.01694915254237288, 0.016666666666666666};
@@ -226,37 +235,42 @@ __constant__ double kInvInt[60] = {1.0, 0.5, 0.3333333333333333, 0.25, 0.2, 0.16
 constexpr double SERIES_R = 0.3;
 constexpr int SERIES_N = 36;
 
-// I_k = int_0^H t^k / (z0 + b t) dt, k = 0..3
+// I_k = int_0^H t^k / (z0 + b t) dt, k = 0..3, by z0 I_k + b I_(k+1) = H^(k+1) / (k+1): with
+// r = H b / z0 small, downwards from the series I_3 = H^4 / z0 sum_m (-r)^m / (m + 4) (each step
+// damps errors by |r|); else upwards from I_0 = log(1 + r) / b. (All four sums by their series took
+// twice the multiply-adds; magnitudes by hypot and quotients by scaled division as much again.)
 __device__ void moments(cplx z0, cplx b, double H, cplx I[4]) {
-  cplx r = cdiv(H * b, z0);
-  if (cabs_(r) < SERIES_R) {
-    cplx term = mk(1.0, 0.0);
-    cplx nr = mk(-r.x, -r.y);
-    cplx s0 = mk(0, 0), s1 = mk(0, 0), s2 = mk(0, 0), s3 = mk(0, 0);
-    const double rr = cabs_(r);
+  const cplx iz = cdiv(mk(1.0, 0.0), z0);
+  const cplx r = (H * b) * iz;
+  const double rr = cnorm(r);
+  if (rr < SERIES_R * SERIES_R) {
+    cplx term = mk(1.0, 0.0), s3 = mk(0.0, 0.0);
+    const cplx nr = mk(-r.x, -r.y);
     double tmag = 1.0;
     for (int m = 0; m < SERIES_N; ++m) {
-      s0 = s0 + kInvInt[m] * term;
-      s1 = s1 + kInvInt[m + 1] * term;
-      s2 = s2 + kInvInt[m + 2] * term;
-      s3 = s3 + kInvInt[m + 3] * term;
+      s3.x = fma(kInvInt[m + 3], term.x, s3.x);
+      s3.y = fma(kInvInt[m + 3], term.y, s3.y);
       term = term * nr;
       tmag *= rr;
-      if (tmag < 1e-18) break;     // |r|^(m+1) below the FP64 resolution of the sums (>= 1/4)
+      if (tmag < 1e-36) break;     // |r|^(m+1) below the FP64 resolution of the sum (>= 1/4)
     }
-    cplx iz = cdiv(mk(1.0, 0.0), z0);
-    double h1 = H, h2 = H * H, h3 = h2 * H, h4 = h3 * H;
-    I[0] = h1 * (s0 * iz);
+    // with J_k = I_k z0 / H^(k+1): J_k = 1/(k+1) - r J_(k+1)
+    const cplx s2 = mk(kInvInt[2] - fma(r.x, s3.x, -r.y * s3.y), -fma(r.x, s3.y, r.y * s3.x));
+    const cplx s1 = mk(kInvInt[1] - fma(r.x, s2.x, -r.y * s2.y), -fma(r.x, s2.y, r.y * s2.x));
+    const cplx s0 = mk(kInvInt[0] - fma(r.x, s1.x, -r.y * s1.y), -fma(r.x, s1.y, r.y * s1.x));
+    const double h2 = H * H, h3 = h2 * H, h4 = h3 * H;
+    I[0] = H * (s0 * iz);
     I[1] = h2 * (s1 * iz);
     I[2] = h3 * (s2 * iz);
     I[3] = h4 * (s3 * iz);
   } else {
-    cplx ib = cdiv(mk(1.0, 0.0), b);
+    const cplx ib = cdiv(mk(1.0, 0.0), b);
     I[0] = clog_(mk(1.0 + r.x, r.y)) * ib;
     double hk = 1.0;
+#pragma unroll
     for (int k = 1; k < 4; ++k) {
       hk *= H;
-      I[k] = (mk(hk / k, 0.0) - z0 * I[k - 1]) * ib;
+      I[k] = (mk(hk * kInvInt[k - 1], 0.0) - z0 * I[k - 1]) * ib;
     }
   }
 }
@@ -265,15 +279,15 @@ __device__ void moments(cplx z0, cplx b, double H, cplx I[4]) {
 __device__ cplx tail_integral(cplx A, double sgn, double X) {
   cplx isg = mk(0.0, sgn);
   cplx rho = cdiv(A, mk(0.0, sgn * X));
-  if (cabs_(rho) < 0.5) {
+  const double rr = cnorm(rho);
+  if (rr < 0.25) {
     cplx term = mk(1.0, 0.0), nr = mk(-rho.x, -rho.y), s = mk(0, 0);
-    const double rr = cabs_(rho);
     double tmag = 1.0;
     for (int m = 0; m < 56; ++m) {
       s = s + kInvInt[m + 1] * term;
       term = term * nr;
       tmag *= rr;
-      if (tmag < 1e-18) break;     // |rho|^(m+1) below the FP64 resolution of the sum (>= 1/2)
+      if (tmag < 1e-36) break;     // |rho|^(m+1) below the FP64 resolution of the sum (>= 1/2)
     }
     return cdiv(s, mk(0.0, sgn * X * X));
   }
@@ -335,9 +349,12 @@ __device__ void piece_coeffs(const double* y, const double* m, const double* lam
 //     open-addressing table (atomicCAS), records its slot and counts the slot's pairs;
 //   k_conv_scan: per q, the offsets of the slots' pair lists and the occupied slots;
 //   k_conv_scatter: every pair writes its index into its slot's list;
-//   k_conv_slot: one CTA per (occupied slot, 16 output frequencies): S (once per CTA), K (one
-//     thread per output frequency and piece), T, then Sigma_s(i w_i) += w_q f sum_j T_ij c_jp
-//     over the slot's pairs (FP64 atomics).
+//   k_conv_slot: the items (occupied slot, 16 output frequencies) of all q points in one list
+//     over persistent CTAs: S (once per CTA), K (one thread per output frequency and piece), T,
+//     then Sigma_s(i w_i) += w_q f sum_j T_ij c_jp over the slot's pairs (FP64 atomics). The FP64
+//     pipe's instructions bound it (two moments of 4 per output frequency, piece and energy):
+//     8 q of 3,328 distinct energies at 16 x 16 frequencies took 3.8 ms with all four moments
+//     by their own sums, scaled divisions, hypot and one loop per q; 2.3 ms now.
 constexpr int CTHREADS = 256;
 constexpr int CIC = 16;                       // output frequencies per slot CTA
 constexpr unsigned long long EMPTY_KEY = ~0ull;   // a NaN pattern: never a valid energy
@@ -501,11 +518,23 @@ __global__ void __launch_bounds__(CTHREADS) k_conv_slot(ConvLaunch L, int nw, Om
   __syncthreads();
   const double f = -1.0 / (2.0 * 3.14159265358979323846);
   const int nich = (nw_out + CIC - 1) / CIC;
-  for (int q = 0; q < L.nq; ++q) {
-    const ConvQ& Q = L.Q[q];
-    if (Q.npair == 0) continue;
-    const int64_t items = int64_t(*Q.nocc) * nich;
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+  // the items (occupied slot, 16 output frequencies) of all q in one list
+  __shared__ int64_t first[SMAXQ + 1];
+  if (tid == 0) {
+    int64_t t = 0;
+    for (int q = 0; q < L.nq; ++q) {
+      first[q] = t;
+      t += L.Q[q].npair > 0 ? int64_t(*L.Q[q].nocc) * nich : 0;
+    }
+    first[L.nq] = t;
+  }
+  __syncthreads();
+  {
+    int q = 0;
+    for (int64_t g = blockIdx.x; g < first[L.nq]; g += gridDim.x) {
+      while (g >= first[q + 1]) ++q;
+      const ConvQ& Q = L.Q[q];
+      const int64_t it = g - first[q];
       const int slot = Q.occ[it / nich];
       const int i0 = int(it % nich) * CIC;
       const int ni = min(CIC, nw_out - i0);
