@@ -278,8 +278,10 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
 // order (sums over points as the warp's butterfly forms them, everything else through shared
 // memory as there), so the results are bit-identical. A block draws its curves from a contiguous
 // range through a counter, the lanes of a curve taking the next one when their fit ends; each trip
-// of the loop is damped solve, cost, accept or reject, and the Jacobian for the curves that
-// accepted. Still bound by the FP64 pipe. One lane per curve was not faster (270 ms for 1e5 curves:
+// of the loop is damped solve, cost, accept or reject for the curves that are not waiting for a
+// Jacobian, and the Jacobian (two thirds of the instructions) for all that accepted, once these
+// are more than half of the warp's curves: about every other step is rejected, so a Jacobian per
+// trip would run with half its lanes. Still bound by the FP64 pipe. One lane per curve was not faster (270 ms for 1e5 curves:
 // its registers hold one curve's matrix, few warps run) and rounds differently.
 // Two-pole fits on 24 points, this kernel against one warp per curve: 1e5 curves 440 -> 248 ms,
 // 32,000 144 -> 91.5, 8,192 40.3 -> 33.6, 6,500 32.7 -> 30.3 ms. Below about 6,000 curves there are too
@@ -289,6 +291,8 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
 constexpr int LM_GROUPS_MIN = 6144;   // curves from which this kernel is taken
 constexpr int LM_GROUPS4_MIN = 8192;  // ... with four lanes per curve
 constexpr int LM_GROUPS_MAXNW = 32;
+// accepted curves of a warp's n that a Jacobian waits for
+__host__ __device__ constexpr int LM_JAC(int n) { return n / 2 + 1; }
 
 // doubles of shared memory per curve (odd, so that the curves of a warp start in other banks)
 __host__ __device__ constexpr int lm_group_doubles(int nw, int P) {
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
   }
   // per curve, the same in its eight lanes
   int cidx = 0, it = 0, st = 1;
-  bool active = false, done = false, init = false;
+  bool active = false, done = false, init = false, jac = false;
   double th[P], thn[P], C = 0.0, cscale = 0.0, mu = -1.0;
   for (int k = 0; k < P; ++k) th[k] = thn[k] = 0.0;
   const double2* y = sigma;
@@ -397,7 +401,8 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
       if (init) cscale = cs;
       if (!__any_sync(0xffffffffu, active)) break;
     }
-    const bool solve = active && !init;
+    const bool trial = active && !jac;            // a new point: the start, or a damped step
+    const bool solve = trial && !init;
     bool ok = true;
     if (__any_sync(0xffffffffu, solve)) {
       if (solve) {
@@ -455,30 +460,33 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
         for (int k = 0; k < P; ++k) thn[k] = th[k] + sb[k];
     }
     // the cost at thn
-    double c4[NL];
+    double Cn = 0.0;
+    if (__any_sync(0xffffffffu, trial)) {
+      double c4[NL];
 #pragma unroll
-    for (int k4 = 0; k4 < NL; ++k4) {
-      double c = 0.0;
-      for (int h = 0; h < 2; ++h) {
-        const int j = sub + LMG * k4 + 32 * h;
-        if (j >= nw || !active) break;
-        double fx = 0.0, fy = 0.0;
-        for (int p = 0; p < npole; ++p) {
-          const double dx = -thn[4 * p + 2], dy = om.v[j] - thn[4 * p + 3];
-          const double inv = 1.0 / (dx * dx + dy * dy);
-          const double px = dx * inv, py = -dy * inv;          // phi = 1 / (i w_j - w_p)
-          fx += thn[4 * p] * px - thn[4 * p + 1] * py;
-          fy += thn[4 * p] * py + thn[4 * p + 1] * px;
+      for (int k4 = 0; k4 < NL; ++k4) {
+        double c = 0.0;
+        for (int h = 0; h < 2; ++h) {
+          const int j = sub + LMG * k4 + 32 * h;
+          if (j >= nw || !trial) break;
+          double fx = 0.0, fy = 0.0;
+          for (int p = 0; p < npole; ++p) {
+            const double dx = -thn[4 * p + 2], dy = om.v[j] - thn[4 * p + 3];
+            const double inv = 1.0 / (dx * dx + dy * dy);
+            const double px = dx * inv, py = -dy * inv;          // phi = 1 / (i w_j - w_p)
+            fx += thn[4 * p] * px - thn[4 * p + 1] * py;
+            fy += thn[4 * p] * py + thn[4 * p + 1] * px;
+          }
+          const double2 yj = y[j];
+          const double rx = fx - yj.x, ry = fy - yj.y;
+          c += rx * rx + ry * ry;
         }
-        const double2 yj = y[j];
-        const double rx = fx - yj.x, ry = fy - yj.y;
-        c += rx * rx + ry * ry;
+        c4[k4] = c;
       }
-      c4[k4] = c;
+      Cn = 0.5 * group_butterfly<LMG>(c4);
     }
-    const double Cn = 0.5 * group_butterfly<LMG>(c4);
-    bool jac = false, end = false;
-    if (active) {
+    bool end = false;
+    if (trial) {
       bool accepted = init;
       double dec = 0.0, Cold = 0.0;
       if (!init) {
@@ -518,7 +526,10 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
         }
       }
     }
-    if (__any_sync(0xffffffffu, jac)) {
+    // the Jacobian once enough curves wait for it, or when no other curve can go on
+    const unsigned waits = __ballot_sync(0xffffffffu, jac);
+    const unsigned goes = __ballot_sync(0xffffffffu, !jac && !done);
+    if (waits != 0 && (__popc(waits) >= LMG * LM_JAC(32 / LMG) || goes == 0)) {
       // Jacobian rows and residuals of this lane's points
       if (jac) {
         for (int j = sub; j < nw; j += LMG) {
@@ -586,6 +597,7 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
           end = true;
         }
         if (mu < 0.0) mu = 1e-3 * dm;
+        jac = false;
       }
     }
     if (end) {
