@@ -270,33 +270,54 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
   status_out[cidx] = st;
 }
 
-// ---- many curves: four or eight lanes per curve, eight or four curves per warp --------------------
+// ---- many curves: four lanes per curve, eight curves per warp -------------------------------------
 // GB300's FP64 pipe takes as long for an instruction with one active lane as for a full one (16
 // cycles per warp instruction and SM), and the warp-per-curve kernel issues most of its FP64
 // instructions with few (the pivots with one, the sweeps with at most P = 4 N_p, the points with nw
-// of 32). Here several curves share a warp's instructions, with the same operations in the same
+// of 32). Here eight curves share a warp's instructions, with the same operations in the same
 // order (sums over points as the warp's butterfly forms them, everything else through shared
 // memory as there), so the results are bit-identical. A block draws its curves from a contiguous
 // range through a counter, the lanes of a curve taking the next one when their fit ends; each trip
 // of the loop is damped solve, cost, accept or reject for the curves that are not waiting for a
 // Jacobian, and the Jacobian (two thirds of the instructions) for all that accepted, once these
 // are more than half of the warp's curves: about every other step is rejected, so a Jacobian per
-// trip would run with half its lanes. Still bound by the FP64 pipe. One lane per curve was not faster (270 ms for 1e5 curves:
-// its registers hold one curve's matrix, few warps run) and rounds differently.
-// Two-pole fits on 24 points, this kernel against one warp per curve: 1e5 curves 440 -> 248 ms,
-// 32,000 144 -> 91.5, 8,192 40.3 -> 33.6, 6,500 32.7 -> 30.3 ms. Below about 6,000 curves there are too
-// few warps (5,000: 26.5 -> 30.9 ms), and from 8,192 on four lanes per curve are the faster split
-// (16,000: 57.4 -> 55.5 ms, 1e5: 276 -> 248 ms). More than 32 points take too much shared
-// memory per curve (9,000 curves on 64 points: 82 -> 167 ms), as do four poles and more.
-constexpr int LM_GROUPS_MIN = 6144;   // curves from which this kernel is taken
-constexpr int LM_GROUPS4_MIN = 8192;  // ... with four lanes per curve
-constexpr int LM_GROUPS_MAXNW = 32;
+// trip would run with half its lanes. Still bound by the FP64 pipe. Not faster: one lane per curve
+// (270 ms for 1e5 curves: its registers hold one curve's matrix, few warps run), eight lanes (216 ms
+// against 182), two lanes (172 ms).
+// The Jacobian takes phi and the residuals from the accepted trial's cost.
+// One warp per curve -> this kernel, 24 points, two poles: 1e5 curves 440 -> 164 ms, 32,000 144 ->
+// 63.6, 8,192 40.2 -> 23.8, 3,500 20.0 -> 17.6; three poles: 8,000 curves 116 -> 42.1 ms; one pole:
+// 30,000 curves 20.4 -> 11.0 ms.
+constexpr int LMG = 4;                // lanes per curve
+// Curves from which this kernel is taken, by the number of poles:
+// below them too few warps run (two poles, 3,000 curves: 17.3 -> 17.4 ms; one pole, 4,096: 4.7 ->
+// 5.1; three poles, 1,500: 30.3 -> 29.6), the more so with the shared memory of more than 32 points
+// (64 points: one pole, 6,500 curves 11.2 -> 11.8; two poles, 3,000 32 -> 34, 9,000 82 -> 70 ms).
+constexpr int LM_GROUPS_MIN[2][3] = {{5000, 3500, 2000}, {8000, 5600, 3200}};   // [nw > 32]
 // accepted curves of a warp's n that a Jacobian waits for
 __host__ __device__ constexpr int LM_JAC(int n) { return n / 2 + 1; }
 
-// doubles of shared memory per curve (odd, so that the curves of a warp start in other banks)
+// Doubles of shared memory per curve: D (which the solve's L, right-hand side and reciprocal pivots
+// share), residuals, A, g, theta and the trial. Lanes read consecutive entries, so curves that start
+// LMG doubles apart (of the 16 that a row of the banks holds) do not collide (171 -> 164 ms).
+__host__ __device__ constexpr int lm_group_d(int nw, int P) {
+  return nw * P > P * (P + 1) / 2 + 2 * P ? nw * P : P * (P + 1) / 2 + 2 * P;
+}
 __host__ __device__ constexpr int lm_group_doubles(int nw, int P) {
-  return (2 * nw * P + 2 * nw + P * (P + 1) + 3 * P) | 1;
+  const int d = lm_group_d(nw, P) + 2 * nw + P * (P + 1) / 2 + 3 * P;
+  return d + (LMG - d % 16 + 16) % 16;
+}
+
+// a b + c d and a b - c d, rounded as the compiler contracts them in k_lm_warp
+__device__ __forceinline__ double lm_sum(double a, double b, double c, double d) {
+  return fma(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ double lm_dif(double a, double b, double c, double d) {
+  return fma(a, b, -__dmul_rn(c, d));
+}
+// x with its sign flipped where bit 31 of m is set
+__device__ __forceinline__ double lm_flip(double x, int m) {
+  return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x));
 }
 
 // the sum the butterfly of warp_sum forms of the lanes' values c(l), l = sub + G k held in c[k]
@@ -318,8 +339,8 @@ __device__ __forceinline__ double group_max(double v) {
   return v;
 }
 
-template <int NPOLE, int LMG>
-__global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __grid_constant__ OmegaArr om,
+template <int NPOLE>
+__global__ void __launch_bounds__(64, 4) k_lm_groups(int ncurve, int nw, const __grid_constant__ OmegaArr om,
                                                    const double2* __restrict__ sigma,
                                                    const double* __restrict__ sign,
                                                    const double* theta_init, double* params,
@@ -330,37 +351,40 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
   constexpr int P = 4 * npole;
   constexpr int NP = P * (P + 1) / 2;
   constexpr int EPL = (NP + LMG - 1) / LMG;     // packed entries per lane
+  constexpr int GPL = (P + LMG - 1) / LMG;      // entries of g per lane
   constexpr int NL = 32 / LMG;                  // lanes of the warp kernel per lane
   extern __shared__ double lsm[];
   __shared__ int next;
   const int lane = threadIdx.x & 31, sub = lane & (LMG - 1);
-  double* rowR = lsm + size_t(threadIdx.x / LMG) * lm_group_doubles(nw, P);
-  double* rowI = rowR + nw * P;
-  double* res = rowI + nw * P;
-  double* sA = res + 2 * nw;
-  double* Ld = sA + NP;
-  double* sg = Ld + NP;
-  double* sb = sg + P;
+  // D[j][a]: (Re phi, Im phi, Re a phi^2, Im a phi^2) of pole a / 4 at point j. The Jacobian's rows
+  // are R[a] = +-D[a] (minus for odd a) and I[a] = D[a ^ 1].
+  double* D = lsm + size_t(threadIdx.x / LMG) * lm_group_doubles(nw, P);
+  // D is dead from the decision on a trial to the next trial's cost: the solve's arrays overlay it.
+  double* Ld = D;
+  double* sb = Ld + NP;
   double* dinv = sb + P;
+  double* res = D + lm_group_d(nw, P);
+  double* sA = res + 2 * nw;
+  double* sg = sA + NP;
+  double* sth = sg + P;
+  double* sthn = sth + P;
   const int per = (ncurve + int(gridDim.x) - 1) / int(gridDim.x);
   const int c_end = min(ncurve, (int(blockIdx.x) + 1) * per);
   if (threadIdx.x == 0) next = int(blockIdx.x) * per;
   __syncthreads();
-  // the packed entries e = sub + 8 h of A this lane sums: row ea[h], column eb[h]
-  int ea[EPL], eb[EPL];
+  // the packed entries e = sub + LMG h of A this lane sums: row (low half) and column
+  int eab[EPL];
 #pragma unroll
   for (int h = 0; h < EPL; ++h) {
     const int e = sub + LMG * h;
     int a = 0;
     while ((a + 1) * (a + 2) / 2 <= e) ++a;
-    ea[h] = e < NP ? a : 0;
-    eb[h] = e < NP ? e - a * (a + 1) / 2 : 0;
+    eab[h] = e < NP ? a | (e - a * (a + 1) / 2) << 16 : 0;
   }
-  // per curve, the same in its eight lanes
+  // per curve, the same in its lanes
   int cidx = 0, it = 0, st = 1;
   bool active = false, done = false, init = false, jac = false;
-  double th[P], thn[P], C = 0.0, cscale = 0.0, mu = -1.0;
-  for (int k = 0; k < P; ++k) th[k] = thn[k] = 0.0;
+  double C = 0.0, cscale = 0.0, mu = -1.0;
   const double2* y = sigma;
   while (true) {
     const bool want = !active && !done;
@@ -379,23 +403,21 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
           mu = -1.0;
           y = sigma + size_t(cidx) * nw;
           if (theta_init) {
-            for (int k = 0; k < P; ++k) thn[k] = theta_init[size_t(cidx) * P + k];
+            for (int k = sub; k < P; k += LMG) sthn[k] = theta_init[size_t(cidx) * P + k];
           } else if (sub == 0) {
             const double s = sign ? (sign[cidx] >= 0.0 ? 1.0 : -1.0) : 1.0;
-            lm_default_start(om.v, y, nw, npole, s, sb);
+            lm_default_start(om.v, y, nw, npole, s, sthn);
           }
         }
       }
       __syncwarp();
-      if (init && !theta_init)
-        for (int k = 0; k < P; ++k) thn[k] = sb[k];
       double c4[NL];
 #pragma unroll
       for (int k = 0; k < NL; ++k) {
         const int l = sub + LMG * k;
         const double2 a = init && l < nw ? y[l] : make_double2(0.0, 0.0);
         const double2 b = init && l + 32 < nw ? y[l + 32] : make_double2(0.0, 0.0);
-        c4[k] = a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y;
+        c4[k] = fma(b.y, b.y, fma(b.x, b.x, lm_sum(a.x, a.x, a.y, a.y)));
       }
       const double cs = 0.5 * group_butterfly<LMG>(c4);
       if (init) cscale = cs;
@@ -457,12 +479,15 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
         __syncwarp();
       }
       if (solve)
-        for (int k = 0; k < P; ++k) thn[k] = th[k] + sb[k];
+        for (int k = sub; k < P; k += LMG) sthn[k] = sth[k] + sb[k];
+      __syncwarp();
     }
-    // the cost at thn
+    // the cost at the new point; phi and the residuals stay for its Jacobian
     double Cn = 0.0;
     if (__any_sync(0xffffffffu, trial)) {
-      double c4[NL];
+      double c4[NL], thn[P];
+#pragma unroll
+      for (int k = 0; k < P; ++k) thn[k] = sthn[k];
 #pragma unroll
       for (int k4 = 0; k4 < NL; ++k4) {
         double c = 0.0;
@@ -470,16 +495,21 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
           const int j = sub + LMG * k4 + 32 * h;
           if (j >= nw || !trial) break;
           double fx = 0.0, fy = 0.0;
+#pragma unroll
           for (int p = 0; p < npole; ++p) {
             const double dx = -thn[4 * p + 2], dy = om.v[j] - thn[4 * p + 3];
-            const double inv = 1.0 / (dx * dx + dy * dy);
+            const double inv = 1.0 / lm_sum(dy, dy, dx, dx);
             const double px = dx * inv, py = -dy * inv;          // phi = 1 / (i w_j - w_p)
-            fx += thn[4 * p] * px - thn[4 * p + 1] * py;
-            fy += thn[4 * p] * py + thn[4 * p + 1] * px;
+            fx += lm_dif(thn[4 * p], px, thn[4 * p + 1], py);
+            fy += lm_sum(thn[4 * p], py, thn[4 * p + 1], px);
+            D[j * P + 4 * p] = px;
+            D[j * P + 4 * p + 1] = py;
           }
           const double2 yj = y[j];
           const double rx = fx - yj.x, ry = fy - yj.y;
-          c += rx * rx + ry * ry;
+          res[2 * j] = rx;
+          res[2 * j + 1] = ry;
+          c += lm_sum(rx, rx, ry, ry);
         }
         c4[k4] = c;
       }
@@ -504,7 +534,7 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
         }
       }
       if (accepted) {
-        for (int k = 0; k < P; ++k) th[k] = thn[k];
+        for (int k = sub; k < P; k += LMG) sth[k] = sthn[k];
         C = Cn;
         if (!init) {
           ++it;
@@ -526,66 +556,66 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
         }
       }
     }
+    __syncwarp();
     // the Jacobian once enough curves wait for it, or when no other curve can go on
     const unsigned waits = __ballot_sync(0xffffffffu, jac);
     const unsigned goes = __ballot_sync(0xffffffffu, !jac && !done);
     if (waits != 0 && (__popc(waits) >= LMG * LM_JAC(32 / LMG) || goes == 0)) {
-      // Jacobian rows and residuals of this lane's points
+      double v[EPL], w[GPL];
+#pragma unroll
+      for (int h = 0; h < EPL; ++h) v[h] = 0.0;
+#pragma unroll
+      for (int h = 0; h < GPL; ++h) w[h] = 0.0;
+      // a phi^2 at this lane's points (a phi as the cost's)
       if (jac) {
         for (int j = sub; j < nw; j += LMG) {
-          double fx = 0.0, fy = 0.0;
+#pragma unroll
           for (int p = 0; p < npole; ++p) {
-            const double ax = th[4 * p], ay = th[4 * p + 1];
-            const double dx = -th[4 * p + 2], dy = om.v[j] - th[4 * p + 3];
-            const double inv = 1.0 / (dx * dx + dy * dy);
-            const double px = dx * inv, py = -dy * inv;        // phi
-            const double tx = ax * px - ay * py, ty = ax * py + ay * px;   // a phi
-            fx += tx;
-            fy += ty;
-            const double qx = tx * px - ty * py, qy = tx * py + ty * px;   // a phi^2
-            double* R = rowR + j * P + 4 * p;
-            double* I = rowI + j * P + 4 * p;
-            R[0] = px;
-            I[0] = py;
-            R[1] = -py;
-            I[1] = px;
-            R[2] = qx;
-            I[2] = qy;
-            R[3] = -qy;
-            I[3] = qx;
+            double* d = D + j * P + 4 * p;
+            const double ax = sth[4 * p], ay = sth[4 * p + 1], px = d[0], py = d[1];
+            const double tx = lm_dif(ax, px, ay, py), ty = lm_sum(ax, py, ay, px);
+            d[2] = lm_dif(tx, px, ty, py);
+            d[3] = lm_sum(tx, py, ty, px);
           }
-          const double2 yj = y[j];
-          res[2 * j] = fx - yj.x;
-          res[2 * j + 1] = fy - yj.y;
         }
       }
       __syncwarp();
       // A (packed lower) and g, summed over points
-      double gm = 0.0, dm = 0.0;
       if (jac) {
-        double v[EPL];
-#pragma unroll
-        for (int h = 0; h < EPL; ++h) v[h] = 0.0;
 #pragma unroll 2
         for (int j = 0; j < nw; ++j) {
-          const double* R = rowR + j * P;
-          const double* I = rowI + j * P;
+          const double* d = D + j * P;
 #pragma unroll
-          for (int h = 0; h < EPL; ++h) v[h] += R[ea[h]] * R[eb[h]] + I[ea[h]] * I[eb[h]];
+          for (int h = 0; h < EPL; ++h) {
+            const int ea = eab[h] & 0xffff, eb = eab[h] >> 16;
+            v[h] += lm_sum(lm_flip(d[ea], (ea ^ eb) << 31), d[eb], d[ea ^ 1], d[eb ^ 1]);
+          }
         }
+#pragma unroll
+        for (int h = 0; h < GPL; ++h) {
+          const int a = sub + LMG * h;
+          if (a < P)
+            for (int j = 0; j < nw; ++j)
+              w[h] += lm_sum(lm_flip(D[j * P + a], a << 31), res[2 * j], D[j * P + (a ^ 1)], res[2 * j + 1]);
+        }
+      }
+      double gm = 0.0, dm = 0.0;
+      if (jac) {
 #pragma unroll
         for (int h = 0; h < EPL; ++h) {
           const int e = sub + LMG * h;
           if (e < NP) {
             sA[e] = v[h];
-            if (ea[h] == eb[h]) dm = fmax(dm, v[h]);
+            if ((eab[h] & 0xffff) == eab[h] >> 16) dm = fmax(dm, v[h]);
           }
         }
-        for (int a = sub; a < P; a += LMG) {
-          double w = 0.0;
-          for (int j = 0; j < nw; ++j) w += rowR[j * P + a] * res[2 * j] + rowI[j * P + a] * res[2 * j + 1];
-          sg[a] = w;
-          gm = fmax(gm, fabs(w));
+#pragma unroll
+        for (int h = 0; h < GPL; ++h) {
+          const int a = sub + LMG * h;
+          if (a < P) {
+            sg[a] = w[h];
+            gm = fmax(gm, fabs(w[h]));
+          }
         }
       }
       __syncwarp();
@@ -604,7 +634,7 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
       active = false;
       // the other start's result stays when it is not worse
       if (sub == 0 && (!keep_better || C < cost_out[cidx])) {
-        for (int k = 0; k < P; ++k) params[size_t(cidx) * P + k] = th[k];
+        for (int k = 0; k < P; ++k) params[size_t(cidx) * P + k] = sth[k];
         cost_out[cidx] = C;
         iters_out[cidx] = it;
         status_out[cidx] = st;
@@ -613,19 +643,21 @@ __global__ void __launch_bounds__(128) k_lm_groups(int ncurve, int nw, const __g
   }
 }
 
-template <int NPOLE, int G>
+template <int NPOLE>
 static int launch_lm_groups(int ncurve, int nw, const OmegaArr& om, const double2* y, const double* sign,
                             const double* theta_init, double* params, double* cost, int* iters,
                             int* status, int keep_better, cudaStream_t s, const DeviceCtx& ctx) {
-  const auto kern = k_lm_groups<NPOLE, G>;
-  const size_t per_warp = size_t(32 / G) * lm_group_doubles(nw, 4 * NPOLE) * sizeof(double);
-  const int warps = int(std::max<size_t>(1, std::min<size_t>(4, (100u << 10) / per_warp)));
+  const auto kern = k_lm_groups<NPOLE>;
+  const size_t per_warp = size_t(32 / LMG) * lm_group_doubles(nw, 4 * NPOLE) * sizeof(double);
+  // Two warps share a range of curves once every SM gets five such blocks; with fewer, blocks of
+  // one warp spread over the SMs more evenly (8,192 curves 29.9 -> 25.9 ms; 1e5: 181 against 186).
+  const int warps = ncurve >= 5 * 2 * (32 / LMG) * ctx.sm_count ? 2 : 1;
   const size_t smem = warps * per_warp;
   int rc = set_max_dyn_smem(reinterpret_cast<const void*>(kern), smem, ctx.device);
   if (rc) return rc;
   int fit = 0;                        // resident blocks per SM
   GW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, 32 * warps, smem));
-  const int curves = warps * 32 / G;
+  const int curves = warps * 32 / LMG;
   const int blocks = int(std::min<int64_t>((int64_t(ncurve) + curves - 1) / curves,
                                            int64_t(ctx.sm_count) * std::max(1, fit)));
   kern<<<blocks, 32 * warps, smem, s>>>(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status,
@@ -640,17 +672,12 @@ int launch_lm(int ncurve, int nw, const OmegaArr& om, const double* sigma, const
   if (ncurve == 0) return GW_OK;
   if (nw > LM_WMAXNW) return set_error(GW_EINVAL, "the fit takes at most %d frequencies", LM_WMAXNW);
   const double2* y = reinterpret_cast<const double2*>(sigma);
-  if (npole <= 3 && nw <= LM_GROUPS_MAXNW && ncurve >= LM_GROUPS_MIN) {
+  if (npole <= 3 && ncurve >= LM_GROUPS_MIN[nw > 32][npole - 1]) {
     DeviceCtx ctx;
     int rc = device_ctx(&ctx);
     if (rc) return rc;
-    auto run = [&](auto f) {
-      return f(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status, keep_better, s, ctx);
-    };
-    const bool four = ncurve >= LM_GROUPS4_MIN;
-    if (npole == 1) return run(four ? launch_lm_groups<1, 4> : launch_lm_groups<1, 8>);
-    if (npole == 2) return run(four ? launch_lm_groups<2, 4> : launch_lm_groups<2, 8>);
-    return run(four ? launch_lm_groups<3, 4> : launch_lm_groups<3, 8>);
+    const auto run = npole == 1 ? launch_lm_groups<1> : npole == 2 ? launch_lm_groups<2> : launch_lm_groups<3>;
+    return run(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status, keep_better, s, ctx);
   }
   auto go = [&](auto kern) {
     kern<<<ncurve, 32, 0, s>>>(ncurve, nw, om, y, sign, theta_init, params, cost, iters, status,

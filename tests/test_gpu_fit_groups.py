@@ -44,3 +44,22 @@ def test_learned_start_many_curves_equal_few(gw):
                                            for i in range(0, n, 3300)))]
         for a, b in zip(many, few):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,nw,npole", [(5000, 4, 1), (8001, 40, 1), (3500, 24, 2), (5607, 33, 2),
+                                        (12200, 16, 2), (2000, 24, 3), (2003, 6, 3), (3210, 64, 3)])
+def test_groups_equal_one_curve_per_warp(gw, n, nw, npole):
+    """From the smallest numbers of curves that several per warp are taken for; the calls of at most
+    1,900 curves take one warp per curve."""
+    om = S.omega_mesh(nw)
+    y, sg = S.model_sigma_curves(6, n, om)
+    y = torch.as_tensor(y, device="cuda")
+    sg = torch.as_tensor(sg, device="cuda")
+    y[2] = 0.0
+    y[4, 3] = complex(0.0, float("inf"))
+    many = gw.continue_fit(y, om, npole=npole, sign=sg)
+    few = [torch.cat(t) for t in zip(*(gw.continue_fit(y[i:i + 1900].contiguous(), om, npole=npole,
+                                                       sign=sg[i:i + 1900].contiguous())
+                                       for i in range(0, n, 1900)))]
+    for a, b in zip(many, few):
+        assert torch.equal(torch.nan_to_num(a.double(), nan=-7.0), torch.nan_to_num(b.double(), nan=-7.0))
