@@ -233,27 +233,45 @@ __device__ __forceinline__ cplx clog_(cplx a) {
 __constant__ double kInvInt[60] = {1.0, 0.5, 0.3333333333333333, 0.25, 0.2, 0.16666666666666666, 0.14285714285714285, 0.125, 0.1111111111111111, 0.1, 0.09090909090909091, 0.08333333333333333, 0.07692307692307693, 0.07142857142857142, 0.06666666666666667, 0.0625, 0.058823529411764705, 0.05555555555555555, 0.05263157894736842, 0.05, 0.047619047619047616, 0.045454545454545456, 0.043478260869565216, 0.041666666666666664, 0.04, 0.038461538461538464, 0.037037037037037035, 0.03571428571428571, 0.034482758620689655, 0.03333333333333333, 0.03225806451612903, 0.03125, 0.030303030303030304, 0.029411764705882353, 0.02857142857142857, 0.027777777777777776, 0.02702702702702703, 0.02631578947368421, 0.02564102564102564, 0.025, 0.024390243902439025, 0.023809523809523808, 0.023255813953488372, 0.022727272727272728, 0.022222222222222223, 0.021739130434782608, 0.02127659574468085, 0.020833333333333332, 0.02040816326530612, 0.02, 0.0196078431372549, 0.019230769230769232, 0.018867924528301886, 0.018518518518518517, 0.01818181818181818, 0.017857142857142856, 0.017543859649122806, 0.017241379310344827, 0.01694915254237288, 0.016666666666666666};
 
 constexpr double SERIES_R = 0.3;
-constexpr int SERIES_N = 36;
+
+// J_3(r) = int_0^1 t^3 / (1 + r t) dt for |r| < SERIES_R by the 8-point Gauss rule of the weight t^3
+// (Golub and Welsch 1969), as one quotient: with x = 2 t - 1 and u = (r/2) / (1 + r/2),
+// J_3 = P(u) / (Q(u) (1 + r/2)), Q = prod_i (1 + u x_i), P = sum_i w_i prod_{j != i} (1 + u x_j).
+// The pole lies at |x| > 5.67, so the rule's error is below 2e-17; against 60 digits the quotient is
+// 5e-16 off at most (the power series with 36 terms: 8e-16). A polynomial of real coefficients at a
+// complex u takes two multiply-adds per coefficient (Goertzel 1958).
+__constant__ double kJ3P[8] = {0.25, 0.16578947368421052632, -0.27748538011695906433,
+                               -0.15498304584991891493, 0.083202286762658279686,
+                               0.033404589906137893754, -0.0058405818467737972382,
+                               -0.00094689356815259808036};
+__constant__ double kJ3Q[9] = {1.0, 1.2631578947368421053, -0.81871345029239766082,
+                               -1.3292053663570691434, 0.072239422084623323013,
+                               0.3660130718954248366, 0.028895768833849329205,
+                               -0.022227514487576407081, -0.0012966050117752904131};
+template <int N>
+__device__ __forceinline__ cplx real_poly(const double (&c)[N], cplx u, double p, double q) {
+  double b1 = c[N - 1], b2 = 0.0;
+#pragma unroll
+  for (int k = N - 2; k > 0; --k) {
+    const double b = fma(p, b1, fma(-q, b2, c[k]));
+    b2 = b1;
+    b1 = b;
+  }
+  return mk(fma(u.x, b1, fma(-q, b2, c[0])), u.y * b1);
+}
 
 // I_k = int_0^H t^k / (z0 + b t) dt, k = 0..3, by z0 I_k + b I_(k+1) = H^(k+1) / (k+1): with
-// r = H b / z0 small, downwards from the series I_3 = H^4 / z0 sum_m (-r)^m / (m + 4) (each step
-// damps errors by |r|); else upwards from I_0 = log(1 + r) / b. (All four sums by their series took
-// twice the multiply-adds; magnitudes by hypot and quotients by scaled division as much again.)
+// r = H b / z0 small, downwards from I_3 = H^4 J_3(r) / z0 (each step damps errors by |r|); else
+// upwards from I_0 = log(1 + r) / b. (All four by power series took eight times the multiply-adds;
+// magnitudes by hypot and quotients by scaled division came on top.)
 __device__ void moments(cplx z0, cplx b, double H, cplx I[4]) {
   const cplx iz = cdiv(mk(1.0, 0.0), z0);
   const cplx r = (H * b) * iz;
   const double rr = cnorm(r);
   if (rr < SERIES_R * SERIES_R) {
-    cplx term = mk(1.0, 0.0), s3 = mk(0.0, 0.0);
-    const cplx nr = mk(-r.x, -r.y);
-    double tmag = 1.0;
-    for (int m = 0; m < SERIES_N; ++m) {
-      s3.x = fma(kInvInt[m + 3], term.x, s3.x);
-      s3.y = fma(kInvInt[m + 3], term.y, s3.y);
-      term = term * nr;
-      tmag *= rr;
-      if (tmag < 1e-36) break;     // |r|^(m+1) below the FP64 resolution of the sum (>= 1/4)
-    }
+    const cplx h = 0.5 * r, d = cdiv(mk(1.0, 0.0), mk(1.0 + h.x, h.y)), u = h * d;
+    const double p = 2.0 * u.x, q = cnorm(u);
+    const cplx s3 = d * cdiv(real_poly(kJ3P, u, p, q), real_poly(kJ3Q, u, p, q));
     // with J_k = I_k z0 / H^(k+1): J_k = 1/(k+1) - r J_(k+1)
     const cplx s2 = mk(kInvInt[2] - fma(r.x, s3.x, -r.y * s3.y), -fma(r.x, s3.y, r.y * s3.x));
     const cplx s1 = mk(kInvInt[1] - fma(r.x, s2.x, -r.y * s2.y), -fma(r.x, s2.y, r.y * s2.x));
@@ -354,7 +372,8 @@ __device__ void piece_coeffs(const double* y, const double* m, const double* lam
 //     then Sigma_s(i w_i) += w_q f sum_j T_ij c_jp over the slot's pairs (FP64 atomics). The FP64
 //     pipe's instructions bound it (two moments of 4 per output frequency, piece and energy):
 //     8 q of 3,328 distinct energies at 16 x 16 frequencies took 3.8 ms with all four moments
-//     by their own sums, scaled divisions, hypot and one loop per q; 2.3 ms now.
+//     by their own sums, scaled divisions, hypot and one loop per q, 2.3 ms with one series and the
+//     recursion, 1.45 ms now.
 constexpr int CTHREADS = 256;
 constexpr int CIC = 16;                       // output frequencies per slot CTA
 constexpr unsigned long long EMPTY_KEY = ~0ull;   // a NaN pattern: never a valid energy
@@ -540,10 +559,11 @@ __global__ void __launch_bounds__(CTHREADS) k_conv_slot(ConvLaunch L, int nw, Om
       const int ni = min(CIC, nw_out - i0);
       const double e = __longlong_as_double(static_cast<long long>(Q.keys[slot]));
       // closed-form integrals of t^k against the kernel on every piece, and the tail
+      // (the tails last: warps that mixed both ran both)
       for (int x = tid; x < ni * (n + 1); x += blockDim.x) {
-        const int i = x / (n + 1), s = x % (n + 1);
+        const int i = x < ni * n ? x / n : x - ni * n, s = x % n;
         const cplx A = mk(-e, om_out.v[i0 + i]);
-        if (s == n) {
+        if (x >= ni * n) {
           tl[i] = tail_integral(A, 1.0, wN) + tail_integral(A, -1.0, wN);
           continue;
         }
