@@ -959,18 +959,32 @@ __global__ void __launch_bounds__(OT) k_oz_slice_rows(const __grid_constant__ Oz
 }
 
 // largest magnitude of the columns of U over 128 of its rows: grid (column blocks, row chunks,
-// problems x frequencies); thread = column. W: the problem's first frequency.
-__global__ void __launch_bounds__(OT) k_oz_uscale(const __grid_constant__ OzBatch batch, int nfmax) {
+// problems x frequencies); thread = column and quarter of the rows. W: the problem's first
+// frequency. The latency of the loads bounds it: N_b = 600, 16 frequencies 174 us with one thread per
+// column and one row at a time, 90 us with quarters and eight rows in flight (N_b = 64: 46 -> 13 us).
+constexpr int UROWS = 4;
+__global__ void __launch_bounds__(OT * UROWS) k_oz_uscale(const __grid_constant__ OzBatch batch, int nfmax) {
   const OzProb& L = batch.q[blockIdx.z / nfmax];
   const int f = blockIdx.z % nfmax, cb = blockIdx.x, ch = blockIdx.y;
   if (f >= L.nf || cb >= L.nbj || ch > cb) return;
   const double2* W = L.M + size_t(f) * L.nb * L.nb;
-  const int c = cb * OT + threadIdx.x;
+  const int n = threadIdx.x % OT, g = threadIdx.x / OT, c = cb * OT + n;
+  const int k0 = ch * OT + g * (OT / UROWS);
   float mx = 0.f, sum = 0.f;
-  for (int k = ch * OT; k < (ch + 1) * OT && k <= c; ++k) {
-    const float v = abs_up(u_entry(W, L.nb, k, c));
+#pragma unroll 8
+  for (int k = 0; k < OT / UROWS; ++k) {
+    const float v = abs_up(u_entry(W, L.nb, k0 + k, c));
     mx = fmaxf(mx, v);
     sum += v;
+  }
+  __shared__ float2 sh[UROWS][OT];
+  sh[g][n] = make_float2(mx, sum);
+  __syncthreads();
+  if (g > 0) return;
+#pragma unroll
+  for (int h = 1; h < UROWS; ++h) {
+    mx = fmaxf(mx, sh[h][n].x);
+    sum += sh[h][n].y;
   }
   L.part[(size_t(f) * L.nbj + ch) * (size_t(L.nbj) * OT) + c] = make_float2(mx, sum);
 }
@@ -1400,7 +1414,7 @@ int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig
     const int64_t cap = int64_t(ctx.sm_count) * 16;
     k_oz_rowexps<<<dim3(unsigned(std::min<int64_t>((nbi * OT * nsb + 7) / 8, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_rowexps");
-    k_oz_uscale<<<dim3(unsigned(nbj), unsigned(nbj), nz), OT, 0, s>>>(b, int(nf));
+    k_oz_uscale<<<dim3(unsigned(nbj), unsigned(nbj), nz), OT * UROWS, 0, s>>>(b, int(nf));
     GW_LAUNCH_CHECK("k_oz_uscale");
     k_oz_uexps<<<dim3(unsigned(std::min<int64_t>((nf * nbj * OT * nsb + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_uexps");
