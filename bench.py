@@ -46,17 +46,6 @@ METRIC = "P(iω)+Σ^c GFLOP/s and % of roofline, mixed vs FP64 on GB300 at ≤1e
 HERK_TRAFFIC_BYTES = {"bf16x3": (5.753e9 + 0.653e9) * 4, "tf32x3": (10.718e9 + 1.184e9) * 4}
 
 
-def cplx_tiles(nb):
-    """HERK tiles of one frequency of a complex q and whether they are the three-product layout
-    (the library's choice: C and the upper half of S over ceil(N_b / 128) blocks where that is
-    fewer than the upper half of the interleaved 2 N_b x 2 N_b Gram matrix)."""
-    nbi4 = (2 * nb + 127) // 128
-    t4 = nbi4 * (nbi4 + 1) // 2
-    nbb = (nb + 127) // 128
-    t3 = nbb * nbb + nbb * (nbb + 1) // 2
-    return (t3, True) if t3 < t4 else (t4, False)
-
-
 def workload_flops(wl):
     nw = wl.nw
     fp = sum(4.0 * wl.K(i) * wl.nb[i] * (wl.nb[i] + 1) * nw for i in range(wl.nq))
@@ -275,35 +264,12 @@ class Pipeline:
         return gw.continue_fit(self.sigma, self.om_out, npole=2, sign=self.sign)
 
     def launches_per_step(self):
-        """Kernel launches of the library in one step (the code paths of the step's calls)."""
-        import torch
-        nq, nw = self.wl.nq, self.wl.nw
-        if self.prec == "fp64":
-            p = 2                                   # FP64 HERK + fixed-order reduction
-        else:
-            # weights + prep per q; one HERK launch per group of q (a group closes at 4 work
-            # items per SM; items = 128-tiles x frequencies); the combination of the
-            # three-product tiles per such q
-            sm = torch.cuda.get_device_properties(self.dev).multi_processor_count
-            groups, items, n3 = 0, None, 0
-            for nb in self.wl.nb:
-                t, p3 = cplx_tiles(nb)
-                if items is None or items >= 4 * sm:
-                    groups, items = groups + 1, 0
-                items += t * nw
-                n3 += 1 if p3 else 0
-            p = 2 * nq + groups + n3
-        # dielectric, per batch of <= 256 systems: eps, per 32-wide panel the diagonal block
-        # (+ panel and trailing update but the last), diagonal inverses, inverse by block
-        # columns, W^c
-        nt = (max(self.wl.nb) + 31) // 32
-        w = (3 * nt + 2) * ((nq * nw + 255) // 256)
-        if self.sprec == "fp64":
-            s = 1 + nq                              # pair coefficients + per-q reductions
-        else:
-            s = 2 * nq + 1                          # A copy + B split per q, one HERK launch
-        s += 5                                      # convolution: init, hash, scan, scatter, slot
-        return p + w + s + 1                        # + LM fit
+        """Kernel launches of the library in one step, counted in a step of its own."""
+        from torch.profiler import ProfilerActivity, profile
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            self.step()
+            self.torch.cuda.synchronize()
+        return sum(e.count for e in p.key_averages() if "gw::" in e.key)
 
 
 def run_gpu(args, rank, world):
@@ -358,6 +324,7 @@ def run_gpu(args, rank, world):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         ms = float(t.item())
 
+    launches = pipe.launches_per_step()
     # end to end through the public API with host buffers: H2D of the step's inputs,
     # the step, D2H of the fitted parameters and Sigma^c
     e2e = e2e_measure(pipe, args, world)
@@ -374,11 +341,12 @@ def run_gpu(args, rank, world):
     ratio = 0.5 if args.precision == "tf32x3" else 1.0
     # the HERK runs inside a step of about half a second: the sustained peak applies
     peak_tf = (pk.get("bf16_tflops_sustained", pk["bf16_tflops"]) * ratio
-               if args.precision != "fp64" else 1.25)
-    # one HERK launch per q here (a q of this size fills a group): algorithmic flop of one q
-    # over the launch's average duration (CUDA events around each launch, on its stream)
+               if args.precision != "fp64" else pk["bf16_tflops"] / 28)   # 28 products of digit slices
+    # the step's algorithmic flop of P over the duration of its HERK launches (one per q in split
+    # precision, several in FP64; CUDA events around each launch, on its stream)
     herk_launch_ms = statistics.mean(herk_ms) if herk_ms else p_launch_ms / wl.nq
-    achieved = fp / wl.nq / (herk_launch_ms * 1e-3) / 1e12
+    herk_step_ms = sum(herk_ms) / args.steps if herk_ms else p_launch_ms
+    achieved = fp / (herk_step_ms * 1e-3) / 1e12
     line = {
         "metric": METRIC, "value": step_flops * world / (ms * 1e-3) / 1e9, "unit": "GFLOP/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
@@ -391,15 +359,15 @@ def run_gpu(args, rank, world):
                    "n_omega": wl.nw, "n_sigma_states": pipe.nsig, "precision": args.precision,
                    "sigma_precision": pipe.sprec, "l2": "inputs larger than L2 (M = "
                    f"{sum(m.numel() * m.element_size() for m in pipe.M) / 1e9:.1f} GB)"},
-        "roofline": {"bound": "tensor" if args.precision != "fp64" else "alu",
+        "roofline": {"bound": "tensor",
                      "kernel": ("k_herk_tc (split-precision HERK, one launch per q; events around "
-                                "each launch)" if args.precision != "fp64" else "k_herk_fp64"),
+                                "each launch)" if args.precision != "fp64" else "k_oz_gemm_pol (FP64 from digit slices)"),
                      "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                      "frac": achieved / peak_tf,
                      "peak_source": (f"{src} bf16 sustained x 0.5 (nominal tf32/bf16)"
                                      if args.precision == "tf32x3"
                                      else f"{src} bf16 sustained" if args.precision == "bf16x3"
-                                     else "nominal FP64 1.25 TFLOP/s"),
+                                     else "measured bf16 peak over the 28 products of an FP64 one by digit slices"),
                      "traffic": HERK_TRAFFIC_BYTES.get(args.precision),
                      "traffic_source": "ncu capture of one q at K = 102,400 scaled by K to one launch",
                      "algorithmic_bytes": wl.K(0) * wl.nb[0] * 8 + wl.nw * wl.nb[0] ** 2 * 16,
@@ -407,7 +375,7 @@ def run_gpu(args, rank, world):
                      "polarization_call_ms": p_launch_ms},
         "clocks": ck,
         "e2e": e2e,
-        "gpu_launches": pipe.launches_per_step() * args.steps,
+        "gpu_launches": launches * args.steps,
         "fp64_gpu_sample": fp64,
         "tf32x3_polarization": tf32,
         "sampled_rel_err_P": err,

@@ -57,8 +57,10 @@ enum gw_status {
  * symmetric, computed as one real SYRK of half the size and stored with zero imaginary parts. */
 enum gw_dtype { GW_C128 = 0, GW_C64 = 1, GW_R32 = 2 };
 
-/* Arithmetic of the P and Sigma contractions. GW_FP64: double precision on the
- * FP64 pipe (M must be GW_C128). GW_TF32X3 ("FP32-split"): tensor-core products of
+/* Arithmetic of the P and Sigma contractions. GW_FP64: double precision (M must be GW_C128), on
+ * the tensor cores from exact digit slices of the operands (7 of 8 bits each, so that no result
+ * is further from the exact one than on the FP64 pipe), on the FP64 pipe below 32 transitions
+ * and where operands span more than the slices hold. GW_TF32X3 ("FP32-split"): tensor-core products of
  * a two-term TF32 split of each FP32 operand (hi*hi + hi*lo + lo*hi), FP32
  * accumulation drained into FP64 partial sums (M must be GW_C64). GW_BF16X3: the
  * same with a two-term BF16 split. */
@@ -247,17 +249,20 @@ int gw_plan_waves(int nq, const int64_t* K_host, const int* nb_host, int nw, int
  * a3. Dielectric matrix and correlation part of the screened interaction in the
  * Coulomb eigenbasis (Eqs. dielec_MB, screen_MB and W^c = W - v, Sec. III.C):
  *   eps = 1 - v^1/2 P v^1/2,   W^c = v^1/2 (eps^{-1} - 1) v^1/2,
- * computed in FP64 from the Cholesky factor of eps (HPD on the imaginary axis).
+ * computed to FP64 accuracy from the Cholesky factor of eps (HPD on the imaginary axis).
  *   v_dev[q]  [N_b] double > 0 Coulomb eigenvalues,
  *   P_dev[q]  [nw][N_b][N_b] complex128 (Hermitian NSD),
  *   Wc_dev[q] [nw][N_b][N_b] complex128 output (may alias P_dev[q]).
- * The factorisation runs over many CTAs (per 32-wide panel: the diagonal block, the panel
- * below it, the trailing update), the inverse factor by block columns, W^c by block rows.
+ * The factorisation runs over many CTAs (per 32-wide panel: the diagonal block with its inverse,
+ * the panel below it, the update) and the inverse factor by block columns, in float-float. From
+ * N_b = 257 on (449 in gw_screened_w_real) the products over 128-wide blocks, the inverse factor
+ * beyond its diagonal blocks and W^c run on the tensor cores, from 7 slices of 8 bits per operand.
  * A failed factorisation (eps not positive definite, or non-finite entries) is reported by
  * gw_check as GW_ENOTHPD (GW_ENONFINITE); the later phases still run on the half-finished
  * factor, so Wc_dev (and P_dev where it aliases Wc_dev) is undefined after such an error.
- * Workspace: gw_screened_w_workspace() bytes, per (q, frequency) system
- * 16 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256. */
+ * Workspace: gw_screened_w_workspace() bytes: per (q, frequency) system
+ * 16 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of the systems from
+ * N_b = 257 on (at most 6 GB, or one system's where that is more; further systems take turns). */
 size_t gw_screened_w_workspace(int nq, const int* nb_host, int nw);
 int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev,
                   const double* const* P_dev, double* const* Wc_dev,
@@ -267,8 +272,8 @@ int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev
  * Sec. II: with inversion symmetry the basis and the wave functions can be chosen real): the
  * Cholesky factor and the inverse are real (a quarter of the FP64 work), the imaginary parts of
  * P_dev are not read (taken as zero), W^c is written with zero imaginary parts. Same layouts
- * and errors as gw_screened_w. Workspace: gw_screened_w_real_workspace() bytes, per system
- * 8 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256. */
+ * and errors as gw_screened_w. Workspace: gw_screened_w_real_workspace() bytes: per system
+ * 8 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of large systems. */
 size_t gw_screened_w_real_workspace(int nq, const int* nb_host, int nw);
 int gw_screened_w_real(int nq, const int* nb_host, int nw, const double* const* v_dev,
                        const double* const* P_dev, double* const* Wc_dev,
