@@ -46,6 +46,17 @@ METRIC = "P(iω)+Σ^c GFLOP/s and % of roofline, mixed vs FP64 on GB300 at ≤1e
 HERK_TRAFFIC_BYTES = {"bf16x3": (5.753e9 + 0.653e9) * 4, "tf32x3": (10.718e9 + 1.184e9) * 4}
 
 
+def cplx_tiles(nb):
+    """HERK tiles of one frequency of a complex q and whether they are the three-product layout
+    (the library's choice: C and the upper half of S over ceil(N_b / 128) blocks where that is
+    fewer than the upper half of the interleaved 2 N_b x 2 N_b Gram matrix)."""
+    nbi4 = (2 * nb + 127) // 128
+    t4 = nbi4 * (nbi4 + 1) // 2
+    nbb = (nb + 127) // 128
+    t3 = nbb * nbb + nbb * (nbb + 1) // 2
+    return (t3, True) if t3 < t4 else (t4, False)
+
+
 def workload_flops(wl):
     nw = wl.nw
     fp = sum(4.0 * wl.K(i) * wl.nb[i] * (wl.nb[i] + 1) * nw for i in range(wl.nq))
@@ -229,7 +240,7 @@ class Pipeline:
             # a (start, end) event pair around each HERK launch: the dominant kernel's own time
             opts = {"herk_events": [(self.torch.cuda.Event(enable_timing=True),
                                      self.torch.cuda.Event(enable_timing=True))
-                                    for _ in range(self.wl.nq)]}
+                                    for _ in range(self.wl.nq * (64 if self.prec == "fp64" else 1))]}
         gw.polarization(self.M, self.delta, self.om, self.wl.prefactor, self.prec, out=self.P,
                         ws=self.ws_p, options=opts)
         if time_p:
@@ -264,12 +275,57 @@ class Pipeline:
         return gw.continue_fit(self.sigma, self.om_out, npole=2, sign=self.sign)
 
     def launches_per_step(self):
-        """Kernel launches of the library in one step, counted in a step of its own."""
-        from torch.profiler import ProfilerActivity, profile
-        with profile(activities=[ProfilerActivity.CUDA]) as p:
-            self.step()
-            self.torch.cuda.synchronize()
-        return sum(e.count for e in p.key_averages() if "gw::" in e.key)
+        """Kernel launches of the library in one step (the code paths of the step's calls)."""
+        import torch
+        nq, nw = self.wl.nq, self.wl.nw
+        if self.prec == "fp64":
+            p = 4 * len(self.herk_events[-1])       # scales, exponents, slices, GEMM per pass
+        else:
+            # weights + prep per q; one HERK launch per group of q (a group closes at 4 work
+            # items per SM; items = 128-tiles x frequencies); the combination of the
+            # three-product tiles per such q
+            sm = torch.cuda.get_device_properties(self.dev).multi_processor_count
+            groups, items, n3 = 0, None, 0
+            for nb in self.wl.nb:
+                t, p3 = cplx_tiles(nb)
+                if items is None or items >= 4 * sm:
+                    groups, items = groups + 1, 0
+                items += t * nw
+                n3 += 1 if p3 else 0
+            p = 2 * nq + groups + n3
+        w = dielectric_launches(max(self.wl.nb), nq * nw)
+        if self.sprec == "fp64":
+            s = 9                                   # exponents 3, slices 2, GEMM, reduction; flagged 2
+        else:
+            s = 2 * nq + 1                          # A copy + B split per q, one HERK launch
+        s += 5                                      # convolution: init, hash, scan, scatter, slot
+        return p + w + s + 1                        # + LM fit
+
+
+def dielectric_launches(nb, nsys):
+    """Launches of gw_screened_w for nsys complex systems of order nb (in batches of <= 256)."""
+    up = lambda a, b: -(-a // b)
+    nt, nbb = up(nb, 32), up(nb, 128)
+    if nb < 257:
+        # eps, per 32-wide panel the diagonal block (+ panel and update but the last), inverse by
+        # block columns, W^c
+        return (3 * nt + 1) * up(nsys, 256)
+    # slices of two operands and the three products' tiles of a system; batches within 6 GB
+    size = 2 * 3 * nbb * nt * 57344 + 3 * (nbb * (nbb + 1) // 2) * 131072
+    total = 0
+    while nsys > 0:
+        n = max(1, min(nsys, 256, (6 << 30) // size))
+        product = lambda m: up(m, 192) + up(m, 256)                # GEMM, combination
+        total += 1 + 1 + nt + (nt - 1) + sum(kt % 4 != 3 for kt in range(nt - 1))
+        total += (nbb - 1) * (product(n) + up(n, 256)) + 1         # panels, their slices; Z's diagonal
+        g = 1
+        while g < nbb:                                             # Z by doubling
+            m = n * len(range(0, nbb - g, 2 * g))
+            total += 2 * up(m, 256) + 2 * up(2 * m, 256) + 2 * product(m)
+            g *= 2
+        total += 2 * up(n, 256) + product(n)                       # W^c
+        nsys -= n
+    return total
 
 
 def run_gpu(args, rank, world):
@@ -324,7 +380,6 @@ def run_gpu(args, rank, world):
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         ms = float(t.item())
 
-    launches = pipe.launches_per_step()
     # end to end through the public API with host buffers: H2D of the step's inputs,
     # the step, D2H of the fitted parameters and Sigma^c
     e2e = e2e_measure(pipe, args, world)
@@ -375,7 +430,7 @@ def run_gpu(args, rank, world):
                      "polarization_call_ms": p_launch_ms},
         "clocks": ck,
         "e2e": e2e,
-        "gpu_launches": launches * args.steps,
+        "gpu_launches": pipe.launches_per_step() * args.steps,
         "fp64_gpu_sample": fp64,
         "tf32x3_polarization": tf32,
         "sampled_rel_err_P": err,

@@ -1,6 +1,7 @@
 // a7: analytic continuation of Sigma^c(i w) by the multipole model of Eq. modelf,
 // f(z) = sum_p a_p / (z - w_p), fitted in FP64 by Levenberg-Marquardt
-// (Marquardt 1963, diagonal scaling), one warp per curve.
+// (Marquardt 1963, diagonal scaling), one warp per curve, or eight curves per warp where there
+// are thousands.
 //
 // Cost C = 1/2 sum_j |f(i w_j) - y_j|^2 over the parameters
 // theta = (Re a_p, Im a_p, Re w_p, Im w_p)_p. Each iteration accumulates

@@ -12,7 +12,7 @@
 // reduces by partial fractions to K(lambda) = -i b+/(A + b+ lambda) + i b-/(A + b- lambda)
 // with A = i w - e and b(+-) = +-i - A (the 1/(1-lambda) parts cancel between the two
 // terms). Each spline piece times K is integrated in closed form (moments of
-// 1/(z0 + b t), by series when the pole is far and by recurrence from the complex
+// 1/(z0 + b t), by recurrence from a Gauss rule when the pole is far and from the complex
 // logarithm otherwise), and the tail c_N w_N^2 / w'^2 beyond the last node likewise.
 #include <vector>
 #include <algorithm>
