@@ -283,7 +283,9 @@ __device__ void moments(cplx z0, cplx b, double H, cplx I[4]) {
     I[3] = h4 * (s3 * iz);
   } else {
     const cplx ib = cdiv(mk(1.0, 0.0), b);
-    I[0] = clog_(mk(1.0 + r.x, r.y)) * ib;
+    // 1 + r as (z0 + H b) / z0: with the pole beside the piece's end the sum 1 + r would cancel to
+    // the roundings of r
+    I[0] = clog_(mk(fma(H, b.x, z0.x), fma(H, b.y, z0.y)) * iz) * ib;
     double hk = 1.0;
 #pragma unroll
     for (int k = 1; k < 4; ++k) {
