@@ -834,8 +834,9 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
 
 // What to slice: blocks of 128 lines (columns of M, or rows with DZ_ROWS) and stages of 32 values
 // along each line, of a float-float matrix M (row-major n x n); DZ_LOWER: entries above the
-// diagonal count as zero, DZ_CONJ: the conjugate.
-enum : int { DZ_ROWS = 1, DZ_LOWER = 2, DZ_CONJ = 4 };
+// diagonal count as zero, DZ_CONJ: the conjugate; DZ_FACTOR: rows of the Cholesky factor, whose
+// magnitudes mx are bounds that hold for a positive definite eps only.
+enum : int { DZ_ROWS = 1, DZ_LOWER = 2, DZ_CONJ = 4, DZ_FACTOR = 8 };
 struct DzSlice {
   const void* M;            // FFC or FF entries
   char* out;                // (set, block, stage) = (0, 0, 0)
@@ -895,9 +896,13 @@ __global__ void __launch_bounds__(OT) k_dz_max(const __grid_constant__ DzSliceBa
   }
 }
 
-// the slices: grid (stages, blocks x 4, jobs), four lanes per line
+// The slices: grid (stages, blocks x 4, jobs), four lanes per line. The digits wrap beyond the
+// line's exponent (an entry of 8 at a bound of 1 would read as zero), so every entry is compared with
+// the bound: a row of the factor beyond sqrt(eps_ii) belongs to an eps that is not positive definite
+// (its pivot would be negative), anything else beyond the largest magnitude is not finite.
 template <typename FT>
-__global__ void __launch_bounds__(OT) k_dz_slice(const __grid_constant__ DzSliceBatch batch) {
+__global__ void __launch_bounds__(OT) k_dz_slice(const __grid_constant__ DzSliceBatch batch,
+                                                 unsigned* status) {
   const DzSlice& J = batch.j[blockIdx.z];
   const int b = blockIdx.y >> 2;
   if (int(blockIdx.x) >= J.nst || b >= J.nblk) return;
@@ -905,18 +910,22 @@ __global__ void __launch_bounds__(OT) k_dz_slice(const __grid_constant__ DzSlice
   if (dz_empty(J, J.blk0 + b, st * OKS)) return;
   const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
   const int line = (J.blk0 + b) * OT + n, k0 = st * OKS + kc * 8;
-  const int E = exponent_of(J.mx[line]);
+  const float mx = J.mx[line], most = fminf(1.0001f * mx, 3.4e38f);
+  const int E = exponent_of(mx);
+  bool bad = false;
   char* out = J.out + (J.blk0 + b) * J.blk + int64_t(st) * OBLK;
   long long xr[8], xi[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const FFC x = dz_entry<FT>(J, line, k0 + k);
+    bad = bad || !(fabsf(x.re.h) <= most) || !(fabsf(x.im.h) <= most);
     xr[k] = fixed_f32(x.re.h, E) + fixed_f32(x.re.l, E);
     if constexpr (sizeof(FT) == sizeof(FFC)) {
       const long long v = fixed_f32(x.im.h, E) + fixed_f32(x.im.l, E);
       xi[k] = (J.mode & DZ_CONJ) ? -v : v;
     }
   }
+  if (bad) raise_status(status, (J.mode & DZ_FACTOR) ? ST_ENOTHPD : ST_ENONFINITE);
   uint32_t w[OSL][4];
   fixed_digits8(xr, w);
   store_digits(out, n, kc, w);
@@ -1071,7 +1080,8 @@ static size_t dz_workspace(const std::vector<int>& ns, bool cplx, int sm) {
 }
 
 template <typename FT>
-static int dz_launch_slices(const std::vector<DzSlice>& jobs, cudaStream_t s, bool find_max) {
+static int dz_launch_slices(const std::vector<DzSlice>& jobs, cudaStream_t s, const DeviceCtx& ctx,
+                            bool find_max) {
   for (size_t j0 = 0; j0 < jobs.size(); j0 += DZ_MAX) {
     const int n = int(std::min<size_t>(DZ_MAX, jobs.size() - j0));
     DzSliceBatch b;
@@ -1087,7 +1097,7 @@ static int dz_launch_slices(const std::vector<DzSlice>& jobs, cudaStream_t s, bo
       k_dz_max<FT><<<dim3(unsigned(nblk), unsigned((nst + SPB - 1) / SPB), unsigned(n)), OT, 0, s>>>(b);
       GW_LAUNCH_CHECK("k_dz_max");
     }
-    k_dz_slice<FT><<<dim3(unsigned(nst), unsigned(4 * nblk), unsigned(n)), OT, 0, s>>>(b);
+    k_dz_slice<FT><<<dim3(unsigned(nst), unsigned(4 * nblk), unsigned(n)), OT, 0, s>>>(b, ctx.status);
     GW_LAUNCH_CHECK("k_dz_slice");
   }
   return GW_OK;
@@ -1253,7 +1263,8 @@ struct DzChunk {
           cb.push_back(combine(y, pr.back(), y.S.E));
         }
         if (kb + 1 < y.p.nbb)
-          sl.push_back(slice(y, y.S.E, y.X1, y.mag(0), DZ_ROWS, kb + 1, y.p.nbb - kb - 1, SPB * kb, SPB));
+          sl.push_back(slice(y, y.S.E, y.X1, y.mag(0), DZ_ROWS | DZ_FACTOR,
+                             kb + 1, y.p.nbb - kb - 1, SPB * kb, SPB));
       }
       int rc = run<DZ_SUB>(pr, cb);
       if (rc) return rc;
@@ -1271,7 +1282,7 @@ struct DzChunk {
         k_chol_update<T><<<dim3(unsigned(tiles), nsys), DTHREADS, smem_u, s>>>(batch, kt, jend);
         GW_LAUNCH_CHECK("k_chol_update");
       }
-      if ((rc = dz_launch_slices<FT>(sl, s, false))) return rc;
+      if ((rc = dz_launch_slices<FT>(sl, s, ctx, false))) return rc;
     }
     return GW_OK;
   }
@@ -1308,9 +1319,9 @@ struct DzChunk {
           tile0 += q.ntile;
         }
       }
-      int rc = dz_launch_slices<FT>(s1, s, true);
+      int rc = dz_launch_slices<FT>(s1, s, ctx, true);
       if (!rc) rc = run<DZ_PUT>(p1, c1);
-      if (!rc) rc = dz_launch_slices<FT>(s2, s, true);
+      if (!rc) rc = dz_launch_slices<FT>(s2, s, ctx, true);
       if (!rc) rc = run<DZ_NEG>(p2, c2);
       if (rc) return rc;
     }
@@ -1327,7 +1338,7 @@ struct DzChunk {
                            OZC_UPPER | OZC_KA | OZC_KB));
       cb.push_back(combine(y, pr.back(), nullptr));
     }
-    int rc = dz_launch_slices<FT>(sl, s, true);
+    int rc = dz_launch_slices<FT>(sl, s, ctx, true);
     return rc ? rc : run<DZ_W>(pr, cb);
   }
 };
