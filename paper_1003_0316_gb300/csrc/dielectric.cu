@@ -835,8 +835,10 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
 // What to slice: blocks of 128 lines (columns of M, or rows with DZ_ROWS) and stages of 32 values
 // along each line, of a float-float matrix M (row-major n x n); DZ_LOWER: entries above the
 // diagonal count as zero, DZ_CONJ: the conjugate; DZ_FACTOR: rows of the Cholesky factor, whose
-// magnitudes mx are bounds that hold for a positive definite eps only.
-enum : int { DZ_ROWS = 1, DZ_LOWER = 2, DZ_CONJ = 4, DZ_FACTOR = 8 };
+// magnitudes mx are bounds that hold for a positive definite eps only. DZ_KUP, DZ_KDOWN: the two
+// operands of a product scaled along K by powers of two that cancel: a line's digits end 2^-55 below
+// its largest entry, so entries that meet large partners must not be small on their line.
+enum : int { DZ_ROWS = 1, DZ_LOWER = 2, DZ_CONJ = 4, DZ_FACTOR = 8, DZ_KUP = 16, DZ_KDOWN = 32 };
 struct DzSlice {
   const void* M;            // FFC or FF entries
   char* out;                // (set, block, stage) = (0, 0, 0)
@@ -844,6 +846,7 @@ struct DzSlice {
   int64_t set, blk;         // strides in bytes
   int n, mode;
   int blk0, nblk, st0, nst;
+  const float* kscale;      // DZ_KUP / DZ_KDOWN: value k times / over 2^(exponent of kscale[k])
 };
 constexpr int DZ_MAX = 256;
 struct DzSliceBatch {
@@ -862,6 +865,14 @@ __device__ __forceinline__ FFC dz_entry(const DzSlice& J, int line, int k) {
   if (!in) return FFC{};
   return ff_cplx((J.mode & DZ_ROWS) ? M[size_t(line) * J.n + k] : M[size_t(k) * J.n + line]);
 }
+
+// the exponent of value k's scale (0 without one)
+__device__ __forceinline__ int dz_kexp(const DzSlice& J, int k) {
+  if (!(J.mode & (DZ_KUP | DZ_KDOWN)) || k >= J.n) return 0;
+  const int e = max(-60, min(60, (int(__float_as_uint(J.kscale[k]) >> 23) & 0xff) - 127));
+  return (J.mode & DZ_KUP) ? e : -e;
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
 // whether values k0 .. k0 + 31 of a block's lines are all above the diagonal (never read)
 __device__ __forceinline__ bool dz_empty(const DzSlice& J, int blk, int k0) {
@@ -883,7 +894,7 @@ __global__ void __launch_bounds__(OT) k_dz_max(const __grid_constant__ DzSliceBa
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = warp; i < OT; i += OT / 32) {
       float m = 0.0f;
-      for (int k = k0 + lane; k < k1; k += 32) m = fmaxf(m, mag(dz_entry<FT>(J, line0 + i, k)));
+      for (int k = k0 + lane; k < k1; k += 32) m = fmaxf(m, mag(dz_entry<FT>(J, line0 + i, k)) * pow2f(dz_kexp(J, k)));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
       if (lane == 0) atomicMax(reinterpret_cast<int*>(J.mx) + line0 + i, __float_as_int(m));
@@ -891,7 +902,7 @@ __global__ void __launch_bounds__(OT) k_dz_max(const __grid_constant__ DzSliceBa
   } else {
     const int line = line0 + threadIdx.x;
     float m = 0.0f;
-    for (int k = k0; k < k1; ++k) m = fmaxf(m, mag(dz_entry<FT>(J, line, k)));
+    for (int k = k0; k < k1; ++k) m = fmaxf(m, mag(dz_entry<FT>(J, line, k)) * pow2f(dz_kexp(J, k)));
     atomicMax(reinterpret_cast<int*>(J.mx) + line, __float_as_int(m));
   }
 }
@@ -911,14 +922,16 @@ __global__ void __launch_bounds__(OT) k_dz_slice(const __grid_constant__ DzSlice
   const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
   const int line = (J.blk0 + b) * OT + n, k0 = st * OKS + kc * 8;
   const float mx = J.mx[line], most = fminf(1.0001f * mx, 3.4e38f);
-  const int E = exponent_of(mx);
+  const int E0 = exponent_of(mx);
   bool bad = false;
   char* out = J.out + (J.blk0 + b) * J.blk + int64_t(st) * OBLK;
   long long xr[8], xi[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const FFC x = dz_entry<FT>(J, line, k0 + k);
-    bad = bad || !(fabsf(x.re.h) <= most) || !(fabsf(x.im.h) <= most);
+    const int e = dz_kexp(J, k0 + k), E = E0 - e;
+    const float sc = pow2f(e);
+    bad = bad || !(fabsf(x.re.h) * sc <= most) || !(fabsf(x.im.h) * sc <= most);
     xr[k] = fixed_f32(x.re.h, E) + fixed_f32(x.re.l, E);
     if constexpr (sizeof(FT) == sizeof(FFC)) {
       const long long v = fixed_f32(x.im.h, E) + fixed_f32(x.im.l, E);
@@ -1185,6 +1198,7 @@ struct DzChunk {
     j.nblk = nblk;
     j.st0 = st0;
     j.nst = nst;
+    j.kscale = y.mag(0);                     // sqrt(eps_kk)
     return j;
   }
   static OzC product(const Sys& y, const char* X, const float* mx, const char* Y, const float* my, int a0,
@@ -1309,9 +1323,12 @@ struct DzChunk {
           q.G += size_t(tile0) * q.nprod * OT * OT;
           p1.push_back(q);
           c1.push_back(combine(y, q, y.S.Z));
-          // -Z22 T from conj(Z22) and T
-          s2.push_back(slice(y, y.S.Z, y.X2, mt, 0, j, g, ks1, ks2 - ks1));
-          s2.push_back(slice(y, y.S.Z, y.X1, m22, DZ_ROWS | DZ_LOWER | DZ_CONJ, h, e - h, ks1, ks2 - ks1));
+          // -Z22 T from conj(Z22) and T, scaled along K to unit diagonal of eps: T has the size of
+          // the rows of L, Z22 that of their reciprocals (with eps_ii over 6 decades, N = 600, the
+          // error of W^c against 80 bits was 3e-10 without it, 1e-13 with it)
+          s2.push_back(slice(y, y.S.Z, y.X2, mt, DZ_KDOWN, j, g, ks1, ks2 - ks1));
+          s2.push_back(slice(y, y.S.Z, y.X1, m22, DZ_ROWS | DZ_LOWER | DZ_CONJ | DZ_KUP, h, e - h, ks1,
+                             ks2 - ks1));
           q = product(y, y.X1, m22, y.X2, mt, h, e, j, h, ks1, ks2, OZC_KTOP);
           q.G += size_t(tile0) * q.nprod * OT * OT;
           p2.push_back(q);

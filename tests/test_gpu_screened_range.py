@@ -1,9 +1,16 @@
 """The screened interaction outside the range of well-behaved matrices: an eps that is not positive
-definite is an error wherever its large entries stand.
+definite is an error wherever its large entries stand, and an eps whose diagonal spans many decades
+is as exact as one with a unit diagonal.
 
 An indefinite eps: the identity but for a pair of off-diagonal entries of magnitude above 1, in a
 32-block, a 128-block or a panel other than the pivot's. The factor's entry passes the bound
 sqrt(eps_ii) of a positive definite matrix, and the pivot 1 - |x|^2 is negative.
+
+Scales: for eps = S B S with S diagonal, eps^-1 = S^-1 B^-1 S^-1, and Cholesky, inverse and product
+keep the errors relative to S, |d eps^-1_IJ| <= c sqrt(eps^-1_II eps^-1_JJ) with c of the order of
+2^-48 times N and the condition number of B. With B within 1 of the identity by 0.5 (condition 3) and
+N <= 700: 1e-11 would be generous, 2e-12 is asked for; the FP64 inverse that it is compared with is
+scaled the same way.
 """
 import pytest
 
@@ -57,3 +64,22 @@ def test_indefinite_random_is_an_error(gw, n, real):
         gw.check()
     assert e.value.code == gw.GW_ENOTHPD
 
+
+
+@pytest.mark.parametrize("n,real", [(200, False), (300, False), (513, True), (640, False)])
+@pytest.mark.parametrize("lo,hi", [(-2, 2), (-3, 3), (0, 6)])
+def test_scaled_diagonal(gw, n, real, lo, hi):
+    g = torch.Generator(device="cuda").manual_seed(n + hi)
+    x = torch.randn((n, n, 2), generator=g, dtype=torch.float64, device="cuda")
+    x = x[..., 0].to(torch.complex128) if real else torch.view_as_complex(x)
+    x = x + x.mH
+    B = torch.eye(n, dtype=torch.complex128, device="cuda") + 0.5 * x / torch.linalg.matrix_norm(x, 2)
+    u = torch.rand(n, generator=g, dtype=torch.float64, device="cuda")
+    s = 2.0 ** torch.round(3.3219 * (lo + (hi - lo) * u))
+    eps = s[:, None] * B * s[None, :]
+    W = w_of(gw, eps, real)
+    gw.check()
+    eye = torch.eye(n, dtype=torch.complex128, device="cuda")
+    inv = torch.linalg.inv((eye - (eye - eps)) / (s[:, None] * s[None, :]))     # of the P passed in
+    off = ~eye.bool()
+    assert float(((W * s[:, None] * s[None, :] - inv).abs())[off].max()) <= 2e-12
