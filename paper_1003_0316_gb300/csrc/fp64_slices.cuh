@@ -83,9 +83,9 @@ __device__ __forceinline__ void store_digits(char* blk, int n, int kc, const uin
     *reinterpret_cast<uint4*>(blk + i * SLB + off) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
 
-// E with 2.01 m < 2^E for an FP32 magnitude m (zero, and what is below the normal range: -126)
+// E with 1.005 m < 2^E for an FP32 magnitude m (zero, and what is below the normal range: -126)
 __device__ __forceinline__ int exponent_of(float m) {
-  return (int(__float_as_uint(2.01f * m) >> 23) & 0xff) - 126;
+  return (int(__float_as_uint(1.005f * m) >> 23) & 0xff) - 126;
 }
 
 // ---- complex products of sliced operands (fp64_tc.cu, k_oz_gemm_cplx) ------------------------------
@@ -97,7 +97,7 @@ enum : int { OZC_UPPER = 1, OZC_KA = 2, OZC_KB = 4, OZC_KTOP = 8 };
 struct OzC {
   const char* X;            // slices: set, block and stage (0, 0, 0); strides in bytes
   const char* Y;
-  const float* mx;          // largest magnitude per row of X, column of Y (block 0)
+  const float* mx;          // bound of the magnitudes of all sets per row of X, column of Y (block 0)
   const float* my;
   float2* G;
   int64_t xset, xblk, yset, yblk;

@@ -14,6 +14,11 @@
 //     K = 32 between drains (g = 5 is drained every 2, see below);
 //   g = 6, 7, 8 (18 pairs, "low") together in one accumulator, 2^-32 below the leading group: their
 //     truncating FP32 chain stays near 2^-50 of the result, where FP64 sums round as well.
+//     The complex products of the dielectric sum g = 6 by itself (exactly) and take g = 9 as well:
+//     the entries of a Cholesky factor are far below the bound of their row, and both the truncation
+//     and what is left out count against that bound, K^1/2 times. 4,096 basis functions, eigenvalues
+//     of eps over six decades, error of eps^-1: 7.1e-9 without the exact g = 6, 3.7e-9 without g = 9,
+//     3.1e-10 with both, 1.1e-9 in float-float; 128 systems of N_b = 600 12.34 -> 13.49 ms.
 // The epilogue keeps three FP32 sums per element, s (groups 2-4), c (exact rounding errors of s,
 // and group 5) and d (exact rounding errors of c, and the low groups), by two-sums, so nothing
 // above 2^-24 of the low groups is lost; a superblock's result (s + c) + d goes to FP64 with the
@@ -38,6 +43,7 @@
 // the low groups and group 5 so that each is drained while C's MMAs run:
 //   even stage: g4; low, drain; g3, g2; g5
 //   odd stage:  g5 (continuing), drain; g4, g3, g2 (drains due every 8 stages); low, drain
+// (with an exact g6, that follows low in D: five drains of D per two stages instead of three)
 // (low starts afresh in every stage, its smallest products first: continuing it over a second
 // stage adds 26 truncating MMAs to a large accumulator and cost 3x the error of P)
 // Eight epilogue warps drain (two per lane quadrant, 64 columns each).
@@ -111,6 +117,9 @@ static_assert(sizeof(OzCBatch) < 32000, "kernel parameter space");
 enum : int { OZ_POL, OZ_QUAD, OZ_CPLX };
 template <int MODE> struct OzBatchOf { using B = OzBatch; using P = OzProb; };
 template <> struct OzBatchOf<OZ_CPLX> { using B = OzCBatch; using P = OzC; };
+
+// whether a mode sums group 6 by itself (exactly), and group 9 as well
+constexpr bool oz_exact6(int mode) { return mode == OZ_CPLX; }
 
 // One work item: its problem, operand slices (stage 0), stage range, stages per superblock, and the
 // indexes that its output needs.
@@ -245,6 +254,7 @@ __device__ __forceinline__ int4 ld_exp4(const int* p) {
 template <int MODE>
 __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch, unsigned* status) {
   constexpr uint32_t IDESC = tc::instr_desc(1u, OT, OT);
+  constexpr bool EXACT6 = oz_exact6(MODE);
   extern __shared__ __align__(1024) char dsmem[];
   char* ring = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
   // full/empty per stage part (0: slices 1-4, 1: slices 5-7); D and C: the accumulators
@@ -326,12 +336,23 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
         for (int i = 0; i < 16; ++i) sp_s[(h * 16 + i) * OT] = sv[i];
       }
     };
-    // D: group 5 into c, the low groups into d; false after an expired wait
-    auto drain_d = [&](bool g5) {
+    // D: group 5 (and an exact group 6) into c, the low groups into d; false after an expired wait
+    auto drain_d = [&](bool exact) {
       if (!oz_wait(&fullD, gD & 1, &s_abort, status)) return false;
       ++gD;
       tc::tc_fence_after();
-      if (g5) {
+      if constexpr (EXACT6) {
+        // five drains per two stages: the accumulator is free as soon as it is in registers
+        uint64_t v[32];
+        tc::tmem_ld64p(base, v);
+        tc::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&emptyD);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) add(d[i], exact ? two_sum(c[i], v[i]) : v[i]);
+        return true;
+      }
+      if (exact) {
 #pragma unroll
         for (int h = 0; h < 8; ++h) {
           uint64_t v[4];
@@ -367,7 +388,9 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
         bool fresh = true;                    // s is zero
         for (int k = 0; k < n; ++k) {
           const bool last = k == n - 1;
-          if (!drain_d(k & 1)) {               // even: low, odd: group 5
+          // even: low, (6,) the accumulators due, group 5 unless the next odd stage continues it;
+          // odd: group 5, the accumulators due, low(, 6)
+          if (!drain_d(k & 1) || (EXACT6 && !(k & 1) && !drain_d(true))) {
             stop = true;
             break;
           }
@@ -388,8 +411,7 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&emptyC);
           }
-          // odd: low; even: group 5, which the next odd stage continues
-          if (((k & 1) || last) && !drain_d(!(k & 1))) {
+          if ((((k & 1) || last) && !drain_d(!(k & 1))) || (EXACT6 && (k & 1) && !drain_d(true))) {
             stop = true;
             break;
           }
@@ -584,9 +606,17 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
               }
             };
             auto low = [&]() {                          // a fresh D, the smallest products first
-              group(8, tm, 0u);
+              if constexpr (EXACT6) group(9, tm, 0u);
+              group(8, tm, EXACT6 ? 1u : 0u);
               group(7, tm, 1u);
-              group(6, tm, 1u);
+              if constexpr (!EXACT6) {
+                group(6, tm, 1u);
+                tc::mma_commit(&empty[slot][1]);
+              }
+              tc::mma_commit(&fullD);
+            };
+            auto g6 = [&]() {                           // EXACT6: a D of its own
+              group(6, tm, 0u);
               tc::mma_commit(&empty[slot][1]);
               tc::mma_commit(&fullD);
             };
@@ -595,6 +625,12 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
               group(3, tm + 2 * OT, (k & 15) ? 1u : 0u);
               group(2, tm + 3 * OT, (k & 31) ? 1u : 0u);
               if (due) tc::mma_commit(&fullC);
+            };
+            // the next D, once the epilogue has drained the last one
+            auto next_d = [&]() {
+              if (!wait(&emptyD, (nD & 1) ^ 1)) return false;
+              tc::tc_fence_after();
+              return true;
             };
             if (odd) {
               if (tc::elect_one()) {
@@ -605,34 +641,51 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
               ++nD;
               if (!wait(&emptyC, (nC & 1) ^ 1)) break;
               tc::tc_fence_after();
+              // (with the drain of the accumulators due, before low, so that it runs beside it)
               if (tc::elect_one()) {
                 g4();
-                g32();
+                if (!EXACT6 || due) g32();
               }
               __syncwarp();
-              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
-              tc::tc_fence_after();
+              if (!next_d()) break;
               if (tc::elect_one()) {
                 low();
-                tc::mma_commit(&empty[slot][0]);
+                if (EXACT6 && !due) g32();
+                if (!EXACT6) tc::mma_commit(&empty[slot][0]);
               }
               __syncwarp();
               ++nD;
+              if constexpr (EXACT6) {
+                if (!next_d()) break;
+                if (tc::elect_one()) {
+                  g6();
+                  tc::mma_commit(&empty[slot][0]);
+                }
+                __syncwarp();
+                ++nD;
+              }
             } else {
               if (!wait(&emptyC, (nC & 1) ^ 1)) break;
               tc::tc_fence_after();
               if (tc::elect_one()) g4();
               __syncwarp();
-              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
-              tc::tc_fence_after();
+              if (!next_d()) break;
               if (tc::elect_one()) {
                 low();
-                g32();
+                if (!EXACT6) g32();
               }
               __syncwarp();
               ++nD;
-              if (!wait(&emptyD, (nD & 1) ^ 1)) break;
-              tc::tc_fence_after();
+              if constexpr (EXACT6) {
+                if (!next_d()) break;
+                if (tc::elect_one()) {
+                  g6();
+                  g32();
+                }
+                __syncwarp();
+                ++nD;
+              }
+              if (!next_d()) break;
               if (tc::elect_one()) {
                 group(5, tm, 0u);
                 tc::mma_commit(&empty[slot][0]);

@@ -1,6 +1,7 @@
 """The screened interaction outside the range of well-behaved matrices: an eps that is not positive
 definite is an error wherever its large entries stand, and an eps whose diagonal spans many decades
-is as exact as one with a unit diagonal.
+is as exact as one with a unit diagonal, and a spectrum of many decades costs no more than the
+float-float storage does.
 
 An indefinite eps: the identity but for a pair of off-diagonal entries of magnitude above 1, in a
 32-block, a 128-block or a panel other than the pivot's. The factor's entry passes the bound
@@ -11,6 +12,12 @@ keep the errors relative to S, |d eps^-1_IJ| <= c sqrt(eps^-1_II eps^-1_JJ) with
 2^-48 times N and the condition number of B. With B within 1 of the identity by 0.5 (condition 3) and
 N <= 700: 1e-11 would be generous, 2e-12 is asked for; the FP64 inverse that it is compared with is
 scaled the same way.
+
+Spectra: eps = H diag(lambda) H^T / N with a Hadamard matrix and powers of two from 1 to kappa is exact
+in FP64, and so is its inverse. Float-float rounds every entry of eps and of the panels' updates by
+2^-49 at most; entries are sqrt(N) below the largest eigenvalue, so the rounding errors (rms 0.3 of
+their bound, the 2-norm of N x N of them 2 sqrt(N) rms) disturb eps by 0.1 to 0.2 of 2^-48 kappa for
+the few updates of an entry: 0.4 2^-48 kappa of eps^-1 in the Frobenius norm.
 """
 import pytest
 
@@ -83,3 +90,27 @@ def test_scaled_diagonal(gw, n, real, lo, hi):
     inv = torch.linalg.inv((eye - (eye - eps)) / (s[:, None] * s[None, :]))     # of the P passed in
     off = ~eye.bool()
     assert float(((W * s[:, None] * s[None, :] - inv).abs())[off].max()) <= 2e-12
+
+
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("decades", [10, 20])
+def test_wide_spectrum(gw, real, decades):
+    n = 1024
+    H = torch.ones((1, 1), dtype=torch.float64, device="cuda")
+    while H.shape[0] < n:
+        H = torch.cat([torch.cat([H, H], 1), torch.cat([H, -H], 1)], 0)
+    g = torch.Generator(device="cuda").manual_seed(decades)
+    k = torch.arange(n, device="cuda") * (decades + 1) // n
+    lam = 2.0 ** k[torch.randperm(n, generator=g, device="cuda")].double()
+    sign = torch.where(torch.rand(n, generator=g, device="cuda") < 0.5, -1.0, 1.0).double()
+    H = H * sign[:, None]                               # not the Sylvester matrix itself: its factors are special
+    eps, inv = ((H * d[None, :] / n) @ H.T for d in (lam, 1.0 / lam))
+    ph = torch.ones(n, dtype=torch.complex128, device="cuda")
+    if not real:
+        ph = torch.exp(0.5j * torch.pi * torch.randint(4, (n,), generator=g, device="cuda"))
+        ph = torch.complex(ph.real.round(), ph.imag.round())
+    eps, inv = (ph[:, None] * x * ph.conj()[None, :] for x in (eps, inv))
+    W = w_of(gw, eps, real)
+    gw.check()
+    ref = inv - torch.eye(n, dtype=torch.complex128, device="cuda")
+    assert float((W - ref).norm() / inv.norm()) <= 0.4 * 2.0 ** (decades - 48)
