@@ -135,9 +135,11 @@ __device__ __forceinline__ FF to_ff(double x) {
 }
 // to_ff by integer arithmetic (each FP64 conversion occupies the FP64 pipe like a multiply-add): h
 // from the magnitude rounded to 24 bits (to nearest, ties to even), l from the remaining bits, whose
-// integer difference is exact. l of a value below 2^-73 is zero.
+// integer difference is exact. Below 2^-73, where the power of two of l leaves the FP32 range, the
+// conversions (rare: entries of eps that small are mostly zeros).
 __device__ __forceinline__ FF split_ff(double x) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x)) & 0x7fffffffffffffffull;
+  if (b != 0 && (b >> 52) < 1023 - 73) return to_ff(x);
   const unsigned long long hb = (b + 0x0fffffffull + ((b >> 29) & 1ull)) & ~0x1fffffffull;
   const int ex = int(b >> 52);                                   // biased by 1023
   const uint32_t sign = static_cast<uint32_t>(__double2hiint(x)) & 0x80000000u;
@@ -145,7 +147,7 @@ __device__ __forceinline__ FF split_ff(double x) {
   const uint32_t hbits = hf < 0x00800000ll ? 0u : hf > 0x7f800000ll ? 0x7f800000u : uint32_t(hf);
   const float d = float(int(static_cast<long long>(b) - static_cast<long long>(hb)));
   const int se = ex - 1023 - 52 + 127;                           // 2^(e - 52)
-  const float l = hbits == 0u || se < 1 ? 0.0f : d * __int_as_float(se << 23);
+  const float l = hbits == 0u ? 0.0f : d * __int_as_float(se << 23);
   return FF{__uint_as_float(hbits | sign), __uint_as_float(__float_as_uint(l) ^ sign)};
 }
 __device__ __forceinline__ FF split_ff_t(double x) { return split_ff(x); }

@@ -1,7 +1,7 @@
-"""The screened interaction outside the range of well-behaved matrices: an eps that is not positive
-definite is an error wherever its large entries stand, and an eps whose diagonal spans many decades
-is as exact as one with a unit diagonal, and a spectrum of many decades costs no more than the
-float-float storage does.
+"""The screened interaction outside the range of well-behaved matrices. An eps that is not positive
+definite is an error wherever its large entries stand; an eps whose diagonal spans many decades is as
+exact as one with a unit diagonal; a spectrum of many decades costs no more than the float-float
+storage does; below 257 basis functions small entries of eps keep their own relative precision.
 
 An indefinite eps: the identity but for a pair of off-diagonal entries of magnitude above 1, in a
 32-block, a 128-block or a panel other than the pivot's. The factor's entry passes the bound
@@ -114,3 +114,20 @@ def test_wide_spectrum(gw, real, decades):
     gw.check()
     ref = inv - torch.eye(n, dtype=torch.complex128, device="cuda")
     assert float((W - ref).norm() / inv.norm()) <= 0.4 * 2.0 ** (decades - 48)
+
+
+@pytest.mark.parametrize("lo", [-20, -26])
+@pytest.mark.parametrize("real", [False, True])
+def test_small_entries_keep_their_precision(gw, lo, real):
+    n = 70
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((n, n, 2), generator=g, dtype=torch.float64, device="cuda")
+    x = x[..., 0].to(torch.complex128) if real else torch.view_as_complex(x)
+    x = torch.tril(x, -1) * 10.0 ** lo
+    x = x + x.mH
+    eye = torch.eye(n, dtype=torch.complex128, device="cuda")
+    W = gw.screened_w([-x[None].contiguous()], [torch.ones(n, dtype=torch.float64, device="cuda")],
+                      real=real)[0][0]
+    gw.check()
+    off = ~eye.bool()
+    assert float(((W + x).abs() / x.abs().clamp(min=1e-300))[off].max()) <= 1e-12
