@@ -1385,6 +1385,12 @@ static int launch_dielectric(std::vector<DieSysT<T>>& sys, WsCursor dz, float* s
   }
   constexpr bool CPLX = sizeof(T) == sizeof(double2);
   const bool by_columns = !sys.empty() && sys[0].D != nullptr;
+  // The systems of the sliced path behind the others, whatever the order of the sizes in the call: a
+  // batch is of one kind, and sizes that alternate around the limit would make a batch (a chain of
+  // three launches per 32 columns) per q: 8 q of 250 and 260 in turn, 16 frequencies, 10.4 -> 4.6 ms.
+  if (by_columns)
+    std::stable_partition(sys.begin(), sys.end(),
+                          [](const DieSysT<T>& S) { return !dz_takes(S.n, CPLX); });
   for (size_t b0 = 0; b0 < sys.size();) {
     // up to DMAXSYS systems; those of the sliced path apart from the others, within the slice budget
     const bool sliced = by_columns && dz_takes(sys[b0].n, CPLX);
