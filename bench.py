@@ -295,7 +295,8 @@ class Pipeline:
             p = 2 * nq + groups + n3
         w = dielectric_launches(max(self.wl.nb), nq * nw)
         if self.sprec == "fp64":
-            s = 9                                   # exponents 3, slices 2, GEMM, reduction; flagged 2
+            # scales, exponents 3, guard, slices 2, GEMM 2, reduction; FP64 kernel 2 (by flags)
+            s = 12
         else:
             s = 2 * nq + 1                          # A copy + B split per q, one HERK launch
         s += 5                                      # convolution: init, hash, scan, scatter, slot

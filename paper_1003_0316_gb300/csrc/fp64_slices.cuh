@@ -75,6 +75,14 @@ __device__ __forceinline__ void digits8(const double (&v)[8], int E, uint32_t (&
   fixed_digits8(X, w);
 }
 
+// the same with an exponent per value (the line's E less the exponent of the value's own scale)
+__device__ __forceinline__ void digits8(const double (&v)[8], const int (&E)[8], uint32_t (&w)[OSL][4]) {
+  long long X[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) X[k] = fixed_f64(v[k], E[k]);
+  fixed_digits8(X, w);
+}
+
 // 16 bytes of every slice of row n at K chunk kc of a stage's block
 __device__ __forceinline__ void store_digits(char* blk, int n, int kc, const uint32_t (&w)[OSL][4]) {
   const uint32_t off = swz64(n, kc);

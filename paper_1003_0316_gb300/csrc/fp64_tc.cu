@@ -68,6 +68,9 @@ constexpr uint64_t OWAIT = 2000000000ull;   // ns per bounded wait
 constexpr int CHROWS = 64;                  // rows per scale chunk (superblocks are multiples)
 constexpr float RATIO_MAX = 1024.0f;        // largest entry against the mean magnitude of a column
 
+// bits of a problem's flag: the FP64 kernel does it; the GEMM with an exact group 6 does it
+enum : int { FLAG_FP64 = 1, FLAG_EXACT6 = 2 };
+
 // One problem: a q point's polarization over a range of rows and frequencies, or (QF) the pair
 // coefficients of a range of pairs and frequencies.
 struct OzProb {
@@ -79,11 +82,13 @@ struct OzProb {
   double* w;                // s_tj [nw][Kall]; wp: of the pass's first row and frequency
   const double* wp;
   const double* x;          // QF: rows of the real operand [nrow][ncol]
-  int* flag;                // set: the FP64 kernel does this problem
+  int* flag;                // FLAG_*: what else does this problem
   // workspace
   float2* part;             // scale partials
   int* EA;                  // exponents [operand block][superblock][128]
   int* EB;
+  int* eq;                  // QF: exponents of the basis functions' scales
+  float2* cols;             // QF: largest magnitude and |diagonal| per column of the scaled U [f][128 nbj]
   char* A;                  // slices: [f (polarization)][block][stage][56 KB]
   char* B;                  // [f (QF)][block][stage][56 KB]
   double* G;                // polarization: [split][f][C, S][nbp][nbp], transposed tiles
@@ -118,9 +123,6 @@ enum : int { OZ_POL, OZ_QUAD, OZ_CPLX };
 template <int MODE> struct OzBatchOf { using B = OzBatch; using P = OzProb; };
 template <> struct OzBatchOf<OZ_CPLX> { using B = OzCBatch; using P = OzC; };
 
-// whether a mode sums group 6 by itself (exactly), and group 9 as well
-constexpr bool oz_exact6(int mode) { return mode == OZ_CPLX; }
-
 // One work item: its problem, operand slices (stage 0), stage range, stages per superblock, and the
 // indexes that its output needs.
 template <int MODE>
@@ -133,8 +135,8 @@ struct OzItem {
 
 // polarization: tiles of C = Mr^T D Mi (all) and S = (Mr+Mi)^T D (Mr+Mi) (upper), the layout of the
 // split-precision polarization; quadratic form: every (row block, column block), whose column block
-// bj needs K < 128 (bj + 1). False: the FP64 kernel does this problem.
-template <int MODE>
+// bj needs K < 128 (bj + 1). False: another kernel does this problem.
+template <int MODE, bool EXACT6>
 __device__ __forceinline__ bool oz_item(const OzBatch& batch, int64_t item, OzItem<MODE>& it) {
   int q = 0;
   while (q + 1 < batch.nq && item >= batch.item0[q + 1]) ++q;
@@ -175,10 +177,10 @@ __device__ __forceinline__ bool oz_item(const OzBatch& batch, int64_t item, OzIt
     it.a = L.A + size_t(it.f * 2 * nbb + it.bi) * L.nst * OBLK;
     it.b = L.B + size_t(it.bj) * L.nst * OBLK;
   }
-  return !__ldg(L.flag);
+  return __ldg(L.flag) == (EXACT6 ? FLAG_EXACT6 : 0);
 }
 // complex products: kind: the product, f: the tile's index, (bi, bj): the tile
-template <int MODE>
+template <int MODE, bool EXACT6>
 __device__ __forceinline__ bool oz_item(const OzCBatch& batch, int64_t item, OzItem<MODE>& it) {
   int lo = 0, hi = batch.nq - 1;        // the last problem that starts at or before the item
   while (lo < hi) {
@@ -251,10 +253,15 @@ __device__ __forceinline__ int4 ld_exp4(const int* p) {
   return r;
 }
 
-template <int MODE>
+// EXACT6: group 6 summed by itself (exactly), and group 9 as well
+template <int MODE, bool EXACT6>
 __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch, unsigned* status) {
   constexpr uint32_t IDESC = tc::instr_desc(1u, OT, OT);
-  constexpr bool EXACT6 = oz_exact6(MODE);
+  if constexpr (MODE != OZ_CPLX) {            // nothing of the batch is this kernel's: whole grid
+    bool any = false;
+    for (int q = 0; q < batch.nq; ++q) any = any || __ldg(batch.q[q].flag) == (EXACT6 ? FLAG_EXACT6 : 0);
+    if (!any) return;
+  }
   extern __shared__ __align__(1024) char dsmem[];
   char* ring = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(dsmem) + 1023) & ~uintptr_t(1023));
   // full/empty per stage part (0: slices 1-4, 1: slices 5-7); D and C: the accumulators
@@ -376,7 +383,7 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
     };
     for (int64_t item = blockIdx.x; item < nitems && !stop; item += gridDim.x) {
       OzItem<MODE> w;
-      if (!oz_item<MODE>(batch, item, w)) continue;
+      if (!oz_item<MODE, EXACT6>(batch, item, w)) continue;
       const auto& L = *w.L;
       const int f = w.f, sp = w.sp, bi = w.bi, bj = w.bj, kind = w.kind;
       double qsum = 0.0;
@@ -541,7 +548,7 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
       bool ok = true;
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
         OzItem<MODE> w;
-        if (!oz_item<MODE>(batch, item, w)) continue;
+        if (!oz_item<MODE, EXACT6>(batch, item, w)) continue;
         const char *a = w.a, *b = w.b;
         for (int st = w.st0; st < w.st1 && ok; ++st, ++g) {
           const int slot = g % ONST;
@@ -574,7 +581,7 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
       const uint64_t desc0 = tc::smem_desc(tc::uniform(tc::smem_u32(ring)), 512, 4);
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
         OzItem<MODE> w;
-        if (!oz_item<MODE>(batch, item, w)) continue;
+        if (!oz_item<MODE, EXACT6>(batch, item, w)) continue;
         for (int sb0 = w.st0; sb0 < w.st1 && ok; sb0 += w.sbst) {
           const int n = min(w.sbst, w.st1 - sb0);
           for (int k = 0; k < n; ++k, ++g) {
@@ -717,27 +724,31 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
 
 __global__ void __launch_bounds__(OTHREADS, 1)
     k_oz_gemm_pol(const __grid_constant__ OzBatch batch, unsigned* status) {
-  oz_gemm<OZ_POL>(batch, status);
+  oz_gemm<OZ_POL, false>(batch, status);
 }
 __global__ void __launch_bounds__(OTHREADS, 1)
     k_oz_gemm_quad(const __grid_constant__ OzBatch batch, unsigned* status) {
-  oz_gemm<OZ_QUAD>(batch, status);
+  oz_gemm<OZ_QUAD, false>(batch, status);
+}
+__global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm_quad6(const __grid_constant__ OzBatch batch, unsigned* status) {
+  oz_gemm<OZ_QUAD, true>(batch, status);
 }
 __global__ void __launch_bounds__(OTHREADS, 1)
     k_oz_gemm_cplx(const __grid_constant__ OzCBatch batch, unsigned* status) {
-  oz_gemm<OZ_CPLX>(batch, status);
+  oz_gemm<OZ_CPLX, true>(batch, status);
 }
 
 // ------------------------------------------------------------------ digits (fp64_slices.cuh)
 // the exponent of a range: E with (largest magnitude) < 0.996 2^E, or a raised flag
 __device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool ratio, int* flag) {
   if (!(sum <= 3.0e38f) || !(mx < 1.2676506e30f)) {        // not finite, or from 2^100 on
-    *flag = 1;
+    atomicOr(flag, FLAG_FP64);
     return 0;
   }
   if (mx == 0.0f) return 0;
   if (mx < 7.8886091e-31f || (ratio && mx * n > RATIO_MAX * sum)) {
-    *flag = 1;
+    atomicOr(flag, FLAG_FP64);
     return 0;
   }
   return ilogbf(mx * 1.005f) + 1;       // 1.005 mx < 2^E
@@ -765,12 +776,12 @@ __global__ void k_oz_weights(const __grid_constant__ OzBatch batch, double pref,
   }
 }
 
-// |v| rounded up to FP32 by integer arithmetic (the FP64 pipe's conversions cost three times the
+// |v| 2^e rounded up to FP32 by integer arithmetic (the FP64 pipe's conversions cost three times the
 // reads of the scale kernel): the exponent re-biased, the top 23 mantissa bits plus one. Zero and
 // magnitudes below 2^-126 become 2^-126, those above the FP32 range (and non-finite ones) infinite.
-__device__ __forceinline__ float abs_up(double v) {
+__device__ __forceinline__ float abs_up(double v, int e = 0) {
   const unsigned long long b = __double_as_longlong(v) & 0x7fffffffffffffffull;
-  const long long f = (long long)(b >> 29) - (896ll << 23) + 1;      // FP32 bits of the next value up
+  const long long f = (long long)(b >> 29) - ((896ll - e) << 23) + 1;  // FP32 bits of the next value up
   const int bits = f < 0x00800000ll ? 0x00800000 : f > 0x7f800000ll ? 0x7f800000 : int(f);
   return __int_as_float(b ? bits : 0);
 }
@@ -872,7 +883,7 @@ __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
 __global__ void __launch_bounds__(OT) k_oz_slice(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.z];
   const int nst = L.nst, nsb = L.nsb, sbst = L.sbst, nbb = L.nbj, nb = L.nb, nf = L.nf;
-  if (int(blockIdx.x) >= nst || int(blockIdx.y) >= 4 * nbb || __ldg(L.flag)) return;
+  if (int(blockIdx.x) >= nst || int(blockIdx.y) >= 4 * nbb || (__ldg(L.flag) & FLAG_FP64)) return;
   const double2* __restrict__ M = L.M;
   const double* __restrict__ w = L.wp;
   const int64_t K = L.K, wld = L.Kall;
@@ -920,7 +931,7 @@ __global__ void __launch_bounds__(OT) k_oz_slice(const __grid_constant__ OzBatch
 // P_ab = -S_ab + C_ab + C_ba + i (C_ab - C_ba), Hermitian exactly (S from its upper element)
 __global__ void k_oz_combine(const __grid_constant__ OzBatch batch, int accumulate) {
   const OzProb& L = batch.q[blockIdx.y];
-  if (__ldg(L.flag)) return;
+  if (__ldg(L.flag) & FLAG_FP64) return;
   double2* __restrict__ P = L.P;
   const double* __restrict__ G = L.G;
   const int nb = L.nb, nbp = L.nbj * OT, nf = L.nf, splits = L.splits;
@@ -963,6 +974,42 @@ __device__ __forceinline__ double u_entry(const double2* __restrict__ W, int nb,
   return u + (a == b ? t.x : b == 0 ? -t.y : t.y);
 }
 
+// The basis is scaled by powers of two first: x'_I = x_I 2^e_I, W'_IJ = W_IJ 2^-(e_I + e_J) with
+// 2^(2 e_I) near the largest |W_II| of the problem's frequencies. It changes no term and rounds
+// nothing (the digits are cut with the shifted exponents), and a (semi)definite W, which W^c is, has
+// |W'_IJ| <= 4 then, whatever units the basis functions have. Without it, scales of 10^+-2 at random left
+// 1e-13 of the sum of the terms' magnitudes, 10^+-8 1e-6.
+// 32 basis functions per CTA, eight threads each (the diagonals lie pages apart: latency).
+constexpr int EQF = 8;
+__global__ void __launch_bounds__(32 * EQF) k_oz_equilibrate(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  if (int(blockIdx.x) * 32 >= L.nb) return;   // whole CTA, before any barrier
+  __shared__ double sm[EQF][32];
+  const int lane = threadIdx.x & 31, f0 = threadIdx.x >> 5, I = blockIdx.x * 32 + lane;
+  double d[GW_MAX_NW / EQF], m = 0.0;
+#pragma unroll
+  for (int k = 0; k < GW_MAX_NW / EQF; ++k) {
+    const int f = f0 + EQF * k;
+    d[k] = f < L.nf && I < L.nb ? __ldg(L.M + (size_t(f) * L.nb + I) * L.nb + I).x : 0.0;
+    m = fmax(m, fabs(d[k]));
+  }
+  sm[f0][lane] = m;
+  __syncthreads();
+  if (I >= L.nb) return;
+#pragma unroll
+  for (int k = 0; k < EQF; ++k) m = fmax(m, sm[k][lane]);
+  const int ex = (__double2hiint(m) >> 20) & 0x7ff;
+  const int e = ex == 0 || ex == 0x7ff ? 0 : max(-64, min(64, (ex - 1023) >> 1));
+  if (f0 == 0) L.eq[I] = e;
+#pragma unroll
+  for (int k = 0; k < GW_MAX_NW / EQF; ++k) {
+    const int f = f0 + EQF * k;
+    if (f >= L.nf) break;
+    float2* c = L.cols + size_t(f) * L.nbj * OT + 2 * I;
+    c[0].y = c[1].y = abs_up(d[k], -2 * e);
+  }
+}
+
 // exponents of the rows of x, one warp per row and superblock (rows beyond nrow: zeros)
 __global__ void __launch_bounds__(256) k_oz_rowexps(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.y];
@@ -975,7 +1022,7 @@ __global__ void __launch_bounds__(256) k_oz_rowexps(const __grid_constant__ OzBa
     if (row < L.nrow) {
       const int64_t c0 = int64_t(sb) * L.sbst * OKS, c1 = min(L.ncol, c0 + int64_t(L.sbst) * OKS);
       for (int64_t c = c0 + lane; c < c1; c += 32) {
-        const float v = abs_up(__ldg(L.x + row * L.ncol + c));
+        const float v = abs_up(__ldg(L.x + row * L.ncol + c), __ldg(L.eq + (c >> 1)));
         mx = fmaxf(mx, v);
         sum += v;
       }
@@ -993,7 +1040,7 @@ __global__ void __launch_bounds__(256) k_oz_rowexps(const __grid_constant__ OzBa
 // digit slices of x: grid (stages, row blocks x 4, problems), four lanes per row
 __global__ void __launch_bounds__(OT) k_oz_slice_rows(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.z];
-  if (int(blockIdx.x) >= L.nst || int(blockIdx.y) >= 4 * L.nbi || __ldg(L.flag)) return;
+  if (int(blockIdx.x) >= L.nst || int(blockIdx.y) >= 4 * L.nbi || (__ldg(L.flag) & FLAG_FP64)) return;
   const int bi = blockIdx.y >> 2, st = blockIdx.x, kc = threadIdx.x & 3;
   const int n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
   const int64_t row = int64_t(bi) * OT + n, c0 = int64_t(st) * OKS + kc * 8;
@@ -1007,7 +1054,11 @@ __global__ void __launch_bounds__(OT) k_oz_slice_rows(const __grid_constant__ Oz
     v[k + 1] = x.y;
   }
   uint32_t dg[OSL][4];
-  digits8(v, L.EA[(size_t(bi) * L.nsb + st / L.sbst) * OT + n], dg);
+  const int E = L.EA[(size_t(bi) * L.nsb + st / L.sbst) * OT + n];
+  int Ek[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) Ek[k] = E - (c0 + k < L.ncol ? __ldg(L.eq + ((c0 + k) >> 1)) : 0);
+  digits8(v, Ek, dg);
   store_digits(L.A + (size_t(bi) * L.nst + st) * OBLK, n, kc, dg);
 }
 
@@ -1023,10 +1074,12 @@ __global__ void __launch_bounds__(OT * UROWS) k_oz_uscale(const __grid_constant_
   const double2* W = L.M + size_t(f) * L.nb * L.nb;
   const int n = threadIdx.x % OT, g = threadIdx.x / OT, c = cb * OT + n;
   const int k0 = ch * OT + g * (OT / UROWS);
+  const int ec = c < 2 * L.nb ? __ldg(L.eq + (c >> 1)) : 0;
   float mx = 0.f, sum = 0.f;
 #pragma unroll 8
   for (int k = 0; k < OT / UROWS; ++k) {
-    const float v = abs_up(u_entry(W, L.nb, k0 + k, c));
+    const int ek = k0 + k < 2 * L.nb ? __ldg(L.eq + ((k0 + k) >> 1)) : 0;
+    const float v = abs_up(u_entry(W, L.nb, k0 + k, c), -(ek + ec));
     mx = fmaxf(mx, v);
     sum += v;
   }
@@ -1042,6 +1095,8 @@ __global__ void __launch_bounds__(OT * UROWS) k_oz_uscale(const __grid_constant_
   L.part[(size_t(f) * L.nbj + ch) * (size_t(L.nbj) * OT) + c] = make_float2(mx, sum);
 }
 
+// exponents of the scaled U's columns, plus that of the column's own scale (what the GEMM's epilogue
+// multiplies with x, unscaled), and the columns' largest magnitudes
 __global__ void k_oz_uexps(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.y];
   const int ncolp = L.nbj * OT, cps = L.sbst * OKS / OT;
@@ -1056,31 +1111,119 @@ __global__ void k_oz_uexps(const __grid_constant__ OzBatch batch) {
       mx = fmaxf(mx, p.x);
       sum += p.y;
     }
-    L.EB[(size_t(f * L.nbj + cb) * L.nsb + sb) * OT + c % OT] = range_exponent(mx, sum, 1.0f, false, L.flag);
+    L.EB[(size_t(f * L.nbj + cb) * L.nsb + sb) * OT + c % OT] =
+        range_exponent(mx, sum, 1.0f, false, L.flag) + (c < 2 * L.nb ? __ldg(L.eq + (c >> 1)) : 0);
+    if (sb > 0) continue;
+    for (int ch = cps; ch <= cb; ++ch)
+      mx = fmaxf(mx, L.part[(size_t(f) * L.nbj + ch) * ncolp + c].x);
+    L.cols[size_t(f) * ncolp + c].x = mx;
   }
+}
+
+// Whether the digits hold the pairs' coefficients. The error of a coefficient from digits is a
+// multiple of 2^-53 max_k |x'_k| (sum_c (x'_c max_k |U'_kc|)^2)^1/2 (independent errors of the columns'
+// sums), that of FP64 sums a multiple of 2^-53 of the sum of the terms' magnitudes, of which the diagonal
+// sum_c |U'_cc| x'_c^2 is a part. R is the largest quotient of the two over pairs and frequencies: at
+// most 1.0 for the W^c of the repository's workloads (N_b = 27 to 600), more where the diagonal of W falls
+// off differently with the frequency for different basis functions, or where W is not definite.
+// Measured errors relative to the sum of the terms' magnitudes, N_b = 16 to 600, rms (the FP64 kernel's:
+// 3e-16 to 9e-16):
+//   R       0.7 to 1         1.4 to 2          4 to 6            32 to 64          64 to 90
+//   digits  3e-16 to 1.4e-15 3.4e-16 to 1.2e-15 7e-16 to 3.4e-15 5e-15 to 2e-14    8e-15 to 3e-14
+//   exact6  3e-16 to 1e-15   2e-16 to 6e-16    3e-16 to 7e-16    4e-16 to 8e-16    6e-16 to 1.1e-15
+// so above 2 a q takes the GEMM with an exact group 6 (6,656 pairs, N_b = 600, 16 frequencies: 5.5 ->
+// 6.8 ms), above 64 the FP64 kernel (262 ms).
+// 16 pairs per CTA, a pair in two lanes, which take different frequencies; 64 columns at a time.
+constexpr float PAIR_EXACT6 = 2.0f, PAIR_FP64 = 64.0f;
+constexpr int GP = 16, GC = 64, GT = 256, GF = GW_MAX_NW * GP / GT;
+static_assert(GF * GT == GW_MAX_NW * GP, "a thread's frequencies");
+__global__ void __launch_bounds__(GT) k_oz_pair_guard(const __grid_constant__ OzBatch batch) {
+  const OzProb& L = batch.q[blockIdx.y];
+  const int64_t p0 = int64_t(blockIdx.x) * GP;
+  if (p0 >= L.nrow) return;                   // whole CTA, before any barrier
+  __shared__ float sx[GC][GP + 1];
+  __shared__ float2 su[GW_MAX_NW][GC];
+  __shared__ int se[GP];
+  const int tid = threadIdx.x, pr = tid & (GP - 1), f0 = tid / GP, ncolp = L.nbj * OT;
+  if (tid < GP) {                             // x' against the row's exponent: no overflow in FP32
+    const int64_t p = p0 + tid;
+    int e = -1000;
+    for (int sb = 0; sb < L.nsb && p < L.nrow; ++sb)
+      e = max(e, L.EA[(size_t(p / OT) * L.nsb + sb) * OT + p % OT]);
+    se[tid] = e;
+  }
+  float top = 0.f, lhs[GF] = {}, rhs[GF] = {};
+  for (int c0 = 0; c0 < int(L.ncol); c0 += GC) {
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < GP * GC / GT; ++j) {
+      const int i = tid + j * GT, c = i % GC, r = i / GC;
+      sx[c][r] = p0 + r < L.nrow && c0 + c < L.ncol
+                     ? abs_up(__ldg(L.x + (p0 + r) * L.ncol + c0 + c), __ldg(L.eq + ((c0 + c) >> 1)) - se[r])
+                     : 0.f;
+    }
+    for (int i = tid; i < L.nf * GC; i += GT) {
+      const int c = i % GC, f = i / GC;
+      float2 u = c0 + c < L.ncol ? L.cols[size_t(f) * ncolp + c0 + c] : make_float2(0.f, 0.f);
+      if (u.x > 0.f) u.x = fmaxf(u.x, 8.7e-19f);                // (the squares stay above the FP32 range)
+      su[f][c] = u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < GF; ++i) {
+      const int f = f0 + GT / GP * i;
+      if (f >= L.nf) break;
+      float a = 0.f, b = 0.f;
+#pragma unroll 16
+      for (int c = 0; c < GC; ++c) {
+        const float x = sx[c][pr];
+        const float2 u = su[f][c];
+        const float t = x * u.x;
+        top = fmaxf(top, x);
+        a = fmaf(t, t, a);
+        b = fmaf(x * x, u.y, b);
+      }
+      lhs[i] += a;
+      rhs[i] += b;
+    }
+  }
+  int bits = 0;
+#pragma unroll
+  for (int i = 0; i < GF; ++i) {
+    const float err = top * sqrtf(lhs[i]);
+    if (!(err <= PAIR_FP64 * rhs[i]) || (err == 0.f && rhs[i] > 0.f)) bits |= FLAG_FP64;
+    else if (err > PAIR_EXACT6 * rhs[i]) bits |= FLAG_EXACT6;
+  }
+  bits = __reduce_or_sync(0xffffffffu, bits);
+  if ((tid & 31) == 0 && bits) atomicOr(L.flag, bits);
 }
 
 // digit slices of U: grid (stages, column blocks x 4, problems x frequencies)
 __global__ void __launch_bounds__(OT) k_oz_slice_u(const __grid_constant__ OzBatch batch, int nfmax) {
   const OzProb& L = batch.q[blockIdx.z / nfmax];
   const int f = blockIdx.z % nfmax, cb = blockIdx.y >> 2, st = blockIdx.x;
-  if (f >= L.nf || cb >= L.nbj || st >= L.nst || st * OKS > cb * OT + OT - 1 || __ldg(L.flag)) return;
+  if (f >= L.nf || cb >= L.nbj || st >= L.nst || st * OKS > cb * OT + OT - 1 || (__ldg(L.flag) & FLAG_FP64)) return;
   const double2* W = L.M + size_t(f) * L.nb * L.nb;
   const int kc = threadIdx.x & 3, n = int(blockIdx.y & 3) * 32 + (threadIdx.x >> 2);
   const int c = cb * OT + n, k0 = st * OKS + kc * 8;
-  double v[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = u_entry(W, L.nb, k0 + k, c);
-  uint32_t dg[OSL][4];
   const size_t blk = size_t(f) * L.nbj + cb;
-  digits8(v, L.EB[(blk * L.nsb + st / L.sbst) * OT + n], dg);
+  const int E = L.EB[(blk * L.nsb + st / L.sbst) * OT + n];
+  double v[8];
+  int Ek[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    v[k] = u_entry(W, L.nb, k0 + k, c);
+    Ek[k] = E + (k0 + k < 2 * L.nb ? __ldg(L.eq + ((k0 + k) >> 1)) : 0);
+  }
+  uint32_t dg[OSL][4];
+  digits8(v, Ek, dg);
   store_digits(L.B + (blk * L.nst + st) * OBLK, n, kc, dg);
 }
 
 // c[f][p] from the column blocks' parts in order; ldc: pairs of the whole q
 __global__ void k_oz_pair_reduce(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.y];
-  if (__ldg(L.flag)) return;
+  if (__ldg(L.flag) & FLAG_FP64) return;
   const int64_t total = L.nrow * L.nf;
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
        e += int64_t(gridDim.x) * blockDim.x) {
@@ -1356,8 +1499,8 @@ struct PairPlan {
   int q, f0, nf;
   int64_t p0, np;
   int nst, nsb, nbi, nbj;
-  size_t digits, b_part, b_ea, b_eb, b_A, b_B, b_c;
-  size_t total() const { return b_part + b_ea + b_eb + b_A + b_B + b_c; }
+  size_t digits, b_part, b_ea, b_eb, b_eq, b_cols, b_A, b_B, b_c;
+  size_t total() const { return b_part + b_ea + b_eb + b_eq + b_cols + b_A + b_B + b_c; }
 };
 
 std::vector<std::vector<PairPlan>> pair_batches(int nq, const int64_t* npair, const int* nb, int nw) {
@@ -1388,6 +1531,8 @@ std::vector<std::vector<PairPlan>> pair_batches(int nq, const int64_t* npair, co
         p.b_part = ws_round(size_t(p.nf) * nbj * nbj * OT * sizeof(float2));
         p.b_ea = ws_round(size_t(p.nbi) * p.nsb * OT * 4);
         p.b_eb = ws_round(size_t(p.nf) * nbj * p.nsb * OT * 4);
+        p.b_eq = ws_round(size_t(nb[q]) * sizeof(int));
+        p.b_cols = ws_round(size_t(p.nf) * nbj * OT * sizeof(float2));
         p.b_c = ws_round(size_t(p.nf) * 2 * nbj * size_t(p.np) * 8);
         if (out.empty() || int(out.back().size()) == OZQ || bytes + p.digits > DIGIT_BUDGET) {
           out.push_back({});
@@ -1426,7 +1571,7 @@ int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig
     OzBatch b{};
     b.nq = int(v.size());
     b.s = ssum;
-    int64_t nst = 0, nbi = 0, nbj = 0, nf = 0, nsb = 0, nred = 0;
+    int64_t nst = 0, nbi = 0, nbj = 0, nf = 0, nsb = 0, nred = 0, nrow = 0, nbmax = 0;
     for (int i = 0; i < b.nq; ++i) {
       const PairPlan& p = v[i];
       OzProb& L = b.q[i];
@@ -1434,10 +1579,12 @@ int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig
       L.part = static_cast<float2*>(cur.take(p.b_part));
       L.EA = static_cast<int*>(cur.take(p.b_ea));
       L.EB = static_cast<int*>(cur.take(p.b_eb));
+      L.eq = static_cast<int*>(cur.take(p.b_eq));
+      L.cols = static_cast<float2*>(cur.take(p.b_cols));
       L.A = static_cast<char*>(cur.take(p.b_A));
       L.B = static_cast<char*>(cur.take(p.b_B));
       L.cpart = static_cast<double*>(cur.take(p.b_c));
-      if (!L.part || !L.EA || !L.EB || !L.A || !L.B || !L.cpart)
+      if (!L.part || !L.EA || !L.EB || !L.eq || !L.cols || !L.A || !L.B || !L.cpart)
         return set_error(GW_EWORKSPACE, "internal: FP64 pair workspace too small");
       L.nb = nb[p.q];
       L.ncol = 2 * int64_t(nb[p.q]);
@@ -1462,20 +1609,27 @@ int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig
       nf = std::max<int64_t>(nf, p.nf);
       nsb = std::max<int64_t>(nsb, p.nsb);
       nred = std::max<int64_t>(nred, p.np * p.nf);
+      nrow = std::max<int64_t>(nrow, p.np);
+      nbmax = std::max<int64_t>(nbmax, L.nb);
     }
     const unsigned nq_ = unsigned(b.nq), nz = unsigned(b.nq * nf);
     const int64_t cap = int64_t(ctx.sm_count) * 16;
+    k_oz_equilibrate<<<dim3(unsigned((nbmax + 31) / 32), nq_), 32 * EQF, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_equilibrate");
     k_oz_rowexps<<<dim3(unsigned(std::min<int64_t>((nbi * OT * nsb + 7) / 8, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_rowexps");
     k_oz_uscale<<<dim3(unsigned(nbj), unsigned(nbj), nz), OT * UROWS, 0, s>>>(b, int(nf));
     GW_LAUNCH_CHECK("k_oz_uscale");
     k_oz_uexps<<<dim3(unsigned(std::min<int64_t>((nf * nbj * OT * nsb + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_uexps");
+    k_oz_pair_guard<<<dim3(unsigned((nrow + GP - 1) / GP), nq_), GT, 0, s>>>(b);
+    GW_LAUNCH_CHECK("k_oz_pair_guard");
     k_oz_slice_rows<<<dim3(unsigned(nst), unsigned(4 * nbi), nq_), OT, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_slice_rows");
     k_oz_slice_u<<<dim3(unsigned(nst), unsigned(4 * nbj), nz), OT, 0, s>>>(b, int(nf));
     GW_LAUNCH_CHECK("k_oz_slice_u");
     int rc = launch_oz<OzBatch>(k_oz_gemm_quad, b, s, ctx);
+    if (!rc) rc = launch_oz<OzBatch>(k_oz_gemm_quad6, b, s, ctx);    // empty unless a flag asks for it
     if (rc) return rc;
     k_oz_pair_reduce<<<dim3(unsigned(std::min<int64_t>((nred + 255) / 256, cap)), nq_), 256, 0, s>>>(b);
     GW_LAUNCH_CHECK("k_oz_pair_reduce");

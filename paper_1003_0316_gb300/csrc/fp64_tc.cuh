@@ -19,7 +19,7 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
            PolOpts& o);
 
 // Pair coefficients c_p (FP64) of every q. The workspace's first 4 nq bytes then hold one int per q
-// that is non-zero when that q needs the FP64 kernel (its c is to be overwritten).
+// that is odd when that q needs the FP64 kernel (its c is to be overwritten).
 size_t oz_pair_workspace(int nq, const int64_t* npair, const int* nb, int nw, int sm);
 int oz_pair(int nq, const int64_t* npair, const int* nb, const void* const* Msig, int nw,
             const double* const* Wc, double* const* c, void* ws, size_t ws_bytes, cudaStream_t s,

@@ -41,14 +41,14 @@ struct PairLaunch {
   int nw;
 };
 
-// only_if: one device word per q of the launch; a q's work is empty when its word is zero (the sliced
-// tensor-core path has its result)
+// only_if: one device word per q of the launch; a q's work is empty when its lowest bit is zero (the
+// sliced tensor-core path has its result)
 __global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __restrict__ part,
                                                        const int* __restrict__ only_if) {
   int64_t blk = blockIdx.x;
   int q = 0;
   while (q + 1 < L.nq && blk >= L.blk0[q + 1]) ++q;
-  if (!only_if[q]) return;
+  if (!(only_if[q] & 1)) return;
   int64_t loc = blk - L.blk0[q];
   const int it = int(loc % L.itiles[q]);
   loc /= L.itiles[q];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __r
 __global__ void k_paircoef_reduce(PairLaunch L, const double* __restrict__ part,
                                   const int* __restrict__ only_if) {
   const int q = blockIdx.y;
-  if (!only_if[q]) return;
+  if (!(only_if[q] & 1)) return;
   const int64_t np = L.npair[q];
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < np * L.nw;
        e += int64_t(gridDim.x) * blockDim.x) {

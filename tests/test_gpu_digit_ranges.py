@@ -1,0 +1,81 @@
+"""FP64 results of operands whose entries differ by many orders of magnitude, against sums of FP64
+terms: where the digit slices of the tensor-core path would lose what FP64 keeps, the call has to
+notice it.
+
+Bound of the pair coefficients: 1e-14 of the sum of the magnitudes of the terms (the bound of the
+digit slices for well-scaled operands; a change of scales s of the basis, x_I -> s_I x_I and W_IJ ->
+W_IJ / (s_I s_J), by powers of two changes neither the terms nor their sum).
+"""
+import pytest
+
+import synth_inputs as S
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gw():
+    import paper_1003_0316_gb300 as g
+    return g
+
+
+def randn(g, *shape):
+    return torch.view_as_complex(torch.randn((*shape, 2), generator=g, dtype=torch.float64, device="cuda"))
+
+
+def pairs(npair, nb, nw, seed, kind):
+    """Projections and W: negative definite, Hermitian without a diagonal, or general."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    M = randn(g, npair, nb)
+    if kind == "definite":
+        X = randn(g, nw, nb, 2 * nb)
+        W = -(X @ X.mH)
+        W = 0.5 * (W + W.mH)
+    else:
+        W = randn(g, nw, nb, nb)
+        if kind == "hollow":
+            W = W + W.mH
+            W.diagonal(dim1=1, dim2=2).zero_()
+    return M, W, g
+
+
+def check_pairs(gw, M, W):
+    c = gw.sigma_pair_coeffs([M], [W])[0]
+    gw.check()
+    r = torch.stack([((M @ w.T) * M.conj()).sum(1).real for w in W])
+    a = torch.stack([((M.abs() @ w.abs().T) * M.abs()).sum(1) for w in W])
+    assert float(((c - r).abs() / a).max()) <= 1e-14
+
+
+@pytest.mark.parametrize("kind", ["definite", "hollow", "general"])
+@pytest.mark.parametrize("npair,nb,nw,decades", [(130, 48, 4, 2), (64, 48, 4, 8), (200, 129, 4, 4),
+                                                 (90, 300, 4, 12), (300, 70, 9, 14)])
+def test_pair_coefficients_of_scaled_basis(gw, npair, nb, nw, decades, kind):
+    M, W, g = pairs(npair, nb, nw, nb + decades, kind)
+    s = 2.0 ** torch.round(3.3219 * decades * (2.0 * torch.rand(nb, generator=g, dtype=torch.float64,
+                                                               device="cuda") - 1.0))
+    check_pairs(gw, M * s, W / (s[:, None] * s[None, :]))
+
+
+@pytest.mark.parametrize("kind", ["definite", "hollow"])
+def test_pair_coefficients_of_frequencies_of_different_shape(gw, kind):
+    """The diagonal of W falls off with the frequency by a different power for every basis function."""
+    M, W, g = pairs(150, 60, 6, 11, kind)
+    p = 3.0 * torch.rand(60, generator=g, dtype=torch.float64, device="cuda")
+    for j in range(6):
+        d = (1.0 + 4.0 * j) ** -p
+        W[j] = d[:, None] * W[j] * d[None, :]
+    check_pairs(gw, M, W)
+
+
+@pytest.mark.parametrize("big", [1e3, 1e6, 1e12])
+def test_pair_coefficients_of_rows_and_columns_with_one_large_entry(gw, big):
+    """A row of M and a column of W whose largest entries meet small ones."""
+    M, W, _ = pairs(140, 66, 4, 21, "general")
+    M[::3, 5] *= big
+    W[:, 5, :] *= 1e-3 / big
+    W[:, :, 5] *= 1e-3 / big
+    W[1, 7, 9] *= big
+    W[2, 11, 11] *= big
+    check_pairs(gw, M, W)
