@@ -788,9 +788,13 @@ __device__ __forceinline__ float abs_up(double v, int e = 0) {
 
 // Bounds (within 2^-21) of the largest magnitude and of the magnitude sum of every column over
 // chunks of 64 rows, in FP32: operand types 0 Mi, 1 Mr + Mi (B), 2 + 2 f and 3 + 2 f: s_f Mr,
-// s_f (Mr + Mi) (A). Thread = column; grid (column blocks, chunks). Bound by the read of M.
+// s_f (Mr + Mi) (A). Thread = column; grid (column blocks, chunks). Bound by the read of M. The products
+// with the weights are rounded up, so that none becomes zero: a column whose largest product is below
+// 2^-100 takes the FP64 kernel, and so do weights that abs_up raises to 2^-126 where an entry of M
+// could lift them above that (and weights from 2^26 on, which lift raised entries of M).
 __global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch batch) {
   __shared__ float sw[4][CHROWS];
+  __shared__ int odd;
   const OzProb& L = batch.q[blockIdx.z];
   const double2* __restrict__ M = L.M;
   const double* __restrict__ w = L.wp;
@@ -805,9 +809,14 @@ __global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch
   for (int f0 = 0; f0 < nf; f0 += 4) {
     const int nj = min(4, nf - f0);
     __syncthreads();
+    if (threadIdx.x == 0) odd = 0;
+    __syncthreads();
     for (int e = threadIdx.x; e < 4 * CHROWS; e += OT) {
       const int j = e / CHROWS, t = e % CHROWS;
-      sw[j][t] = j < nj && t < n ? abs_up(w[size_t(f0 + j) * wld + t0 + t]) : 0.0f;
+      const double v = j < nj && t < n ? w[size_t(f0 + j) * wld + t0 + t] : 0.0;
+      sw[j][t] = abs_up(v);
+      if (v != 0.0 && fabs(v) < 1.1754944e-38) atomicOr(&odd, 1);
+      if (fabs(v) >= 6.7108864e7) atomicOr(&odd, 2);
     }
     __syncthreads();
     float mi = 0.f, ms = 0.f, si = 0.f, ss = 0.f, ma[4][2] = {}, sa[4][2] = {};
@@ -825,7 +834,7 @@ __global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch
         ss += s;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float pr = r * sw[j][t], ps = s * sw[j][t];
+          const float pr = __fmul_ru(r, sw[j][t]), ps = __fmul_ru(s, sw[j][t]);
           ma[j][0] = fmaxf(ma[j][0], pr);
           sa[j][0] += pr;
           ma[j][1] = fmaxf(ma[j][1], ps);
@@ -833,6 +842,7 @@ __global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch
         }
       }
     }
+    if ((odd & 2) || (odd && (mi >= 3.3e7f || ms >= 3.3e7f))) atomicOr(L.flag, FLAG_FP64);
     if (f0 == 0) {
       out[0] = make_float2(mi, si);
       out[ncolp] = make_float2(ms, ss);

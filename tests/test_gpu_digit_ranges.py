@@ -79,3 +79,21 @@ def test_pair_coefficients_of_rows_and_columns_with_one_large_entry(gw, big):
     W[1, 7, 9] *= big
     W[2, 11, 11] *= big
     check_pairs(gw, M, W)
+
+
+@pytest.mark.parametrize("m,f", [(1e-20, 1e-40), (1e-25, 1.0), (1e-12, 1e-60), (1e20, 1e-60)])
+def test_polarization_of_small_weights(gw, m, f):
+    """Products of M and the weights below the FP32 range: the sum over 200 transitions against the
+    sum of magnitudes (FP64 sums, 2^-53 per term)."""
+    g = torch.Generator(device="cuda").manual_seed(4)
+    K, nb, om = 200, 40, S.omega_mesh(4)[:2]
+    M = randn(g, K, nb) * m
+    d = 0.05 + 2.0 * torch.rand(K, generator=g, dtype=torch.float64, device="cuda")
+    ft = torch.full((K,), f, dtype=torch.float64, device="cuda")
+    P = gw.polarization([M], [d], om, 0.25, "fp64", fs=[ft])[0]
+    gw.check()
+    for j, w in enumerate(om):
+        s = -0.5 * f * d / (d * d + float(w) ** 2)
+        r = (M * s[:, None]).T @ M.conj()
+        a = ((M.abs() * s.abs()[:, None]).T @ M.abs())
+        assert float(((P[j] - r).abs() / a).max()) <= 3e-14
