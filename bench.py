@@ -279,7 +279,7 @@ class Pipeline:
         import torch
         nq, nw = self.wl.nq, self.wl.nw
         if self.prec == "fp64":
-            p = 4 * len(self.herk_events[-1])       # scales, exponents, slices, GEMM per pass
+            p = 5 * len(self.herk_events[-1])       # scales, exponents, slices, GEMM 2 per pass
         else:
             # weights + prep per q; one HERK launch per group of q (a group closes at 4 work
             # items per SM; items = 128-tiles x frequencies); the combination of the

@@ -83,6 +83,7 @@ struct OzProb {
   const double* wp;
   const double* x;          // QF: rows of the real operand [nrow][ncol]
   int* flag;                // FLAG_*: what else does this problem
+  int* spread;              // polarization: largest spreads of the columns of A and of B (FP32 bits)
   // workspace
   float2* part;             // scale partials
   int* EA;                  // exponents [operand block][superblock][128]
@@ -727,6 +728,10 @@ __global__ void __launch_bounds__(OTHREADS, 1)
   oz_gemm<OZ_POL, false>(batch, status);
 }
 __global__ void __launch_bounds__(OTHREADS, 1)
+    k_oz_gemm_pol6(const __grid_constant__ OzBatch batch, unsigned* status) {
+  oz_gemm<OZ_POL, true>(batch, status);
+}
+__global__ void __launch_bounds__(OTHREADS, 1)
     k_oz_gemm_quad(const __grid_constant__ OzBatch batch, unsigned* status) {
   oz_gemm<OZ_QUAD, false>(batch, status);
 }
@@ -741,7 +746,8 @@ __global__ void __launch_bounds__(OTHREADS, 1)
 
 // ------------------------------------------------------------------ digits (fp64_slices.cuh)
 // the exponent of a range: E with (largest magnitude) < 0.996 2^E, or a raised flag
-__device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool ratio, int* flag) {
+__device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool ratio, int* flag,
+                                              float* spread = nullptr) {
   if (!(sum <= 3.0e38f) || !(mx < 1.2676506e30f)) {        // not finite, or from 2^100 on
     atomicOr(flag, FLAG_FP64);
     return 0;
@@ -751,6 +757,7 @@ __device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool
     atomicOr(flag, FLAG_FP64);
     return 0;
   }
+  if (spread) *spread = mx * n / sum;
   return ilogbf(mx * 1.005f) + 1;       // 1.005 mx < 2^E
 }
 
@@ -759,7 +766,7 @@ __device__ __forceinline__ int range_exponent(float mx, float sum, float n, bool
 __global__ void k_oz_weights(const __grid_constant__ OzBatch batch, double pref, int nw, OmegaArr om,
                              unsigned* status) {
   const OzProb& L = batch.q[blockIdx.y];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *L.flag = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *L.flag = L.spread[0] = L.spread[1] = 0;
   for (int64_t t = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; t < L.Kall;
        t += int64_t(gridDim.x) * blockDim.x) {
     const double d = L.delta[t];
@@ -854,7 +861,16 @@ __global__ void __launch_bounds__(OT) k_oz_scale(const __grid_constant__ OzBatch
   }
 }
 
-// exponents of every (type, column, superblock) from the chunk partials
+// Exponents of every (type, column, superblock) from the chunk partials, and the largest spreads: for a
+// column of n rows with magnitudes of maximum m and mean a, m / (a n^1/4). The error of an element from
+// digits is a multiple of 2^-53 n^1/2 m_A m_B, that of FP64 sums one of 2^-53 n (A^2 B^2 in the mean)^1/2,
+// so the quotient of the two is at most the product of the spreads of A and B. Measured against sums
+// in twice FP64's precision, rms relative to sqrt(P_II P_JJ) (FP64 kernel): Gaussian M and gaps from
+// 0.05 Ha on, product 4 to 19: 1.0e-16 (1.1e-16) for K = 512, 2.7e-17 (2.6e-17) for 8,192; gaps of 0.003
+// Ha, 100: 4.3e-16 (2.8e-16); entries of 30 to 300 times the others, 300 on: 5e-16 to 9e-16 (1e-16 to
+// 2.4e-16). Above SPREAD_EXACT6 the GEMM with an exact group 6 takes over: 2.5e-17 to 7e-17 in all of
+// these (5.85 -> 7.5 ms for K = 102,400, N_b = 600, 2 frequencies).
+constexpr float SPREAD_EXACT6 = 32.0f;
 __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.y];
   const float2* __restrict__ part = L.part;
@@ -877,7 +893,12 @@ __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
     }
     const int64_t r0 = int64_t(sb) * sbst * OKS;
     const float rows = float(min(int64_t(sbst) * OKS, K - r0));
-    const int E = range_exponent(mx, sum, rows, true, L.flag);
+    float sp = 0.f;
+    const int E = range_exponent(mx, sum, rows, true, L.flag, &sp);
+    sp *= rsqrtf(sqrtf(rows));
+    const unsigned act = __activemask(), kind = __match_any_sync(act, int(type < 2));
+    const int top = __reduce_max_sync(kind, __float_as_int(sp));
+    if ((threadIdx.x & 31) == __ffs(kind) - 1) atomicMax(L.spread + (type < 2), top);
     const int cb = col / OT, n = col % OT;
     if (type < 2)
       EB[(size_t(type * nbb + cb) * nsb + sb) * OT + n] = E;
@@ -893,7 +914,10 @@ __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
 __global__ void __launch_bounds__(OT) k_oz_slice(const __grid_constant__ OzBatch batch) {
   const OzProb& L = batch.q[blockIdx.z];
   const int nst = L.nst, nsb = L.nsb, sbst = L.sbst, nbb = L.nbj, nb = L.nb, nf = L.nf;
-  if (int(blockIdx.x) >= nst || int(blockIdx.y) >= 4 * nbb || (__ldg(L.flag) & FLAG_FP64)) return;
+  if (int(blockIdx.x) >= nst || int(blockIdx.y) >= 4 * nbb || (__ldcg(L.flag) & FLAG_FP64)) return;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 &&
+      __int_as_float(L.spread[0]) * __int_as_float(L.spread[1]) > SPREAD_EXACT6)
+    atomicOr(L.flag, FLAG_EXACT6);            // read by the GEMMs
   const double2* __restrict__ M = L.M;
   const double* __restrict__ w = L.wp;
   const int64_t K = L.K, wld = L.Kall;
@@ -1404,6 +1428,7 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
   const std::vector<OzPlan> plans = oz_plans(idx, K.data(), nb.data(), nw, ctx.sm_count);
   WsCursor cur{static_cast<char*>(ws), ws_bytes, 0};
   int* flags = static_cast<int*>(cur.take(256));
+  static_assert(3 * OZQ * sizeof(int) <= 256, "flags and spreads");
   OzBatch b{};
   b.nq = n;
   b.s = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));
@@ -1414,6 +1439,7 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
     const PolQ& Q = qs[group[i]];
     OzProb& L = b.q[i];
     L.flag = flags + i;
+    L.spread = flags + OZQ + 2 * i;
     L.w = static_cast<double*>(cur.take(p.b_w));
     L.part = static_cast<float2*>(cur.take(p.b_part));
     exps[i] = static_cast<char*>(cur.take(size_t(p.npass) * p.nchunk * (p.b_ea + p.b_eb)));
@@ -1488,6 +1514,7 @@ int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, c
       int rc = record_herk_event(o, o.launches, false, s);
       if (rc) return rc;
       if ((rc = launch_oz<OzBatch>(k_oz_gemm_pol, b, s, ctx))) return rc;
+      if ((rc = launch_oz<OzBatch>(k_oz_gemm_pol6, b, s, ctx))) return rc;   // empty unless flagged
       if ((rc = record_herk_event(o, o.launches, true, s))) return rc;
       ++o.launches;
     }

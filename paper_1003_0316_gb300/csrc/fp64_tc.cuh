@@ -13,7 +13,7 @@ std::vector<std::vector<int>> oz_pol_groups(const std::vector<int>& qs, const in
                                             int nw);
 size_t oz_pol_workspace(const std::vector<int>& group, const int64_t* K, const int* nb, int nw, int sm);
 // P of one group. The workspace's first 256 bytes then hold one int per q of the group that is
-// non-zero when that q's input needs the FP64 kernel (its P is untouched).
+// odd when that q's input needs the FP64 kernel (its P is untouched).
 int oz_pol(const std::vector<int>& group, const PolQ* qs, double pref, int nw, const OmegaArr& om,
            bool accumulate, void* ws, size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx,
            PolOpts& o);

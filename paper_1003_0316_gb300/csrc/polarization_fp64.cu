@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k_herk_fp64(PolLaunch L, double pref, Ome
   int64_t item = blockIdx.x;
   int q = 0;
   while (q + 1 < L.nq && item >= L.item0[q + 1]) ++q;
-  if (only_if && !only_if[q]) return;         // whole CTA: the sliced path has this q's result
+  if (only_if && !(only_if[q] & 1)) return;   // whole CTA: the sliced path has this q's result
   int64_t local = item - L.item0[q];
   const int S = L.splits[q];
   const int T = L.tside[q];
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(256) k_herk_reduce(PolLaunch L, const double2*
     if (blk < acc_blocks + nblk) break;
     acc_blocks += nblk;
   }
-  if (only_if && !only_if[q]) return;
+  if (only_if && !(only_if[q] & 1)) return;
   int64_t rest = blk - acc_blocks;
   const int S = L.splits[q];
   const int nw = L.nw;
@@ -333,7 +333,7 @@ size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const
 }
 
 // the FP64 kernel over the given q points; only_if: one device word per q point (MAXQ at most), whose
-// work is empty when it is zero (these launches are not counted as HERK launches)
+// work is empty when it is even (these launches are not counted as HERK launches)
 static int pol_fp64_plain(const std::vector<PolQ>& qs, double pref, int nw, const OmegaArr& om,
                           void* ws, size_t ws_bytes, const int* only_if, cudaStream_t s,
                           const DeviceCtx& ctx, PolOpts& o) {

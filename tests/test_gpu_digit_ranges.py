@@ -97,3 +97,43 @@ def test_polarization_of_small_weights(gw, m, f):
         r = (M * s[:, None]).T @ M.conj()
         a = ((M.abs() * s.abs()[:, None]).T @ M.abs())
         assert float(((P[j] - r).abs() / a).max()) <= 3e-14
+
+
+@pytest.mark.parametrize("K", [300, 700, 5000])
+@pytest.mark.parametrize("kind,f", [("spike", 20.0), ("spike", 200.0), ("spike", 600.0), ("gap", 1e-2),
+                                    ("gap", 1e-3), ("half", 1e-6)])
+def test_polarization_of_uneven_columns(gw, K, kind, f):
+    """A few large entries per column, in the same rows for pairs of columns; small gaps; columns that are
+    large in one half of the rows. Root mean square error relative to sqrt(P_II P_JJ): the FP64 kernel's
+    sums of K terms, about 2^-53 (1.1e-16) per partial sum, give at most 3e-16 for any of these; digits
+    with a share of that from every term would give more."""
+    g = torch.Generator(device="cuda").manual_seed(K)
+    nb = 70
+    M = randn(g, K, nb)
+    d = 0.05 + 2.0 * torch.rand(K, generator=g, dtype=torch.float64, device="cuda")
+    col = torch.arange(nb, device="cuda")
+    if kind == "spike":
+        rows = torch.randint(K, (nb // 2 + 1,), generator=g, device="cuda")[col // 2]
+        M[rows, col] *= f
+    elif kind == "gap":
+        d = d - 0.05 + f
+        d[3], d[K // 2] = f, 1.1 * f
+    else:
+        M[: K // 2, ::2] *= f
+        M[K // 2:, 1::2] *= f
+    P = gw.polarization([M], [d], [0.0, 1.0], 0.25, "fp64")[0]
+    gw.check()
+    for j, w in enumerate((0.0, 1.0)):
+        s = -0.5 * d / (d * d + w * w)
+        hi = torch.zeros((nb, nb, 2), dtype=torch.float64, device="cuda")
+        lo = hi.clone()
+        for t in range(0, K, 32):                    # FP64 sums of 32 terms, added without rounding
+            m = M[t:t + 32]
+            x = torch.view_as_real(((m * s[t:t + 32, None]).T @ m.conj()).contiguous())
+            a = hi + x
+            b = a - hi
+            lo += (hi - (a - b)) + (x - b)
+            hi = a
+        R = torch.view_as_complex(hi + lo)
+        dg = R.diagonal().real.abs().sqrt()
+        assert float(((P[j] - R).abs() / (dg[:, None] * dg)).square().mean().sqrt()) <= 3e-16
