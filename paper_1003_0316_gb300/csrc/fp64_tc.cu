@@ -545,13 +545,13 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
     tc::setmaxnreg_dec<REG_P>();
     if (warp == EPI_WARPS && lane == 0) {
       // ---------------------------------------------- bulk copies of the slices
-      uint32_t g = 0;
+      uint32_t g = 0, half = 0;               // stages copied; 1: and slices 5-7 of the next one
       bool ok = true;
       for (int64_t item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
         OzItem<MODE> w;
         if (!oz_item<MODE, EXACT6>(batch, item, w)) continue;
         const char *a = w.a, *b = w.b;
-        for (int st = w.st0; st < w.st1 && ok; ++st, ++g) {
+        for (int st = w.st0; st < w.st1; ++st, ++g) {
           const int slot = g % ONST;
           const uint32_t par = ((g / ONST) & 1) ^ 1;
           char* dst = ring + slot * OSTAGE;
@@ -559,6 +559,7 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
           for (int h = 1; h >= 0; --h) {              // slices 5-7 are free first
             if (!tc::mbar_wait(&empty[slot][h], par, &s_abort, OWAIT)) {
               ok = false;
+              half = h ? 0 : 1;
               break;
             }
             const int nb = h ? LOB : HIB;
@@ -568,12 +569,22 @@ __device__ __forceinline__ void oz_gemm(const typename OzBatchOf<MODE>::B& batch
             tc::bulk_g2s(to, a + off, nb, &full[slot][h]);
             tc::bulk_g2s(to + nb, b + off, nb, &full[slot][h]);
           }
+          if (!ok) break;
         }
       }
       if (!ok && !s_abort) {
         s_abort = 1;
         raise_status(status, ST_ETIMEOUT);
       }
+      // However the loop ended (its consumers may have given up): no copy into this CTA's shared
+      // memory outlives the CTA. The last phase of every barrier that was armed.
+      int never = 0;
+      for (int h = 0; h < 2; ++h)
+        for (uint32_t i = 0; i < ONST; ++i) {
+          const uint32_t armed = (g + ONST - 1 - i) / ONST + (h && half && g % ONST == i ? 1 : 0);
+          if (armed)
+            tc::mbar_wait(&full[i][h], (armed - 1) & 1, reinterpret_cast<volatile int*>(&never), OWAIT);
+        }
     } else if (warp == EPI_WARPS + 1) {
       // ---------------------------------------------- MMA issue (tc::elect_one)
       const uint32_t tm = tc::uniform(tmem);
