@@ -477,6 +477,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           s_abort = 1;
           raise_status(status, ST_ETIMEOUT);
         }
+        // however the loop ended (the consumers may have given up): no copy into this CTA's shared
+        // memory outlives the CTA; g copies were issued, in turn to the NSB barriers
+        int never = 0;
+        for (uint64_t i = 0; i < NSB; ++i) {
+          const uint64_t armed = (g + NSB - 1 - i) / NSB;
+          if (armed)
+            tc::mbar_wait(&fullB[i], uint32_t(armed - 1) & 1, reinterpret_cast<volatile int*>(&never),
+                          WAIT_LIMIT);
+        }
         if (kWaitProfile) {
           hp_flush(HP_BP_TOTAL, hp_now() - hp0);
           hp_flush(HP_BP_WAIT, hp_w);
@@ -529,6 +538,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         if (!ok && !s_abort) {
           s_abort = 1;
           raise_status(status, ST_ETIMEOUT);
+        }
+        int never = 0;                        // as for the B tiles
+        for (uint64_t i = 0; i < NWS; ++i) {
+          const uint64_t armed = (g + NWS - 1 - i) / NWS;
+          if (armed)
+            tc::mbar_wait(&fullW[i], uint32_t(armed - 1) & 1, reinterpret_cast<volatile int*>(&never),
+                          WAIT_LIMIT);
         }
         if (kWaitProfile) {
           hp_flush(HP_WP_TOTAL, hp_now() - hp0);
