@@ -41,6 +41,16 @@ struct LmWarpSmem {
   int flag;
 };
 
+// a b + c d and a b - c d with their roundings written out: both kernels use them, since a compiler may
+// contract either product, and their results are equal bit for bit. (A single product added to a
+// value can be contracted in one way only.)
+__device__ __forceinline__ double lm_sum(double a, double b, double c, double d) {
+  return fma(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ double lm_dif(double a, double b, double c, double d) {
+  return fma(a, b, -__dmul_rn(c, d));
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -63,13 +73,13 @@ __device__ __forceinline__ double warp_cost(const double* om, const double2* yl,
     double fx = 0.0, fy = 0.0;
     for (int p = 0; p < npole; ++p) {
       const double dx = -t[4 * p + 2], dy = om[j] - t[4 * p + 3];
-      const double inv = 1.0 / (dx * dx + dy * dy);
+      const double inv = 1.0 / lm_sum(dy, dy, dx, dx);
       const double px = dx * inv, py = -dy * inv;          // phi = 1 / (i w_j - w_p)
-      fx += t[4 * p] * px - t[4 * p + 1] * py;
-      fy += t[4 * p] * py + t[4 * p + 1] * px;
+      fx += lm_dif(t[4 * p], px, t[4 * p + 1], py);
+      fy += lm_sum(t[4 * p], py, t[4 * p + 1], px);
     }
     const double rx = fx - yl[h].x, ry = fy - yl[h].y;
-    c += rx * rx + ry * ry;
+    c += lm_sum(rx, rx, ry, ry);
   }
   return 0.5 * warp_sum(c);
 }
@@ -109,8 +119,8 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
   __syncwarp();
   double th[P], thn[P];
   for (int k = 0; k < P; ++k) th[k] = S.th[k];
-  const double cscale = 0.5 * warp_sum(yl[0].x * yl[0].x + yl[0].y * yl[0].y +
-                                       yl[1].x * yl[1].x + yl[1].y * yl[1].y);
+  const double cscale = 0.5 * warp_sum(fma(yl[1].y, yl[1].y,
+                                           fma(yl[1].x, yl[1].x, lm_sum(yl[0].x, yl[0].x, yl[0].y, yl[0].y))));
   double C = warp_cost(om.v, yl, nw, npole, th);
   // the packed entries e = lane + 32 h of A this lane sums: row ea[h], column eb[h]
   constexpr int EPL = (NP + 31) / 32;
@@ -138,12 +148,12 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
       for (int p = 0; p < npole; ++p) {
         const double ax = th[4 * p], ay = th[4 * p + 1];
         const double dx = -th[4 * p + 2], dy = om.v[j] - th[4 * p + 3];
-        const double inv = 1.0 / (dx * dx + dy * dy);
+        const double inv = 1.0 / lm_sum(dy, dy, dx, dx);
         const double px = dx * inv, py = -dy * inv;        // phi
-        const double tx = ax * px - ay * py, ty = ax * py + ay * px;   // a phi
+        const double tx = lm_dif(ax, px, ay, py), ty = lm_sum(ax, py, ay, px);   // a phi
         fx += tx;
         fy += ty;
-        const double qx = tx * px - ty * py, qy = tx * py + ty * px;   // a phi^2
+        const double qx = lm_dif(tx, px, ty, py), qy = lm_sum(tx, py, ty, px);   // a phi^2
         // d f / d Re a = phi, d f / d Im a = i phi, d f / d Re w = a phi^2, d f / d Im w = i a phi^2
         S.rowR[j][4 * p] = px;
         S.rowI[j][4 * p] = py;
@@ -165,12 +175,12 @@ __global__ void __launch_bounds__(32) k_lm_warp(int ncurve, int nw, OmegaArr om,
       if (e >= NP) break;
       const int a = ea[h], bcol = eb[h];
       double v = 0.0;
-      for (int j = 0; j < nw; ++j) v += S.rowR[j][a] * S.rowR[j][bcol] + S.rowI[j][a] * S.rowI[j][bcol];
+      for (int j = 0; j < nw; ++j) v += lm_sum(S.rowR[j][a], S.rowR[j][bcol], S.rowI[j][a], S.rowI[j][bcol]);
       S.A[e] = v;
     }
     if (lane < P) {
       double v = 0.0;
-      for (int j = 0; j < nw; ++j) v += S.rowR[j][lane] * S.res[j][0] + S.rowI[j][lane] * S.res[j][1];
+      for (int j = 0; j < nw; ++j) v += lm_sum(S.rowR[j][lane], S.res[j][0], S.rowI[j][lane], S.res[j][1]);
       S.g[lane] = v;
     }
     __syncwarp();
@@ -309,13 +319,6 @@ __host__ __device__ constexpr int lm_group_doubles(int nw, int P) {
   return d + (LMG - d % 16 + 16) % 16;
 }
 
-// a b + c d and a b - c d, rounded as the compiler contracts them in k_lm_warp
-__device__ __forceinline__ double lm_sum(double a, double b, double c, double d) {
-  return fma(a, b, __dmul_rn(c, d));
-}
-__device__ __forceinline__ double lm_dif(double a, double b, double c, double d) {
-  return fma(a, b, -__dmul_rn(c, d));
-}
 // x with its sign flipped where bit 31 of m is set
 __device__ __forceinline__ double lm_flip(double x, int m) {
   return __hiloint2double(__double2hiint(x) ^ m, __double2loint(x));
