@@ -262,7 +262,9 @@ int gw_plan_waves(int nq, const int64_t* K_host, const int* nb_host, int nw, int
  * factor, so Wc_dev (and P_dev where it aliases Wc_dev) is undefined after such an error.
  * Workspace: gw_screened_w_workspace() bytes: per (q, frequency) system
  * 16 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of the systems from
- * N_b = 257 on (at most 6 GB, or one system's where that is more; further systems take turns). */
+ * N_b = 257 on (at most 6 GB, or one system's where that is more; further systems take turns). A
+ * smaller workspace, down to the first part alone, is accepted: systems whose slices find no room
+ * are solved in float-float throughout. */
 size_t gw_screened_w_workspace(int nq, const int* nb_host, int nw);
 int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev,
                   const double* const* P_dev, double* const* Wc_dev,
@@ -273,7 +275,8 @@ int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev
  * Cholesky factor and the inverse are real (a quarter of the FP64 work), the imaginary parts of
  * P_dev are not read (taken as zero), W^c is written with zero imaginary parts. Same layouts
  * and errors as gw_screened_w. Workspace: gw_screened_w_real_workspace() bytes: per system
- * 8 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of large systems. */
+ * 8 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of large systems (or
+ * less, as above). */
 size_t gw_screened_w_real_workspace(int nq, const int* nb_host, int nw);
 int gw_screened_w_real(int nq, const int* nb_host, int nw, const double* const* v_dev,
                        const double* const* P_dev, double* const* Wc_dev,

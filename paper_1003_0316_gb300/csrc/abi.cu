@@ -342,7 +342,7 @@ int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev
     if (nb_host[q] < 1 || nb_host[q] > 8192) return set_error(GW_EINVAL, "nb[%d]=%d", q, nb_host[q]);
     if (!v_dev[q] || !P_dev[q] || !Wc_dev[q]) return set_error(GW_EINVAL, "NULL pointer for q=%d", q);
   }
-  size_t need = dielectric_workspace(nq, nb_host, nw);
+  size_t need = dielectric_workspace(nq, nb_host, nw, false);
   int rc = check_ws(ws_dev, ws_bytes, need);
   if (rc) return rc;
   DeviceCtx ctx;
@@ -368,7 +368,7 @@ int gw_screened_w_real(int nq, const int* nb_host, int nw, const double* const* 
     if (nb_host[q] < 1 || nb_host[q] > 8192) return set_error(GW_EINVAL, "nb[%d]=%d", q, nb_host[q]);
     if (!v_dev[q] || !P_dev[q] || !Wc_dev[q]) return set_error(GW_EINVAL, "NULL pointer for q=%d", q);
   }
-  int rc = check_ws(ws_dev, ws_bytes, dielectric_real_workspace(nq, nb_host, nw));
+  int rc = check_ws(ws_dev, ws_bytes, dielectric_real_workspace(nq, nb_host, nw, false));
   if (rc) return rc;
   DeviceCtx ctx;
   if ((rc = device_ctx(&ctx))) return rc;

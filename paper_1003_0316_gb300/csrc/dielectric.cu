@@ -1385,24 +1385,29 @@ static int launch_dielectric(std::vector<DieSysT<T>>& sys, WsCursor dz, float* s
   }
   constexpr bool CPLX = sizeof(T) == sizeof(double2);
   const bool by_columns = !sys.empty() && sys[0].D != nullptr;
+  // a caller's workspace without room for the slices (of all, or of large systems): float-float
+  const size_t room = ssum ? dz.size - std::min(dz.size, (dz.used + 255) & ~size_t(255)) : 0;
+  auto sliced_path = [&](const DieSysT<T>& S) {
+    return dz_takes(S.n, CPLX) && DzPlan(S.n, CPLX).total() <= room;
+  };
   // The systems of the sliced path behind the others, whatever the order of the sizes in the call: a
   // batch is of one kind, and sizes that alternate around the limit would make a batch (a chain of
   // three launches per 32 columns) per q: 8 q of 250 and 260 in turn, 16 frequencies, 10.4 -> 4.6 ms.
   if (by_columns)
     std::stable_partition(sys.begin(), sys.end(),
-                          [](const DieSysT<T>& S) { return !dz_takes(S.n, CPLX); });
+                          [&](const DieSysT<T>& S) { return !sliced_path(S); });
   for (size_t b0 = 0; b0 < sys.size();) {
     // up to DMAXSYS systems; those of the sliced path apart from the others, within the slice budget
-    const bool sliced = by_columns && dz_takes(sys[b0].n, CPLX);
+    const bool sliced = by_columns && sliced_path(sys[b0]);
     size_t nb_ = 0, bytes = 0;
     DieBatchT<T> batch;
     int ntmax = 1;
     while (b0 + nb_ < sys.size() && nb_ < DMAXSYS) {
       const DieSysT<T>& S = sys[b0 + nb_];
-      if (by_columns && dz_takes(S.n, CPLX) != sliced) break;
+      if (by_columns && sliced_path(S) != sliced) break;
       if (sliced) {
         const size_t need = DzPlan(S.n, CPLX).total();
-        if (nb_ > 0 && bytes + need > DZ_BUDGET) break;
+        if (nb_ > 0 && bytes + need > std::min(DZ_BUDGET, room)) break;
         bytes += need;
       }
       batch.s[nb_++] = S;
@@ -1438,16 +1443,16 @@ static int launch_dielectric(std::vector<DieSysT<T>>& sys, WsCursor dz, float* s
   return GW_OK;
 }
 
-// E, Z, D of every system
+// E, Z, D of every system (what a call needs), and the slices of large ones
 template <typename T>
-static size_t dielectric_ws_t(int nq, const int* nb, int nw) {
+static size_t dielectric_ws_t(int nq, const int* nb, int nw, bool slices) {
   size_t b = 0;
   std::vector<int> large;
   for (int q = 0; q < nq; ++q) {
     size_t n = size_t(nb[q]);
     const size_t nt = (n + DB - 1) / DB;
     b += size_t(nw) * ws_round((2 * n * n + nt * DB * DB) * sizeof(T));
-    if (dz_takes(nb[q], sizeof(T) == sizeof(double2))) large.insert(large.end(), nw, nb[q]);
+    if (slices && dz_takes(nb[q], sizeof(T) == sizeof(double2))) large.insert(large.end(), nw, nb[q]);
   }
   if (large.empty()) return b;
   int sm = 152, dev = 0;
@@ -1483,18 +1488,15 @@ static int dielectric_t(int nq, const int* nb, int nw, const double* const* v,
   float* ssum = nullptr;
   bool large = false;
   for (int q = 0; q < nq; ++q) large = large || dz_takes(nb[q], sizeof(T) == sizeof(double2));
-  if (large) {
-    ssum = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));
-    if (!ssum) return set_error(GW_EWORKSPACE, "internal: dielectric workspace too small");
-  }
+  if (large) ssum = static_cast<float*>(cur.take(oz_sum_bytes(ctx.sm_count)));    // NULL: no room for slices
   return launch_dielectric<T>(sys, cur, ssum, s, ctx);
 }
 
-size_t dielectric_workspace(int nq, const int* nb, int nw) {
-  return dielectric_ws_t<double2>(nq, nb, nw);
+size_t dielectric_workspace(int nq, const int* nb, int nw, bool slices) {
+  return dielectric_ws_t<double2>(nq, nb, nw, slices);
 }
-size_t dielectric_real_workspace(int nq, const int* nb, int nw) {
-  return dielectric_ws_t<double>(nq, nb, nw);
+size_t dielectric_real_workspace(int nq, const int* nb, int nw, bool slices) {
+  return dielectric_ws_t<double>(nq, nb, nw, slices);
 }
 
 int dielectric_wc(int nq, const int* nb, int nw, const double* const* v, const double* const* P,

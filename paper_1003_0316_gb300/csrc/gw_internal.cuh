@@ -132,12 +132,13 @@ int sigma_extrapolar(int nq, const double* wq, const int* nb, int nsig, const do
                      size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx);
 
 // a3
-size_t dielectric_workspace(int nq, const int* nb, int nw);
+// (without the slices: the least that a call takes)
+size_t dielectric_workspace(int nq, const int* nb, int nw, bool slices = true);
 int dielectric_wc(int nq, const int* nb, int nw, const double* const* v, const double* const* P,
                   double* const* Wc, void* ws, size_t ws_bytes, cudaStream_t s,
                   const DeviceCtx& ctx);
 // real symmetric systems (inversion symmetry): real factor and inverse, W^c imaginary parts 0
-size_t dielectric_real_workspace(int nq, const int* nb, int nw);
+size_t dielectric_real_workspace(int nq, const int* nb, int nw, bool slices = true);
 int dielectric_wc_real(int nq, const int* nb, int nw, const double* const* v,
                        const double* const* P, double* const* Wc, void* ws, size_t ws_bytes,
                        cudaStream_t s, const DeviceCtx& ctx);

@@ -1,0 +1,52 @@
+"""Workspaces without room for the digit slices: a call takes what its FP64 (or float-float) arithmetic
+needs by itself and gives the same results within the bounds of the two (1e-12 of the Frobenius norm);
+one byte less is an error."""
+import pytest
+
+import synth_inputs as S
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gw():
+    import paper_1003_0316_gb300 as g
+    return g
+
+
+def buf(n):
+    return torch.empty(int(n), dtype=torch.uint8, device="cuda")
+
+
+def randn(g, *shape):
+    return torch.view_as_complex(torch.randn((*shape, 2), generator=g, dtype=torch.float64, device="cuda"))
+
+
+def err(a, b):
+    return float((a - b).norm() / b.norm())
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_screened_w(gw, real):
+    """The size in gw.h: 16 (8 for real systems) x (2 N^2 + 1024 ceil(N / 32)) per system."""
+    ns, nw = [300, 40, 520, 600], 2
+    g = torch.Generator(device="cuda").manual_seed(2)
+    Ps, vs = [], []
+    for n in ns:
+        X = randn(g, nw, n, 2 * n) / (1.0 + torch.arange(n, device="cuda", dtype=torch.float64)[:, None] / 16.0)
+        if real:
+            X = X.real.to(torch.complex128)
+        P = -(X @ X.mH) / n
+        Ps.append(0.5 * (P + P.mH))
+        vs.append(torch.as_tensor(S.coulomb_eigenvalues(n), device="cuda"))
+    ref = gw.screened_w(Ps, vs, real=real)
+    gw.check()
+    least = sum(nw * -(-(8 if real else 16) * (2 * n * n + 1024 * -(-n // 32)) // 256) * 256 for n in ns)
+    for more in (0, 3 << 20, 30 << 20, 60 << 20, 150 << 20, 400 << 20):
+        W = gw.screened_w(Ps, vs, ws=buf(least + more), real=real)
+        gw.check()
+        assert max(err(a, b) for a, b in zip(W, ref)) <= 1e-12
+    with pytest.raises(gw.GWError) as e:
+        gw.screened_w(Ps, vs, ws=buf(least - 1), real=real)
+    assert e.value.code == gw.GW_EWORKSPACE
