@@ -121,7 +121,11 @@ int gw_transition_weights(int64_t K, const double* delta_dev, const double* f_de
  *   omega_host    [nw] double, 1 <= nw <= GW_MAX_NW,
  *   P_dev[q]      [nw][N_b][N_b] complex128 output, both triangles written.
  * precision: GW_FP64 needs GW_C128; GW_TF32X3 and GW_BF16X3 need GW_C64.
- * Workspace: gw_polarization_workspace() bytes. */
+ * Workspace: gw_polarization_workspace() bytes. For GW_FP64 that is mostly the digit slices: up to
+ * 6 GB (further q points, rows and frequencies take turns), and the weights and the partial sums of
+ * P. A smaller GW_FP64 workspace is accepted down to the partial sums of the FP64 pipe (64 KB per 64 x 64
+ * tile of P, frequency and split of K; a fraction of P's size for large N_b): the call then runs on
+ * that pipe, which takes about 40 times as long for large K. */
 size_t gw_polarization_workspace(int nq, const int64_t* K_host, const int* nb_host,
                                  int nw, int precision);
 int gw_polarization(int nq, const int64_t* K_host, const int* nb_host,
@@ -240,8 +244,9 @@ int gw_polarization_extrapolar(int nq, const int64_t* K_host, const int* nb_host
  * larger than device memory). Assigns each q to a wave so that, per wave, the projections
  * (complex128 for GW_FP64, complex64 otherwise), the gw_polarization workspace of the wave and
  * the P outputs fit in budget_bytes; first-fit decreasing by footprint. Host only.
- *   wave_of_q [nq] output (0-based), *nwaves_out the number of waves. GW_EINVAL if one q
- *   alone exceeds the budget. */
+ *   wave_of_q [nq] output (0-based), *nwaves_out the number of waves. A q that fits alone only
+ *   with the smallest workspace that gw_polarization accepts is a wave of its own. GW_EINVAL if
+ *   one q alone exceeds the budget even so. */
 int gw_plan_waves(int nq, const int64_t* K_host, const int* nb_host, int nw, int precision,
                   size_t budget_bytes, int* wave_of_q, int* nwaves_out);
 

@@ -257,7 +257,12 @@ static int polarization_impl(int nq, const int64_t* K_host, const int* nb_host,
     if (precision != GW_FP64 && (reinterpret_cast<uintptr_t>(qs[q].M) & 15u))
       return set_error(GW_EINVAL, "M_dev[%d] not 16-byte aligned", q);
   }
-  size_t need = polarization_workspace_impl(nq, K_host, nb_host, nw, precision, po);
+  const size_t full = polarization_workspace_impl(nq, K_host, nb_host, nw, precision, po);
+  size_t need = full;
+  if (precision == GW_FP64 && ws_bytes < full) {
+    po.fp64_slices = false;
+    need = pol_fp64_least_workspace(nq, K_host, nb_host, nw, po);
+  }
   if ((rc = check_ws(ws_dev, ws_bytes, need))) return rc;
   DeviceCtx ctx;
   if ((rc = device_ctx(&ctx))) return rc;

@@ -97,12 +97,15 @@ struct PolOpts {
   void* const* input_events = nullptr;   // per q: cudaEvent_t to wait for before reading its inputs
   void* const* events = nullptr;   // cudaEvent_t pairs around the HERK launches
   int n_events = 0;
+  bool fp64_slices = true;         // the workspace has room for FP64's digit slices
   int launches = 0;                // out: HERK launches of the call
 };
 int resolve_pol_options(const gw_pol_options* o, PolOpts* out);
 // records the pair's start (end = false) or end event of HERK launch `idx`, if one was given
 int record_herk_event(PolOpts& o, int idx, bool end, cudaStream_t s);
 size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o);
+// the least that a call takes (its q points then run on the FP64 pipe)
+size_t pol_fp64_least_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o);
 int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, void* ws,
              size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx, PolOpts& o);
 size_t pol_tc_workspace(int nq, const int64_t* K, const int* nb, int nw, int precision,

@@ -309,12 +309,20 @@ static void split_q(int nq, const int64_t* K, std::vector<int>& oz, std::vector<
   for (int q = 0; q < nq; ++q) (oz_pol_eligible(K[q]) ? oz : plain).push_back(q);
 }
 
-size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o) {
-  int sm = 152;
-  int dev = 0;
+static int sm_count_here() {
+  int sm = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess)
     cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
   cudaGetLastError();
+  return sm;
+}
+
+size_t pol_fp64_least_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o) {
+  return plain_fp64_workspace(nq, K, nb, nw, sm_count_here(), o.fp64_waves);
+}
+
+size_t pol_fp64_workspace(int nq, const int64_t* K, const int* nb, int nw, const PolOpts& o) {
+  const int sm = sm_count_here();
   std::vector<int> oz, plain;
   split_q(nq, K, oz, plain);
   auto plain_need = [&](const std::vector<int>& qs) {
@@ -398,6 +406,8 @@ int pol_fp64(int nq, const PolQ* qs, double pref, int nw, const OmegaArr& om, vo
     for (int q = 0; q < nq; ++q)
       if (o.input_events[q])
         GW_CUDA_TRY(cudaStreamWaitEvent(s, static_cast<cudaEvent_t>(o.input_events[q]), 0));
+  if (!o.fp64_slices)                  // no room for the digit slices: the FP64 kernel does all
+    return pol_fp64_plain(std::vector<PolQ>(qs, qs + nq), pref, nw, om, ws, ws_bytes, nullptr, s, ctx, o);
   std::vector<int64_t> K(nq);
   std::vector<int> nb(nq);
   for (int q = 0; q < nq; ++q) {

@@ -17,6 +17,11 @@ static size_t pol_ws(int nq, const int64_t* K, const int* nb, int nw, int precis
   return precision == GW_FP64 ? pol_fp64_workspace(nq, K, nb, nw, PolOpts{})
                               : pol_tc_workspace(nq, K, nb, nw, precision, PolOpts{});
 }
+// the least workspace of one q
+static size_t pol_ws_least(int64_t K, int nb, int nw, int precision) {
+  return precision == GW_FP64 ? pol_fp64_least_workspace(1, &K, &nb, nw, PolOpts{})
+                              : pol_ws(1, &K, &nb, nw, precision);
+}
 
 int plan_waves(int nq, const int64_t* K, const int* nb, int nw, int precision, size_t budget,
                int* wave_of_q, int* nwaves) {
@@ -42,9 +47,10 @@ int plan_waves(int nq, const int64_t* K, const int* nb, int nw, int precision, s
   std::vector<size_t> foot(nq);
   for (int q = 0; q < nq; ++q) {
     foot[q] = cost({q});
-    if (foot[q] > budget)
-      return set_error(GW_EINVAL, "q=%d alone needs %zu bytes, above the budget of %zu", q,
-                       foot[q], budget);
+    if (foot[q] <= budget) continue;
+    const size_t least = data[q] + pol_ws_least(K[q], nb[q], nw, precision);
+    if (least > budget)
+      return set_error(GW_EINVAL, "q=%d alone needs %zu bytes, above the budget of %zu", q, least, budget);
   }
   std::vector<int> order(nq);
   std::iota(order.begin(), order.end(), 0);

@@ -50,3 +50,26 @@ def test_screened_w(gw, real):
     with pytest.raises(gw.GWError) as e:
         gw.screened_w(Ps, vs, ws=buf(least - 1), real=real)
     assert e.value.code == gw.GW_EWORKSPACE
+
+
+def test_polarization(gw):
+    """64 KB per 64 x 64 tile of P, frequency and split of K hold the FP64 kernel's partial sums; at most
+    K / 512 splits."""
+    sizes, om = [(3000, 100), (20, 30), (1500, 64), (500, 200)], S.omega_mesh(4)[:2]
+    g = torch.Generator(device="cuda").manual_seed(3)
+    Ms = [randn(g, K, nb) for K, nb in sizes]
+    ds = [0.05 + 2.0 * torch.rand(K, generator=g, dtype=torch.float64, device="cuda") for K, _ in sizes]
+    ref = gw.polarization(Ms, ds, om, 0.25, "fp64")
+    gw.check()
+    least = 0
+    for K, nb in sizes:
+        t = -(-nb // 64)
+        least += t * (t + 1) // 2 * len(om) * max(1, K // 512) * 65536
+    full = gw.polarization_workspace([K for K, _ in sizes], [nb for _, nb in sizes], len(om), "fp64")
+    assert least < full
+    P = gw.polarization(Ms, ds, om, 0.25, "fp64", ws=buf(least))
+    gw.check()
+    assert max(err(a, b) for a, b in zip(P, ref)) <= 1e-12
+    with pytest.raises(gw.GWError) as e:
+        gw.polarization(Ms, ds, om, 0.25, "fp64", ws=buf(65536))
+    assert e.value.code == gw.GW_EWORKSPACE
