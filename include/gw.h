@@ -368,7 +368,12 @@ int gw_sigma_extrapolar(int nq, const double* wq_host, const int* nb_host, int n
                         double* sigma_dev, double* cbar_dev, void* ws_dev, size_t ws_bytes,
                         gw_stream_t stream);
 
-/* a5 + a6 in one call (the Sigma^c step of the hot path). */
+/* a5 + a6 in one call (the Sigma^c step of the hot path). Workspace: gw_sigma_workspace() bytes; for
+ * GW_FP64 mostly the digit slices of the projections and of W^c, up to 6 GB. A smaller GW_FP64
+ * workspace is accepted, here and in gw_sigma_pair_coeffs, down to the coefficients (here) and the
+ * larger of the FP64 pipe's partial sums (8 nw npair ceil(N_b / 64) bytes, summed over q) and
+ * gw_sigma_convolve_workspace(): the coefficients then come from that pipe, 40 times as slow for large
+ * N_b. */
 size_t gw_sigma_workspace(int nq, const int64_t* npair_host, const int* nb_host, int nw,
                           int precision);
 int gw_sigma_c(int nq, const double* wq_host, const int64_t* npair_host,

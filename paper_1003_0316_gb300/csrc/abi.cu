@@ -421,12 +421,16 @@ int gw_sigma_pair_coeffs(int nq, const int64_t* npair_host, const int* nb_host,
     if (precision != GW_FP64 && (reinterpret_cast<uintptr_t>(Msig_dev[q]) & 15u))
       return set_error(GW_EINVAL, "Msig_dev[%d] not 16-byte aligned", q);
   }
-  size_t need = paircoef_workspace(nq, npair_host, nb_host, nw, precision);
-  if ((rc = check_ws(ws_dev, ws_bytes, need))) return rc;
+  const bool full =
+      ws_dev != nullptr && ws_bytes >= paircoef_workspace(nq, npair_host, nb_host, nw, precision);
+  if (!full) {
+    const size_t need = paircoef_least_workspace(nq, npair_host, nb_host, nw, precision);
+    if ((rc = check_ws(ws_dev, ws_bytes, need))) return rc;
+  }
   DeviceCtx ctx;
   if ((rc = device_ctx(&ctx))) return rc;
   return paircoef(nq, npair_host, nb_host, Msig_dev, m_dtype, nw, Wc_dev, c_dev, precision,
-                  ws_dev, ws_bytes, stream, ctx);
+                  ws_dev, ws_bytes, full, stream, ctx);
 }
 
 size_t gw_sigma_convolve_workspace(int nq, const int64_t* npair_host) {
@@ -513,8 +517,8 @@ int gw_sigma_extrapolar(int nq, const double* wq_host, const int* nb_host, int n
                           ws_dev, ws_bytes, stream, ctx);
 }
 
-size_t gw_sigma_workspace(int nq, const int64_t* npair_host, const int* nb_host, int nw,
-                          int precision) {
+static size_t sigma_workspace(int nq, const int64_t* npair_host, const int* nb_host, int nw,
+                              int precision, bool least) {
   if (nq < 1 || !npair_host || !nb_host || nw < 1 || nw > GW_MAX_NW) return 0;
   size_t b = 0;
   for (int q = 0; q < nq; ++q) {
@@ -522,8 +526,14 @@ size_t gw_sigma_workspace(int nq, const int64_t* npair_host, const int* nb_host,
     b += ws_round(sizeof(double) * size_t(nw) * size_t(npair_host[q]));
   }
   // the pair-coefficient scratch and the convolution's share the space after the coefficients
-  return b + std::max(paircoef_workspace(nq, npair_host, nb_host, nw, precision),
+  return b + std::max(least ? paircoef_least_workspace(nq, npair_host, nb_host, nw, precision)
+                            : paircoef_workspace(nq, npair_host, nb_host, nw, precision),
                       convolve_workspace(nq, npair_host, nw, 0));
+}
+
+size_t gw_sigma_workspace(int nq, const int64_t* npair_host, const int* nb_host, int nw,
+                          int precision) {
+  return sigma_workspace(nq, npair_host, nb_host, nw, precision, false);
 }
 
 int gw_sigma_c(int nq, const double* wq_host, const int64_t* npair_host, const int* nb_host,
@@ -534,8 +544,8 @@ int gw_sigma_c(int nq, const double* wq_host, const int64_t* npair_host, const i
                gw_stream_t stream) {
   int rc = validate_pairs(nq, npair_host, nb_host, precision, m_dtype);
   if (rc) return rc;
-  size_t need = gw_sigma_workspace(nq, npair_host, nb_host, nw, precision);
-  if ((rc = check_ws(ws_dev, ws_bytes, need))) return rc;
+  if ((rc = check_ws(ws_dev, ws_bytes, sigma_workspace(nq, npair_host, nb_host, nw, precision, true))))
+    return rc;
   if (nw < 4 || nw > GW_MAX_NW) return set_error(GW_EINVAL, "nw=%d outside [4, %d]", nw, GW_MAX_NW);
   WsCursor cur{static_cast<char*>(ws_dev), ws_bytes, 0};
   std::vector<double*> cbuf(nq);

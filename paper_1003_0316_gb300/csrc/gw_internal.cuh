@@ -150,7 +150,9 @@ int dielectric_wc_real(int nq, const int* nb, int nw, const double* const* v,
 size_t paircoef_workspace(int nq, const int64_t* npair, const int* nb, int nw, int precision);
 int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msig, int dtype,
              int nw, const double* const* Wc, double* const* c, int precision, void* ws,
-             size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx);
+             size_t ws_bytes, bool slices, cudaStream_t s, const DeviceCtx& ctx);
+// (slices: the workspace has room for FP64's digit slices) the least that a call takes
+size_t paircoef_least_workspace(int nq, const int64_t* npair, const int* nb, int nw, int precision);
 
 // a6
 size_t convolve_workspace(int nq, const int64_t* npair, int nw, int nw_out);

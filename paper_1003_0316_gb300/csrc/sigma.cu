@@ -41,14 +41,14 @@ struct PairLaunch {
   int nw;
 };
 
-// only_if: one device word per q of the launch; a q's work is empty when its lowest bit is zero (the
-// sliced tensor-core path has its result)
+// only_if: NULL, or one device word per q of the launch; a q's work is empty when its lowest bit is zero
+// (the sliced tensor-core path has its result)
 __global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __restrict__ part,
                                                        const int* __restrict__ only_if) {
   int64_t blk = blockIdx.x;
   int q = 0;
   while (q + 1 < L.nq && blk >= L.blk0[q + 1]) ++q;
-  if (!(only_if[q] & 1)) return;
+  if (only_if && !(only_if[q] & 1)) return;
   int64_t loc = blk - L.blk0[q];
   const int it = int(loc % L.itiles[q]);
   loc /= L.itiles[q];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_paircoef_fp64(PairLaunch L, double* __r
 __global__ void k_paircoef_reduce(PairLaunch L, const double* __restrict__ part,
                                   const int* __restrict__ only_if) {
   const int q = blockIdx.y;
-  if (!(only_if[q] & 1)) return;
+  if (only_if && !(only_if[q] & 1)) return;
   const int64_t np = L.npair[q];
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < np * L.nw;
        e += int64_t(gridDim.x) * blockDim.x) {
@@ -139,6 +139,19 @@ __global__ void k_paircoef_reduce(PairLaunch L, const double* __restrict__ part,
   }
 }
 
+static size_t paircoef_partials(int nq, const int64_t* npair, const int* nb, int nw) {
+  size_t b = 0;
+  for (int q = 0; q < nq; ++q) {
+    int it = (nb[q] + ST - 1) / ST;
+    b += size_t(nw) * it * size_t(npair[q]);
+  }
+  return ws_round(b * sizeof(double));
+}
+// the least that a call takes: the FP64 kernel's partial sums
+size_t paircoef_least_workspace(int nq, const int64_t* npair, const int* nb, int nw, int precision) {
+  return precision == GW_FP64 ? paircoef_partials(nq, npair, nb, nw)
+                              : paircoef_workspace(nq, npair, nb, nw, precision);
+}
 // FP64: the sliced tensor-core path (fp64_tc.cu), and the FP64 kernel for the q points whose flag it
 // raised, with its partial sums behind the flags.
 size_t paircoef_workspace(int nq, const int64_t* npair, const int* nb, int nw, int precision) {
@@ -146,25 +159,24 @@ size_t paircoef_workspace(int nq, const int64_t* npair, const int* nb, int nw, i
   int sm = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
   cudaGetLastError();
-  size_t b = 0;
-  for (int q = 0; q < nq; ++q) {
-    int it = (nb[q] + ST - 1) / ST;
-    b += size_t(nw) * it * size_t(npair[q]);
-  }
-  return std::max(ws_round(size_t(nq) * sizeof(int)) + ws_round(b * sizeof(double)),
+  return std::max(ws_round(size_t(nq) * sizeof(int)) + paircoef_partials(nq, npair, nb, nw),
                   oz_pair_workspace(nq, npair, nb, nw, sm));
 }
 
 int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msig, int dtype,
              int nw, const double* const* Wc, double* const* c, int precision, void* ws,
-             size_t ws_bytes, cudaStream_t s, const DeviceCtx& ctx) {
+             size_t ws_bytes, bool slices, cudaStream_t s, const DeviceCtx& ctx) {
   if (precision != GW_FP64)
     return quad_tc(nq, npair, nb, Msig, nw, Wc, c, precision, dtype == GW_R32, ws, ws_bytes, s,
                    ctx);
-  int rc = oz_pair(nq, npair, nb, Msig, nw, Wc, c, ws, ws_bytes, s, ctx);
-  if (rc) return rc;
-  const int* flags = static_cast<const int*>(ws);
-  double* part = reinterpret_cast<double*>(static_cast<char*>(ws) + ws_round(size_t(nq) * sizeof(int)));
+  const int* flags = nullptr;          // no room for the digit slices: the FP64 kernel does all
+  double* part = static_cast<double*>(ws);
+  if (slices) {
+    int rc = oz_pair(nq, npair, nb, Msig, nw, Wc, c, ws, ws_bytes, s, ctx);
+    if (rc) return rc;
+    flags = static_cast<const int*>(ws);
+    part = reinterpret_cast<double*>(static_cast<char*>(ws) + ws_round(size_t(nq) * sizeof(int)));
+  }
   for (int q0 = 0; q0 < nq; q0 += SMAXQ) {
     int n = std::min(SMAXQ, nq - q0);
     PairLaunch L{};
@@ -188,9 +200,10 @@ int paircoef(int nq, const int64_t* npair, const int* nb, const void* const* Msi
     }
     L.blk0[n] = blk;
     if (blk == 0) continue;
-    k_paircoef_fp64<<<unsigned(blk), 256, 0, s>>>(L, part, flags + q0);
+    k_paircoef_fp64<<<unsigned(blk), 256, 0, s>>>(L, part, flags ? flags + q0 : nullptr);
     GW_LAUNCH_CHECK("k_paircoef_fp64");
-    k_paircoef_reduce<<<dim3(unsigned(ctx.sm_count), unsigned(n)), 256, 0, s>>>(L, part, flags + q0);
+    k_paircoef_reduce<<<dim3(unsigned(ctx.sm_count), unsigned(n)), 256, 0, s>>>(
+        L, part, flags ? flags + q0 : nullptr);
     GW_LAUNCH_CHECK("k_paircoef_reduce");
   }
   return GW_OK;

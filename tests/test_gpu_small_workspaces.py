@@ -73,3 +73,32 @@ def test_polarization(gw):
     with pytest.raises(gw.GWError) as e:
         gw.polarization(Ms, ds, om, 0.25, "fp64", ws=buf(65536))
     assert e.value.code == gw.GW_EWORKSPACE
+
+
+def test_sigma(gw):
+    """The FP64 kernel's partial sums: 8 nw npair ceil(N_b / 64) bytes, rounded up to 256."""
+    sizes, nw = [(500, 100), (130, 64), (0, 20), (77, 300)], 5
+    om = S.omega_mesh(nw)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    Ms = [randn(g, n, nb) for n, nb in sizes]
+    Ws = []
+    for _, nb in sizes:
+        X = randn(g, nw, nb, 2 * nb)
+        Ws.append(-(X @ X.mH))
+    es = [torch.rand(n, generator=g, dtype=torch.float64, device="cuda") + 0.1 for n, _ in sizes]
+    ps = [torch.arange(n, dtype=torch.int32, device="cuda") % 7 for n, _ in sizes]
+    args = ([0.25] * 4, Ms, ps, es, Ws, om, om, 7)
+    ref = gw.sigma_c(*args)
+    gw.check()
+    up = lambda b: -(-b // 256) * 256
+    c = sum(up(8 * nw * n) for n, _ in sizes)
+    part = up(sum(8 * nw * n * -(-nb // 64) for n, nb in sizes))
+    conv = gw._lib.gw_sigma_convolve_workspace(4, gw._arr(gw._i64, [n for n, _ in sizes]))
+    least = c + max(part, conv)
+    assert least < gw.sigma_workspace([n for n, _ in sizes], [nb for _, nb in sizes], nw, "fp64")
+    sig = gw.sigma_c(*args, ws=buf(least))
+    gw.check()
+    assert err(sig, ref) <= 1e-12
+    with pytest.raises(gw.GWError) as e:
+        gw.sigma_c(*args, ws=buf(least - 1))
+    assert e.value.code == gw.GW_EWORKSPACE
