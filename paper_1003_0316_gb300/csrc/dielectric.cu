@@ -135,19 +135,19 @@ __device__ __forceinline__ FF to_ff(double x) {
 }
 // to_ff by integer arithmetic (each FP64 conversion occupies the FP64 pipe like a multiply-add): h
 // from the magnitude rounded to 24 bits (to nearest, ties to even), l from the remaining bits, whose
-// integer difference is exact. Below 2^-73, where the power of two of l leaves the FP32 range, the
-// conversions (rare: entries of eps that small are mostly zeros).
+// integer difference is exact. For small x the power of two of l leaves the FP32 range (from 2^-73 on) and
+// is applied in two steps; |x| < 2^-126, where h is not normal, counts as zero.
 __device__ __forceinline__ FF split_ff(double x) {
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x)) & 0x7fffffffffffffffull;
-  if (b != 0 && (b >> 52) < 1023 - 73) return to_ff(x);
   const unsigned long long hb = (b + 0x0fffffffull + ((b >> 29) & 1ull)) & ~0x1fffffffull;
   const int ex = int(b >> 52);                                   // biased by 1023
   const uint32_t sign = static_cast<uint32_t>(__double2hiint(x)) & 0x80000000u;
   const long long hf = static_cast<long long>(hb >> 29) - (896ll << 23);
   const uint32_t hbits = hf < 0x00800000ll ? 0u : hf > 0x7f800000ll ? 0x7f800000u : uint32_t(hf);
   const float d = float(int(static_cast<long long>(b) - static_cast<long long>(hb)));
-  const int se = ex - 1023 - 52 + 127;                           // 2^(e - 52)
-  const float l = hbits == 0u ? 0.0f : d * __int_as_float(se << 23);
+  const bool small = ex < 1023 - 32;
+  const int se = min(ex - 1023 - 52 + 127 + (small ? 64 : 0), 254);              // 2^(e - 52), or 2^64 of it
+  const float l = hbits == 0u ? 0.0f : d * __int_as_float(se << 23) * (small ? 5.42101086e-20f : 1.0f);
   return FF{__uint_as_float(hbits | sign), __uint_as_float(__float_as_uint(l) ^ sign)};
 }
 __device__ __forceinline__ FF split_ff_t(double x) { return split_ff(x); }
