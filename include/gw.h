@@ -58,9 +58,16 @@ enum gw_status {
 enum gw_dtype { GW_C128 = 0, GW_C64 = 1, GW_R32 = 2 };
 
 /* Arithmetic of the P and Sigma contractions. GW_FP64: double precision (M must be GW_C128), on
- * the tensor cores from exact digit slices of the operands (7 of 8 bits each, so that no result
- * is further from the exact one than on the FP64 pipe), on the FP64 pipe below 32 transitions
- * and where operands span more than the slices hold. GW_TF32X3 ("FP32-split"): tensor-core products of
+ * the tensor cores from exact digit slices of the operands (7 of 8 bits each), on the FP64 pipe
+ * below 32 transitions and where operands span more than the slices hold. Errors are those of FP64
+ * sums: of the polarization relative to sqrt(P_II P_JJ) (an element that is small because its two
+ * columns of M are large in different rows keeps that error, not one relative to itself), of a pair
+ * coefficient relative to the sum of the magnitudes of its terms. Operands are looked at first, per q:
+ * even ones take the GEMM as it is, uneven ones (columns of M w with few large entries, gaps below
+ * about 0.01 Ha; W^c whose diagonals fall off differently with the frequency) one that takes a quarter
+ * longer, and a column whose largest entry exceeds 1,024 times its mean magnitude, magnitudes outside
+ * 2^+-100, non-finite ones and the like the FP64 pipe, all frequencies of the q at about 40 times the
+ * time for large K. GW_TF32X3 ("FP32-split"): tensor-core products of
  * a two-term TF32 split of each FP32 operand (hi*hi + hi*lo + lo*hi), FP32
  * accumulation drained into FP64 partial sums (M must be GW_C64). GW_BF16X3: the
  * same with a two-term BF16 split. */
@@ -148,11 +155,15 @@ int gw_polarization(int nq, const int64_t* K_host, const int* nb_host,
  *                       less workspace.
  *   b_stages            split-precision paths: shared-memory stages of the B operand, 4 or 6
  *                       (two rounds more in flight, less L1 for the A loads); 0 means 4.
- *   fp64_waves          GW_FP64: the K splits fill at least this many waves of CTAs; 0 means 4.
+ *   fp64_waves          GW_FP64, the FP64 pipe's part (q points of fewer than 32 transitions, of
+ *                       operands that the digit slices do not hold, or without workspace for them):
+ *                       the K splits fill at least this many waves of CTAs; 0 means 4.
  *   herk_events         NULL, or n_herk_events pairs of cudaEvent_t (created by the caller,
  *                       layout [start, end] per pair): the call records the pair around each
  *                       of its first n_herk_events HERK launches, on the stream the HERK runs
- *                       on (the dominant kernel alone, without the per-q preparation);
+ *                       on (the dominant kernel alone, without the per-q preparation); for
+ *                       GW_FP64 a launch is one pass of the digit slices' GEMM over a group of
+ *                       q points, a range of their transitions and of the frequencies;
  *   n_herk_events       the number of pairs in herk_events;
  *   herk_launches_out   NULL, or (host) the number of HERK launches of the call;
  *   serial_prep         split-precision paths with more than one group: nonzero runs each
@@ -254,14 +265,16 @@ int gw_plan_waves(int nq, const int64_t* K_host, const int* nb_host, int nw, int
  * a3. Dielectric matrix and correlation part of the screened interaction in the
  * Coulomb eigenbasis (Eqs. dielec_MB, screen_MB and W^c = W - v, Sec. III.C):
  *   eps = 1 - v^1/2 P v^1/2,   W^c = v^1/2 (eps^{-1} - 1) v^1/2,
- * computed to FP64 accuracy from the Cholesky factor of eps (HPD on the imaginary axis).
+ * computed to FP64 accuracy (errors relative to sqrt(eps^-1_II eps^-1_JJ), whatever the scales of the
+ * diagonal of eps) from the Cholesky factor of eps (HPD on the imaginary axis).
  *   v_dev[q]  [N_b] double > 0 Coulomb eigenvalues,
  *   P_dev[q]  [nw][N_b][N_b] complex128 (Hermitian NSD),
  *   Wc_dev[q] [nw][N_b][N_b] complex128 output (may alias P_dev[q]).
  * The factorisation runs over many CTAs (per 32-wide panel: the diagonal block with its inverse,
  * the panel below it, the update) and the inverse factor by block columns, in float-float. From
  * N_b = 257 on (449 in gw_screened_w_real) the products over 128-wide blocks, the inverse factor
- * beyond its diagonal blocks and W^c run on the tensor cores, from 7 slices of 8 bits per operand.
+ * beyond its diagonal blocks and W^c run on the tensor cores, from 7 slices of 8 bits per operand. An
+ * eps that is not positive definite is found on either path.
  * A failed factorisation (eps not positive definite, or non-finite entries) is reported by
  * gw_check as GW_ENOTHPD (GW_ENONFINITE); the later phases still run on the half-finished
  * factor, so Wc_dev (and P_dev where it aliases Wc_dev) is undefined after such an error.
@@ -277,7 +290,7 @@ int gw_screened_w(int nq, const int* nb_host, int nw, const double* const* v_dev
 
 /* The same for real symmetric P (inversion-symmetric systems, e.g. the GW_R32 polarization;
  * Sec. II: with inversion symmetry the basis and the wave functions can be chosen real): the
- * Cholesky factor and the inverse are real (a quarter of the FP64 work), the imaginary parts of
+ * Cholesky factor and the inverse are real (a quarter of the multiplications), the imaginary parts of
  * P_dev are not read (taken as zero), W^c is written with zero imaginary parts. Same layouts
  * and errors as gw_screened_w. Workspace: gw_screened_w_real_workspace() bytes: per system
  * 8 (2 N_b^2 + 1024 ceil(N_b / 32)) bytes rounded up to 256, and the slices of large systems (or

@@ -1,7 +1,7 @@
 // a3: dielectric matrix and W^c in FP64 (Eqs. dielec_MB, screen_MB; W^c = W - v).
 //
 //   eps = 1 - v^1/2 P v^1/2      (Hermitian positive definite on the imaginary axis)
-//   eps = L L^H                   blocked right-looking Cholesky
+//   eps = L L^H                   blocked Cholesky
 //   Z   = L^{-1}                  blocked triangular inversion
 //   W^c = v^1/2 (Z^H Z - 1) v^1/2
 //
@@ -611,11 +611,13 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T>
 }
 
 // ---- the factorisation over many CTAs (the caller-workspace entry points) -----------------
-// A right-looking blocked Cholesky with one launch per step and panel kt: the diagonal block
-// (one CTA per system), the panel below it (one CTA per system and 256 rows, one row per
-// thread), the trailing update of the lower tiles (one CTA per system and 32 x 32 tile). Every
-// SM takes part however few systems there are (20 systems of N_b = 4096 would leave 132 of
-// 152 SMs idle with one CTA per system).
+// One launch per step and 32-wide panel kt: the diagonal block with its inverse (one CTA per system),
+// the panel below it (one CTA per system and 32 rows, a tile product with that inverse), the update of
+// the lower tiles (one CTA per system and 32 x 32 tile): of all tiles behind the panel (right-looking)
+// in small systems, of those inside the current 128 columns in large ones, whose panels of 128 first
+// take one product with all columns before them (left-looking, DzChunk below). Every SM takes part
+// however few systems there are (20 systems of N_b = 4096 would leave 132 of 152 SMs idle with
+// one CTA per system).
 
 // the lower triangle of eps = 1 - v^1/2 P v^1/2 (what the factorisation reads), with the whole of P
 // checked for non-finite values: grid (32-row blocks, system). Three FP64 multiplications per
@@ -830,8 +832,8 @@ static int launch_cholesky_grid(const DieBatchT<T>& batch, int nsys, int ntmax, 
 // ---- large systems: the products on the tensor cores ------------------------------------------
 // The float-float tile products take 52 FP32 operations per complex multiply-add and keep the FP32
 // pipe 80 % busy. For larger systems the products run as digit-slice products of 128 x 128 tiles on
-// the tensor cores instead (fp64_slices.cuh, k_oz_gemm_cplx: 56-bit digits, more than the 48 of
-// the float-float storage): the float-float operands are cut into slices, a launch forms the products
+// the tensor cores instead (fp64_slices.cuh, k_oz_gemm_cplx: 56 bits below the bound of a row or
+// column, against the 48 of the float-float storage below the entry itself): the float-float operands are cut into slices, a launch forms the products
 // C1, C2, S of all systems' tiles, and k_dz_combine turns them into W^c or float-float blocks.
 
 // What to slice: blocks of 128 lines (columns of M, or rows with DZ_ROWS) and stages of 32 values
@@ -1058,10 +1060,14 @@ __global__ void __launch_bounds__(256) k_dz_combine(const __grid_constant__ DzCo
 }
 
 // Systems that take this path, and the slice workspace of one of them. Chunks of systems share a
-// launch while their slices stay within DZ_BUDGET. Float-float tiles against slices, whole solve:
-// complex N = 200 (20 systems) 0.93 / 1.00 ms, 300 (30) 2.07 / 1.97, 450 (32) 5.54 / 3.33, 600 (128)
-// 30.3 / 12.3, 2048 (2) 39.8 / 9.9; real N = 333 (32) 1.16 / 1.38, 600 (128) 9.72 / 5.63, 1100 (3)
-// 5.6 / 3.5 (a real product is a third of a complex one, but its slicing costs half).
+// launch while their slices stay within DZ_BUDGET. The lines lie where the slices win for many systems
+// and lose little for few. Float-float tiles / slices, whole solve of 8, 32 and 128 systems in ms:
+//   complex  257: 1.31 / 1.42, 1.73 / 1.99, 4.20 / 3.87    300: 1.58 / 1.58, 2.26 / 2.19, 5.49 / 4.34
+//            449: 3.02 / 2.28, 5.43 / 3.61, 15.1 / 8.4     600: 4.68 / 3.20, 9.71 / 5.42, 29.6 / 13.6
+//            2048 (2 systems): 39.9 / 10.9
+//   real     400: 1.16 / 1.40, 1.55 / 1.82, 3.75 / 3.55    449: 1.43 / 1.56, 2.01 / 2.02, 5.04 / 3.99
+//            600: 2.18 / 2.14, 3.37 / 2.95, 9.31 / 6.29    2048 (2 systems): 16.7 / 7.4
+// (a real product is a third of a complex one, but its slicing costs half).
 constexpr int DZ_MIN_N = 257, DZ_MIN_N_REAL = 449;
 constexpr size_t DZ_BUDGET = size_t(6) << 30;
 struct DzPlan {

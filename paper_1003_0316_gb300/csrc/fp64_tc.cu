@@ -13,8 +13,10 @@
 //     accumulators of the tensor core while pairs x K x 2^14 <= 2^24: 32, 16, 8 and 8 stages of
 //     K = 32 between drains (g = 5 is drained every 2, see below);
 //   g = 6, 7, 8 (18 pairs, "low") together in one accumulator, 2^-32 below the leading group: their
-//     truncating FP32 chain stays near 2^-50 of the result, where FP64 sums round as well.
-//     The complex products of the dielectric sum g = 6 by itself (exactly) and take g = 9 as well:
+//     truncating FP32 chain stays near 2^-50 of the product of the two bounds, where FP64 sums of evenly
+//     distributed entries round as well. Uneven ones lie below their bounds and would lose: for them
+//     the kernels ..6 sum g = 6 by itself (exactly) and take g = 9 as well (a quarter more time).
+//     The complex products of the dielectric always do:
 //     the entries of a Cholesky factor are far below the bound of their row, and both the truncation
 //     and what is left out count against that bound, K^1/2 times. 4,096 basis functions, eigenvalues
 //     of eps over six decades, error of eps^-1: 7.1e-9 without the exact g = 6, 3.7e-9 without g = 9,
@@ -28,12 +30,16 @@
 // 7.2 ms (41 TFLOP/s FP64-equivalent): k_oz_gemm 5.8 ms, slices 1.05, scales 0.25; relative error of
 // P against 64-bit sums 1.1e-15 -> 5e-16. K = 896, N_b = 64, 8 frequencies 3.7 -> 0.14 ms. The MMAs
 // take about 85 cycles instead of 64 (both operands from shared memory) and set the pace. Pair
-// coefficients of 6,656 pairs, N_b = 600, 16 frequencies: 262 -> 5.9 ms (k_oz_gemm 5.5 ms).
+// coefficients of 6,656 pairs, N_b = 600, 16 frequencies: 262 -> 5.8 ms (k_oz_gemm 5.5 ms).
 //
 // What an input may contain: the scale kernels see every operand first. A non-finite value, one
-// outside [2^-100, 2^100], or a column whose largest entry exceeds 1024 times its mean magnitude
-// (where fixed-point slices would lose what FP64 keeps) sets a device flag: the sliced kernels
-// then return at once and the FP64 kernel, launched behind them and otherwise empty, does the work.
+// outside [2^-100, 2^100], weights outside the FP32 range that count, a column of the polarization whose
+// largest entry exceeds 1024 times its mean magnitude, or a pair whose digits would be off by more than
+// FP64 sums (k_oz_pair_guard) set a bit of a device flag: the sliced kernels then return at once and
+// the FP64 kernel, launched behind them and otherwise empty, does the work. A second bit sends uneven
+// operands (k_oz_exps, k_oz_pair_guard) to the GEMM with the exact g = 6. The polarization's guards
+// look at columns one by one: its errors are those of FP64 sums relative to sqrt(P_II P_JJ), not to
+// an element that is small because its columns are large in different rows.
 //
 // Layout and roles of k_oz_gemm_* (384 threads, one persistent CTA per SM): 128 x 128 tiles; per stage
 // (K = 32) 7 slices of A and of B, pre-split in global memory as 8 KB K-major, 64-byte-swizzled

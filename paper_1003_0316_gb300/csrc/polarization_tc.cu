@@ -1054,7 +1054,8 @@ __global__ void k_prep_xpad(const float* __restrict__ x, int64_t nrow, int ncol,
 // of R = Re W^c for real projections (REAL): U_kk = R_kk, U_kc = R_kc + R_ck for k < c, 0 below
 // the diagonal, so that x U x^T = x R x^T for every real row x (the form sees only the
 // symmetric part of R) with about half the products. Split and swizzled like the
-// polarization's B tiles, [c block][k chunk]; chunks below the diagonal block are zero.
+// polarization's B tiles, [c block][k chunk]; chunks below the diagonal block are not written (no
+// item of the column block reads them).
 template <bool BF16, bool REAL>
 __global__ void __launch_bounds__(128) k_prep_quad(const double2* __restrict__ W0, int nb,
                                                    int64_t nch, char* __restrict__ bsp0,
