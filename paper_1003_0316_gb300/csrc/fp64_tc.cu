@@ -898,6 +898,7 @@ __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
   const int64_t total = int64_t(ntype) * ncolp * nsb;
   const int cps = sbst * OKS / CHROWS;              // chunks per superblock
   const int nch = int((K + CHROWS - 1) / CHROWS);
+  float top_a = 0.f, top_b = 0.f;
   for (int64_t e = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; e < total;
        e += int64_t(gridDim.x) * blockDim.x) {
     const int col = int(e % ncolp), type = int(e / ncolp % ntype), sb = int(e / ncolp / ntype);
@@ -913,14 +914,19 @@ __global__ void k_oz_exps(const __grid_constant__ OzBatch batch) {
     float sp = 0.f;
     const int E = range_exponent(mx, sum, rows, true, L.flag, &sp);
     sp *= rsqrtf(sqrtf(rows));
-    const unsigned act = __activemask(), kind = __match_any_sync(act, int(type < 2));
-    const int top = __reduce_max_sync(kind, __float_as_int(sp));
-    if ((threadIdx.x & 31) == __ffs(kind) - 1) atomicMax(L.spread + (type < 2), top);
+    (type < 2 ? top_b : top_a) = fmaxf(type < 2 ? top_b : top_a, sp);
     const int cb = col / OT, n = col % OT;
     if (type < 2)
       EB[(size_t(type * nbb + cb) * nsb + sb) * OT + n] = E;
     else
       EA[(size_t((type - 2) / 2 * 2 * nbb + (type & 1) * nbb + cb) * nsb + sb) * OT + n] = E;
+  }
+  __syncwarp();
+  const int a = __reduce_max_sync(0xffffffffu, __float_as_int(top_a));      // (positive: ordered as integers)
+  const int b = __reduce_max_sync(0xffffffffu, __float_as_int(top_b));
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(L.spread, a);
+    atomicMax(L.spread + 1, b);
   }
 }
 
