@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(DTHREADS) k_dielectric_zcol(const DieBatchT<T>
 
 // ---- the factorisation over many CTAs (the caller-workspace entry points) -----------------
 // One launch per step and 32-wide panel kt: the diagonal block with its inverse (one CTA per system),
-// the panel below it (one CTA per system and 32 rows, a tile product with that inverse), the update of
+// the panel below it (one CTA per system and 32 rows, a triangular solve in steps of 8 columns), the update of
 // the lower tiles (one CTA per system and 32 x 32 tile): of all tiles behind the panel (right-looking)
 // in small systems, of those inside the current 128 columns in large ones, whose panels of 128 first
 // take one product with all columns before them (left-looking, DzChunk below). Every SM takes part
@@ -723,16 +723,24 @@ __global__ void __launch_bounds__(DTHREADS) k_chol_diag(const DieBatchT<T> batch
   if (tid == 0 && fail) raise_status(status, ST_ENOTHPD);
 }
 
-// step 2: the panel X = A_ik L_kk^{-H} = A_ik D_kt^H below the diagonal block, in float-float; one
-// CTA per (32-row block, system): 1.3 ms for the 18 panels of 128 systems of N_b = 600. (A row per
-// thread solving against L_kk took 4.1 ms, one dependent chain of 26,000 FP32 operations per row.)
+// step 2: the panel X L_kk^H = A_ik below the diagonal block, in float-float; one CTA per (32-row
+// block, system). A triangular solve in steps of PB = 8 columns, X_s = (A_s - sum_{t<s} X_t L_st^H)
+// D_ss^H with the inverse of the 8 x 8 diagonal block of L (a block of D_kt: the inverse of a lower
+// triangle has its blocks' inverses on the diagonal). One thread per row and column of a step, so a row
+// stays in a quarter of a warp. Errors grow with the condition of the 8 x 8 blocks: with one product
+// by the whole D_kt they grew with that of the 32 x 32 block (N_b = 64, condition of
+// eps 1e6 / 1e9, mean over 24 matrices: W^c 1.5e-9 / 1.3e-6 off; 9.6e-10 / 7.2e-7 here, 1.0e-9 / 7.7e-7
+// by substitution). 128 systems of N_b = 600, 18 panels: 0.91 ms (1.31 with the one product; a row
+// per thread substituting one column after the other 4.1).
+constexpr int PB = 8;
+static_assert(DTHREADS == DB * PB && 32 % PB == 0, "a thread per row and column of a step");
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS) k_chol_panel(const DieBatchT<T> batch, int kt) {
   using FT = typename FFOf<T>::tile;
   using FA = typename FFOf<T>::acc;
   extern __shared__ __align__(16) unsigned char dsm_raw[];
-  FT* SA = reinterpret_cast<FT*>(dsm_raw);
-  FT* SB = SA + DB * DLD;
+  FT* SA = reinterpret_cast<FT*>(dsm_raw);   // A, then X
+  FT* SL = SA + DB * DLD;                    // L_kk below the diagonal blocks, D_ss in them
   const DieSysT<T>& sys = batch.s[blockIdx.y];
   const int n = sys.n, nt = (n + DB - 1) / DB;
   const int it = kt + 1 + blockIdx.x;
@@ -741,16 +749,32 @@ __global__ void __launch_bounds__(DTHREADS) k_chol_panel(const DieBatchT<T> batc
   FT* E = stor(sys.E);
   load_tile_s(SA, E, n, n, n, it * DB, k0, 0);
   const FT* Dr = stor(sys.D) + size_t(kt) * DB * DB;
-  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS)       // SB[k][c] = conj(D[c][k])
-    SB[(e % DB) * DLD + e / DB] = ff_conj(Dr[e]);
+  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS) {
+    const int r = e / DB, c = e % DB;
+    SL[r * DLD + c] = r / PB == c / PB ? Dr[e] : c < r ? E[size_t(k0 + r) * n + k0 + c] : FT{};
+  }
   __syncthreads();
-  const int tr = threadIdx.x >> 3, tc = threadIdx.x & 7;
-  FA acc[4] = {};
-  tile_mac_ff<false>(acc, SA, SB, tr, tc);
-  const int R = it * DB + tr;
-  if (R < n) {
+  const int tr = threadIdx.x / PB, tc = threadIdx.x % PB;
+  FT* row = SA + tr * DLD;
+#pragma unroll 1
+  for (int s = 0; s < DB; s += PB) {
+    const FT* lc = SL + (s + tc) * DLD;
+    FA acc = ff_acc(row[s + tc]);
+#pragma unroll 4
+    for (int k = 0; k < s; ++k) ff_csubmul_conj(acc, row[k], lc[k]);
+    row[s + tc] = ff_renorm_t(acc);
+    __syncwarp();
+    acc = FA{};
 #pragma unroll
-    for (int b = 0; b < 4; ++b) E[size_t(R) * n + k0 + tc + 8 * b] = ff_renorm_t(acc[b]);
+    for (int k = 0; k < PB; ++k) ff_cmac(acc, row[s + k], ff_conj(lc[s + k]));    // D_ss is lower: zeros beyond
+    __syncwarp();
+    row[s + tc] = ff_renorm_t(acc);
+    __syncwarp();
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < DB * DB; e += DTHREADS) {
+    const int r = e / DB, c = e % DB;
+    if (it * DB + r < n) E[size_t(it * DB + r) * n + k0 + c] = SA[r * DLD + c];
   }
 }
 
