@@ -1086,11 +1086,11 @@ __global__ void __launch_bounds__(256) k_dz_combine(const __grid_constant__ DzCo
 // Systems that take this path, and the slice workspace of one of them. Chunks of systems share a
 // launch while their slices stay within DZ_BUDGET. The lines lie where the slices win for many systems
 // and lose little for few. Float-float tiles / slices, whole solve of 8, 32 and 128 systems in ms:
-//   complex  257: 1.31 / 1.42, 1.73 / 1.99, 4.20 / 3.87    300: 1.58 / 1.58, 2.26 / 2.19, 5.49 / 4.34
-//            449: 3.02 / 2.28, 5.43 / 3.61, 15.1 / 8.4     600: 4.68 / 3.20, 9.71 / 5.42, 29.6 / 13.6
-//            2048 (2 systems): 39.9 / 10.9
-//   real     400: 1.16 / 1.40, 1.55 / 1.82, 3.75 / 3.55    449: 1.43 / 1.56, 2.01 / 2.02, 5.04 / 3.99
-//            600: 2.18 / 2.14, 3.37 / 2.95, 9.31 / 6.29    2048 (2 systems): 16.7 / 7.4
+//   complex  257: 1.28 / 1.37, 1.69 / 1.94, 4.07 / 3.74    300: 1.54 / 1.53, 2.20 / 2.13, 5.32 / 4.18
+//            449: 2.98 / 2.22, 5.33 / 3.47, 14.7 / 8.0     600: 4.62 / 3.11, 9.53 / 5.22, 29.1 / 13.1
+//            2048 (2 systems): 40.1 / 10.6
+//   real     400: 1.14 / 1.38, 1.54 / 1.80, 3.69 / 3.50    449: 1.41 / 1.53, 1.98 / 1.99, 4.95 / 3.89
+//            600: 2.14 / 2.11, 3.34 / 2.91, 9.16 / 6.13    2048 (2 systems): 16.5 / 7.4
 // (a real product is a third of a complex one, but its slicing costs half).
 constexpr int DZ_MIN_N = 257, DZ_MIN_N_REAL = 449;
 constexpr size_t DZ_BUDGET = size_t(6) << 30;
